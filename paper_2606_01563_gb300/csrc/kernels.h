@@ -76,19 +76,22 @@ struct EvictArgs {
   int32_t budget;
   float tau;
   void* ws;
-  float* scratch;  // [units][G][cap] logits (single-CTA kernel)
-  void* stage;     // [units][cap] rows staged by the cluster kernel's compaction
+  float* scratch;  // [units][cap][G] softmax terms that shared memory does not hold (large kernel)
+  void* stage;     // [units][cap] rows staged by the compaction
+  float* Yw;       // [units][cap][D] y rows that shared memory does not hold (large kernel)
   float* Y;          // optional fp32 [units][cap][D]: y_j = S_tilde k_j of each row (mkv_cache.y)
   int32_t* y_len;    // optional [units]: rows 0..y_len-1 of Y are current (mkv_cache.y_len)
-  int32_t rows_max;  // cluster kernel: rows per CTA slice = ceil(cap / CTAs per unit)
-  int32_t kv_smem;   // cluster kernel: the slice's K/V rows are cached in shared memory
+  int32_t rows_max;  // rows per CTA slice = ceil(cap / CTAs per unit)
+  int32_t kv_smem;   // register kernel: the slice's K/V rows are cached in shared memory
   int32_t batch;
   int32_t n_kv;
 };
 
+size_t evict_large_y_bytes(const mkv_geom& g, int32_t capacity);
 size_t evict_workspace_bytes(const mkv_geom& g, int32_t capacity);
 void evict_carve(EvictArgs& a, const mkv_geom& g, int32_t capacity, void* ws);
 cudaError_t launch_evict(const EvictArgs& a, int head_dim, int group, cudaStream_t stream);
+cudaError_t launch_evict_large(const EvictArgs& a, int head_dim, int group, cudaStream_t stream);
 
 // ---------------------------------------------------------------- compress
 struct CompressArgs {

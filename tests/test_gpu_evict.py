@@ -155,6 +155,25 @@ def test_evict_slice_sizes(cap):
     check(gpu, st)
 
 
+@pytest.mark.parametrize("units,G,D,cap,evict,tau", [
+    (2, 4, 128, 1153, 3, 1e-6),   # the smallest capacity past the register kernel: all state in shared memory
+    (8, 4, 128, 2500, 3, 1e-6),   # K/V rows stay in the cache
+    (9, 2, 128, 3300, 2, 1e-6),   # 8-CTA clusters: y rows in the workspace
+    (9, 8, 64, 12500, 2, 1e-6),   # softmax terms in the workspace too
+    (1, 1, 64, 1201, 3, 0.05),    # a few clamped entries or the direct clamped product, slices of 76 rows
+    (2, 1, 128, 1300, 2, 0.5),    # the direct clamped product
+])
+def test_evict_large_slices(units, G, D, cap, evict, tau):
+    """Capacities above 1152 rows, at the sizes where the rows' state moves
+    from shared memory to the workspace and where the cluster size changes;
+    ragged lengths, a unit with no evicted token, appended tokens."""
+    rng = np.random.default_rng(61 + cap)
+    lens = [cap - 1 - 7 * (i % 3) for i in range(units)]
+    st = setup(rng, 1, units, G, D, lens, cap, [0 if i == 1 else 300 for i in range(units)])
+    gpu = run_case(st, 1, units, G, D, cap - 14 - evict, True, tau=tau)
+    check(gpu, st)
+
+
 def test_evict_many_units():
     """24 units at capacity 200: three waves of 8-CTA clusters of the register
     kernel (5 rows per warp)."""
