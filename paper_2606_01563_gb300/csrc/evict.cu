@@ -13,11 +13,16 @@
 // their products out of y_j; above kMaxClamp such entries that iteration
 // computes C' k_j directly.
 //
-// Two kernels, chosen by the capacity: evict_reg_kernel here (row slices of up
-// to 144 rows, capacity 1152), and evict_large_kernel (evict_large.cu).
+// Two kernels, chosen by the capacity: evict_reg_kernel here (up to kRegCap =
+// 1152 rows, the capacity up to which y rows are kept across calls), and
+// evict_large_kernel (evict_large.cu).
 #include <cooperative_groups.h>
 
+#include <algorithm>
+#include <mutex>
+
 #include "evict_common.cuh"
+#include "warp_mma.cuh"
 
 namespace cg = cooperative_groups;
 
@@ -25,148 +30,150 @@ namespace mkv {
 
 namespace {
 
-constexpr int kCL = 8;           // CTAs per unit (one cluster)
-constexpr int kLPR = 8;          // lanes per row in the set-up passes
-constexpr int kTWR = 8;          // warps that run the 32x32 tile transposes
-// dynamic shared memory available next to the kernel's static arrays
-constexpr size_t kSmemBudget = 192 * 1024;
-
 // ---------------------------------------------------------------------------
-// Register-resident cluster kernel, used while a row slice has at most
-// kRW * RPW rows.  8 CTAs of 512 threads per unit (one cluster); warp w of a
-// CTA owns the slice rows w, w + 16, ... and lane l owns the dims
-// [l*DPL, (l+1)*DPL) of each.  State in the raw co-moment form S_tilde = n C:
-// y_j = S_tilde k_j of the warp's rows stays in registers, and so does a
-// 1/512 share of S_tilde (rows a of the lane's dims, columns c = w + 16 i),
-// which every iteration folds and scans for the clamp list.  Set-up: each CTA
-// takes the logits and softmax (max, sum) of its own rows, and one cluster
-// exchange gives the unit's maximum and normaliser.  Every thread computes the
-// Welford fold of its own dims from the evicted row, so the only barriers of
-// an iteration are one block barrier (the block's minimum key) and one
-// cluster barrier (every CTA's key, candidate row and its softmax terms,
-// written into every CTA's mailbox beforehand).  Scores are computed assuming
-// an empty clamp list; when the list is not empty they are recomputed with it.
+// Register kernel: a cluster of 8, 4 or 2 CTAs of 512 threads per unit, each
+// with a contiguous slice of at most 16 RPW rows.  Warp w owns the slice rows
+// w, w + 16, ... and lane l the dims [l*DPL, (l+1)*DPL) of each, with
+// y_j = S_tilde k_j (raw co-moment form, S_tilde = n C) in registers.  The CTAs
+// share out S_tilde itself by rows, in shared memory: a fold costs a warp one
+// row or a few, and every CTA lists the clamped entries of its own rows.
+// Every thread computes the Welford fold of its own dims from the evicted row,
+// so the only barriers of an iteration are one block barrier (the block's
+// minimum key) and one cluster barrier (every CTA's key, candidate row, its
+// softmax terms and its count of clamped entries, written into every CTA's
+// mailbox beforehand).  Scores assume that no entry is clamped; when a mailbox
+// says otherwise, the lists are exchanged and the rows scored again.
+//
+// What bounds it: a chain of dependent steps, not memory: about 2 us per
+// eviction and a fixed part of a few round trips (length, rows and moments,
+// one cluster exchange of the softmax maxima and sums, rows out).  Logits and
+// S_tilde k of rows without a kept y run on the tensor cores from the rows in
+// shared memory; survivors are written straight from there to their compacted
+// places (every CTA has seen every evicted row, so no count is exchanged).
+constexpr int kRegCap = 1152;  // largest capacity of this kernel
 constexpr int kRT = 512;       // threads per CTA
 constexpr int kRW = kRT / 32;  // warps per CTA
+constexpr int kMaxCL = 8;      // CTAs per unit at most
+constexpr int kBlk = 32;       // rows per block of the set-up products
 
-template <int D, int G>
+template <int D, int G, int RPW>
 struct RegLayout {
-  size_t Ct, lg, Ks, Vs, alive, total;
-  __host__ __device__ RegLayout(int R, int cap, int kv) {
-    size_t off = 0;
-    Ct = off; off += (size_t)D * D * 4;
-    lg = off; off += align_up((size_t)G * R * 4, 16);
-    Ks = off; off += kv ? (size_t)R * D * 2 : 0;
-    Vs = off; off += kv ? (size_t)R * D * 2 : 0;
-    alive = off; off += align_up((size_t)cap, 16);
-    total = off;
-  }
+  static constexpr int R = kRW * RPW;  // rows of a slice at most
+  static constexpr int LDK = D + 8;    // row stride of K: conflict-free matrix loads
+  static constexpr int LDY = D + 4;    // row stride of a block of set-up products
+  static constexpr size_t K = 0, V = K + (size_t)R * LDK * 2, lg = V + (size_t)R * D * 2,
+                          pos = lg + (size_t)G * R * 4, yb = pos + (size_t)R * 4, S = yb + (size_t)kBlk * LDY * 4;
+  static __host__ __device__ size_t total(int cl) { return S + (size_t)(D / cl) * D * 4; }
 };
 
 template <int D, int G, int RPW>
-__global__ void __cluster_dims__(kCL, 1, 1) __launch_bounds__(kRT, 1)
-    evict_reg_kernel(const EvictArgs a) {
-  constexpr int NC = D / 32;   // float4 chunks per row for 8-lane row groups (set-up)
+__global__ void __launch_bounds__(kRT, 1) evict_reg_kernel(const EvictArgs a) {
+  using L = RegLayout<D, G, RPW>;
   constexpr int DPL = D / 32;  // dims per lane
-  constexpr int CJ = D / kRW;  // C columns per thread
-  constexpr int kRP = kRW * (32 / kLPR);  // rows per pass of 8-lane groups
+  constexpr int KS = D / 16, NT = D / 8, CH = D / 8;
+  constexpr int P = RPW <= 8 ? 8 : 16;  // padded row count of the transposing sums
+  constexpr int SH = P == 8 ? 2 : 1;    // lane l scores row l >> SH
   extern __shared__ __align__(16) uint8_t dsmem[];
-  const int R = a.rows_max;
-  const RegLayout<D, G> lay(R, a.cap, a.kv_smem);
-  float* Ct = reinterpret_cast<float*>(dsmem + lay.Ct);  // Ct[c*D + a] = C[a][c] (set-up, direct mode, write-back)
-  float* lg = reinterpret_cast<float*>(dsmem + lay.lg);  // [G][R] e_hj of this CTA's rows
-  uint8_t* alive_all = dsmem + lay.alive;
-  __shared__ __align__(16) float s_mu_k[D];
-  __shared__ __align__(16) float s_mu_v[D];
-  __shared__ __align__(16) float s_q[G][D];
-  __shared__ float s_red[kRW][G];
-  __shared__ float s_zpart[kRW][G];
-  __shared__ float s_M[G];        // this CTA's largest logit per head (read remotely), then the unit's
-  __shared__ float s_Z[G];        // this CTA's sum of exp(l - s_M) per head (read remotely)
-  __shared__ float mail_e[2][kCL][G];  // e_h of each CTA's candidate row
+  __nv_bfloat16* Ks = reinterpret_cast<__nv_bfloat16*>(dsmem + L::K);  // [R][LDK]
+  __nv_bfloat16* Vs = reinterpret_cast<__nv_bfloat16*>(dsmem + L::V);  // [R][D]
+  float* lg = reinterpret_cast<float*>(dsmem + L::lg);                 // [G][R] logits, then e_hj
+  int32_t* s_pos = reinterpret_cast<int32_t*>(dsmem + L::pos);
+  float* yb = reinterpret_cast<float*>(dsmem + L::yb);  // [kBlk][LDY]
+  float* S = reinterpret_cast<float*>(dsmem + L::S);    // [D / CL][D] this CTA's rows of S_tilde
+  __shared__ __align__(16) __nv_bfloat16 s_q[8][L::LDK];  // heads past G are zero
+  __shared__ float s_mw[kRW][8], s_zw[kRW][8];          // (max, sum) of each warp's rows
+  __shared__ float mail_m[kMaxCL][G], mail_z[kMaxCL][G];  // every CTA's (max, sum)
+  __shared__ float mail_e[2][kMaxCL][G];                  // e_h of each CTA's candidate row
   __shared__ unsigned long long s_best[2];
-  __shared__ unsigned long long mail_key[2][kCL];
-  __shared__ __align__(16) __nv_bfloat16 mail_row[2][kCL][2 * D];
-  __shared__ int ex_cnt;
-  __shared__ uint32_t s_zidx[kMaxClamp];
-  __shared__ float s_zval[kMaxClamp];
+  __shared__ unsigned long long mail_key[2][kMaxCL];
+  __shared__ int mail_nz[2][kMaxCL];
+  __shared__ __align__(16) __nv_bfloat16 mail_row[2][kMaxCL][2 * D];
+  __shared__ uint32_t s_zidx[kMaxClamp], s_gidx[kMaxClamp];  // this CTA's clamped entries, the unit's
+  __shared__ float s_zval[kMaxClamp], s_gval[kMaxClamp];
   __shared__ int s_nz;
-  __shared__ float s_tile[kTWR][32 * 33];
+  __shared__ uint32_t s_mask[kRW];  // survivors of each warp
 
+  // The next kernel in the stream may be placed on free SMs while this one
+  // runs (it waits for this one's end); not before this one's own wait.
+  grid_dependency_wait();
+  grid_launch_dependents();
   cg::cluster_group cluster = cg::this_cluster();
-  const int rank = static_cast<int>(cluster.block_rank());
-  const int u = blockIdx.x / kCL;
+  const int rank = static_cast<int>(cluster.block_rank()), CL = static_cast<int>(cluster.num_blocks());
+  const int u = blockIdx.x / CL;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const int q = lane & 7;
-  const int rsub = warp * (32 / kLPR) + (lane >> 3);
   const size_t row0 = (size_t)u * a.cap;
   __nv_bfloat16* Kg = reinterpret_cast<__nv_bfloat16*>(a.K) + row0 * D;
   __nv_bfloat16* Vg = reinterpret_cast<__nv_bfloat16*>(a.V) + row0 * D;
   int32_t* Pg = a.pos + row0;
-  const int len_in = a.len[u];
-  const int seen_in = a.seen[u];
+  const int len_in = a.len[u], seen_in = a.seen[u];
+  int n = a.n[u];
+  const bool has_y = a.Y != nullptr && a.y_len != nullptr;
+  const int y_len_in = has_y ? a.y_len[u] : 0;
   const bool has_new = a.k_new != nullptr;
   if (len_in < 0 || len_in > a.cap || (has_new && len_in + 1 > a.cap)) {
     if (rank == 0 && tid == 0) record_error(a.ws, MKV_ERR_CAPACITY, u);
     return;  // uniform over the cluster
   }
   const int len = len_in + (has_new ? 1 : 0);
-  // rows 0..y_cur-1 of the cache's y rows are current (none without them)
-  const int y_cur = (a.Y != nullptr && a.y_len != nullptr) ? max(0, min(a.y_len[u], len_in)) : 0;
-  const int rows_per = (len + kCL - 1) / kCL;
+  const int rows_per = (len + CL - 1) / CL;
   const int j0 = min(len, rank * rows_per), j1 = min(len, j0 + rows_per);
   const int nr = j1 - j0;
-  if (has_new && len_in >= j0 && len_in < j1) {  // the owning CTA appends the token
-    const __nv_bfloat16* kn = reinterpret_cast<const __nv_bfloat16*>(a.k_new) + (size_t)u * D;
-    const __nv_bfloat16* vn = reinterpret_cast<const __nv_bfloat16*>(a.v_new) + (size_t)u * D;
+  const int jn = has_new ? len_in - j0 : -1;  // the appended token's slice row, if it is here
+  const __nv_bfloat16* kn = reinterpret_cast<const __nv_bfloat16*>(a.k_new) + (size_t)u * D;
+  const __nv_bfloat16* vn = reinterpret_cast<const __nv_bfloat16*>(a.v_new) + (size_t)u * D;
+  if (jn >= 0 && jn < nr) {  // the owning CTA appends the token
     for (int i = tid; i < D; i += kRT) {
-      Kg[(size_t)len_in * D + i] = kn[i];
-      Vg[(size_t)len_in * D + i] = vn[i];
+      const __nv_bfloat16 k = kn[i], v = vn[i];
+      Kg[(size_t)len_in * D + i] = k;
+      Vg[(size_t)len_in * D + i] = v;
+      Ks[jn * L::LDK + i] = k;
+      Vs[jn * D + i] = v;
     }
-    if (tid == 0) Pg[len_in] = seen_in;
-    __threadfence();
+    if (tid == 0) {
+      Pg[len_in] = seen_in;
+      s_pos[jn] = seen_in;
+    }
   }
-  __syncthreads();
+  cluster_arrive_release();  // every CTA has read the length; awaited before the first remote store
   if (len <= a.budget) {
+    cluster_wait_acquire();
     if (rank == 0 && tid == 0) {
       a.len[u] = len;
       a.seen[u] = seen_in + (has_new ? 1 : 0);
     }
     return;
   }
-  // other CTAs' rows (the appended one included) are read below
-  cluster.sync();
+  // rows 0..y_cur-1 of the cache's y rows are current (none without them)
+  const int y_cur = max(0, min(y_len_in, len_in));
 
-  int n = a.n[u];
-  {
-    float* tb = s_tile[warp % kTWR];
-    for (int t = warp; warp < kTWR && t < (D / 32) * (D / 32); t += kTWR) {
-      const int r0 = (t / (D / 32)) * 32, c0 = (t % (D / 32)) * 32;
-      for (int i = 0; i < 32; ++i)
-        tb[i * 33 + lane] = (n > 0) ? a.C[(size_t)u * D * D + (size_t)(r0 + i) * D + c0 + lane] : 0.f;
-      __syncwarp();
-      for (int i = 0; i < 32; ++i) Ct[(size_t)(c0 + i) * D + r0 + lane] = tb[lane * 33 + i];
-      __syncwarp();
-    }
+  // ---- this slice's rows, the query, this CTA's rows of S_tilde, the means
+  for (int idx = tid; idx < nr * CH; idx += kRT) {
+    const int r = idx / CH, c = idx % CH;
+    if (r == jn) continue;
+    const uint4 k4 = reinterpret_cast<const uint4*>(Kg + (size_t)(j0 + r) * D)[c];
+    const uint4 v4 = reinterpret_cast<const uint4*>(Vg + (size_t)(j0 + r) * D)[c];
+    *reinterpret_cast<uint4*>(Ks + r * L::LDK + c * 8) = k4;
+    *reinterpret_cast<uint4*>(Vs + r * D + c * 8) = v4;
   }
-  for (int i = tid; i < D; i += kRT) {
-    s_mu_k[i] = (n > 0) ? a.mu_k[(size_t)u * D + i] : 0.f;
-    s_mu_v[i] = (n > 0) ? a.mu_v[(size_t)u * D + i] : 0.f;
-  }
-  const float scale = rsqrtf(static_cast<float>(D));
+  for (int r = tid; r < nr; r += kRT)
+    if (r != jn) s_pos[r] = Pg[j0 + r];
   const __nv_bfloat16* qg = reinterpret_cast<const __nv_bfloat16*>(a.q) + (size_t)u * G * D;
-  for (int i = tid; i < G * D; i += kRT) s_q[i / D][i % D] = __bfloat162float(qg[i]) * scale;
-  const __nv_bfloat16* Kr = Kg + (size_t)j0 * D;
-  const __nv_bfloat16* Vr = Vg + (size_t)j0 * D;
-  if (a.kv_smem) {
-    __nv_bfloat16* Ks = reinterpret_cast<__nv_bfloat16*>(dsmem + lay.Ks);
-    __nv_bfloat16* Vs = reinterpret_cast<__nv_bfloat16*>(dsmem + lay.Vs);
-    for (int idx = tid; idx < nr * (D / 8); idx += kRT) {
-      reinterpret_cast<uint4*>(Ks)[idx] = reinterpret_cast<const uint4*>(Kr)[idx];
-      reinterpret_cast<uint4*>(Vs)[idx] = reinterpret_cast<const uint4*>(Vr)[idx];
-    }
-    Kr = Ks;
-    Vr = Vs;
+  for (int i = tid; i < 8 * D; i += kRT)
+    s_q[i / D][i % D] = i / D < G ? qg[i] : __float2bfloat16_rn(0.f);
+  const float nf0 = static_cast<float>(n);
+  const int SR = D / CL, a0 = rank * SR;  // rows [a0, a0 + SR) of S_tilde
+  const float* Cg = a.C + (size_t)u * D * D;
+  for (int idx = tid; idx < SR * (D / 4); idx += kRT) {
+    float4 c4 = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (n > 0) c4 = reinterpret_cast<const float4*>(Cg + (size_t)a0 * D)[idx];
+    reinterpret_cast<float4*>(S)[idx] = make_float4(c4.x * nf0, c4.y * nf0, c4.z * nf0, c4.w * nf0);
+  }
+  float mk[DPL], mv[DPL], sdk[DPL], sdv[DPL];
+#pragma unroll
+  for (int d = 0; d < DPL; ++d) {
+    mk[d] = n > 0 ? a.mu_k[(size_t)u * D + lane * DPL + d] : 0.f;
+    mv[d] = n > 0 ? a.mu_v[(size_t)u * D + lane * DPL + d] : 0.f;
+    sdk[d] = sdv[d] = 0.f;
   }
   if (tid == 0) {
     s_nz = 0;
@@ -174,294 +181,247 @@ __global__ void __cluster_dims__(kCL, 1, 1) __launch_bounds__(kRT, 1)
   }
   __syncthreads();
 
-  // ---- logits of this CTA's rows (8 lanes per row)
-  for (int base = 0; base < nr; base += kRP) {
-    const int j = base + rsub;
-    const bool ok = j < nr;
-    float kf[NC][4];
+  // ---- logits of this CTA's rows: warp w takes rows 16 w .. 16 w + 15 against
+  // the heads as the 8-column side, and their (max, sum of exp) per head
+  const float scale = rsqrtf(static_cast<float>(D));
+  {
+    const int g = lane >> 2, t = lane & 3;
+    float m0 = -INFINITY, m1 = -INFINITY, z0 = 0.f, z1 = 0.f;  // heads 2t, 2t + 1
+    if (warp * 16 < nr) {
+      float c0[4] = {0.f, 0.f, 0.f, 0.f}, c1[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll
-    for (int c = 0; c < NC; ++c) {
-      if (ok) load4_bf16<D>(Kr + (size_t)j * D + chunk_dim<D>(q, c), kf[c]);
-      else kf[c][0] = kf[c][1] = kf[c][2] = kf[c][3] = 0.f;
-    }
-#pragma unroll
-    for (int h = 0; h < G; ++h) {
-      float acc = 0.f;
-#pragma unroll
-      for (int c = 0; c < NC; ++c) {
-        const float4 q4 = *reinterpret_cast<const float4*>(&s_q[h][chunk_dim<D>(q, c)]);
-        acc = fmaf(q4.x, kf[c][0], fmaf(q4.y, kf[c][1], fmaf(q4.z, kf[c][2], fmaf(q4.w, kf[c][3], acc))));
+      for (int kk = 0; kk < KS; ++kk) {
+        uint32_t k4[4];
+        ldsm_x4(k4, Ks + (warp * 16 + (lane & 7) + ((lane >> 3) & 1) * 8) * L::LDK + kk * 16 + (lane >> 4) * 8);
+        const uint32_t b0 = *reinterpret_cast<const uint32_t*>(&s_q[g][kk * 16 + 2 * t]);
+        const uint32_t b1 = *reinterpret_cast<const uint32_t*>(&s_q[g][kk * 16 + 8 + 2 * t]);
+        if (kk & 1) mma_m16n8k16(c1, k4[0], k4[1], k4[2], k4[3], b0, b1);
+        else mma_m16n8k16(c0, k4[0], k4[1], k4[2], k4[3], b0, b1);
       }
-      acc = group_sum(acc);
-      if (ok && q == 0) lg[h * R + j] = acc;
+      const int ra = warp * 16 + g, rb = ra + 8;
+      const float x0 = ra < nr ? (c0[0] + c1[0]) * scale : -INFINITY, x1 = ra < nr ? (c0[1] + c1[1]) * scale : -INFINITY;
+      const float x2 = rb < nr ? (c0[2] + c1[2]) * scale : -INFINITY, x3 = rb < nr ? (c0[3] + c1[3]) * scale : -INFINITY;
+      if (2 * t < G) {
+        if (ra < nr) lg[2 * t * L::R + ra] = x0;
+        if (rb < nr) lg[2 * t * L::R + rb] = x2;
+      }
+      if (2 * t + 1 < G) {
+        if (ra < nr) lg[(2 * t + 1) * L::R + ra] = x1;
+        if (rb < nr) lg[(2 * t + 1) * L::R + rb] = x3;
+      }
+      m0 = fmaxf(x0, x2);
+      m1 = fmaxf(x1, x3);
+#pragma unroll
+      for (int o = 4; o < 32; o <<= 1) {
+        m0 = fmaxf(m0, __shfl_xor_sync(kFull, m0, o));
+        m1 = fmaxf(m1, __shfl_xor_sync(kFull, m1, o));
+      }
+      if (m0 != -INFINITY) z0 = expf(x0 - m0) + expf(x2 - m0);
+      if (m1 != -INFINITY) z1 = expf(x1 - m1) + expf(x3 - m1);
+#pragma unroll
+      for (int o = 4; o < 32; o <<= 1) {
+        z0 += __shfl_xor_sync(kFull, z0, o);
+        z1 += __shfl_xor_sync(kFull, z1, o);
+      }
+    }
+    if (g == 0) {
+      s_mw[warp][2 * t] = m0;
+      s_mw[warp][2 * t + 1] = m1;
+      s_zw[warp][2 * t] = z0;
+      s_zw[warp][2 * t + 1] = z1;
     }
   }
   __syncthreads();
-  // softmax is shift-invariant: e_hj = exp(l_hj - M0_h) with M0_h the
-  // unit's largest logit at the start.  Each CTA takes (max, sum) over its
-  // rows; one cluster exchange gives M0_h and Z_h, and the CTA rescales its
-  // e_hj by exp(m_h - M0_h).
-  {
-    float mx[G];
+  cluster_wait_acquire();  // every CTA of the cluster has started
+  if (tid < CL * G) {      // this CTA's (max, sum) of head h to rank r
+    const int r = tid / G, h = tid % G;
+    float m = -INFINITY, z = 0.f;
 #pragma unroll
-    for (int h = 0; h < G; ++h) mx[h] = -INFINITY;
-    for (int jj = tid; jj < nr; jj += kRT)
+    for (int w = 0; w < kRW; ++w) m = fmaxf(m, s_mw[w][h]);
 #pragma unroll
-      for (int h = 0; h < G; ++h) mx[h] = fmaxf(mx[h], lg[h * R + jj]);
+    for (int w = 0; w < kRW; ++w)
+      if (s_mw[w][h] != -INFINITY) z += s_zw[w][h] * expf(s_mw[w][h] - m);
+    *cluster.map_shared_rank(&mail_m[rank][h], r) = m;
+    *cluster.map_shared_rank(&mail_z[rank][h], r) = z;
+  }
+  cluster_arrive_release();
+
+  // ---- y_j = S_tilde k_j.  Rows below the cache's y_len carry it from the call
+  // that last changed the moments; the others (appended since) are computed
+  // here: n (C k_j) on the tensor cores, C as three bf16 parts (exact to 24
+  // bits), warp w taking 8 value dims, in blocks of 32 rows
+  float y[RPW][DPL];
+  unsigned alive = 0u;
 #pragma unroll
-    for (int h = 0; h < G; ++h) {
-      mx[h] = warp_max(mx[h]);
-      if (lane == 0) s_red[warp][h] = mx[h];
-    }
-    __syncthreads();
-    if (tid < G) {
-      float m = -INFINITY;
-      for (int w = 0; w < kRW; ++w) m = fmaxf(m, s_red[w][tid]);
-      s_M[tid] = m;
-    }
-    __syncthreads();
-    float zs[G];
+  for (int i = 0; i < RPW; ++i) {
+    const int r = warp + kRW * i;
 #pragma unroll
-    for (int h = 0; h < G; ++h) zs[h] = 0.f;
-    for (int jj = tid; jj < nr; jj += kRT)
-#pragma unroll
-      for (int h = 0; h < G; ++h) zs[h] += expf(lg[h * R + jj] - s_M[h]);
-#pragma unroll
-    for (int h = 0; h < G; ++h) {
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) zs[h] += __shfl_xor_sync(kFull, zs[h], o);
-      if (lane == 0) s_zpart[warp][h] = zs[h];
-    }
-    for (int jj = len + tid; jj < a.cap; jj += kRT) alive_all[jj] = 0;
-    __syncthreads();
-    if (tid < G) {
-      float z = 0.f;
-      for (int w = 0; w < kRW; ++w) z += s_zpart[w][tid];
-      s_Z[tid] = z;
+    for (int d = 0; d < DPL; ++d) y[i][d] = 0.f;
+    if (r < nr) {
+      alive |= 1u << i;
+      if (n > 0 && j0 + r < y_cur) ld_vec<DPL>(a.Y + (row0 + j0 + r) * D + lane * DPL, y[i]);
     }
   }
-  cluster.sync();  // every CTA's (max, sum) is published
-  constexpr int P = RPW <= 8 ? 8 : 16;       // padded row count of the transposing sums
-  constexpr int SH = P == 8 ? 2 : 1;         // lane l scores row l >> SH
-  // Z_h lives in lane h < G of every warp as a compensated (Kahan) float,
-  // decremented per eviction: value zf - zc.  Every CTA combines the
-  // published partials in the same order, so all hold identical values.
-  float zf = 1.f, zc = 0.f, zinv = 1.f;
-  {
-    __shared__ float s_Mg[G], s_Zg[G];
-    if (tid < G) {  // thread h: the unit's maximum and normaliser of head h
-      float mr[kCL], m = -INFINITY;
+  if (n > 0 && nr > 0 && j1 > y_cur) {  // uniform over the CTA
+    constexpr int kHalves = kRW / NT;   // warps sharing 8 value dims: 1 at D = 128 (both 16-row halves), 2 at D = 64
+    const int g = lane >> 2, t = lane & 3, nt = warp % NT, half = warp / NT;
+    uint32_t b3[3][KS][2];
 #pragma unroll
-      for (int r = 0; r < kCL; ++r) {
-        mr[r] = cluster.map_shared_rank(s_M, r)[tid];
-        m = fmaxf(m, mr[r]);
+    for (int kk = 0; kk < KS; ++kk)
+#pragma unroll
+      for (int hf = 0; hf < 2; ++hf) {
+        const float2 c2 = *reinterpret_cast<const float2*>(Cg + (size_t)(nt * 8 + g) * D + kk * 16 + hf * 8 + 2 * t);
+        float x = c2.x, w = c2.y;
+#pragma unroll
+        for (int part = 0; part < 3; ++part) {
+          b3[part][kk][hf] = pack_bf16x2(x, w);
+          x = bf16_residual(x);
+          w = bf16_residual(w);
+        }
       }
-      float z = 0.f;
 #pragma unroll
-      for (int r = 0; r < kCL; ++r)
-        if (mr[r] != -INFINITY) z += cluster.map_shared_rank(s_Z, r)[tid] * expf(mr[r] - m);
-      s_Mg[tid] = m;
-      s_Zg[tid] = z;
+    for (int blk = 0; blk < (RPW + 1) / 2; ++blk) {
+      const int rlo = blk * kBlk, rhi = min(nr, rlo + kBlk);
+      if (rlo < nr && j0 + rhi > y_cur) {  // a row of the block has no kept y
+#pragma unroll
+        for (int hh = 0; hh < 2 / kHalves; ++hh) {
+          const int rt = kHalves == 1 ? hh : half;
+          if (rlo + rt * 16 < L::R) {
+            float d0[4] = {0.f, 0.f, 0.f, 0.f}, d1[4] = {0.f, 0.f, 0.f, 0.f}, d2[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+            for (int kk = 0; kk < KS; ++kk) {
+              uint32_t k4[4];
+              ldsm_x4(k4, Ks + (rlo + rt * 16 + (lane & 7) + ((lane >> 3) & 1) * 8) * L::LDK + kk * 16 + (lane >> 4) * 8);
+              mma_m16n8k16(d0, k4[0], k4[1], k4[2], k4[3], b3[0][kk][0], b3[0][kk][1]);
+              mma_m16n8k16(d1, k4[0], k4[1], k4[2], k4[3], b3[1][kk][0], b3[1][kk][1]);
+              mma_m16n8k16(d2, k4[0], k4[1], k4[2], k4[3], b3[2][kk][0], b3[2][kk][1]);
+            }
+            float* ya = yb + (rt * 16 + g) * L::LDY + nt * 8 + 2 * t;
+            ya[0] = (d0[0] + (d1[0] + d2[0])) * nf0;
+            ya[1] = (d0[1] + (d1[1] + d2[1])) * nf0;
+            ya[8 * L::LDY] = (d0[2] + (d1[2] + d2[2])) * nf0;
+            ya[8 * L::LDY + 1] = (d0[3] + (d1[3] + d2[3])) * nf0;
+          }
+        }
+        __syncthreads();
+#pragma unroll
+        for (int i = 2 * blk; i < 2 * blk + 2 && i < RPW; ++i) {
+          const int r = warp + kRW * i;
+          if (r < nr && j0 + r >= y_cur) ld_vec<DPL>(yb + (r - rlo) * L::LDY + lane * DPL, y[i]);
+        }
+        __syncthreads();
+      }
     }
-    __syncthreads();
-    float f[G];  // this CTA's rescale to the unit's maximum
-#pragma unroll
-    for (int h = 0; h < G; ++h) f[h] = s_M[h] != -INFINITY ? expf(s_M[h] - s_Mg[h]) : 0.f;
-    for (int jj = tid; jj < nr; jj += kRT)
-#pragma unroll
-      for (int h = 0; h < G; ++h) lg[h * R + jj] = expf(lg[h * R + jj] - s_M[h]) * f[h];
-    if (lane < G) {
-      zf = s_Zg[lane];
-      zinv = 1.f / zf;
-    }
-    // once no CTA reads this one's partials any more, the unit's maxima
-    // replace its own (Phase 2 reads them)
-    cluster.sync();
-    if (tid < G) s_M[tid] = s_Mg[tid];
   }
+  // clamp list of the initial moments: this CTA's entries with 0 < |S_tilde_ab| < tau
+  const float tau = a.tau;
+  auto scan_row = [&](int j, const float (&s)[DPL]) {
+#pragma unroll
+    for (int d = 0; d < DPL; ++d)
+      if (s[d] != 0.f && fabsf(s[d]) < tau) {
+        const int slot = atomicAdd(&s_nz, 1);
+        if (slot < kMaxClamp) {
+          s_zidx[slot] = static_cast<uint32_t>((a0 + j) * D + lane * DPL + d);
+          s_zval[slot] = s[d];
+        }
+      }
+  };
+  if (n > 0 && tau > 0.f)
+    for (int j = warp; j < SR; j += kRW) {
+      float s[DPL];
+      ld_vec<DPL>(S + (size_t)j * D + lane * DPL, s);
+      scan_row(j, s);
+    }
+
+  // ---- softmax is shift-invariant: e_hj = exp(l_hj - M_h) with M_h the unit's
+  // largest logit.  Z_h lives in lane h < G of every warp as a compensated
+  // (Kahan) float, decremented per eviction: value zf - zc.  Every CTA
+  // combines the same partials in the same order, so all hold the same values.
+  cluster_wait_acquire();
+  float zf = 1.f, zc = 0.f, zinv = 1.f, Mh = 0.f;
+  if (lane < G) {
+    float m = -INFINITY, z = 0.f;
+    for (int r = 0; r < CL; ++r) m = fmaxf(m, mail_m[r][lane]);
+    for (int r = 0; r < CL; ++r)
+      if (mail_m[r][lane] != -INFINITY) z += mail_z[r][lane] * expf(mail_m[r][lane] - m);
+    Mh = m;
+    zf = z;
+    zinv = 1.f / zf;
+  }
+  for (int jj = warp * 32 + lane; jj - lane < nr; jj += kRT)  // whole warps: the maxima come by shuffles
+#pragma unroll
+    for (int h = 0; h < G; ++h) {
+      const float m = __shfl_sync(kFull, Mh, h);
+      if (jj < nr) lg[h * L::R + jj] = expf(lg[h * L::R + jj] - m);
+    }
   __syncthreads();
   // e_hj of the row this lane scores
   float ereg[G];
   {
     const int i = lane >> SH, r = warp + kRW * i;
 #pragma unroll
-    for (int h = 0; h < G; ++h) ereg[h] = (i < RPW && r < nr) ? lg[h * R + r] : 0.f;
+    for (int h = 0; h < G; ++h) ereg[h] = (i < RPW && r < nr) ? lg[h * L::R + r] : 0.f;
   }
 
-  // ---- registers, in the raw co-moment form S_tilde = n C (Eq. app_S_tilde):
-  // y_j = S_tilde k_j of the warp's rows, the thread's share of S_tilde, the
-  // means.  A Welford fold then adds (k - mu_k)(v - mu_v')^T to S_tilde and
-  // ((k - mu_k) . k_j)(v - mu_v') to y_j: one FMA per element, and the clamp
-  // test is |S_tilde_ab| < tau with no scaling.
-  const float nf0 = static_cast<float>(n);
-  float y[RPW][DPL];
-  unsigned alive = 0u;
+  // y_j' = y_j + (dk . k_j) dv of the warp's surviving rows
+  auto fold_y = [&]() {
+    float pv[P];
 #pragma unroll
-  for (int i = 0; i < RPW; ++i) {
+    for (int i = 0; i < P; ++i) {
+      pv[i] = 0.f;
+      if (i < RPW && ((alive >> i) & 1u)) {
+        float kf[DPL];
+        load_bf16<DPL>(Ks + (warp + kRW * i) * L::LDK + lane * DPL, kf);
 #pragma unroll
-    for (int d = 0; d < DPL; ++d) y[i][d] = 0.f;
-    if (warp + kRW * i < nr) alive |= 1u << i;
-  }
-  if (n > 0) {
-    // rows below the cache's y_len carry y_j = S_tilde k_j from the call that
-    // last changed the moments (kept in the cache across calls); the others
-    // (the rows appended since) are computed here, O(d^2) each
-    unsigned fresh = 0u;
+        for (int d = 0; d < DPL; ++d) pv[i] = fmaf(sdk[d], kf[d], pv[i]);
+      }
+    }
+    const float dsum = transpose_sum<P>(pv, lane);
 #pragma unroll
     for (int i = 0; i < RPW; ++i) {
-      const int r = warp + kRW * i;
-      if (r < nr && j0 + r < y_cur) {
-        const float* src = a.Y + (row0 + j0 + r) * D + lane * DPL;
-        if constexpr (DPL == 4) {
-          const float4 t = *reinterpret_cast<const float4*>(src);
-          y[i][0] = t.x;
-          y[i][1] = t.y;
-          y[i][2] = t.z;
-          y[i][3] = t.w;
-        } else {
-          const float2 t = *reinterpret_cast<const float2*>(src);
-          y[i][0] = t.x;
-          y[i][1] = t.y;
-        }
-      } else if (r < nr) {
-        fresh |= 1u << i;
-      }
+      const float dot = __shfl_sync(kFull, dsum, i << SH);
+#pragma unroll
+      for (int d = 0; d < DPL; ++d) y[i][d] = fmaf(dot, sdv[d], y[i][d]);
     }
-    if (fresh != 0u) {  // warp-uniform
-      for (int c = 0; c < D; ++c) {
-        float cv[DPL];
-        ld_vec<DPL>(Ct + (size_t)c * D + lane * DPL, cv);
-#pragma unroll
-        for (int i = 0; i < RPW; ++i) {
-          if ((fresh >> i) & 1u) {
-            const float kv = __bfloat162float(Kr[(size_t)(warp + kRW * i) * D + c]);
-#pragma unroll
-            for (int d = 0; d < DPL; ++d) y[i][d] = fmaf(cv[d], kv, y[i][d]);
-          }
-        }
-      }
-#pragma unroll
-      for (int i = 0; i < RPW; ++i)
-        if ((fresh >> i) & 1u)
-#pragma unroll
-          for (int d = 0; d < DPL; ++d) y[i][d] *= nf0;
-    }
-  }
-  float creg[CJ][DPL];
-#pragma unroll
-  for (int jj = 0; jj < CJ; ++jj) {
-    ld_vec<DPL>(Ct + (size_t)(warp + kRW * jj) * D + lane * DPL, creg[jj]);
-#pragma unroll
-    for (int d = 0; d < DPL; ++d) creg[jj][d] *= nf0;
-  }
-  float mk[DPL], mv[DPL], sdk[DPL], sdv[DPL];
-#pragma unroll
-  for (int d = 0; d < DPL; ++d) {
-    mk[d] = s_mu_k[lane * DPL + d];
-    mv[d] = s_mu_v[lane * DPL + d];
-    sdk[d] = sdv[d] = 0.f;
-  }
-  // clamp list of the initial moments: entries with 0 < |S_tilde_ab| < tau
-  const float tau = a.tau;
-  if (n > 0 && tau > 0.f) {
-#pragma unroll
-    for (int jj = 0; jj < CJ; ++jj)
-#pragma unroll
-      for (int d = 0; d < DPL; ++d) {
-        const float v = creg[jj][d];
-        if (v != 0.f && fabsf(v) < tau) {
-          const int k = atomicAdd(&s_nz, 1);
-          if (k < kMaxClamp) {
-            s_zidx[k] = static_cast<uint32_t>((warp + kRW * jj) * D + lane * DPL + d);
-            s_zval[k] = v;
-          }
-        }
-      }
-  }
-  __syncthreads();
-
-  const int n_evict = max(0, len - a.budget);
+  };
+  const int n_evict = len - a.budget;
+  int base = j0;  // where this slice's first survivor goes: the evicted rows below the slice move it down
   for (int e = 0;; ++e) {
     const int par = e & 1;
-    // ---- fold the previous eviction into this thread's share of S_tilde and
-    // build the clamp list: S_tilde' = S_tilde + dk dv^T
-    if (e > 0) {
-      const float mydk = select_n<DPL>(sdk, warp % DPL);
-#pragma unroll
-      for (int jj = 0; jj < CJ; ++jj) {
-        const int c = warp + kRW * jj;
-        const float kd = __shfl_sync(kFull, mydk, c / DPL);  // dk[c]: lane c/DPL, component warp % DPL
+    // ---- fold the previous eviction into this CTA's rows of S_tilde and list
+    // its clamped entries: S_tilde' = S_tilde + dv dk^T
+    if (e > 0)
+      for (int j = warp; j < SR; j += kRW) {
+        const int ra = a0 + j;
+        const float vd = __shfl_sync(kFull, select_n<DPL>(sdv, ra % DPL), ra / DPL);  // dv[ra]
+        float s[DPL];
         bool any = false;
+        ld_vec<DPL>(S + (size_t)j * D + lane * DPL, s);
 #pragma unroll
         for (int d = 0; d < DPL; ++d) {
-          creg[jj][d] = fmaf(kd, sdv[d], creg[jj][d]);
-          any |= fabsf(creg[jj][d]) < tau;
+          s[d] = fmaf(vd, sdk[d], s[d]);
+          any |= fabsf(s[d]) < tau;
         }
-        if (any) {
-#pragma unroll
-          for (int d = 0; d < DPL; ++d)
-            if (creg[jj][d] != 0.f && fabsf(creg[jj][d]) < tau) {
-              const int slot = atomicAdd(&s_nz, 1);
-              if (slot < kMaxClamp) {
-                s_zidx[slot] = static_cast<uint32_t>(c * D + lane * DPL + d);
-                s_zval[slot] = creg[jj][d];
-              }
-            }
-        }
+        st_vec<DPL>(S + (size_t)j * D + lane * DPL, s);
+        if (any) scan_row(j, s);
       }
-    }
     if (e == n_evict) break;  // uniform over the cluster
     if (tid == 0) s_best[par ^ 1] = ~0ull;  // its readers finished one iteration ago
 
-    // ---- y_j' = y_j + (dk . k_j) dv, then the residual norms of the warp's
-    // rows: r_j = v_j - mu_v - (scale / n) y_j
+    // ---- y_j', then the residual norms of the warp's rows:
+    // r_j = v_j - mu_v - (scale / n) y_j
     const float rs = (n > 0) ? scale / static_cast<float>(n) : 0.f;
-    float part[RPW];
-    if (e > 0) {
+    if (e > 0) fold_y();
+    float invz[G];
 #pragma unroll
-      for (int i = 0; i < RPW; ++i) {
-        part[i] = 0.f;
-        if ((alive >> i) & 1u) {
-          float kf[DPL];
-          load_bf16<DPL>(Kr + (size_t)(warp + kRW * i) * D + lane * DPL, kf);
-#pragma unroll
-          for (int d = 0; d < DPL; ++d) part[i] = fmaf(sdk[d], kf[d], part[i]);
-        }
-      }
-      float pv[P];
-#pragma unroll
-      for (int i = 0; i < P; ++i) pv[i] = i < RPW ? part[i] : 0.f;
-      const float dsum = transpose_sum<P>(pv, lane);
-#pragma unroll
-      for (int i = 0; i < RPW; ++i) {
-        const float dot = __shfl_sync(kFull, dsum, i << SH);
-#pragma unroll
-        for (int d = 0; d < DPL; ++d) y[i][d] = fmaf(dot, sdv[d], y[i][d]);
-      }
-    }
-#pragma unroll
-    for (int i = 0; i < RPW; ++i) {
-      part[i] = 0.f;
-      if ((alive >> i) & 1u) {
-        float vf[DPL];
-        load_bf16<DPL>(Vr + (size_t)(warp + kRW * i) * D + lane * DPL, vf);
-#pragma unroll
-        for (int d = 0; d < DPL; ++d) {
-          const float rr = vf[d] - mv[d] - rs * y[i][d];
-          part[i] = fmaf(rr, rr, part[i]);
-        }
-      }
-    }
+    for (int h = 0; h < G; ++h) invz[h] = __shfl_sync(kFull, zinv, h);
     // residual norms reduced so that lane l holds row l >> SH's; those lanes
     // score their row, and the warp's minimum key goes to the block minimum
-    auto post_keys = [&](const float (&ss)[RPW]) {
+    auto post_keys = [&](const float (&ss)[P]) {
       float pv[P];
 #pragma unroll
-      for (int i = 0; i < P; ++i) pv[i] = i < RPW ? ss[i] : 0.f;
+      for (int i = 0; i < P; ++i) pv[i] = ss[i];
       const float sum = transpose_sum<P>(pv, lane);
-      float invz[G];
-#pragma unroll
-      for (int h = 0; h < G; ++h) invz[h] = __shfl_sync(kFull, zinv, h);
       const int i = lane >> SH;
       unsigned long long key = ~0ull;
       if ((lane & ((1 << SH) - 1)) == 0 && i < RPW && ((alive >> i) & 1u)) {
@@ -479,30 +439,73 @@ __global__ void __cluster_dims__(kCL, 1, 1) __launch_bounds__(kRT, 1)
       }
       if (lane == 0 && key != ~0ull) atomicMin(&s_best[par], key);
     };
+    // warp w < CL posts this CTA's key, candidate row and clamp count into rank w's mailbox
+    auto post_mail = [&](int nz) {
+      if (warp < CL) {
+        const unsigned long long b = s_best[par];
+        const int jb = (b == ~0ull) ? -1 : static_cast<int>(b & 0xffffffffu) - j0;
+        if (lane == 0) {
+          *cluster.map_shared_rank(&mail_key[par][rank], warp) = b;
+          *cluster.map_shared_rank(&mail_nz[par][rank], warp) = nz;
+        }
+        if (jb >= 0 && lane < G) *cluster.map_shared_rank(&mail_e[par][rank][lane], warp) = lg[lane * L::R + jb];
+        if (jb >= 0 && lane < D / 4) {  // lanes 0..D/8-1 carry k, the next D/8 carry v
+          const bool is_v = lane >= D / 8;
+          const int i = is_v ? lane - D / 8 : lane;
+          const uint4 w4 = *reinterpret_cast<const uint4*>(is_v ? Vs + jb * D + i * 8 : Ks + jb * L::LDK + i * 8);
+          reinterpret_cast<uint4*>(cluster.map_shared_rank(&mail_row[par][rank][is_v ? D : 0], warp))[i] = w4;
+        }
+      }
+    };
+    float part[P];
+#pragma unroll
+    for (int i = 0; i < P; ++i) {
+      part[i] = 0.f;
+      if (i < RPW && ((alive >> i) & 1u)) {
+        float vf[DPL];
+        load_bf16<DPL>(Vs + (warp + kRW * i) * D + lane * DPL, vf);
+#pragma unroll
+        for (int d = 0; d < DPL; ++d) {
+          const float rr = vf[d] - mv[d] - rs * y[i < RPW ? i : 0][d];
+          part[i] = fmaf(rr, rr, part[i]);
+        }
+      }
+    }
     post_keys(part);
     __syncthreads();
-    const int nz = s_nz;
-    if (nz > 0) {  // uniform: clamped entries of C' change y; score again with them
+    post_mail(s_nz);
+    cluster.sync();
+    const int my_nz = lane < CL ? mail_nz[par][lane] : 0;
+    if (__any_sync(kFull, my_nz > 0)) {  // uniform over the cluster: clamped entries of C' change y; score again
+      const int nz = __reduce_add_sync(kFull, min(my_nz, kMaxClamp + 1));
       const bool direct = nz > kMaxClamp;
-      if (tid == 0) s_best[par] = ~0ull;
+      float* St = a.C + (size_t)u * D * D;  // direct: S_tilde transposed, in C's memory (C is written at the end)
       if (direct) {
+        for (int j = warp; j < SR; j += kRW)
 #pragma unroll
-        for (int jj = 0; jj < CJ; ++jj) st_vec<DPL>(Ct + (size_t)(warp + kRW * jj) * D + lane * DPL, creg[jj]);
+          for (int d = 0; d < DPL; ++d) St[(size_t)(lane * DPL + d) * D + a0 + j] = S[(size_t)j * D + lane * DPL + d];
+        __threadfence();
+      } else if (tid < nz) {  // the unit's list: rank by rank
+        int z = tid, r = 0;
+        while (z >= mail_nz[par][r]) z -= mail_nz[par][r++];
+        s_gidx[tid] = cluster.map_shared_rank(s_zidx, r)[z];
+        s_gval[tid] = cluster.map_shared_rank(s_zval, r)[z];
       }
-      __syncthreads();
+      if (tid == 0) s_best[par] = ~0ull;
+      cluster.sync();  // lists and mailboxes read, S_tilde written
 #pragma unroll
-      for (int i = 0; i < RPW; ++i) {
+      for (int i = 0; i < P; ++i) {
         part[i] = 0.f;
-        if ((alive >> i) & 1u) {
+        if (i < RPW && ((alive >> i) & 1u)) {
           const int r = warp + kRW * i;
           float yc[DPL];
           if (!direct) {
 #pragma unroll
-            for (int d = 0; d < DPL; ++d) yc[d] = y[i][d];
+            for (int d = 0; d < DPL; ++d) yc[d] = y[i < RPW ? i : 0][d];
             for (int z = 0; z < nz; ++z) {  // y'_a -= S_tilde_ab k_b for clamped (a, b)
-              const int kb = static_cast<int>(s_zidx[z] / D), va = static_cast<int>(s_zidx[z] % D);
+              const int va = static_cast<int>(s_gidx[z] / D), kb = static_cast<int>(s_gidx[z] % D);
               if (va / DPL == lane) {
-                const float corr = s_zval[z] * __bfloat162float(Kr[(size_t)r * D + kb]);
+                const float corr = s_gval[z] * __bfloat162float(Ks[r * L::LDK + kb]);
 #pragma unroll
                 for (int d = 0; d < DPL; ++d)
                   if (va % DPL == d) yc[d] -= corr;
@@ -512,15 +515,16 @@ __global__ void __cluster_dims__(kCL, 1, 1) __launch_bounds__(kRT, 1)
 #pragma unroll
             for (int d = 0; d < DPL; ++d) yc[d] = 0.f;
             for (int c = 0; c < D; ++c) {
-              const float kv = __bfloat162float(Kr[(size_t)r * D + c]);
-              float cv[DPL];
-              ld_vec<DPL>(Ct + (size_t)c * D + lane * DPL, cv);
+              const float kv = __bfloat162float(Ks[r * L::LDK + c]);
 #pragma unroll
-              for (int d = 0; d < DPL; ++d) yc[d] = fmaf((fabsf(cv[d]) < tau) ? 0.f : cv[d], kv, yc[d]);
+              for (int d = 0; d < DPL; ++d) {
+                const float cv = __ldcg(St + (size_t)c * D + lane * DPL + d);
+                yc[d] = fmaf((fabsf(cv) < tau) ? 0.f : cv, kv, yc[d]);
+              }
             }
           }
           float vf[DPL];
-          load_bf16<DPL>(Vr + (size_t)r * D + lane * DPL, vf);
+          load_bf16<DPL>(Vs + r * D + lane * DPL, vf);
 #pragma unroll
           for (int d = 0; d < DPL; ++d) {
             const float rr = vf[d] - mv[d] - rs * yc[d];
@@ -530,27 +534,14 @@ __global__ void __cluster_dims__(kCL, 1, 1) __launch_bounds__(kRT, 1)
       }
       post_keys(part);
       __syncthreads();
-      if (tid == 0) s_nz = 0;  // every reader of the list is past the barrier above
+      if (tid == 0) s_nz = 0;  // the next entries are listed after the cluster barrier below
+      post_mail(0);
+      cluster.sync();
     }
-
-    // ---- warp w < 8 posts this CTA's key and candidate row into rank w's mailbox
-    if (warp < kCL) {
-      const unsigned long long b = s_best[par];
-      const int jb = (b == ~0ull) ? -1 : static_cast<int>(b & 0xffffffffu) - j0;
-      if (lane == 0) *cluster.map_shared_rank(&mail_key[par][rank], warp) = b;
-      if (jb >= 0 && lane < G) *cluster.map_shared_rank(&mail_e[par][rank][lane], warp) = lg[lane * R + jb];
-      if (jb >= 0 && lane < D / 4) {  // lanes 0..D/8-1 carry k, the next D/8 carry v
-        const bool is_v = lane >= D / 8;
-        const int i = is_v ? lane - D / 8 : lane;
-        const uint4 w4 = reinterpret_cast<const uint4*>((is_v ? Vr : Kr) + (size_t)jb * D)[i];
-        reinterpret_cast<uint4*>(cluster.map_shared_rank(&mail_row[par][rank][is_v ? D : 0], warp))[i] = w4;
-      }
-    }
-    cluster.sync();
 
     // ---- every warp: the cluster's minimum key (ties cannot happen: rows
     // differ), by two warp-wide minimum reductions (score bits, then row)
-    const unsigned long long bk = (lane < kCL) ? mail_key[par][lane] : ~0ull;
+    const unsigned long long bk = (lane < CL) ? mail_key[par][lane] : ~0ull;
     const unsigned khi = static_cast<unsigned>(bk >> 32), klo = static_cast<unsigned>(bk);
     const unsigned mhi = __reduce_min_sync(kFull, khi);
     const unsigned mlo = __reduce_min_sync(kFull, khi == mhi ? klo : 0xffffffffu);
@@ -577,6 +568,7 @@ __global__ void __cluster_dims__(kCL, 1, 1) __launch_bounds__(kRT, 1)
       n += 1;
     }
     const int jr = js - j0;
+    if (jr < 0) --base;
     if (jr >= 0 && jr < nr && jr % kRW == warp) alive &= ~(1u << (jr / kRW));
     if (lane < G) {  // compensated Z_h -= e_h,js
       const float yk = -mail_e[par][src][lane] - zc;
@@ -586,168 +578,148 @@ __global__ void __cluster_dims__(kCL, 1, 1) __launch_bounds__(kRT, 1)
       zinv = 1.f / zf;
     }
   }
+  // every CTA's reads of the cache, y and C lie before the loop's cluster
+  // barriers, and no remote access follows them
 
-  // ---- state back to shared memory: survivors, C (transposed), means
-#pragma unroll
-  for (int i = 0; i < RPW; ++i)
-    if (lane == 0 && warp + kRW * i < nr) alive_all[j0 + warp + kRW * i] = (alive >> i) & 1u;
-#pragma unroll
-  for (int jj = 0; jj < CJ; ++jj) {
-    float cv[DPL];
-#pragma unroll
-    for (int d = 0; d < DPL; ++d) cv[d] = n > 0 ? creg[jj][d] / static_cast<float>(n) : 0.f;
-    st_vec<DPL>(Ct + (size_t)(warp + kRW * jj) * D + lane * DPL, cv);
-  }
-  if (warp == 0) {
-#pragma unroll
-    for (int d = 0; d < DPL; ++d) {
-      s_mu_k[lane * DPL + d] = mk[d];
-      s_mu_v[lane * DPL + d] = mv[d];
-    }
-  }
+  // ---- survivors to their places, in order, from shared memory
+  if (has_y) fold_y();  // the loop left the last eviction out of y
+  if (lane == 0) s_mask[warp] = alive;
   __syncthreads();
-  const uint8_t* alv = alive_all + j0;
-
-  // ---- ordered compaction across the cluster through the staging buffer
-  {
-    int cnt = 0;
-    for (int r = tid; r < nr; r += kRT) cnt += alv[r];
+  const uint32_t mask = lane < kRW ? s_mask[lane] : 0u;
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) cnt += __shfl_xor_sync(kFull, cnt, o);
-    if (lane == 0) s_red[warp][0] = static_cast<float>(cnt);
-    __syncthreads();
-    if (tid == 0) {
-      int c = 0;
-      for (int w = 0; w < kRW; ++w) c += static_cast<int>(s_red[w][0]);
-      ex_cnt = c;
-    }
-  }
-  cluster.sync();
-  int base = 0;
-  for (int r = 0; r < rank; ++r) base += *cluster.map_shared_rank(&ex_cnt, r);
-  const int mine = ex_cnt;
-  if (a.Y != nullptr && a.y_len != nullptr) {
-    // the loop left the last eviction folded into S_tilde but not yet into
-    // y: y_j += (dk . k_j) dv for the surviving rows, as in the loop
-    {
-      float part[RPW];
-#pragma unroll
-      for (int i = 0; i < RPW; ++i) {
-        part[i] = 0.f;
-        if ((alive >> i) & 1u) {
-          float kf[DPL];
-          load_bf16<DPL>(Kr + (size_t)(warp + kRW * i) * D + lane * DPL, kf);
-#pragma unroll
-          for (int d = 0; d < DPL; ++d) part[i] = fmaf(sdk[d], kf[d], part[i]);
-        }
-      }
-      float pv[P];
-#pragma unroll
-      for (int i = 0; i < P; ++i) pv[i] = i < RPW ? part[i] : 0.f;
-      const float dsum = transpose_sum<P>(pv, lane);
-#pragma unroll
-      for (int i = 0; i < RPW; ++i) {
-        const float dot = __shfl_sync(kFull, dsum, i << SH);
-#pragma unroll
-        for (int d = 0; d < DPL; ++d) y[i][d] = fmaf(dot, sdv[d], y[i][d]);
-      }
-    }
-    // y_j of the surviving rows to their compacted rows: each warp writes its
-    // own rows' registers (every read of the y rows was in the set-up, before
-    // the cluster barriers of the loop)
-#pragma unroll
-    for (int i = 0; i < RPW; ++i) {
+  for (int i = 0; i < RPW; ++i) {
+    if ((alive >> i) & 1u) {  // warp-uniform
       const int r = warp + kRW * i;
-      if (r < nr && ((alive >> i) & 1u)) {  // warp-uniform
-        int before = 0;  // survivors of this CTA ahead of row r
-        for (int c0 = 0; c0 < r; c0 += 32)
-          before += __popc(__ballot_sync(kFull, c0 + lane < r && alv[c0 + lane]));
-        float* dst = a.Y + (row0 + base + before) * D + lane * DPL;
-        if constexpr (DPL == 4) *reinterpret_cast<float4*>(dst) = make_float4(y[i][0], y[i][1], y[i][2], y[i][3]);
-        else *reinterpret_cast<float2*>(dst) = make_float2(y[i][0], y[i][1]);
-      }
-    }
-    if (rank == 0 && tid == 0) a.y_len[u] = a.budget;  // ordered after the other CTAs' writes by the kernel end
-  }
-  uint8_t* st = static_cast<uint8_t*>(a.stage) + (size_t)u * stage_stride(a.cap, D);
-  __nv_bfloat16* SK = reinterpret_cast<__nv_bfloat16*>(st);
-  __nv_bfloat16* SV = SK + (size_t)a.cap * D;
-  int32_t* SP = reinterpret_cast<int32_t*>(SV + (size_t)a.cap * D);
-  for (int c0 = 0; c0 < nr; c0 += 32) {
-    const bool al = (c0 + lane < nr) && alv[c0 + lane];
-    const unsigned m = __ballot_sync(kFull, al);
-    int before = 0;  // survivors in earlier chunks
-    for (int c1 = 0; c1 < c0; c1 += 32) {
-      const bool a1 = (c1 + lane < nr) && alv[c1 + lane];
-      before += __popc(__ballot_sync(kFull, a1));
-    }
-    for (int bit = warp; bit < 32; bit += kRW) {  // warp w moves rows c0 + w, c0 + w + 16
-      if ((m >> bit) & 1u) {
-        const int r = c0 + bit;
-        const int dst = base + before + __popc(m & ((1u << bit) - 1u));
-        for (int i = lane; i < D / 8; i += 32) {
-          reinterpret_cast<uint4*>(SK + (size_t)dst * D)[i] = reinterpret_cast<const uint4*>(Kr + (size_t)r * D)[i];
-          reinterpret_cast<uint4*>(SV + (size_t)dst * D)[i] = reinterpret_cast<const uint4*>(Vr + (size_t)r * D)[i];
+      // survivors of the slice ahead of row r: lane w counts warp w's
+      const int dst = base + static_cast<int>(__reduce_add_sync(
+                                 kFull, __popc(mask & ((1u << i) - 1u)) + (lane < warp ? (mask >> i) & 1u : 0u)));
+      if (dst != j0 + r) {
+        const size_t o = (size_t)dst * D + lane * DPL;
+        if constexpr (DPL == 4) {
+          *reinterpret_cast<uint2*>(Kg + o) = *reinterpret_cast<const uint2*>(Ks + r * L::LDK + lane * DPL);
+          *reinterpret_cast<uint2*>(Vg + o) = *reinterpret_cast<const uint2*>(Vs + r * D + lane * DPL);
+        } else {
+          *reinterpret_cast<uint32_t*>(Kg + o) = *reinterpret_cast<const uint32_t*>(Ks + r * L::LDK + lane * DPL);
+          *reinterpret_cast<uint32_t*>(Vg + o) = *reinterpret_cast<const uint32_t*>(Vs + r * D + lane * DPL);
         }
-        if (lane == 0) SP[dst] = Pg[j0 + r];
+        if (lane == 0) Pg[dst] = s_pos[r];
       }
+      if (has_y) st_vec<DPL>(a.Y + (row0 + dst) * D + lane * DPL, y[i]);
     }
   }
-  __threadfence();
-  cluster.sync();
-  for (int idx = tid; idx < mine * (D / 8); idx += kRT) {
-    const int row = base + idx / (D / 8), i = idx % (D / 8);
-    reinterpret_cast<uint4*>(Kg + (size_t)row * D)[i] = reinterpret_cast<const uint4*>(SK + (size_t)row * D)[i];
-    reinterpret_cast<uint4*>(Vg + (size_t)row * D)[i] = reinterpret_cast<const uint4*>(SV + (size_t)row * D)[i];
+  // ---- the moments back: this CTA's rows of C = S_tilde / n (each warp folded its own)
+  const float nf1 = static_cast<float>(n);
+  for (int j = warp; j < SR; j += kRW) {
+    float s[DPL];
+    ld_vec<DPL>(S + (size_t)j * D + lane * DPL, s);
+#pragma unroll
+    for (int d = 0; d < DPL; ++d) s[d] = n > 0 ? s[d] / nf1 : 0.f;
+    st_vec<DPL>(a.C + (size_t)u * D * D + (size_t)(a0 + j) * D + lane * DPL, s);
   }
-  for (int r = tid; r < mine; r += kRT) Pg[base + r] = SP[base + r];
-  {  // C back to global, its 32 x 32 tiles shared out over the cluster's CTAs
-    float* tb = s_tile[warp % kTWR];
-    for (int t = rank + kCL * warp; warp < kTWR && t < (D / 32) * (D / 32); t += kCL * kTWR) {
-      const int c0 = (t / (D / 32)) * 32, r0 = (t % (D / 32)) * 32;
-      for (int i = 0; i < 32; ++i) tb[i * 33 + lane] = Ct[(size_t)(c0 + i) * D + r0 + lane];
-      __syncwarp();
-      for (int i = 0; i < 32; ++i) a.C[(size_t)u * D * D + (size_t)(r0 + i) * D + c0 + lane] = tb[lane * 33 + i];
-      __syncwarp();
+  if (rank == 0 && warp == 0) {
+#pragma unroll
+    for (int d = 0; d < DPL; ++d) {  // single elements: mu_k is only 8-byte aligned
+      a.mu_k[(size_t)u * D + lane * DPL + d] = mk[d];
+      a.mu_v[(size_t)u * D + lane * DPL + d] = mv[d];
     }
-  }
-  if (rank == 0) {
-    for (int i = tid; i < D; i += kRT) {
-      a.mu_k[(size_t)u * D + i] = s_mu_k[i];
-      a.mu_v[(size_t)u * D + i] = s_mu_v[i];
-    }
-    if (tid == 0) {
+    if (lane == 0) {
       a.n[u] = n;
       a.len[u] = a.budget;
       a.seen[u] = seen_in + (has_new ? 1 : 0);
+      if (has_y) a.y_len[u] = a.budget;  // ordered after the other CTAs' writes by the kernel end
     }
   }
 }
 
+// Clusters of `cl` CTAs of an instance that the device holds at once (0: none).
 template <int D, int G, int RPW>
-cudaError_t launch_reg(EvictArgs a, cudaStream_t stream) {
-  a.rows_max = (a.cap + kCL - 1) / kCL;
-  a.kv_smem = 1;
-  size_t smem = RegLayout<D, G>(a.rows_max, a.cap, 1).total;
-  if (smem > kSmemBudget) {
-    a.kv_smem = 0;
-    smem = RegLayout<D, G>(a.rows_max, a.cap, 0).total;
+int active_clusters(int cl) {
+  constexpr int kMaxDev = 64;
+  static std::mutex mu;
+  static int known[kMaxDev][kMaxCL + 1] = {};
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDev) return 0;
+  std::lock_guard<std::mutex> lock(mu);
+  if (known[dev][cl] == 0) {
+    int n = 0;
+    const size_t smem = RegLayout<D, G, RPW>::total(2);
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3(cl, 1, 1);
+    cfg.blockDim = dim3(kRT, 1, 1);
+    cfg.dynamicSmemBytes = RegLayout<D, G, RPW>::total(cl);
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = cl;
+    at[0].val.clusterDim.y = 1;
+    at[0].val.clusterDim.z = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    if (cudaFuncSetAttribute(evict_reg_kernel<D, G, RPW>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             static_cast<int>(smem)) != cudaSuccess ||
+        cudaOccupancyMaxActiveClusters(&n, evict_reg_kernel<D, G, RPW>, &cfg) != cudaSuccess) {
+      (void)cudaGetLastError();
+      n = 0;
+    }
+    known[dev][cl] = n > 0 ? n : -1;
   }
-  cudaError_t e = cudaFuncSetAttribute(evict_reg_kernel<D, G, RPW>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       static_cast<int>(smem));
-  if (e != cudaSuccess) return e;
-  evict_reg_kernel<D, G, RPW><<<a.batch * a.n_kv * kCL, kRT, smem, stream>>>(a);
-  return cudaGetLastError();
+  return std::max(0, known[dev][cl]);
 }
 
-// Rows of one CTA's slice at most: warps of the register kernel hold 5 or 9
-// each.  Larger slices keep their state in shared memory and the workspace.
+template <int D, int G, int RPW>
+cudaError_t launch_reg(const EvictArgs& a, int cl, cudaStream_t stream) {
+  if (active_clusters<D, G, RPW>(cl) < 1) return cudaErrorLaunchOutOfResources;  // and the instance's attributes
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3(static_cast<unsigned>((long)a.batch * a.n_kv * cl), 1, 1);
+  cfg.blockDim = dim3(kRT, 1, 1);
+  cfg.dynamicSmemBytes = RegLayout<D, G, RPW>::total(cl);
+  cfg.stream = stream;
+  cudaLaunchAttribute at[2];
+  at[0].id = cudaLaunchAttributeClusterDimension;
+  at[0].val.clusterDim.x = cl;
+  at[0].val.clusterDim.y = 1;
+  at[0].val.clusterDim.z = 1;
+  at[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[1].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = 2;
+  return cudaLaunchKernelEx(&cfg, evict_reg_kernel<D, G, RPW>, a);
+}
+
+template <int D, int G>
+cudaError_t launch_rows(const EvictArgs& a, int cl, cudaStream_t stream) {
+  const int slice = (a.cap + cl - 1) / cl;  // rows of one CTA's slice at most
+  if (slice <= kRW * 5) return launch_reg<D, G, 5>(a, cl, stream);
+  if (slice <= kRW * 9) return launch_reg<D, G, 9>(a, cl, stream);
+  return launch_reg<D, G, 16>(a, cl, stream);
+}
+template <int D, int G>
+int active_rows(int slice, int cl) {
+  if (slice <= kRW * 5) return active_clusters<D, G, 5>(cl);
+  if (slice <= kRW * 9) return active_clusters<D, G, 9>(cl);
+  return active_clusters<D, G, 16>(cl);
+}
+
+// Of 8, 4 and 2 CTAs per unit (slices of at most 256 rows) the one that takes
+// the fewest waves, at a tie the larger: an eviction is a chain of barriers
+// whose length hardly depends on the rows of a CTA, a second wave doubles it.
 template <int D, int G>
 cudaError_t launch_dg(const EvictArgs& a, cudaStream_t stream) {
-  const int slice = (a.cap + kCL - 1) / kCL;
-  if (slice <= kRW * 5) return launch_reg<D, G, 5>(a, stream);
-  if (slice <= kRW * 9) return launch_reg<D, G, 9>(a, stream);
-  return launch_evict_large(a, D, G, stream);
+  if (a.cap > kRegCap) return launch_evict_large(a, D, G, stream);
+  const long units = (long)a.batch * a.n_kv;
+  int cl = kMaxCL;
+  long best = -1;
+  for (int c = kMaxCL; c >= 2; c /= 2) {
+    const int slice = (a.cap + c - 1) / c;
+    if (slice > kRW * 16) break;
+    const int act = active_rows<D, G>(slice, c);
+    if (act < 1) continue;
+    const long waves = (units + act - 1) / act;
+    if (best < 0 || waves < best) {
+      best = waves;
+      cl = c;
+    }
+  }
+  return launch_rows<D, G>(a, cl, stream);
 }
 
 }  // namespace

@@ -5,9 +5,9 @@
 // One cluster of 8, 12 or 16 CTAs per unit; CTA r owns a contiguous slice of
 // the unit's rows, warp w of it the slice rows w, w + 16, ..., and lane l the
 // dims [l*DPL, (l+1)*DPL) of each row.  The loop is the register kernel's: the
-// raw co-moment S_tilde = n C in registers (each CTA holds all of it, a thread
-// 1/512), one FMA per element and eviction for the fold, an exact list of the
-// clamped entries, one block barrier and one cluster barrier per eviction.
+// raw co-moment S_tilde = n C shared out over the CTAs by rows (a warp holds at
+// most one), a list of the clamped entries exchanged when there are any, one
+// block barrier and one cluster barrier per eviction.
 // What differs is where the rows' state lives: y_j = S_tilde k_j (512 bytes a
 // row at d = 128), the softmax terms and the K/V rows are in shared memory as
 // far as they fit (y first: it is read and written at every eviction), else in
@@ -91,7 +91,6 @@ template <int D, int G>
 __global__ void __launch_bounds__(kLT, 1) evict_large_kernel(const EvictArgs a) {
   constexpr int NC = D / 32;   // float4 chunks per row for 8-lane row groups (logits)
   constexpr int DPL = D / 32;  // dims per lane
-  constexpr int CJ = D / kLW;  // rows of S_tilde per thread (DPL columns each)
   constexpr int kRP = kLW * 4; // rows per pass of 8-lane groups
   constexpr int KS = D / 16, NT = D / 8;
   constexpr int P = kRB, SH = 2;  // transposing sums: lane l holds row l >> SH
@@ -107,8 +106,9 @@ __global__ void __launch_bounds__(kLT, 1) evict_large_kernel(const EvictArgs a) 
   // the mailboxes of candidate rows, and before the loop two K blocks of the set-up products
   constexpr int kMailBytes = 2 * kMaxCL * 2 * D * 2, kBlkBytes = 2 * kBlk * (D + 8) * 2;
   __shared__ __align__(16) uint8_t s_rows[kMailBytes > kBlkBytes ? kMailBytes : kBlkBytes];
-  __shared__ uint32_t s_zidx[kMaxClamp];
-  __shared__ float s_zval[kMaxClamp];
+  __shared__ int mail_nz[2][kMaxCL];
+  __shared__ uint32_t s_zidx[kMaxClamp], s_gidx[kMaxClamp];  // this CTA's clamped entries, the unit's
+  __shared__ float s_zval[kMaxClamp], s_gval[kMaxClamp];
   __shared__ int s_nz;
   __shared__ uint32_t s_alive[kLW][kWords];  // bit i of warp w: slice row w + 16 i
   __shared__ uint32_t s_bits[kMaxSlice / 32];
@@ -118,6 +118,10 @@ __global__ void __launch_bounds__(kLT, 1) evict_large_kernel(const EvictArgs a) 
     return reinterpret_cast<__nv_bfloat16*>(s_rows) + ((size_t)par * kMaxCL + r) * 2 * D;
   };
 
+  // The next kernel in the stream may be placed on free SMs while this one
+  // runs (it waits for this one's end); not before this one's own wait.
+  grid_dependency_wait();
+  grid_launch_dependents();
   cg::cluster_group cluster = cg::this_cluster();
   const int rank = static_cast<int>(cluster.block_rank()), CL = static_cast<int>(cluster.num_blocks());
   const int u = blockIdx.x / CL;
@@ -148,6 +152,7 @@ __global__ void __launch_bounds__(kLT, 1) evict_large_kernel(const EvictArgs a) 
     __threadfence();
   }
   if (len <= a.budget) {
+    cluster.sync();  // every CTA has read the length
     if (rank == 0 && tid == 0) {
       a.len[u] = len;
       a.seen[u] = seen_in + (has_new ? 1 : 0);
@@ -319,36 +324,34 @@ __global__ void __launch_bounds__(kLT, 1) evict_large_kernel(const EvictArgs a) 
     for (int i = tid; i < nr * (D / 4); i += kLT) reinterpret_cast<float4*>(Y)[i] = make_float4(0.f, 0.f, 0.f, 0.f);
   }
 
-  // ---- registers: rows a = warp + 16 jj of S_tilde, columns lane*DPL..; the means
-  float creg[CJ][DPL];
+  // ---- registers: warp w < SR holds row a0 + w of S_tilde (the CTAs share out
+  // its rows), lane l columns l*DPL..; the means
+  const int a0 = rank * D / CL, SR = (rank + 1) * D / CL - a0, arow = a0 + warp;
+  const bool holds = warp < SR;
+  float creg[DPL], mk[DPL], mv[DPL], sdk[DPL], sdv[DPL];
 #pragma unroll
-  for (int jj = 0; jj < CJ; ++jj) {
-    if (n > 0) ld_vec<DPL>(Cg + (size_t)(warp + kLW * jj) * D + lane * DPL, creg[jj]);
-#pragma unroll
-    for (int d = 0; d < DPL; ++d) creg[jj][d] = n > 0 ? creg[jj][d] * nf0 : 0.f;
-  }
-  float mk[DPL], mv[DPL], sdk[DPL], sdv[DPL];
+  for (int d = 0; d < DPL; ++d) creg[d] = 0.f;
+  if (holds && n > 0) ld_vec<DPL>(Cg + (size_t)arow * D + lane * DPL, creg);
 #pragma unroll
   for (int d = 0; d < DPL; ++d) {
+    creg[d] *= nf0;
     mk[d] = n > 0 ? a.mu_k[(size_t)u * D + lane * DPL + d] : 0.f;
     mv[d] = n > 0 ? a.mu_v[(size_t)u * D + lane * DPL + d] : 0.f;
     sdk[d] = sdv[d] = 0.f;
   }
   const float tau = a.tau;
-  auto list_entry = [&](int jj, int d) {  // an entry with 0 < |S_tilde_ab| < tau
-    const int slot = atomicAdd(&s_nz, 1);
-    if (slot < kMaxClamp) {
-      s_zidx[slot] = static_cast<uint32_t>((warp + kLW * jj) * D + lane * DPL + d);
-      s_zval[slot] = creg[jj][d];
-    }
+  auto scan_row = [&]() {  // this CTA's entries with 0 < |S_tilde_ab| < tau
+#pragma unroll
+    for (int d = 0; d < DPL; ++d)
+      if (creg[d] != 0.f && fabsf(creg[d]) < tau) {
+        const int slot = atomicAdd(&s_nz, 1);
+        if (slot < kMaxClamp) {
+          s_zidx[slot] = static_cast<uint32_t>(arow * D + lane * DPL + d);
+          s_zval[slot] = creg[d];
+        }
+      }
   };
-  if (n > 0 && tau > 0.f) {
-#pragma unroll
-    for (int jj = 0; jj < CJ; ++jj)
-#pragma unroll
-      for (int d = 0; d < DPL; ++d)
-        if (creg[jj][d] != 0.f && fabsf(creg[jj][d]) < tau) list_entry(jj, d);
-  }
+  if (holds && n > 0) scan_row();
 
   // ---- the unit's maximum and normaliser per head; this CTA's e_hj rescaled to it
   cluster_wait_acquire();
@@ -388,25 +391,13 @@ __global__ void __launch_bounds__(kLT, 1) evict_large_kernel(const EvictArgs a) 
   const int n_evict = len - a.budget;
   for (int e = 0;; ++e) {
     const int par = e & 1;
-    // ---- fold the previous eviction into this thread's share of S_tilde and
-    // build the clamp list: S_tilde' = S_tilde + dv dk^T
-    if (e > 0) {
-      const float mydv = select_n<DPL>(sdv, warp % DPL);
+    // ---- fold the previous eviction into this CTA's rows of S_tilde and list
+    // its clamped entries: S_tilde' = S_tilde + dv dk^T
+    if (e > 0 && holds) {
+      const float vd = __shfl_sync(kFull, select_n<DPL>(sdv, arow % DPL), arow / DPL);  // dv[arow]
 #pragma unroll
-      for (int jj = 0; jj < CJ; ++jj) {
-        const float vd = __shfl_sync(kFull, mydv, (warp + kLW * jj) / DPL);  // dv[a]: lane a/DPL, component warp % DPL
-        bool any = false;
-#pragma unroll
-        for (int d = 0; d < DPL; ++d) {
-          creg[jj][d] = fmaf(vd, sdk[d], creg[jj][d]);
-          any |= fabsf(creg[jj][d]) < tau;
-        }
-        if (any) {
-#pragma unroll
-          for (int d = 0; d < DPL; ++d)
-            if (creg[jj][d] != 0.f && fabsf(creg[jj][d]) < tau) list_entry(jj, d);
-        }
-      }
+      for (int d = 0; d < DPL; ++d) creg[d] = fmaf(vd, sdk[d], creg[d]);
+      scan_row();
     }
     if (e == n_evict) break;  // uniform over the cluster
     if (tid == 0) s_best[par ^ 1] = ~0ull;  // its readers finished one iteration ago
@@ -437,6 +428,24 @@ __global__ void __launch_bounds__(kLT, 1) evict_large_kernel(const EvictArgs a) 
     auto post_key = [&]() {
       const unsigned long long b = shfl_min_u64(key);
       if (lane == 0 && b != ~0ull) atomicMin(&s_best[par], b);
+    };
+    // warp w < CL posts this CTA's key, candidate row and clamp count into rank w's mailbox
+    auto post_mail = [&](int nz) {
+      if (warp < CL) {
+        const unsigned long long b = s_best[par];
+        const int jb = (b == ~0ull) ? -1 : static_cast<int>(b & 0xffffffffu) - j0;
+        if (lane == 0) {
+          *cluster.map_shared_rank(&mail_key[par][rank], warp) = b;
+          *cluster.map_shared_rank(&mail_nz[par][rank], warp) = nz;
+        }
+        if (jb >= 0 && lane < G) *cluster.map_shared_rank(&mail_e[par][rank][lane], warp) = eb[(size_t)lane * es + jb];
+        if (jb >= 0 && lane < D / 4) {  // lanes 0..D/8-1 carry k, the next D/8 carry v
+          const bool is_v = lane >= D / 8;
+          const int i = is_v ? lane - D / 8 : lane;
+          const uint4 w4 = reinterpret_cast<const uint4*>((is_v ? Vr : Kr) + (size_t)jb * D)[i];
+          reinterpret_cast<uint4*>(cluster.map_shared_rank(mail_row(par, rank) + (is_v ? D : 0), warp))[i] = w4;
+        }
+      }
     };
     // ---- y_j' = y_j + (dk . k_j) dv, then ||v_j - mu_v - (scale / n) y_j||, 8 rows at a time
     for (int i0 = 0; i0 < nri; i0 += kRB) {
@@ -492,24 +501,27 @@ __global__ void __launch_bounds__(kLT, 1) evict_large_kernel(const EvictArgs a) 
     }
     post_key();
     __syncthreads();
-    const int nz = s_nz;
-    if (nz > 0) {  // uniform over the cluster: clamped entries of C' change y; score again with them
+    post_mail(s_nz);
+    cluster.sync();
+    const int my_nz = lane < CL ? mail_nz[par][lane] : 0;
+    if (__any_sync(kFull, my_nz > 0)) {  // uniform over the cluster: clamped entries of C' change y; score again
+      const int nz = __reduce_add_sync(kFull, min(my_nz, kMaxClamp + 1));
       const bool direct = nz > kMaxClamp;
-      if (tid == 0) s_best[par] = ~0ull;
-      key = ~0ull;
       float* St = a.C + (size_t)u * D * D;  // direct: S_tilde transposed, in C's memory (C is written at the end)
       if (direct) {
-        if (rank == 0) {
+        if (holds)
 #pragma unroll
-          for (int jj = 0; jj < CJ; ++jj)
-#pragma unroll
-            for (int d = 0; d < DPL; ++d) St[(size_t)(lane * DPL + d) * D + warp + kLW * jj] = creg[jj][d];
-          __threadfence();
-        }
-        cluster.sync();
-      } else {
-        __syncthreads();
+          for (int d = 0; d < DPL; ++d) St[(size_t)(lane * DPL + d) * D + arow] = creg[d];
+        __threadfence();
+      } else if (tid < nz) {  // the unit's list: rank by rank
+        int z = tid, r = 0;
+        while (z >= mail_nz[par][r]) z -= mail_nz[par][r++];
+        s_gidx[tid] = cluster.map_shared_rank(s_zidx, r)[z];
+        s_gval[tid] = cluster.map_shared_rank(s_zval, r)[z];
       }
+      if (tid == 0) s_best[par] = ~0ull;
+      key = ~0ull;
+      cluster.sync();  // lists and mailboxes read, S_tilde written
       for (int i0 = 0; i0 < nri; i0 += kRB) {
         const unsigned m = (s_alive[warp][i0 >> 5] >> (i0 & 31)) & 0xffu;
         if (m == 0u) continue;
@@ -523,9 +535,9 @@ __global__ void __launch_bounds__(kLT, 1) evict_large_kernel(const EvictArgs a) 
             if (!direct) {
               ld_vec<DPL>(Y + (size_t)r * D + lane * DPL, yc);
               for (int z = 0; z < nz; ++z) {  // y'_a -= S_tilde_ab k_b for clamped (a, b)
-                const int va = static_cast<int>(s_zidx[z] / D), kb = static_cast<int>(s_zidx[z] % D);
+                const int va = static_cast<int>(s_gidx[z] / D), kb = static_cast<int>(s_gidx[z] % D);
                 if (va / DPL == lane) {
-                  const float corr = s_zval[z] * __bfloat162float(Kr[(size_t)r * D + kb]);
+                  const float corr = s_gval[z] * __bfloat162float(Kr[(size_t)r * D + kb]);
 #pragma unroll
                   for (int d = 0; d < DPL; ++d)
                     if (va % DPL == d) yc[d] -= corr;
@@ -556,23 +568,10 @@ __global__ void __launch_bounds__(kLT, 1) evict_large_kernel(const EvictArgs a) 
       }
       post_key();
       __syncthreads();
-      if (tid == 0) s_nz = 0;  // every reader of the list is past the barrier above
+      if (tid == 0) s_nz = 0;  // the next entries are listed after the cluster barrier below
+      post_mail(0);
+      cluster.sync();
     }
-
-    // ---- warp w < CL posts this CTA's key and candidate row into rank w's mailbox
-    if (warp < CL) {
-      const unsigned long long b = s_best[par];
-      const int jb = (b == ~0ull) ? -1 : static_cast<int>(b & 0xffffffffu) - j0;
-      if (lane == 0) *cluster.map_shared_rank(&mail_key[par][rank], warp) = b;
-      if (jb >= 0 && lane < G) *cluster.map_shared_rank(&mail_e[par][rank][lane], warp) = eb[(size_t)lane * es + jb];
-      if (jb >= 0 && lane < D / 4) {  // lanes 0..D/8-1 carry k, the next D/8 carry v
-        const bool is_v = lane >= D / 8;
-        const int i = is_v ? lane - D / 8 : lane;
-        const uint4 w4 = reinterpret_cast<const uint4*>((is_v ? Vr : Kr) + (size_t)jb * D)[i];
-        reinterpret_cast<uint4*>(cluster.map_shared_rank(mail_row(par, rank) + (is_v ? D : 0), warp))[i] = w4;
-      }
-    }
-    cluster.sync();
 
     // ---- every warp: the cluster's minimum key (rows differ, so no ties), by
     // two warp-wide minimum reductions (score bits, then row)
@@ -676,21 +675,18 @@ __global__ void __launch_bounds__(kLT, 1) evict_large_kernel(const EvictArgs a) 
       if (i == 0) Pg[d] = SP[d];
     }
   }
-  // ---- the moments back: C = S_tilde / n, its rows shared out over the CTAs
+  // ---- the moments back: this CTA's rows of C = S_tilde / n
+  if (holds) {
 #pragma unroll
-  for (int jj = 0; jj < CJ; ++jj) {
-    const int row = warp + kLW * jj;
-    if (row % CL == rank) {
-      float cv[DPL];
-#pragma unroll
-      for (int d = 0; d < DPL; ++d) cv[d] = n > 0 ? creg[jj][d] / static_cast<float>(n) : 0.f;
-      st_vec<DPL>(a.C + (size_t)u * D * D + (size_t)row * D + lane * DPL, cv);
-    }
+    for (int d = 0; d < DPL; ++d) creg[d] = n > 0 ? creg[d] / static_cast<float>(n) : 0.f;
+    st_vec<DPL>(a.C + (size_t)u * D * D + (size_t)arow * D + lane * DPL, creg);
   }
   if (rank == 0 && warp == 0) {
-    st_vec<DPL>(a.mu_k + (size_t)u * D + lane * DPL, mk);
 #pragma unroll
-    for (int d = 0; d < DPL; ++d) a.mu_v[(size_t)u * D + lane * DPL + d] = mv[d];
+    for (int d = 0; d < DPL; ++d) {  // single elements: mu_k is only 8-byte aligned
+      a.mu_k[(size_t)u * D + lane * DPL + d] = mk[d];
+      a.mu_v[(size_t)u * D + lane * DPL + d] = mv[d];
+    }
     if (lane == 0) {
       a.n[u] = n;
       a.len[u] = a.budget;
@@ -754,13 +750,15 @@ cudaError_t launch_large(EvictArgs a, cudaStream_t stream) {
   cfg.blockDim = dim3(kLT, 1, 1);
   cfg.dynamicSmemBytes = lay.total;
   cfg.stream = stream;
-  cudaLaunchAttribute at[1];
+  cudaLaunchAttribute at[2];
   at[0].id = cudaLaunchAttributeClusterDimension;
   at[0].val.clusterDim.x = cl;
   at[0].val.clusterDim.y = 1;
   at[0].val.clusterDim.z = 1;
+  at[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[1].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = at;
-  cfg.numAttrs = 1;
+  cfg.numAttrs = 2;
   return cudaLaunchKernelEx(&cfg, evict_large_kernel<D, G>, a);
 }
 

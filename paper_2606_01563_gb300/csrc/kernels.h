@@ -81,8 +81,7 @@ struct EvictArgs {
   float* Yw;       // [units][cap][D] y rows that shared memory does not hold (large kernel)
   float* Y;          // optional fp32 [units][cap][D]: y_j = S_tilde k_j of each row (mkv_cache.y)
   int32_t* y_len;    // optional [units]: rows 0..y_len-1 of Y are current (mkv_cache.y_len)
-  int32_t rows_max;  // rows per CTA slice = ceil(cap / CTAs per unit)
-  int32_t kv_smem;   // register kernel: the slice's K/V rows are cached in shared memory
+  int32_t rows_max;  // large kernel: rows per CTA slice = ceil(cap / CTAs per unit)
   int32_t batch;
   int32_t n_kv;
 };
