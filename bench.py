@@ -345,11 +345,11 @@ class Run:
         self.graphs = self.graph_sets[0]
 
     def launches(self):
-        """Kernels of ours one pass launches (9 per per-unit compress, one
+        """Kernels of ours one pass launches (7 per per-unit compress, one
         pack of C' after each compress and eviction)."""
         s = self.st
         n_ev = (s.S // self.ev_every) if self.ev_every else 0
-        return s.L * (9 + 1 + s.S + 2 * n_ev)
+        return s.L * (7 + 1 + s.S + 2 * n_ev)
 
     def check_errors(self, stream):
         for ws in (self.ws_c, self.ws_d, self.ws_e):
@@ -621,7 +621,7 @@ def run_gpu(args):
         per_launch, src = dec_bytes / dec_launches, kernel_sources("decode_cl.cu")
         avg_us = tot["decode"] * 1e3 / dec_launches
     else:
-        kern, achieved = "compress (9 launches per layer)", cmp_bytes / (tot["compress"] / 1e3) / 1e9
+        kern, achieved = "compress (7 launches per layer)", cmp_bytes / (tot["compress"] / 1e3) / 1e9
         per_launch, src = cmp_bytes / (stack.L * len(runs)), kernel_sources("compress.cu")
         avg_us = tot["compress"] * 1e3 / (stack.L * len(runs))
     tr = NCU_TRAFFIC.get(kern)

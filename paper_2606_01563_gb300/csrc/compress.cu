@@ -11,23 +11,24 @@
 //   select    (8-CTA cluster per unit) R0 = protected + top-k(s): radix select
 //                            with 8-bit digits, histograms summed through
 //                            distributed shared memory, ties to the lower
-//                            position; R0's rows gathered densely
-//   stats_tc  (chunk, unit)  moments of the gathered R0 rows (no logits)
-//   finalize  (rows, unit)   M0 = moments(all) - moments(R0) (Chan merges); the
-//                            all-token record is merged once and kept
-//   residual_tc (chunk, unit) Y = K C0'^T on the tensor cores (C0' split into
-//                            three bf16 parts) -> score2 = s_t ||v - mu_v0 - scale y||
-//   select    (cluster, unit) R = protected + top-k(score2), gathered into the cache
-//   stats_tc  (chunk, unit)  moments of the retained rows
-//   finalize  (rows, unit)   moments of E = all \ R -> caller's mkv_moments
+//                            position
+//   rset      (cluster, unit) M0 = moments(all) - moments(R0): the chunk records
+//                            merged, R0's rows gathered and their co-moment
+//                            removed; C0' written as three bf16 operand parts
+//   residual_tc (chunk, unit) Y = K C0'^T on the tensor cores -> score2 =
+//                            s_t ||v - mu_v0 - scale y||
+//   select    (cluster, unit) R = protected + top-k(score2)
+//   rset      (cluster, unit) R's rows into the cache, moments of E = all \ R
+//                            into the caller's mkv_moments
+// Every launch is a programmatic dependent of the one before it: a kernel's
+// set-up, and what it reads of the prompt or of launches further back, run
+// while its predecessor drains.
 //
 // With the budget shared by the KV heads of a batch item (adaptive), each
 // select ranks the (head, position) pairs of the batch item together: a
 // per-unit select first keeps each head's own top k as candidates (the joint
 // top k lies among them) when that prunes at least half the pairs, then one
-// cluster per batch item ranks the candidates.  gather_kernel copies the
-// unequal per-head row sets, and stats_tc / gather_kernel take a grid over
-// each batch item's actual 128-row tiles.
+// cluster per batch item ranks the candidates.
 //
 // The tensor-core kernels are warp-specialised: warp 0 issues the TMA copies
 // (3-D tensor maps over per-unit slabs: rows past a unit's end read as zeros),
@@ -42,6 +43,7 @@
 #include "common.cuh"
 #include "kernels.h"
 #include "tc.cuh"
+#include "warp_mma.cuh"
 
 namespace cg = cooperative_groups;
 
@@ -64,26 +66,19 @@ struct Layout {
   int D, G, W, RW, RWb;  // head dim, group, window, window rows = G*W, 128-row blocks of them
   int T, B;
   int hs;    // units per selection group: 1, or the KV heads of a batch item (adaptive budget)
-  int Bcap;  // rows of each unit's gathered slab: B, or the adaptive maximum rounded up to kTok
   int Tc;    // joint selection entries per unit: T, or the length of its candidate list
   int units, n_chunks, chunk;
   size_t rec;         // floats per moment record: 4 + 2D + D*D (padded)
   float* rowpart;     // [units][n_chunks][RW][2]  (max in log2 units, sum)
   float* mpart;       // [units][n_chunks][rec]    all-token chunk moments
-  float* rpart;       // [units][n_rchunks][rec]   retained-set chunk moments
-  int n_rchunks;      // chunks of kTok retained rows
   float* s;           // [units][T]
   float* s2;          // [units][T]
   int32_t* idx;       // [units / hs][hs * B] selection lists (h * T + t), ascending
   int32_t* cnt;       // [units] rows each unit retains
   int32_t* cand;      // [units][Tc] per-unit candidates of a joint selection (when Tc < T)
   int32_t* hbeg;      // [units] first slot of each unit in idx
-  int32_t* tile0;     // [units / hs][hs + 1] first retained-row tile of each unit in its group (joint)
-  int gtiles;         // bound on a group's retained-row tiles (joint)
-  __nv_bfloat16* gK;  // [units][Bcap][D] rows of R0
-  __nv_bfloat16* gV;
-  float* m0;    // [units][rec] moments of E0
-  float* mall;  // [units][rec] moments of all tokens (the merged chunk records)
+  uint8_t* cimg;      // [units][3][128 x 128] C0' as three bf16 parts, in the residual's operand layout
+  float* mv0;         // [units][kDP] mu_v of E0
 };
 
 __host__ __device__ inline size_t rec_floats(int D) { return align_up(4 + 2 * (size_t)D + (size_t)D * D, 4); }
@@ -99,19 +94,15 @@ Layout make_layout(const mkv_geom& g, int T, int B, int W, int sink, int keep_wi
                    int num_sms) {
   Layout L{};
   L.hs = 1;
-  L.Bcap = B;
   L.Tc = T;
   if (adaptive && T > B) {  // a unit keeps its protected rows plus up to every joint selection
     const long prot = protected_count(T, W, sink, keep_window);
     const long most = std::min<long>(T, (long)g.n_kv_heads * (B - prot) + prot);
     L.hs = g.n_kv_heads;
-    L.Bcap = static_cast<int>((most + kTok - 1) / kTok * kTok);
     // every pair of the joint top k is in its own head's top k, so a first
     // per-unit selection of those (`most` rows with the protected ones)
     // leaves the joint one fewer entries when they are well below T
     if (2 * most <= T) L.Tc = static_cast<int>(most);
-    // sum_h ceil(c_h / kTok) with sum_h c_h = hs * B
-    L.gtiles = static_cast<int>(((long)L.hs * B + (long)L.hs * (kTok - 1)) / kTok);
   }
   L.D = g.head_dim;
   L.G = g.group;
@@ -128,7 +119,6 @@ Layout make_layout(const mkv_geom& g, int T, int B, int W, int sink, int keep_wi
   L.chunk = static_cast<int>(((tiles + per - 1) / per) * kTok);
   L.n_chunks = (T + L.chunk - 1) / L.chunk;
   L.rec = rec_floats(L.D);
-  L.n_rchunks = (L.Bcap + kTok - 1) / kTok;
   return L;
 }
 
@@ -143,23 +133,30 @@ size_t carve(Layout& L, void* ws) {
   const size_t U = L.units;
   L.rowpart = reinterpret_cast<float*>(take(U * L.n_chunks * L.RW * 2 * sizeof(float)));
   L.mpart = reinterpret_cast<float*>(take(U * L.n_chunks * L.rec * sizeof(float)));
-  L.rpart = reinterpret_cast<float*>(take(U * L.n_rchunks * L.rec * sizeof(float)));
   L.s = reinterpret_cast<float*>(take(U * (size_t)L.T * sizeof(float)));
   L.s2 = reinterpret_cast<float*>(take(U * (size_t)L.T * sizeof(float)));
   L.idx = reinterpret_cast<int32_t*>(take(U * (size_t)L.B * sizeof(int32_t)));
   L.cnt = reinterpret_cast<int32_t*>(take(U * sizeof(int32_t)));
   L.cand = L.Tc < L.T ? reinterpret_cast<int32_t*>(take(U * (size_t)L.Tc * sizeof(int32_t))) : nullptr;
   L.hbeg = reinterpret_cast<int32_t*>(take(U * sizeof(int32_t)));
-  L.tile0 = reinterpret_cast<int32_t*>(take((U / L.hs) * (size_t)(L.hs + 1) * sizeof(int32_t)));
-  L.gK = reinterpret_cast<__nv_bfloat16*>(take(U * (size_t)L.Bcap * L.D * 2));
-  L.gV = reinterpret_cast<__nv_bfloat16*>(take(U * (size_t)L.Bcap * L.D * 2));
-  L.m0 = reinterpret_cast<float*>(take(U * L.rec * sizeof(float)));
-  L.mall = reinterpret_cast<float*>(take(U * L.rec * sizeof(float)));
+  L.cimg = take(U * (size_t)3 * kTileBytes);
+  L.mv0 = reinterpret_cast<float*>(take(U * (size_t)kDP * sizeof(float)));
   return off;
 }
 
 __device__ __forceinline__ bool is_protected(int t, int T, int W, int sink, int keep_window) {
   return t < sink || (keep_window && t >= T - W);
+}
+
+// eight bf16 of a 16-byte chunk as floats
+__device__ __forceinline__ void unpack8(const uint4& w, float (&f)[8]) {
+  const uint32_t x[4] = {w.x, w.y, w.z, w.w};
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    const float2 v = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&x[i]));
+    f[2 * i] = v.x;
+    f[2 * i + 1] = v.y;
+  }
 }
 
 __device__ __forceinline__ void epi_sync() { asm volatile("bar.sync 1, 128;" ::: "memory"); }
@@ -204,9 +201,6 @@ __device__ __forceinline__ void drain_after_abort(uint64_t* full, int kS, int is
 
 struct TcArgs {
   int n_rows;  // rows of each unit's slab that take part
-  const int32_t* rows_u;  // optional per-unit row counts (<= n_rows) that replace n_rows
-  const int32_t* tile0;   // optional [groups][hs + 1]: grid (tiles of a group, groups), as in gather_kernel
-  int hs;
   int chunk;   // rows per CTA (multiple of kTok)
   int n_chunks;
   int D, RW, RWb, W, T, causal, sink, keep_window, pool;
@@ -217,57 +211,39 @@ struct TcArgs {
   const float* s_in;
   float* s_out;
   float* diag;
-  const float* m0;
+  const uint8_t* cimg;  // [units][3][128 x 128] operand image of C0'
+  const float* mv0;     // [units][kDP]
   void* ws;
   uint32_t polls;  // poll limit of the pipeline waits
 };
 
 // --------------------------------------------------------------- stats_tc
-// LOGITS = 1: window-row statistics and chunk moments of the prompt;
-// LOGITS = 0: moments only (a dense row set).
-template <int LOGITS>
+// Window-row statistics and chunk moments of the prompt.
 __global__ void __launch_bounds__(kStatsThreads, 1)
     stats_tc(const TcArgs p, const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtensorMap tmV,
              const __grid_constant__ CUtensorMap tmQ) {
-  // without logits (moments of a gathered row set, one tile per CTA): one
-  // stage, no Q, and half the TMEM, so that several CTAs share an SM
-  constexpr int kS = LOGITS ? 2 : 1;
-  constexpr uint32_t kTmemCols = LOGITS ? 512 : 256;
-  constexpr int cS = LOGITS ? 256 : 0, cSum = LOGITS ? 384 : 128;  // TMEM columns of V^T K and the sums
+  constexpr int kS = 2;
+  constexpr uint32_t kTmemCols = 512;
+  constexpr int cS = 256, cSum = 384;  // TMEM columns of V^T K and the sums
   extern __shared__ __align__(1024) uint8_t smraw[];
   uint8_t* sm = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smraw) + 1023) & ~uintptr_t(1023));
   uint8_t* sK = sm;                        // [kS][128 x 128]
   uint8_t* sV = sm + kS * kTileBytes;      // [kS][128 x 128]
   uint8_t* sQ = sm + 2 * kS * kTileBytes;  // [2 boxes][RWb*128 rows][128 B]
-  uint8_t* sOnes = sQ + (LOGITS ? 2 * 2 * kBoxBytes : 0);  // [2 boxes][16 rows][128 B] of bf16 1.0
+  uint8_t* sOnes = sQ + 2 * 2 * kBoxBytes;  // [2 boxes][16 rows][128 B] of bf16 1.0
   __shared__ __align__(8) uint64_t full[kS], empty[kS], lfull, lempty, qfull, sdone;
   __shared__ uint32_t tmem_base;
   __shared__ int abort_flag, s_issued;
   __shared__ float sum_k[kDP], sum_v[kDP];
   __shared__ float s_m1[2][128], s_l1[2][128];  // the second epilogue group's row stats
 
-  int chunk = blockIdx.x, u = blockIdx.y;
-  if (!LOGITS && p.tile0 != nullptr) {  // the group's tiles, unit by unit
-    const int32_t* t0 = p.tile0 + (size_t)blockIdx.y * (p.hs + 1);
-    if (chunk >= t0[p.hs]) return;
-    int h = 0;
-    while (h + 1 < p.hs && t0[h + 1] <= chunk) ++h;
-    u = blockIdx.y * p.hs + h;
-    chunk -= t0[h];
-  }
+  const int chunk = blockIdx.x, u = blockIdx.y;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int t_begin = chunk * p.chunk;
-  const int n_rows = (!LOGITS && p.rows_u != nullptr) ? p.rows_u[u] : p.n_rows;
-  const int t_end = min(n_rows, t_begin + p.chunk);
+  const int t_end = min(p.n_rows, t_begin + p.chunk);
   const int n_tiles = (max(0, t_end - t_begin) + kTok - 1) / kTok;
   const int RWb = p.RWb;
   volatile int* abrt = &abort_flag;
-  if (!LOGITS && n_tiles == 0) {  // a chunk past this unit's rows: an empty record (n = 0, zero means)
-    float* rec = p.mrec + ((size_t)u * p.n_chunks + chunk) * rec_floats(p.D);
-    for (int i = tid; i < 4 + 2 * p.D; i += kStatsThreads) rec[i] = 0.f;
-    return;
-  }
-
   if (tid == 0) {
     for (int i = 0; i < kS; ++i) {
       mbar_init(&full[i], 1);
@@ -291,13 +267,13 @@ __global__ void __launch_bounds__(kStatsThreads, 1)
   __syncthreads();
   tc_fence_after();
   const uint32_t tm = tmem_base;
+  grid_dependency_wait();
+  grid_launch_dependents();
 
   if (warp == 0) {
     if (lane == 0) {  // ---- producer
-      if (LOGITS) {
-        mbar_arrive_expect_tx(&qfull, 2u * RWb * kBoxBytes);
-        for (int bx = 0; bx < 2; ++bx) tma_load_3d(sQ + bx * RWb * kBoxBytes, &tmQ, bx * 64, 0, u, &qfull);
-      }
+      mbar_arrive_expect_tx(&qfull, 2u * RWb * kBoxBytes);
+      for (int bx = 0; bx < 2; ++bx) tma_load_3d(sQ + bx * RWb * kBoxBytes, &tmQ, bx * 64, 0, u, &qfull);
       for (int i = 0; i < min(kPF, n_tiles); ++i)
         for (int bx = 0; bx < 2; ++bx) {
           tma_prefetch_3d(&tmK, bx * 64, t_begin + i * kTok, u);
@@ -325,24 +301,22 @@ __global__ void __launch_bounds__(kStatsThreads, 1)
       const uint32_t idS = idesc_bf16(128, 128, 1, 1);  // V^T K: both MN-major (reduction over tokens)
       const uint32_t id1 = idesc_bf16(128, 16, 1, 0);   // X^T 1: X MN-major, ones K-major
       const uint32_t aQ = smem_addr(sQ), a1 = smem_addr(sOnes);
-      const bool ok = !LOGITS || pwait(&qfull, 0, abrt, p.ws, u, p.polls);
+      const bool ok = pwait(&qfull, 0, abrt, p.ws, u, p.polls);
       for (int i = 0; ok && i < n_tiles; ++i) {
         const int s = i % kS, j = i / kS;
         if (!pwait(&full[s], j & 1, abrt, p.ws, u, p.polls)) break;
         tc_fence_after();
         const uint32_t aK = smem_addr(sK + s * kTileBytes), aV = smem_addr(sV + s * kTileBytes);
-        if (LOGITS) {
-          if (i >= 1 && !pwait(&lempty, (i - 1) & 1, abrt, p.ws, u, p.polls)) break;
-          tc_fence_after();
-          for (int rb = 0; rb < RWb; ++rb)
-            for (int kk = 0; kk < 8; ++kk) {
-              const uint64_t dq =
-                  sdesc_sw128(aQ + (kk >> 2) * RWb * kBoxBytes + rb * kBoxBytes + (kk & 3) * 32, 16, 1024);
-              const uint64_t dk = sdesc_sw128(aK + (kk >> 2) * kBoxBytes + (kk & 3) * 32, 16, 1024);
-              umma_bf16(tm + rb * 128, dq, dk, idL, kk > 0 ? 1u : 0u);
-            }
-          umma_commit(&lfull);
-        }
+        if (i >= 1 && !pwait(&lempty, (i - 1) & 1, abrt, p.ws, u, p.polls)) break;
+        tc_fence_after();
+        for (int rb = 0; rb < RWb; ++rb)
+          for (int kk = 0; kk < 8; ++kk) {
+            const uint64_t dq =
+                sdesc_sw128(aQ + (kk >> 2) * RWb * kBoxBytes + rb * kBoxBytes + (kk & 3) * 32, 16, 1024);
+            const uint64_t dk = sdesc_sw128(aK + (kk >> 2) * kBoxBytes + (kk & 3) * 32, 16, 1024);
+            umma_bf16(tm + rb * 128, dq, dk, idL, kk > 0 ? 1u : 0u);
+          }
+        umma_commit(&lfull);
         for (int kk = 0; kk < 8; ++kk) {
           const uint64_t dv = sdesc_sw128(aV + kk * 2048, kBoxBytes, 1024);
           const uint64_t dk = sdesc_sw128(aK + kk * 2048, kBoxBytes, 1024);
@@ -369,7 +343,7 @@ __global__ void __launch_bounds__(kStatsThreads, 1)
       tmax_vis[rb] = p.causal ? p.T - p.W + r % p.W : 0x7fffffff;
     }
     const int t_safe = p.causal ? p.T - p.W : 0x7fffffff;  // tokens every window row sees
-    for (int i = 0; LOGITS && i < n_tiles; ++i) {
+    for (int i = 0; i < n_tiles; ++i) {
       if (!pwait(&lfull, i & 1, abrt, p.ws, u, p.polls)) break;
       tc_fence_after();
       const int tt0 = t_begin + i * kTok;
@@ -414,7 +388,7 @@ __global__ void __launch_bounds__(kStatsThreads, 1)
       __syncwarp();
       if (lane == 0) mbar_arrive(&lempty);
     }
-    if (LOGITS) {  // merge the two groups' (max, sum) of each row
+    {  // merge the two groups' (max, sum) of each row
       if (grp == 1)
 #pragma unroll
         for (int rb = 0; rb < 2; ++rb) {
@@ -489,7 +463,7 @@ __global__ void __launch_bounds__(kStatsThreads, 1)
   tc_fence_before();
   __syncthreads();
   if (abort_flag) {  // uniform: every role has left its loop
-    if (tid == 0) drain_after_abort(full, kS, s_issued, LOGITS ? &qfull : nullptr, &sdone);
+    if (tid == 0) drain_after_abort(full, kS, s_issued, &qfull, &sdone);
     __syncthreads();
   }
   if (warp == 1) {
@@ -540,6 +514,12 @@ __global__ void __launch_bounds__(kStatsThreads, 1)
   __syncthreads();
   tc_fence_after();
   const uint32_t tm = tmem_base;
+  // The prompt and the queries were complete before stats_tc passed its own
+  // wait, so the copies need not wait for stats_tc; its row statistics do.
+  if (warp != 0) {
+    grid_dependency_wait();
+    grid_launch_dependents();
+  }
 
   if (warp == 0) {
     if (lane == 0) {
@@ -656,7 +636,7 @@ __global__ void __launch_bounds__(kStatsThreads, 1)
   uint8_t* sK = sm;                        // [kS][128 x 128]
   uint8_t* sV = sm + kS * kTileBytes;      // [kS][128 x 128]
   uint8_t* sC = sm + 2 * kS * kTileBytes;  // [3 parts][128 x 128]: C0' = hi + mid + lo
-  __shared__ __align__(8) uint64_t full[kS], empty[kS], yfull[2], yempty[2], mma_done;
+  __shared__ __align__(8) uint64_t full[kS], empty[kS], yfull[2], yempty[2], cfull, mma_done;
   __shared__ uint32_t tmem_base;
   __shared__ int abort_flag, s_issued;
   __shared__ float s_mv[kDP];
@@ -668,7 +648,6 @@ __global__ void __launch_bounds__(kStatsThreads, 1)
   const int n_tiles = (max(0, t_end - t_begin) + kTok - 1) / kTok;
   volatile int* abrt = &abort_flag;
   const int D = p.D;
-  const float* m0 = p.m0 + (size_t)u * rec_floats(D);
 
   if (tid == 0) {
     for (int i = 0; i < kS; ++i) {
@@ -679,10 +658,12 @@ __global__ void __launch_bounds__(kStatsThreads, 1)
       mbar_init(&yfull[i], 1);
       mbar_init(&yempty[i], 4);
     }
+    mbar_init(&cfull, 1);
     mbar_init(&mma_done, 1);
     abort_flag = 0;
     mbar_fence_init();
-    // the first stages' copies go out while C0' is being prepared
+    // the first stages' copies go out before the dependency wait: the prompt
+    // was complete before the compression began
     for (int i = kS; i < min(kS + kPF, n_tiles); ++i)
       for (int bx = 0; bx < 2; ++bx) {
         tma_prefetch_3d(&tmK, bx * 64, t_begin + i * kTok, u);
@@ -698,35 +679,21 @@ __global__ void __launch_bounds__(kStatsThreads, 1)
     s_issued = min(kS, n_tiles);
   }
   if (warp == 1) tmem_alloc(&tmem_base, 256);
-  if (warp >= 2 && warp < 6) {
-    // C0' (clamped where |n0 C0| < tau) as three bf16 parts in the K-major
-    // swizzled layout: row a = value dim (N), 128-byte rows over key dims (K)
-    const int a = tid - 64;
-    const float n0 = m0[0];
-    const float tau = p.tau;
-    for (int c = 0; c < kDP; c += 2) {
-      float v0 = 0.f, v1 = 0.f;
-      if (n0 > 0.f && a < D) {
-        if (c < D) v0 = m0[4 + 2 * D + (size_t)a * D + c];
-        if (c + 1 < D) v1 = m0[4 + 2 * D + (size_t)a * D + c + 1];
-        if (fabsf(v0 * n0) < tau) v0 = 0.f;
-        if (fabsf(v1 * n0) < tau) v1 = 0.f;
-      }
-      float r0 = v0, r1 = v1;
-#pragma unroll
-      for (int part = 0; part < 3; ++part) {
-        const __nv_bfloat16 h0 = __float2bfloat16_rn(r0), h1 = __float2bfloat16_rn(r1);
-        __nv_bfloat162 hv;
-        hv.x = h0;
-        hv.y = h1;
-        *reinterpret_cast<__nv_bfloat162*>(sC + part * kTileBytes + swz_off(a, c, kTok)) = hv;
-        r0 -= __bfloat162float(h0);
-        r1 -= __bfloat162float(h1);
-      }
-    }
-    s_mv[a] = (n0 > 0.f && a < D) ? m0[4 + D + a] : 0.f;
+  if (D < kDP) {  // no second box of key dims: that part of the operand image is zero
+    for (int i = tid; i < 3 * kBoxBytes / 16; i += kStatsThreads)
+      reinterpret_cast<uint4*>(sC + (i / (kBoxBytes / 16)) * kTileBytes + kBoxBytes)[i % (kBoxBytes / 16)] =
+          make_uint4(0u, 0u, 0u, 0u);
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");  // generic writes -> tensor-core reads
   }
+  grid_dependency_wait();
+  grid_launch_dependents();
+  if (tid == 0) {  // C0' as rset_kernel left it: three bf16 parts in the operand layout
+    const uint32_t part_bytes = D < kDP ? kBoxBytes : kTileBytes;
+    mbar_arrive_expect_tx(&cfull, 3 * part_bytes);
+    for (int part = 0; part < 3; ++part)
+      bulk_g2s(sC + part * kTileBytes, p.cimg + ((size_t)u * 3 + part) * kTileBytes, part_bytes, &cfull);
+  }
+  if (tid < kDP) s_mv[tid] = p.mv0[(size_t)u * kDP + tid];
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
@@ -755,7 +722,8 @@ __global__ void __launch_bounds__(kStatsThreads, 1)
     if (lane == 0) {
       const uint32_t id = idesc_bf16(128, 128, 0, 0);
       const uint32_t aC = smem_addr(sC);
-      for (int i = 0; i < n_tiles; ++i) {
+      const bool ok = pwait(&cfull, 0, abrt, p.ws, u, p.polls);
+      for (int i = 0; ok && i < n_tiles; ++i) {
         const int s = i % kS, j = i / kS, b = i & 1;
         if (!pwait(&full[s], j & 1, abrt, p.ws, u, p.polls)) break;
         if (i >= 2 && !pwait(&yempty[b], ((i >> 1) - 1) & 1, abrt, p.ws, u, p.polls)) break;
@@ -823,7 +791,7 @@ __global__ void __launch_bounds__(kStatsThreads, 1)
   tc_fence_before();
   __syncthreads();
   // the MMA thread's final commit, and after an abort the copies in flight
-  if (tid == 0) drain_after_abort(full, kS, abort_flag ? s_issued : 0, nullptr, &mma_done);
+  if (tid == 0) drain_after_abort(full, kS, abort_flag ? s_issued : 0, &cfull, &mma_done);
   __syncthreads();
   if (warp == 1) {
     tc_fence_after();
@@ -836,10 +804,7 @@ __global__ void __launch_bounds__(kStatsThreads, 1)
 // adaptive budget the hs KV heads of a batch item, whose (head, position)
 // pairs f = h * T + t are ranked together.  R = protected + the k highest
 // keys among the other pairs (ties to the lower f), written ascending, with
-// each unit's count and first slot.  For one unit per group the kernel also
-// gathers R's rows into dst_K/dst_V [unit][dst_cap][D] (with positions when
-// the destination is a cache); a joint selection's rows are gathered by
-// gather_kernel.
+// each unit's count and first slot.
 // Exclusive block-wide prefix sum of one int per thread; *total gets the sum.
 __device__ __forceinline__ int block_excl_sum(int v, int* wsum, int* total) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -870,27 +835,17 @@ __device__ __forceinline__ int block_excl_sum(int v, int* wsum, int* total) {
 
 struct SelectArgs {
   const float* scores;  // [units][T]
-  int T, W, B, sink, keep_window, D;
-  const __nv_bfloat16* K;  // prompt [units][T][D]
-  const __nv_bfloat16* V;
+  int T, W, B, sink, keep_window;
   int32_t* idx;          // [groups][hs * B] selection lists, h * T + position, ascending (workspace)
   int32_t* diag_idx;     // optional copy
-  __nv_bfloat16* dst_K;  // optional (one unit per group): the rows are gathered here, [units][dst_cap][D]
-  __nv_bfloat16* dst_V;
-  int dst_cap;
-  int32_t* dst_pos;      // optional cache bookkeeping
-  int32_t* dst_len;
-  int32_t* dst_seen;
   int smem_keys;  // keys of a CTA's range that the dynamic shared memory holds
   int hs;         // units per selection group (1: one unit; > 1: the KV heads of a batch item)
   const int32_t* cand;  // optional [units][Tc] ascending candidate positions per unit (null: all T)
   int Tc;               // entries per unit taking part: T, or the candidate lists' length
   int32_t* cnt;    // optional [units] rows retained per unit
   int32_t* hbeg;   // optional [units] the unit's first slot in idx
-  int32_t* tile0;  // optional [groups][hs + 1] first kTok-row tile of each unit within its group, and the total
 };
 
-constexpr int kFinRB = 16;  // rows of C per finalize CTA
 constexpr int kSelCL = 8;  // CTAs per selection group (one cluster), each over a contiguous range of pairs
 constexpr int kSelSmemKeys = 49152;  // keys of a CTA's range cached in shared memory (192 KB)
 constexpr int kMaxHs = 64;           // KV heads of a batch item with the adaptive budget
@@ -907,6 +862,8 @@ __global__ void __cluster_dims__(kSelCL, 1, 1) __launch_bounds__(kSelThreads, 2)
   __shared__ int s_before[2];
   __shared__ int s_hstart[kMaxHs + 1];  // first slot of each head in the group's selection list
   __shared__ int s_hcnt[kMaxHs];        // this CTA's selections per head (read remotely)
+  grid_dependency_wait();
+  grid_launch_dependents();
   cg::cluster_group cluster = cg::this_cluster();
   const int rank = static_cast<int>(cluster.block_rank());
   const int grp = blockIdx.x / kSelCL, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -1044,7 +1001,6 @@ __global__ void __cluster_dims__(kSelCL, 1, 1) __launch_bounds__(kSelThreads, 2)
   int tb = cta_ties_before + tie_excl;
   const int my_sel = n_sure + min(max(need - tb, 0), n_tie);
   const int sel_excl = block_excl_sum(my_sel, wsum, &tot);
-  const int my_first = cta_sel_before;
   int o = cta_sel_before + sel_excl;
   const int n_sel = hs * a.B;  // the group's selections (protected included)
   int32_t* out = a.idx + (size_t)grp * n_sel;
@@ -1094,269 +1050,384 @@ __global__ void __cluster_dims__(kSelCL, 1, 1) __launch_bounds__(kSelThreads, 2)
     s_hstart[1] = a.B;
   }
   __syncthreads();
-  if (hs == 1 && a.dst_K) {
-    // gather the rows this CTA selected (16-byte chunks); a joint selection's
-    // rows are gathered by gather_kernel over the whole GPU instead
-    const int D = a.D, per_row = D / 8, u = grp;
-    const int o0 = min(my_first, n_sel), o1 = min(my_first + tot, n_sel);
-    for (int i = tid; i < (o1 - o0) * per_row; i += kSelThreads) {
-      const int r = o0 + i / per_row, c = i % per_row;
-      const int t = min(max(out[r], 0), T - 1);  // never read outside the unit's slab
-      const size_t src = ((size_t)u * T + t) * D;
-      const size_t dst = ((size_t)u * a.dst_cap + r) * D;
-      reinterpret_cast<uint4*>(a.dst_K + dst)[c] = reinterpret_cast<const uint4*>(a.K + src)[c];
-      reinterpret_cast<uint4*>(a.dst_V + dst)[c] = reinterpret_cast<const uint4*>(a.V + src)[c];
-    }
-    if (a.dst_pos)
-      for (int r = o0 + tid; r < o1; r += kSelThreads) a.dst_pos[(size_t)u * a.dst_cap + r] = out[r];
-  }
   if (rank == 0 && tid < hs) {
     const int u = grp * hs + tid, c = s_hstart[tid + 1] - s_hstart[tid];
     if (a.cnt) a.cnt[u] = c;
     if (a.hbeg) a.hbeg[u] = grp * n_sel + s_hstart[tid];
-    if (a.dst_len) {
-      a.dst_len[u] = c;
-      a.dst_seen[u] = T;
-    }
-  }
-  if (rank == 0 && tid == 0 && a.tile0) {
-    int acc = 0;
-    for (int h = 0; h < hs; ++h) {
-      a.tile0[grp * (hs + 1) + h] = acc;
-      acc += (s_hstart[h + 1] - s_hstart[h] + kTok - 1) / kTok;
-    }
-    a.tile0[grp * (hs + 1) + hs] = acc;
   }
   cluster.sync();  // no CTA leaves while another may still read its shared memory
 }
 
-// ----------------------------------------------------------------- gather
-// Copies each unit's retained rows (in list order) into dst_K/dst_V
-// [unit][dst_cap][D], one kTok-row tile per CTA, with the positions when the
-// destination is a cache.  With zero_pad the tile's rows past the unit's count
-// are written as zeros (the moments of the slab read whole tiles).  With tile0
-// the grid is (tiles of a group, groups) and each CTA finds its unit there.
-struct GatherArgs {
-  const int32_t* idx;    // selection lists, h * T + position
-  const int32_t* hbeg;   // [units] the unit's first slot in idx
-  const int32_t* cnt;    // [units] its rows
-  const int32_t* tile0;  // optional [groups][hs + 1]
-  int hs, T, D;
-  const __nv_bfloat16* K;  // prompt [units][T][D]
-  const __nv_bfloat16* V;
-  __nv_bfloat16* dst_K;
-  __nv_bfloat16* dst_V;
-  int dst_cap;
-  int32_t* dst_pos;  // optional
-  int zero_pad;
-};
-
-constexpr int kGatherThreads = 512;
-
-__global__ void __launch_bounds__(kGatherThreads) gather_kernel(const GatherArgs a) {
-  int u = blockIdx.y, tile = blockIdx.x, h = 0;
-  if (a.tile0) {
-    const int32_t* t0 = a.tile0 + (size_t)blockIdx.y * (a.hs + 1);
-    if (tile >= t0[a.hs]) return;
-    while (h + 1 < a.hs && t0[h + 1] <= tile) ++h;
-    u = blockIdx.y * a.hs + h;
-    tile -= t0[h];
-  }
-  const int c = a.cnt[u];
-  const int r0 = tile * kTok;
-  const int r1 = min(a.zero_pad ? a.dst_cap : c, r0 + kTok);
-  const int per_row = a.D / 8, per2 = 2 * per_row;  // 16-byte chunks of a row of K and V
-  const int n_items = max(0, r1 - r0) * per2;
-  const int32_t* lst = a.idx + a.hbeg[u];
-  const int hT = h * a.T;
-  constexpr int UG = 4;  // chunks in flight per thread
-  for (int base = threadIdx.x; base < n_items; base += kGatherThreads * UG) {
-    uint4 v[UG];
-    size_t dst[UG];
-    bool isV[UG];
-#pragma unroll
-    for (int q = 0; q < UG; ++q) {
-      const int i = base + q * kGatherThreads;
-      const int r = r0 + i / per2, cc = i % per2;
-      isV[q] = cc >= per_row;
-      const int ch = isV[q] ? cc - per_row : cc;
-      dst[q] = ((size_t)u * a.dst_cap + r) * a.D + ch * 8;
-      v[q] = make_uint4(0u, 0u, 0u, 0u);
-      if (i < n_items && r < c) {
-        const int t = min(max(lst[r] - hT, 0), a.T - 1);  // never read outside the unit's slab
-        const __nv_bfloat16* src = (isV[q] ? a.V : a.K) + ((size_t)u * a.T + t) * a.D + ch * 8;
-        v[q] = *reinterpret_cast<const uint4*>(src);
-      }
-    }
-#pragma unroll
-    for (int q = 0; q < UG; ++q)
-      if (base + q * kGatherThreads < n_items)
-        *reinterpret_cast<uint4*>((isV[q] ? a.dst_V : a.dst_K) + dst[q]) = v[q];
-  }
-  if (a.dst_pos)
-    for (int r = r0 + threadIdx.x; r < min(c, r0 + kTok); r += kGatherThreads)
-      a.dst_pos[(size_t)u * a.dst_cap + r] = lst[r] - hT;
-}
-
-// --------------------------------------------------------------- finalize
-// Moments of E = all \ R for kFinRB value dims (rows of C) per CTA.  Each
-// set's co-moment is the multi-way Chan merge of its chunk records, taken
-// about the first chunk's means x0 so that no global mean is needed first:
+// ------------------------------------------------------------------- rset
+// Moments of E = all \ R for the rows R a selection kept, in one kernel per
+// stage: the rows are gathered by their list straight into the tensor-core
+// operand layout (no dense copy of them), V^T K of them accumulates in TMEM,
+// and the epilogue takes their centred co-moment out of the all-token set's.
+// The first stage writes C0' as the residual pass's operand image, the final
+// one the caller's moments and, from the same tiles, the retained cache.
+//
+// Grid (CL * D/64, units), clusters of CL CTAs: CTA (rank, kh) takes the row
+// tiles rank, rank + CL, ... and the key dims [64 kh, 64 kh + 64); the CL
+// partial sums meet through distributed shared memory, each rank finishing
+// 128 / CL value dims.  A set of 128..1024 rows is one tile per CTA: the kernel
+// is a chain of round trips (list, rows, MMA, exchange), 5-7 us, where the
+// dense gather, the per-tile records and their merge took 25-40.
+//
+// The all-token co-moment is the multi-way Chan merge of the chunk records,
+// taken about the first chunk's means x0 so that no global mean is needed first:
 //   M = sum_ch [M_ch + n_ch d_ch d_ch^T] - n dbar dbar^T,  d_ch = mu_ch - x0,
 //   dbar = sum_ch n_ch d_ch / n,  mu = x0 + dbar.
+// It is merged before the dependency wait, while the selection runs: the
+// records are stats_tc's, complete before the selection's predecessor (which
+// the selection has waited for when this kernel may start) began.
 // R's centred record is then removed with the reverse pairwise formula.
-// merge_all = 1: the all-token set is the chunk records (its merge is kept
-// in L.mall); merge_all = 0: it is L.mall itself.
-//
-// Thread (row ar = tid / 16, lane group cq = tid % 16) takes the columns
-// cq*4 + 64h (h < D/64) of its row as float4s.  The counts and means of up to
-// kFinCH records of both sets are staged in one pass; then every record's
-// co-moment values are loaded with several records in flight.
-constexpr int kFinCH = 32;  // records staged per pass and set
-__global__ void __launch_bounds__(256) finalize_kernel(const Layout L, float* out_rec, mkv_moments out_mom,
-                                                       int final_out, int merge_all) {
-  constexpr int RB = kFinRB, NV = kDP / 64;  // NV float4s per thread (D = 128; one at D = 64)
-  __shared__ float s_n[2][kFinCH];
-  __shared__ __align__(16) float s_mv[2][kFinCH][RB];
-  __shared__ __align__(16) float s_mk[2][kFinCH][kDP];
-  const int D = L.D;
-  const int nv = D / 64;
-  const int rb = blockIdx.x, u = blockIdx.y, tid = threadIdx.x;
-  const size_t rf = rec_floats(D);
-  const int ar = tid / 16, cq = tid % 16;
-  const int row = rb * RB + ar;
+constexpr int kRsThreads = 256;
+constexpr int kFinCH = 32;              // chunk records staged per pass
+constexpr int kRsRed = 64 + 4;          // row stride of a CTA's partial sums (floats)
+constexpr size_t kRsSmem = 1024 + kBoxBytes + kTileBytes;  // one K half, one V tile
 
-  const int n_rec = merge_all ? L.n_chunks : 1;
-  const float* recA = merge_all ? L.mpart + (size_t)u * L.n_chunks * rf : L.mall + (size_t)u * rf;
-  const float* recR = L.rpart + (size_t)u * L.n_rchunks * rf;
-  // a joint selection leaves the unit's rows in its first ceil(cnt / kTok) records
-  const int n_rrec = L.hs > 1 ? min(L.n_rchunks, (L.cnt[u] + kTok - 1) / kTok) : L.n_rchunks;
+struct RsetArgs {
+  Layout L;
+  const __nv_bfloat16* K;  // prompt [units][T][D]
+  const __nv_bfloat16* V;
+  float tau;
+  __nv_bfloat16* dst_K;  // final stage: the cache
+  __nv_bfloat16* dst_V;
+  int dst_cap;
+  int32_t *dst_pos, *dst_len, *dst_seen;
+  mkv_moments mom;
+  void* ws;
+  uint32_t polls;
+};
 
-  struct Set {
-    float n, sv, sk[4 * NV], M[4 * NV];
-    float x0v, x0k[4 * NV];
-  };
-  Set A{}, R{};
-  auto merge = [&](Set& st, int set, const float* rbase, int g0, int nb) {
+__device__ __forceinline__ void cp_async16(void* dst, const void* src, uint32_t src_bytes) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(smem_addr(dst)), "l"(src), "r"(src_bytes)
+               : "memory");
+}
+
+template <int CL, bool FINAL>
+__global__ void __launch_bounds__(kRsThreads, 2) rset_kernel(const RsetArgs a) {
+  constexpr int NI = 8 / CL;       // value dims per thread in the merges (16 apart)
+  constexpr int RW = kDP / CL;     // value dims a rank finishes
+  extern __shared__ __align__(1024) uint8_t smraw[];
+  uint8_t* sm = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smraw) + 1023) & ~uintptr_t(1023));
+  uint8_t* sK = sm;              // [128 rows][64 key dims]
+  uint8_t* sV = sm + kBoxBytes;  // [2 boxes][128 rows][64 value dims]
+  float* red = reinterpret_cast<float*>(sm);  // [128][kRsRed] this CTA's V^T K (after the tiles)
+  __shared__ __align__(8) uint64_t done;
+  __shared__ uint32_t tmem_base;
+  __shared__ int s_ok;
+  __shared__ __align__(16) float s_pk[32][64], s_pv[16][kDP];  // column sums per row group
+  __shared__ __align__(16) float s_sk[64], s_sv[kDP];          // this CTA's column sums (read remotely)
+  const Layout& L = a.L;
+  const int D = L.D, T = L.T;
+  const int rank = blockIdx.x % CL, kh = blockIdx.x / CL, u = blockIdx.y;
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int cq = tid % 16, ar = tid / 16;  // merges: columns kh*64 + 4 cq.., value dims rank*RW + ar + 16 i
+
+  if (tid == 0) {
+    mbar_init(&done, 1);
+    mbar_fence_init();
+    s_ok = 1;
+  }
+  if (warp == 0) tmem_alloc(&tmem_base, 64);
+
+  // ---- the all-token set: this thread's elements of M and its means
+  const size_t rf = L.rec;
+  const float* recs = L.mpart + (size_t)u * L.n_chunks * rf;
+  float n = 0.f, sk[4] = {0.f, 0.f, 0.f, 0.f}, x0k[4] = {0.f, 0.f, 0.f, 0.f};
+  float sv[NI], x0v[NI], M[NI][4];
+#pragma unroll
+  for (int i = 0; i < NI; ++i) {
+    sv[i] = x0v[i] = 0.f;
+#pragma unroll
+    for (int j = 0; j < 4; ++j) M[i][j] = 0.f;
+  }
+  {
+    float* s_n = reinterpret_cast<float*>(sm);  // [kFinCH]
+    float* s_mk = s_n + kFinCH;                 // [kFinCH][64]
+    float* s_mv = s_mk + kFinCH * 64;           // [kFinCH][RW]
+    for (int g0 = 0; g0 < L.n_chunks; g0 += kFinCH) {
+      const int nb = min(kFinCH, L.n_chunks - g0);
+      if (g0 > 0) __syncthreads();
+      constexpr int per = 1 + 16 + RW / 4;  // float4s per record: n, 64 key means, RW value means
 #pragma unroll 4
-    for (int ch = 0; ch < nb; ++ch) {
-      const float* m = rbase + (size_t)(g0 + ch) * rf + 4 + 2 * D + (size_t)row * D;
-      float4 mv4[NV];
+      for (int i = tid; i < nb * per; i += kRsThreads) {
+        const int ch = i / per, j = i % per;
+        const float* r = recs + (size_t)(g0 + ch) * rf;
+        if (j == 0) {
+          s_n[ch] = r[0];
+        } else if (j <= 16) {
+          *reinterpret_cast<float4*>(s_mk + ch * 64 + (j - 1) * 4) =
+              *reinterpret_cast<const float4*>(r + 4 + kh * 64 + (j - 1) * 4);
+        } else {
+          const int c = rank * RW + (j - 17) * 4;
+          *reinterpret_cast<float4*>(s_mv + ch * RW + (j - 17) * 4) =
+              c < D ? *reinterpret_cast<const float4*>(r + 4 + D + c) : make_float4(0.f, 0.f, 0.f, 0.f);
+        }
+      }
+      __syncthreads();
+      if (g0 == 0) {
 #pragma unroll
-      for (int h = 0; h < NV; ++h)
-        mv4[h] = h < nv ? *reinterpret_cast<const float4*>(m + h * 64 + cq * 4) : make_float4(0.f, 0.f, 0.f, 0.f);
-      const float nc = s_n[set][ch];
-      if (nc > 0.f) {  // an empty record's co-moment is never written
-        const float dv = s_mv[set][ch][ar] - st.x0v;
-        st.n += nc;
-        st.sv = fmaf(nc, dv, st.sv);
+        for (int j = 0; j < 4; ++j) x0k[j] = s_mk[cq * 4 + j];
 #pragma unroll
-        for (int h = 0; h < NV; ++h) {
-          if (h >= nv) break;
-          const float4 k4 = *reinterpret_cast<const float4*>(&s_mk[set][ch][h * 64 + cq * 4]);
-          const float kk[4] = {k4.x, k4.y, k4.z, k4.w}, mm[4] = {mv4[h].x, mv4[h].y, mv4[h].z, mv4[h].w};
+        for (int i = 0; i < NI; ++i) x0v[i] = s_mv[ar + 16 * i];
+      }
+#pragma unroll(CL >= 4 ? 8 : 2)
+      for (int ch = 0; ch < nb; ++ch) {
+        const float* m = recs + (size_t)(g0 + ch) * rf + 4 + 2 * D + kh * 64 + cq * 4;
+        float4 m4[NI];
 #pragma unroll
-          for (int i = 0; i < 4; ++i) {
-            const float dk = kk[i] - st.x0k[h * 4 + i];
-            st.sk[h * 4 + i] = fmaf(nc, dk, st.sk[h * 4 + i]);
-            st.M[h * 4 + i] += mm[i] + nc * dv * dk;
+        for (int i = 0; i < NI; ++i) {
+          const int row = rank * RW + ar + 16 * i;
+          m4[i] = row < D ? *reinterpret_cast<const float4*>(m + (size_t)row * D) : make_float4(0.f, 0.f, 0.f, 0.f);
+        }
+        const float nc = s_n[ch];
+        if (nc > 0.f) {  // an empty record's co-moment is never written
+          const float4 k4 = *reinterpret_cast<const float4*>(s_mk + ch * 64 + cq * 4);
+          const float dk[4] = {k4.x - x0k[0], k4.y - x0k[1], k4.z - x0k[2], k4.w - x0k[3]};
+          n += nc;
+#pragma unroll
+          for (int j = 0; j < 4; ++j) sk[j] = fmaf(nc, dk[j], sk[j]);
+#pragma unroll
+          for (int i = 0; i < NI; ++i) {
+            const float dv = s_mv[ch * RW + ar + 16 * i] - x0v[i];
+            sv[i] = fmaf(nc, dv, sv[i]);
+            const float mm[4] = {m4[i].x, m4[i].y, m4[i].z, m4[i].w};
+#pragma unroll
+            for (int j = 0; j < 4; ++j) M[i][j] += mm[j] + nc * dv * dk[j];
           }
         }
       }
     }
-  };
-  for (int g0 = 0; g0 < max(n_rec, n_rrec); g0 += kFinCH) {
-    const int nbA = max(0, min(kFinCH, n_rec - g0)), nbR = max(0, min(kFinCH, n_rrec - g0));
-    if (g0 > 0) __syncthreads();
-    // per record: (n, ...), the CTA's RB mu_v rows and mu_k as float4s;
-    // four loads per thread in flight before their stores
-    const int per = 1 + RB / 4 + D / 4, totA = nbA * per, tot = totA + nbR * per;
-    for (int i0 = 0; i0 < tot; i0 += 4 * 256) {
-      float4 v[4];
+  }
+  __syncthreads();  // the staged records give way to the row tiles
+  if (D < kDP)      // no second box of value dims
+    for (int i = tid; i < kBoxBytes / 16; i += kRsThreads)
+      reinterpret_cast<uint4*>(sV + kBoxBytes)[i] = make_uint4(0u, 0u, 0u, 0u);
+  grid_dependency_wait();
+  grid_launch_dependents();
+
+  // ---- row tiles
+  const int cnt = L.cnt[u];
+  const int32_t* lst = L.idx + L.hbeg[u];
+  const int hT = (u % L.hs) * T;  // list entries are h * T + position
+  const int n_tiles = (cnt + kTok - 1) / kTok;
+  const __nv_bfloat16* Ku = a.K + (size_t)u * T * D + kh * 64;
+  const __nv_bfloat16* Vu = a.V + (size_t)u * T * D;
+  const uint32_t id = idesc_bf16(128, 64, 1, 1);  // V^T K: both MN-major (reduction over rows)
+  const uint32_t aK = smem_addr(sK), aV = smem_addr(sV);
+  const int vch = D / 8;  // 16-byte chunks of a value row
+  float ks[8], vs[8];     // this thread's column sums: key chunk tid % 8, value chunk tid % 16
 #pragma unroll
-      for (int k = 0; k < 4; ++k) {
-        const int i = i0 + k * 256 + tid;
-        if (i < tot) {
-          const int set = i >= totA, kk = set ? i - totA : i, ch = kk / per, j = kk % per;
-          const float* r = (set ? recR : recA) + (size_t)(g0 + ch) * rf;
-          const float* src = j == 0 ? r : (j <= RB / 4 ? r + 4 + D + rb * RB + (j - 1) * 4 : r + 4 + (j - 1 - RB / 4) * 4);
-          v[k] = *reinterpret_cast<const float4*>(src);
-        }
+  for (int j = 0; j < 8; ++j) ks[j] = vs[j] = 0.f;
+  int it = 0;
+  bool ok = true;
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  const uint32_t tm = tmem_base;
+  for (int ti = rank; ti < n_tiles; ti += CL, ++it) {
+    if (it > 0) {  // the operands are free once their MMAs have completed
+      if (tid == 0 && !mbar_wait(&done, (it - 1) & 1, a.polls)) {
+        s_ok = 0;
+        record_error(a.ws, MKV_ERR_TIMEOUT, u);
       }
+      __syncthreads();
+      ok = s_ok != 0;
+      if (!ok) break;  // uniform: s_ok changes only before a barrier
+    }
+    const int r0 = ti * kTok;
 #pragma unroll
-      for (int k = 0; k < 4; ++k) {
-        const int i = i0 + k * 256 + tid;
-        if (i < tot) {
-          const int set = i >= totA, kk = set ? i - totA : i, ch = kk / per, j = kk % per;
-          if (j == 0) s_n[set][ch] = v[k].x;
-          else if (j <= RB / 4) *reinterpret_cast<float4*>(&s_mv[set][ch][(j - 1) * 4]) = v[k];
-          else *reinterpret_cast<float4*>(&s_mk[set][ch][(j - 1 - RB / 4) * 4]) = v[k];
-        }
+    for (int j = 0; j < 4; ++j) {  // 128 rows x 8 chunks of the key half
+      const int r = tid / 8 + 32 * j, c = tid % 8;
+      const int t = r0 + r < cnt ? min(max(lst[r0 + r] - hT, 0), T - 1) : 0;  // never outside the unit's slab
+      cp_async16(sK + r * 128 + ((c ^ (r & 7)) << 4), Ku + (size_t)t * D + c * 8, r0 + r < cnt ? 16u : 0u);
+    }
+#pragma unroll
+    for (int j = 0; j < 8; ++j) {  // 128 rows x 16 chunks of the value rows
+      const int r = tid / 16 + 16 * j, c = tid % 16;
+      const int t = r0 + r < cnt ? min(max(lst[r0 + r] - hT, 0), T - 1) : 0;
+      if (c < vch)
+        cp_async16(sV + (c >> 3) * kBoxBytes + r * 128 + (((c & 7) ^ (r & 7)) << 4), Vu + (size_t)t * D + c * 8,
+                   r0 + r < cnt ? 16u : 0u);
+    }
+    asm volatile("cp.async.wait_all;" ::: "memory");
+    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");  // generic writes -> tensor-core reads
+    __syncthreads();
+    if (tid == 0) {
+      for (int kk = 0; kk < 8; ++kk)
+        umma_bf16(tm, sdesc_sw128(aV + kk * 2048, kBoxBytes, 1024), sdesc_sw128(aK + kk * 2048, kBoxBytes, 1024), id,
+                  (it > 0 || kk > 0) ? 1u : 0u);
+      umma_commit(&done);
+    }
+    // column sums, and in the final stage the cache rows, from the same tile
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      const int r = tid / 8 + 32 * j, c = tid % 8, row = r0 + r;
+      const uint4 w = *reinterpret_cast<const uint4*>(sK + r * 128 + ((c ^ (r & 7)) << 4));
+      float f[8];
+      unpack8(w, f);
+#pragma unroll
+      for (int e = 0; e < 8; ++e) ks[e] += f[e];
+      // (a joint selection's cache is zero up to the next tile past a unit's rows)
+      if (FINAL && (row < cnt || (L.hs > 1 && row < a.dst_cap)))
+        *reinterpret_cast<uint4*>(a.dst_K + ((size_t)u * a.dst_cap + row) * D + kh * 64 + c * 8) = w;
+    }
+#pragma unroll
+    for (int j = 0; j < 8; ++j) {
+      const int r = tid / 16 + 16 * j, c = tid % 16, row = r0 + r;
+      if (c < vch) {
+        const uint4 w = *reinterpret_cast<const uint4*>(sV + (c >> 3) * kBoxBytes + r * 128 + (((c & 7) ^ (r & 7)) << 4));
+        float f[8];
+        unpack8(w, f);
+#pragma unroll
+        for (int e = 0; e < 8; ++e) vs[e] += f[e];
+        if (FINAL && (c >> 3) == kh && (row < cnt || (L.hs > 1 && row < a.dst_cap)))
+          *reinterpret_cast<uint4*>(a.dst_V + ((size_t)u * a.dst_cap + row) * D + c * 8) = w;
       }
+    }
+    if (FINAL && kh == 0 && tid < kTok && r0 + tid < cnt)
+      a.dst_pos[(size_t)u * a.dst_cap + r0 + tid] = lst[r0 + tid] - hT;
+  }
+  // ---- this CTA's sums and V^T K into shared memory
+  if (it > 0 && ok) {
+    if (tid == 0 && !mbar_wait(&done, (it - 1) & 1, a.polls)) {
+      s_ok = 0;
+      record_error(a.ws, MKV_ERR_TIMEOUT, u);
     }
     __syncthreads();
-    if (g0 == 0) {  // the first record's means (zero when a set has none)
-      A.x0v = nbA > 0 ? s_mv[0][0][ar] : 0.f;
-      R.x0v = nbR > 0 ? s_mv[1][0][ar] : 0.f;
-#pragma unroll
-      for (int h = 0; h < NV; ++h)
-#pragma unroll
-        for (int i = 0; i < 4; ++i) {
-          const int c = h * 64 + cq * 4 + i;
-          A.x0k[h * 4 + i] = (nbA > 0 && h < nv) ? s_mk[0][0][c] : 0.f;
-          R.x0k[h * 4 + i] = (nbR > 0 && h < nv) ? s_mk[1][0][c] : 0.f;
-        }
-    }
-    merge(A, 0, recA, g0, nbA);
-    merge(R, 1, recR, g0, nbR);
+    ok = s_ok != 0;
   }
+  if (!ok && tid == 0) (void)mbar_wait(&done, (it - 1) & 1);  // drain: the MMAs still read shared memory
+  __syncthreads();
+  tc_fence_after();
+#pragma unroll
+  for (int e = 0; e < 8; ++e) {
+    s_pk[tid / 8][(tid % 8) * 8 + e] = ks[e];
+    s_pv[tid / 16][(tid % 16) * 8 + e] = vs[e];
+  }
+  {
+    float x[32];
+    const int row = (warp & 3) * 32 + lane, c0 = (warp >> 2) * 32;
+    if (it > 0 && ok) {
+      tmem_ld32(tm + (static_cast<uint32_t>((warp & 3) * 32) << 16) + c0, x);
+    } else {
+#pragma unroll
+      for (int j = 0; j < 32; ++j) x[j] = 0.f;
+    }
+#pragma unroll
+    for (int j = 0; j < 32; j += 4)
+      *reinterpret_cast<float4*>(red + row * kRsRed + c0 + j) = make_float4(x[j], x[j + 1], x[j + 2], x[j + 3]);
+  }
+  tc_fence_before();
+  __syncthreads();
+  if (warp == 0) {
+    tc_fence_after();
+    tmem_dealloc(tm, 64);
+  }
+  if (tid < 64) {
+    float x = 0.f;
+    for (int g = 0; g < 32; ++g) x += s_pk[g][tid];
+    s_sk[tid] = x;
+  } else if (tid < 64 + kDP) {
+    float x = 0.f;
+    for (int g = 0; g < 16; ++g) x += s_pv[g][tid - 64];
+    s_sv[tid - 64] = x;
+  }
+  cg::cluster_group cluster = cg::this_cluster();
+  if constexpr (CL > 1) cluster.sync();
+  else __syncthreads();
 
-  const float n = A.n, nR = R.n, nE = n - nR;
-  const float mv = A.x0v + A.sv / n;
-  const float mvR = nR > 0.f ? R.x0v + R.sv / nR : 0.f;
-  const float mvE = nE > 0.f ? (n * mv - nR * mvR) / nE : 0.f;
-  float* mall = L.mall + (size_t)u * rf;
-  float* o = final_out ? nullptr : out_rec + (size_t)u * rf;
+  // ---- R's sums over the cluster, and E = all \ R
+  const float nR = ok ? static_cast<float>(cnt) : 0.f;
+  float SR[NI][4], rv[NI], rk[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll
-  for (int h = 0; h < NV; ++h) {
-    if (h >= nv) break;
-    float Mo[4], CE[4];
+  for (int i = 0; i < NI; ++i) {
+    rv[i] = 0.f;
 #pragma unroll
-    for (int i = 0; i < 4; ++i) {
-      const int j = h * 4 + i, c = h * 64 + cq * 4 + i;
-      const float mk = A.x0k[j] + A.sk[j] / n;
-      const float M = A.M[j] - A.sv * A.sk[j] / n;
-      const float mkR = nR > 0.f ? R.x0k[j] + R.sk[j] / nR : 0.f;
-      const float MR = nR > 0.f ? R.M[j] - R.sv * R.sk[j] / nR : 0.f;
-      Mo[i] = M;
-      CE[i] = 0.f;
-      float mkE = 0.f;
+    for (int j = 0; j < 4; ++j) SR[i][j] = 0.f;
+  }
+#pragma unroll
+  for (int r = 0; r < CL; ++r) {
+    const float* pr = CL > 1 ? cluster.map_shared_rank(red, r) : red;
+    const float* pk = CL > 1 ? cluster.map_shared_rank(s_sk, r) : s_sk;
+    const float* pv = CL > 1 ? cluster.map_shared_rank(s_sv, r) : s_sv;
+    const float4 k4 = *reinterpret_cast<const float4*>(pk + cq * 4);
+    rk[0] += k4.x;
+    rk[1] += k4.y;
+    rk[2] += k4.z;
+    rk[3] += k4.w;
+#pragma unroll
+    for (int i = 0; i < NI; ++i) {
+      const int row = rank * RW + ar + 16 * i;
+      const float4 s4 = *reinterpret_cast<const float4*>(pr + row * kRsRed + cq * 4);
+      SR[i][0] += s4.x;
+      SR[i][1] += s4.y;
+      SR[i][2] += s4.z;
+      SR[i][3] += s4.w;
+      rv[i] += pv[row];
+    }
+  }
+  const float nE = n - nR;
+  float mk[4], mkR[4], mkE[4];
+#pragma unroll
+  for (int j = 0; j < 4; ++j) {
+    mk[j] = x0k[j] + sk[j] / n;
+    mkR[j] = nR > 0.f ? rk[j] / nR : 0.f;
+    mkE[j] = nE > 0.f ? (n * mk[j] - nR * mkR[j]) / nE : 0.f;
+  }
+#pragma unroll
+  for (int i = 0; i < NI; ++i) {
+    const int row = rank * RW + ar + 16 * i;
+    const float mv = x0v[i] + sv[i] / n;
+    const float mvR = nR > 0.f ? rv[i] / nR : 0.f;
+    const float mvE = nE > 0.f ? (n * mv - nR * mvR) / nE : 0.f;
+    float CE[4];
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      CE[j] = 0.f;
       if (nE > 0.f) {
-        mkE = (n * mk - nR * mkR) / nE;
-        const float ME = M - MR - (nE * nR / n) * (mvR - mvE) * (mkR - mkE);
-        CE[i] = ME / nE;
-      }
-      if (rb == 0 && ar == 0) {  // the k means: row 0's threads
-        if (merge_all) mall[4 + c] = mk;
-        if (final_out) out_mom.mu_k[(size_t)u * D + c] = mkE;
-        else o[4 + c] = mkE;
+        const float Mall = M[i][j] - sv[i] * sk[j] / n;
+        const float MR = nR > 0.f ? SR[i][j] - rv[i] * rk[j] / nR : 0.f;
+        const float ME = Mall - MR - (nE * nR / n) * (mvR - mvE) * (mkR[j] - mkE[j]);
+        CE[j] = ME / nE;
       }
     }
-    const size_t e = (size_t)row * D + h * 64 + cq * 4;
-    if (merge_all) *reinterpret_cast<float4*>(mall + 4 + 2 * D + e) = make_float4(Mo[0], Mo[1], Mo[2], Mo[3]);
-    if (final_out) *reinterpret_cast<float4*>(out_mom.C + (size_t)u * D * D + e) = make_float4(CE[0], CE[1], CE[2], CE[3]);
-    else *reinterpret_cast<float4*>(o + 4 + 2 * D + e) = make_float4(CE[0], CE[1], CE[2], CE[3]);
+    if constexpr (FINAL) {
+      if (row < D) {
+        *reinterpret_cast<float4*>(a.mom.C + ((size_t)u * D + row) * D + kh * 64 + cq * 4) =
+            make_float4(CE[0], CE[1], CE[2], CE[3]);
+        if (kh == 0 && cq == 0) a.mom.mu_v[(size_t)u * D + row] = mvE;
+        if (row == 0)
+#pragma unroll
+          for (int j = 0; j < 4; ++j) a.mom.mu_k[(size_t)u * D + kh * 64 + cq * 4 + j] = mkE[j];
+      }
+    } else {
+      // C0' (clamped where |n0 C0| < tau) as three bf16 parts, K-major operand
+      // rows (value dims; zero past D) in the swizzled layout
+      float r4[4];
+#pragma unroll
+      for (int j = 0; j < 4; ++j) r4[j] = (row < D && !(fabsf(CE[j] * nE) < a.tau)) ? CE[j] : 0.f;
+      uint8_t* img = L.cimg + (size_t)u * 3 * kTileBytes + swz_off(row, kh * 64 + cq * 4, kTok);
+#pragma unroll
+      for (int part = 0; part < 3; ++part) {
+        uint2 w;
+        w.x = pack_bf16x2(r4[0], r4[1]);
+        w.y = pack_bf16x2(r4[2], r4[3]);
+        *reinterpret_cast<uint2*>(img + (size_t)part * kTileBytes) = w;
+#pragma unroll
+        for (int j = 0; j < 4; ++j) r4[j] = bf16_residual(r4[j]);
+      }
+      if (kh == 0 && cq == 0) L.mv0[(size_t)u * kDP + row] = row < D ? mvE : 0.f;
+    }
   }
-  if (cq == 0) {  // the v means: one thread per row
-    if (merge_all) mall[4 + D + row] = mv;
-    if (final_out) out_mom.mu_v[(size_t)u * D + row] = mvE;
-    else o[4 + D + row] = mvE;
+  if (FINAL && kh == 0 && rank == 0 && tid == 0) {
+    a.mom.n[u] = static_cast<int32_t>(nE);
+    a.dst_len[u] = cnt;
+    a.dst_seen[u] = T;
   }
-  if (rb == 0 && tid == 0) {
-    if (merge_all) mall[0] = n;
-    if (final_out) out_mom.n[u] = static_cast<int32_t>(nE);
-    else o[0] = nE;
-  }
+  if constexpr (CL > 1) cluster.sync();  // no CTA leaves while another reads its shared memory
 }
 
 // ---------------------------------------------------------- keep-all path
@@ -1392,41 +1463,82 @@ __global__ void __launch_bounds__(256) keep_all_kernel(const CompressArgs a, int
 
 // ------------------------------------------------------------------- host
 constexpr size_t kStatsSmem = 1024 + 2 * 2 * kTileBytes + 2 * 2 * kBoxBytes + 4096;  // K, V stages, Q, ones
-constexpr size_t kStats0Smem = 1024 + 2 * kTileBytes + 4096;                            // one K, V stage, ones
 constexpr size_t kScoresSmem = 1024 + 3 * kTileBytes + 2 * 2 * kBoxBytes;
 constexpr size_t kResidualSmem = 1024 + 2 * 2 * kTileBytes + 3 * kTileBytes;
+
+// A launch that may begin while the kernel before it on the stream drains (it
+// waits for that kernel's end by itself); cl > 0: in clusters of cl CTAs
+// (select_kernel declares its own).
+template <typename... P, typename... A>
+cudaError_t launch_pdl(void (*f)(P...), dim3 grid, int threads, size_t smem, cudaStream_t st, int cl, A&&... args) {
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = grid;
+  cfg.blockDim = dim3(threads, 1, 1);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cudaLaunchAttribute at[2];
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  at[1].id = cudaLaunchAttributeClusterDimension;
+  at[1].val.clusterDim.x = cl;
+  at[1].val.clusterDim.y = 1;
+  at[1].val.clusterDim.z = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = cl > 0 ? 2 : 1;
+  return cudaLaunchKernelEx(&cfg, f, std::forward<A>(args)...);
+}
+
+cudaError_t smem_attr(const void* f, size_t bytes) {
+  return cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(bytes));
+}
+
+// CTAs per unit and key half of rset_kernel: one row tile each, and no more
+// chunk records to merge than about 300 KB, as long as all CTAs run at once
+// (two per SM).
+int rset_cluster(const Layout& L, int num_sms) {
+  const long tiles = (L.B + kTok - 1) / kTok, nh = L.D / 64;
+  const long want = std::max(tiles, (long)L.n_chunks / 9);
+  int cl = 1;
+  while (cl < 8 && cl < want && 2L * cl * nh * L.units <= 2L * num_sms) cl *= 2;
+  return cl;
+}
+
+template <bool FINAL>
+cudaError_t launch_rset(const RsetArgs& a, int cl, cudaStream_t st) {
+  const dim3 grid(cl * (a.L.D / 64), a.L.units);
+  auto go = [&](void (*f)(RsetArgs)) -> cudaError_t {
+    const cudaError_t e = smem_attr(reinterpret_cast<const void*>(f), kRsSmem);
+    return e != cudaSuccess ? e : launch_pdl(f, grid, kRsThreads, kRsSmem, st, cl, a);
+  };
+  switch (cl) {
+    case 8: return go(rset_kernel<8, FINAL>);
+    case 4: return go(rset_kernel<4, FINAL>);
+    case 2: return go(rset_kernel<2, FINAL>);
+    default: return go(rset_kernel<1, FINAL>);
+  }
+}
 
 cudaError_t run(const CompressArgs& a, const mkv_geom& g, int num_sms, cudaStream_t st) {
   Layout L = make_layout(g, a.T, a.budget, a.window, a.sink, a.keep_window, a.adaptive, num_sms);
   carve(L, a.ws);
-  const int D = g.head_dim, T = a.T, B = a.budget, U = L.units, Bc = L.Bcap;
-  const bool joint = L.hs > 1;
+  const int D = g.head_dim, T = a.T, B = a.budget, U = L.units;
   const bool keep_all = T <= B;
   cudaError_t e = cudaSuccess;
-  auto attr = [](const void* f, size_t bytes) {
-    return cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(bytes));
-  };
-  if ((e = attr((const void*)stats_tc<1>, kStatsSmem)) != cudaSuccess) return e;
-  if ((e = attr((const void*)stats_tc<0>, kStats0Smem)) != cudaSuccess) return e;
-  if ((e = attr((const void*)scores_tc, kScoresSmem)) != cudaSuccess) return e;
-  if ((e = attr((const void*)residual_tc, kResidualSmem)) != cudaSuccess) return e;
+  if ((e = smem_attr((const void*)stats_tc, kStatsSmem)) != cudaSuccess) return e;
+  if ((e = smem_attr((const void*)scores_tc, kScoresSmem)) != cudaSuccess) return e;
+  if ((e = smem_attr((const void*)residual_tc, kResidualSmem)) != cudaSuccess) return e;
 
-  CUtensorMap tmK, tmV, tmQ, tmGK, tmGV, tmCK, tmCV;
+  CUtensorMap tmK, tmV, tmQ;
   const uint64_t rs = (uint64_t)D * 2;
-  bool ok = encode_tmap_bf16_3d(&tmK, a.K, D, T, U, rs, (uint64_t)T * rs, kTok) &&
-            encode_tmap_bf16_3d(&tmV, a.V, D, T, U, rs, (uint64_t)T * rs, kTok) &&
-            encode_tmap_bf16_3d(&tmQ, a.Q, D, L.RW, U, rs, (uint64_t)L.RW * rs, L.RWb * 128);
-  // the retained rows: B per unit, or (joint) up to the capacity with the
-  // rows past each unit's count zero up to the tile (or outside the map)
-  const int cache_rows = joint ? a.cache.capacity : B;
-  if (!keep_all)
-    ok = ok && encode_tmap_bf16_3d(&tmGK, L.gK, D, Bc, U, rs, (uint64_t)Bc * rs, kTok) &&
-         encode_tmap_bf16_3d(&tmGV, L.gV, D, Bc, U, rs, (uint64_t)Bc * rs, kTok) &&
-         encode_tmap_bf16_3d(&tmCK, a.cache.K, D, cache_rows, U, rs, (uint64_t)a.cache.capacity * rs, kTok) &&
-         encode_tmap_bf16_3d(&tmCV, a.cache.V, D, cache_rows, U, rs, (uint64_t)a.cache.capacity * rs, kTok);
-  if (!ok) return cudaErrorInvalidValue;
+  if (!encode_tmap_bf16_3d(&tmK, a.K, D, T, U, rs, (uint64_t)T * rs, kTok) ||
+      !encode_tmap_bf16_3d(&tmV, a.V, D, T, U, rs, (uint64_t)T * rs, kTok) ||
+      !encode_tmap_bf16_3d(&tmQ, a.Q, D, L.RW, U, rs, (uint64_t)L.RW * rs, L.RWb * 128))
+    return cudaErrorInvalidValue;
 
   TcArgs tp{};
+  tp.n_rows = T;
+  tp.chunk = L.chunk;
+  tp.n_chunks = L.n_chunks;
   tp.D = D;
   tp.RW = L.RW;
   tp.RWb = L.RWb;
@@ -1437,23 +1549,18 @@ cudaError_t run(const CompressArgs& a, const mkv_geom& g, int num_sms, cudaStrea
   tp.keep_window = a.keep_window;
   tp.pool = a.pool;
   tp.qscale = rsqrtf(static_cast<float>(D)) * kLog2e;
-  tp.tau = a.tau;
+  tp.rowpart = L.rowpart;
+  tp.mrec = L.mpart;
   tp.ws = a.ws;
   tp.polls = pipeline_poll_limit();
   const dim3 cg(L.n_chunks, U);
 
   if (!keep_all || a.diag_scores != nullptr) {
-    TcArgs p1 = tp;
-    p1.n_rows = T;
-    p1.chunk = L.chunk;
-    p1.n_chunks = L.n_chunks;
-    p1.rowpart = L.rowpart;
-    p1.mrec = L.mpart;
-    stats_tc<1><<<cg, kStatsThreads, kStatsSmem, st>>>(p1, tmK, tmV, tmQ);
-    TcArgs p2 = p1;
+    if ((e = launch_pdl(stats_tc, cg, kStatsThreads, kStatsSmem, st, 0, tp, tmK, tmV, tmQ)) != cudaSuccess) return e;
+    TcArgs p2 = tp;
     p2.s_out = L.s;
     p2.diag = a.diag_scores;
-    scores_tc<<<cg, kStatsThreads, kScoresSmem, st>>>(p2, tmK, tmQ);
+    if ((e = launch_pdl(scores_tc, cg, kStatsThreads, kScoresSmem, st, 0, p2, tmK, tmQ)) != cudaSuccess) return e;
   }
   if (keep_all) {
     if (D == 128) keep_all_kernel<128><<<dim3((T + 7) / 8, U), 256, 0, st>>>(a, T);
@@ -1469,7 +1576,7 @@ cudaError_t run(const CompressArgs& a, const mkv_geom& g, int num_sms, cudaStrea
   sa.smem_keys = cached_keys((L.hs * (long)L.Tc + kSelCL - 1) / kSelCL);
   const int pf_keys = cached_keys((T + kSelCL - 1) / kSelCL);
   const size_t sel_smem = (size_t)sa.smem_keys * sizeof(uint32_t), pf_smem = (size_t)pf_keys * sizeof(uint32_t);
-  if ((e = attr((const void*)select_kernel, std::max(sel_smem, pf_smem))) != cudaSuccess) return e;
+  if ((e = smem_attr((const void*)select_kernel, std::max(sel_smem, pf_smem))) != cudaSuccess) return e;
   sa.T = T;
   sa.Tc = L.Tc;
   sa.cand = L.cand;
@@ -1477,103 +1584,61 @@ cudaError_t run(const CompressArgs& a, const mkv_geom& g, int num_sms, cudaStrea
   sa.B = B;
   sa.sink = a.sink;
   sa.keep_window = a.keep_window;
-  sa.D = D;
-  sa.K = static_cast<const __nv_bfloat16*>(a.K);
-  sa.V = static_cast<const __nv_bfloat16*>(a.V);
   sa.idx = L.idx;
   sa.hs = L.hs;
   sa.cnt = L.cnt;
   sa.hbeg = L.hbeg;
-  sa.tile0 = joint ? L.tile0 : nullptr;
-  // the candidates of a joint selection over `scores`: each unit's protected
-  // rows and its top Tc - |protected| (a per-unit selection)
-  auto prefilter_launch = [&](const float* scores) {
-    if (!prefilter) return;
-    SelectArgs pf = sa;
-    pf.scores = scores;
-    pf.hs = 1;
-    pf.Tc = T;
-    pf.cand = nullptr;
-    pf.B = L.Tc;
-    pf.idx = L.cand;
-    pf.smem_keys = pf_keys;
-    pf.cnt = nullptr;
-    pf.hbeg = nullptr;
-    pf.tile0 = nullptr;
-    select_kernel<<<U * kSelCL, kSelThreads, pf_smem, st>>>(pf);
-  };
-  // the retained rows' tiles: (chunks, units), or (a group's tiles, groups)
-  const dim3 tiles = joint ? dim3(L.gtiles, n_groups) : dim3(L.n_rchunks, U);
-  GatherArgs ga{};
-  ga.idx = L.idx;
-  ga.hbeg = L.hbeg;
-  ga.cnt = L.cnt;
-  ga.tile0 = sa.tile0;
-  ga.hs = L.hs;
-  ga.T = T;
-  ga.D = D;
-  ga.K = sa.K;
-  ga.V = sa.V;
-  ga.zero_pad = joint ? 1 : 0;
-  TcArgs rset = tp;  // moments of a dense row set: chunks of kTok rows
-  rset.n_rows = Bc;
-  rset.rows_u = joint ? L.cnt : nullptr;
-  rset.tile0 = sa.tile0;
-  rset.hs = L.hs;
-  rset.chunk = kTok;
-  rset.n_chunks = L.n_rchunks;
-  rset.mrec = L.rpart;
-
-  if (a.mi) {
-    SelectArgs s0 = sa;
-    s0.scores = L.s;
-    s0.diag_idx = a.diag_idx1;
-    GatherArgs g0 = ga;
-    g0.dst_K = L.gK;
-    g0.dst_V = L.gV;
-    g0.dst_cap = Bc;
-    if (!joint) {
-      s0.dst_K = g0.dst_K;
-      s0.dst_V = g0.dst_V;
-      s0.dst_cap = g0.dst_cap;
+  // one selection over `scores`; a joint one first keeps each unit's protected
+  // rows and its top Tc - |protected| as candidates (a per-unit selection)
+  auto select = [&](const float* scores, int32_t* diag_idx) -> cudaError_t {
+    if (prefilter) {
+      SelectArgs pf = sa;
+      pf.scores = scores;
+      pf.hs = 1;
+      pf.Tc = T;
+      pf.cand = nullptr;
+      pf.B = L.Tc;
+      pf.idx = L.cand;
+      pf.smem_keys = pf_keys;
+      pf.cnt = nullptr;
+      pf.hbeg = nullptr;
+      const cudaError_t pe = launch_pdl(select_kernel, dim3(U * kSelCL), kSelThreads, pf_smem, st, 0, pf);
+      if (pe != cudaSuccess) return pe;
     }
-    prefilter_launch(L.s);
-    select_kernel<<<n_groups * kSelCL, kSelThreads, sel_smem, st>>>(s0);
-    if (joint) gather_kernel<<<tiles, kGatherThreads, 0, st>>>(g0);
-    stats_tc<0><<<tiles, kStatsThreads, kStats0Smem, st>>>(rset, tmGK, tmGV, tmQ);
-    finalize_kernel<<<dim3(D / kFinRB, U), 256, 0, st>>>(L, L.m0, a.mom, 0, 1);
+    SelectArgs s0 = sa;
+    s0.scores = scores;
+    s0.diag_idx = diag_idx;
+    return launch_pdl(select_kernel, dim3(n_groups * kSelCL), kSelThreads, sel_smem, st, 0, s0);
+  };
+  RsetArgs ra{};
+  ra.L = L;
+  ra.K = static_cast<const __nv_bfloat16*>(a.K);
+  ra.V = static_cast<const __nv_bfloat16*>(a.V);
+  ra.tau = a.tau;
+  ra.dst_K = static_cast<__nv_bfloat16*>(a.cache.K);
+  ra.dst_V = static_cast<__nv_bfloat16*>(a.cache.V);
+  ra.dst_cap = a.cache.capacity;
+  ra.dst_pos = a.cache.pos;
+  ra.dst_len = a.cache.len;
+  ra.dst_seen = a.cache.seen;
+  ra.mom = a.mom;
+  ra.ws = a.ws;
+  ra.polls = tp.polls;
+  const int cl = rset_cluster(L, num_sms);
+
+  if ((e = select(L.s, a.diag_idx1)) != cudaSuccess) return e;
+  if (a.mi) {
+    if ((e = launch_rset<false>(ra, cl, st)) != cudaSuccess) return e;
     TcArgs r = tp;
-    r.n_rows = T;
-    r.chunk = L.chunk;
-    r.n_chunks = L.n_chunks;
-    r.m0 = L.m0;
+    r.cimg = L.cimg;
+    r.mv0 = L.mv0;
     r.s_in = L.s;
     r.s_out = L.s2;
     r.diag = a.diag_score2;
-    residual_tc<<<cg, kStatsThreads, kResidualSmem, st>>>(r, tmK, tmV);
+    if ((e = launch_pdl(residual_tc, cg, kStatsThreads, kResidualSmem, st, 0, r, tmK, tmV)) != cudaSuccess) return e;
+    if ((e = select(L.s2, nullptr)) != cudaSuccess) return e;
   }
-  SelectArgs s1 = sa;
-  s1.scores = a.mi ? L.s2 : L.s;
-  s1.diag_idx = a.mi ? nullptr : a.diag_idx1;
-  s1.dst_len = a.cache.len;
-  s1.dst_seen = a.cache.seen;
-  GatherArgs g1 = ga;
-  g1.dst_K = static_cast<__nv_bfloat16*>(a.cache.K);
-  g1.dst_V = static_cast<__nv_bfloat16*>(a.cache.V);
-  g1.dst_cap = a.cache.capacity;
-  g1.dst_pos = a.cache.pos;
-  if (!joint) {
-    s1.dst_K = g1.dst_K;
-    s1.dst_V = g1.dst_V;
-    s1.dst_cap = g1.dst_cap;
-    s1.dst_pos = g1.dst_pos;
-  }
-  prefilter_launch(s1.scores);
-  select_kernel<<<n_groups * kSelCL, kSelThreads, sel_smem, st>>>(s1);
-  if (joint) gather_kernel<<<tiles, kGatherThreads, 0, st>>>(g1);
-  stats_tc<0><<<tiles, kStatsThreads, kStats0Smem, st>>>(rset, tmCK, tmCV, tmQ);
-  finalize_kernel<<<dim3(D / kFinRB, U), 256, 0, st>>>(L, nullptr, a.mom, 1, a.mi ? 0 : 1);
-  return cudaGetLastError();
+  return launch_rset<true>(ra, cl, st);
 }
 
 }  // namespace

@@ -150,9 +150,9 @@ def test_clock_samples_and_throttle_reasons():
 
 class _CountingBinding:
     """Stands in for the binding: counts the kernels each entry point launches
-    (a per-unit compress with T > budget: 9; a decode step, an eviction and a
+    (a per-unit compress with T > budget: 7; a decode step, an eviction and a
     pack of C': 1 each)."""
-    KERNELS = {"mkv_compress": 9, "mkv_decode_step": 1, "mkv_evict_append": 1, "mkv_moments_pack_split": 1}
+    KERNELS = {"mkv_compress": 7, "mkv_decode_step": 1, "mkv_evict_append": 1, "mkv_moments_pack_split": 1}
 
     def __init__(self):
         self.launched = 0
