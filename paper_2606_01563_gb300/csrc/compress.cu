@@ -8,10 +8,9 @@
 //                            sums -> the chunk's centred moments
 //   scores_tc (chunk, unit)  logits again (token-major) -> s_t = sum over rows
 //                            of exp(l - m_row) / l_row, pooled
-//   select    (8-CTA cluster per unit) R0 = protected + top-k(s): radix select
-//                            with 8-bit digits, histograms summed through
-//                            distributed shared memory, ties to the lower
-//                            position
+//   select    (8-CTA cluster per unit) R0 = protected + top-k(s): the bin of the
+//                            k-th key from counts the score kernels keep, the
+//                            bin's keys ranked, ties to the lower position
 //   rset      (cluster, unit) M0 = moments(all) - moments(R0): the chunk records
 //                            merged, R0's rows gathered and their co-moment
 //                            removed; C0' written as three bf16 operand parts
@@ -25,10 +24,7 @@
 // while its predecessor drains.
 //
 // With the budget shared by the KV heads of a batch item (adaptive), each
-// select ranks the (head, position) pairs of the batch item together: a
-// per-unit select first keeps each head's own top k as candidates (the joint
-// top k lies among them) when that prunes at least half the pairs, then one
-// cluster per batch item ranks the candidates.
+// select ranks the (head, position) pairs of the batch item together.
 //
 // The tensor-core kernels are warp-specialised: warp 0 issues the TMA copies
 // (3-D tensor maps over per-unit slabs: rows past a unit's end read as zeros),
@@ -58,7 +54,7 @@ constexpr int kBoxBytes = kTok * 128;
 // stats_tc: two epilogue groups of 4 warps (2..5 and 6..9), each taking half
 // of a tile's tokens, so that two warps per scheduler share the softmax work
 constexpr int kStatsThreads = 320;
-constexpr int kSelThreads = 1024;
+constexpr int kBins = 2048;  // bins of the scores' keys (select_kernel)
 constexpr int kPF = 0;  // tiles prefetched into L2 ahead of the one being loaded (0: none)
 constexpr unsigned kFull = 0xffffffffu;
 
@@ -66,7 +62,6 @@ struct Layout {
   int D, G, W, RW, RWb;  // head dim, group, window, window rows = G*W, 128-row blocks of them
   int T, B;
   int hs;    // units per selection group: 1, or the KV heads of a batch item (adaptive budget)
-  int Tc;    // joint selection entries per unit: T, or the length of its candidate list
   int units, n_chunks, chunk;
   size_t rec;         // floats per moment record: 4 + 2D + D*D (padded)
   float* rowpart;     // [units][n_chunks][RW][2]  (max in log2 units, sum)
@@ -75,7 +70,7 @@ struct Layout {
   float* s2;          // [units][T]
   int32_t* idx;       // [units / hs][hs * B] selection lists (h * T + t), ascending
   int32_t* cnt;       // [units] rows each unit retains
-  int32_t* cand;      // [units][Tc] per-unit candidates of a joint selection (when Tc < T)
+  uint32_t* hist;     // [2][units][kBins] keys of the unprotected scores per bin (s, s2)
   int32_t* hbeg;      // [units] first slot of each unit in idx
   uint8_t* cimg;      // [units][3][128 x 128] C0' as three bf16 parts, in the residual's operand layout
   float* mv0;         // [units][kDP] mu_v of E0
@@ -90,20 +85,10 @@ __host__ __device__ __forceinline__ int protected_count(int T, int W, int sink, 
   return s + w - overlap;
 }
 
-Layout make_layout(const mkv_geom& g, int T, int B, int W, int sink, int keep_window, int adaptive,
-                   int num_sms) {
+Layout make_layout(const mkv_geom& g, int T, int B, int W, int adaptive, int num_sms) {
   Layout L{};
   L.hs = 1;
-  L.Tc = T;
-  if (adaptive && T > B) {  // a unit keeps its protected rows plus up to every joint selection
-    const long prot = protected_count(T, W, sink, keep_window);
-    const long most = std::min<long>(T, (long)g.n_kv_heads * (B - prot) + prot);
-    L.hs = g.n_kv_heads;
-    // every pair of the joint top k is in its own head's top k, so a first
-    // per-unit selection of those (`most` rows with the protected ones)
-    // leaves the joint one fewer entries when they are well below T
-    if (2 * most <= T) L.Tc = static_cast<int>(most);
-  }
+  if (adaptive && T > B) L.hs = g.n_kv_heads;
   L.D = g.head_dim;
   L.G = g.group;
   L.W = W;
@@ -137,7 +122,7 @@ size_t carve(Layout& L, void* ws) {
   L.s2 = reinterpret_cast<float*>(take(U * (size_t)L.T * sizeof(float)));
   L.idx = reinterpret_cast<int32_t*>(take(U * (size_t)L.B * sizeof(int32_t)));
   L.cnt = reinterpret_cast<int32_t*>(take(U * sizeof(int32_t)));
-  L.cand = L.Tc < L.T ? reinterpret_cast<int32_t*>(take(U * (size_t)L.Tc * sizeof(int32_t))) : nullptr;
+  L.hist = reinterpret_cast<uint32_t*>(take(2 * U * (size_t)kBins * sizeof(uint32_t)));
   L.hbeg = reinterpret_cast<int32_t*>(take(U * sizeof(int32_t)));
   L.cimg = take(U * (size_t)3 * kTileBytes);
   L.mv0 = reinterpret_cast<float*>(take(U * (size_t)kDP * sizeof(float)));
@@ -148,15 +133,11 @@ __device__ __forceinline__ bool is_protected(int t, int T, int W, int sink, int 
   return t < sink || (keep_window && t >= T - W);
 }
 
-// eight bf16 of a 16-byte chunk as floats
-__device__ __forceinline__ void unpack8(const uint4& w, float (&f)[8]) {
-  const uint32_t x[4] = {w.x, w.y, w.z, w.w};
-#pragma unroll
-  for (int i = 0; i < 4; ++i) {
-    const float2 v = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&x[i]));
-    f[2 * i] = v.x;
-    f[2 * i + 1] = v.y;
-  }
+// Order-preserving key of a score, at least 1, and its bin: exponent and three
+// mantissa bits of a score that is not negative (all others: bin 0).
+__device__ __forceinline__ uint32_t score_key(float s) { return max(1u, float_key(s)); }
+__device__ __forceinline__ int key_bin(uint32_t key) {
+  return (key & 0x80000000u) ? static_cast<int>((key >> 20) & (kBins - 1)) : 0;
 }
 
 __device__ __forceinline__ void epi_sync() { asm volatile("bar.sync 1, 128;" ::: "memory"); }
@@ -210,6 +191,8 @@ struct TcArgs {
   float* mrec;  // moment records, [units][n_chunks][rec]
   const float* s_in;
   float* s_out;
+  uint32_t* hist;  // stats_tc: both tables, zeroed; scores_tc, residual_tc: the table their scores are counted in
+  int units;
   float* diag;
   const uint8_t* cimg;  // [units][3][128 x 128] operand image of C0'
   const float* mv0;     // [units][kDP]
@@ -269,6 +252,11 @@ __global__ void __launch_bounds__(kStatsThreads, 1)
   const uint32_t tm = tmem_base;
   grid_dependency_wait();
   grid_launch_dependents();
+  if (chunk == 0)  // the unit's two tables of key counts
+    for (int i = tid; i < 2 * kBins / 4; i += kStatsThreads) {
+      const int tab = i / (kBins / 4), b4 = i % (kBins / 4);
+      reinterpret_cast<uint4*>(p.hist + ((size_t)tab * p.units + u) * kBins)[b4] = make_uint4(0u, 0u, 0u, 0u);
+    }
 
   if (warp == 0) {
     if (lane == 0) {  // ---- producer
@@ -612,6 +600,8 @@ __global__ void __launch_bounds__(kStatsThreads, 1)
       for (int o = 1; o < p.pool; o <<= 1) acc += __shfl_xor_sync(kFull, acc, o);  // aligned chunks
       if (t < t_end) {
         p.s_out[(size_t)u * p.T + t] = acc;
+        if (!is_protected(t, p.T, p.W, p.sink, p.keep_window))
+          atomicAdd(p.hist + (size_t)u * kBins + key_bin(score_key(acc)), 1u);
         if (p.diag) p.diag[(size_t)u * p.T + t] = acc;
       }
     }
@@ -781,9 +771,10 @@ __global__ void __launch_bounds__(kStatsThreads, 1)
       }
       const int t = t_begin + i * kTok + row;
       if (t < t_end) {
-        const float v =
-            is_protected(t, p.T, p.W, p.sink, p.keep_window) ? 0.f : p.s_in[(size_t)u * p.T + t] * sqrtf(ss);
+        const bool prot = is_protected(t, p.T, p.W, p.sink, p.keep_window);
+        const float v = prot ? 0.f : p.s_in[(size_t)u * p.T + t] * sqrtf(ss);
         p.s_out[(size_t)u * p.T + t] = v;
+        if (!prot) atomicAdd(p.hist + (size_t)u * kBins + key_bin(score_key(v)), 1u);
         if (p.diag) p.diag[(size_t)u * p.T + t] = v;
       }
     }
@@ -805,255 +796,233 @@ __global__ void __launch_bounds__(kStatsThreads, 1)
 // pairs f = h * T + t are ranked together.  R = protected + the k highest
 // keys among the other pairs (ties to the lower f), written ascending, with
 // each unit's count and first slot.
-// Exclusive block-wide prefix sum of one int per thread; *total gets the sum.
-__device__ __forceinline__ int block_excl_sum(int v, int* wsum, int* total) {
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  int x = v;
-#pragma unroll
-  for (int o = 1; o < 32; o <<= 1) {
-    const int y = __shfl_up_sync(kFull, x, o);
-    if (lane >= o) x += y;
-  }
-  if (lane == 31) wsum[warp] = x;
-  __syncthreads();
-  if (warp == 0) {
-    const int w = lane < (int)(blockDim.x >> 5) ? wsum[lane] : 0;
-    int xw = w;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-      const int y = __shfl_up_sync(kFull, xw, o);
-      if (lane >= o) xw += y;
-    }
-    wsum[lane] = xw - w;
-    if (lane == 31) *total = xw;
-  }
-  __syncthreads();
-  const int r = wsum[warp] + x - v;
-  __syncthreads();  // wsum is reused by the next call
-  return r;
-}
-
+//
+// The kernel that computed the scores has counted their keys into kBins bins
+// (exponent and three mantissa bits), so the bin of the k-th highest is known
+// from one scan.  The keys of that bin (about a sixth of k) are exchanged
+// over the cluster and ranked by counting, which gives the last selected
+// (key, f); one more pass counts and one writes.  Two cluster barriers, where
+// a radix select over the keys took four passes of three barriers each.  When
+// a CTA holds more than kMaxCont keys of that bin (many equal scores), the
+// cluster bisects the key and then f instead.
 struct SelectArgs {
-  const float* scores;  // [units][T]
+  const float* scores;   // [units][T]
+  const uint32_t* hist;  // [units][kBins] counts of the unprotected scores' keys
   int T, W, B, sink, keep_window;
-  int32_t* idx;          // [groups][hs * B] selection lists, h * T + position, ascending (workspace)
-  int32_t* diag_idx;     // optional copy
-  int smem_keys;  // keys of a CTA's range that the dynamic shared memory holds
-  int hs;         // units per selection group (1: one unit; > 1: the KV heads of a batch item)
-  const int32_t* cand;  // optional [units][Tc] ascending candidate positions per unit (null: all T)
-  int Tc;               // entries per unit taking part: T, or the candidate lists' length
-  int32_t* cnt;    // optional [units] rows retained per unit
-  int32_t* hbeg;   // optional [units] the unit's first slot in idx
+  int32_t* idx;       // [groups][hs * B] selection lists, h * T + position, ascending (workspace)
+  int32_t* diag_idx;  // optional copy
+  int hs;             // units per selection group (1: one unit; > 1: the KV heads of a batch item)
+  int32_t* cnt;       // [units] rows retained per unit
+  int32_t* hbeg;      // [units] the unit's first slot in idx
 };
 
-constexpr int kSelCL = 8;  // CTAs per selection group (one cluster), each over a contiguous range of pairs
-constexpr int kSelSmemKeys = 49152;  // keys of a CTA's range cached in shared memory (192 KB)
-constexpr int kMaxHs = 64;           // KV heads of a batch item with the adaptive budget
+constexpr int kSelThreads = 512;
+constexpr int kSelWarps = kSelThreads / 32;
+constexpr int kSelCL = 8;      // CTAs per selection group (one cluster), each over a contiguous range of pairs
+constexpr int kMaxCont = 256;  // keys of the contested bin a CTA may hold
+constexpr int kMaxHs = 64;     // KV heads of a batch item with the adaptive budget
 
 __global__ void __cluster_dims__(kSelCL, 1, 1) __launch_bounds__(kSelThreads, 2) select_kernel(const SelectArgs a) {
-  __shared__ uint32_t hist[2][256];   // this CTA's histogram, double-buffered by pass parity (read remotely)
-  __shared__ uint32_t whist[8][256];  // private histograms for groups of 4 warps (less atomic contention)
-  __shared__ uint32_t ghist[256];     // the cluster's histogram
-  __shared__ int wsum[32];
-  __shared__ int tot;
-  __shared__ uint32_t s_prefix;
-  __shared__ int s_need;
-  __shared__ int ex_cnt[2];  // this CTA's ties and certain selections (protected or above the threshold)
-  __shared__ int s_before[2];
-  __shared__ int s_hstart[kMaxHs + 1];  // first slot of each head in the group's selection list
-  __shared__ int s_hcnt[kMaxHs];        // this CTA's selections per head (read remotely)
-  grid_dependency_wait();
-  grid_launch_dependents();
+  __shared__ int s_w[kSelWarps];
+  __shared__ int s_bin, s_need;
+  __shared__ int s_n;                                          // this CTA's contested keys
+  __shared__ int s_cn[kSelCL];                                 // every CTA's (written remotely)
+  __shared__ unsigned long long s_cont[kSelCL][kMaxCont];      // every CTA's contested (key, ~f) (written remotely)
+  __shared__ unsigned long long s_last;                        // the last selected (key, ~f)
+  __shared__ int s_tot[2][kSelCL];                             // every CTA's counts (written remotely)
+  __shared__ int s_hcnt[kMaxHs], s_hstart[kMaxHs + 1];         // selections per head
   cg::cluster_group cluster = cg::this_cluster();
   const int rank = static_cast<int>(cluster.block_rank());
   const int grp = blockIdx.x / kSelCL, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const int T = a.T, W = a.W, hs = a.hs;
-  // entries f = h * Tc + j of the group stand for (head h, position t), t = j
-  // or the candidate cand[h][j]; either way f ascending is (h, t) ascending
-  const int Tc = a.Tc;
-  const int N = hs * Tc;
-  const int per = (N + kSelCL - 1) / kSelCL;
-  const int r0 = min(N, rank * per), r1 = min(N, r0 + per);
-  const float* sc = a.scores + (size_t)grp * hs * T;  // the group's units are consecutive
-  const int32_t* cand = a.cand ? a.cand + (size_t)grp * N : nullptr;
-  auto pos_of = [&](int f, int& h) -> int {  // (head, position) of entry f
-    h = hs == 1 ? 0 : f / Tc;
-    const int j = f - h * Tc;
-    return cand ? cand[f] : j;
-  };
-  // >= 0 (validated), < candidates
-  const int k = hs * (a.B - protected_count(T, W, a.sink, a.keep_window));
-
-  // The CTA's keys are cached in shared memory when they fit (protected
-  // positions hold key 0; every other position's key is at least 1, whatever
-  // the bits of its score, so at most k of them are ever selected); larger
-  // ranges are read from global memory on every pass.
-  extern __shared__ uint32_t ks[];
-  const int nk = r1 - r0;
-  const bool cached = nk <= a.smem_keys;
-  auto key_of = [&](int f) -> uint32_t {
-    int h;
-    const int t = pos_of(f, h);
-    return is_protected(t, T, W, a.sink, a.keep_window) ? 0u : max(1u, float_key(sc[(size_t)h * T + t]));
-  };
-  auto key_at = [&](int f) -> uint32_t {  // 0 for protected positions
-    return cached ? ks[f - r0] : key_of(f);
-  };
-  for (int h = tid; h < hs; h += kSelThreads) s_hcnt[h] = 0;
-  if (cached)
-    for (int i = tid; i < nk; i += kSelThreads) ks[i] = key_of(r0 + i);
-  __syncthreads();
-  // thread tid owns the contiguous positions [t0, t1) in the ordered passes
-  const int E = (nk + kSelThreads - 1) / kSelThreads;
-  const int t0 = min(r1, r0 + tid * E), t1 = min(r1, t0 + E);
-
-  uint32_t prefix = 0, pmask = 0;
-  int need = k;
-  if (k > 0) {
-    for (int pass = 0; pass < 4; ++pass) {
-      const int shift = 24 - 8 * pass;
-      for (int i = tid; i < 8 * 256; i += kSelThreads) (&whist[0][0])[i] = 0;
-      __syncthreads();
-      uint32_t* wh = whist[warp & 7];
-#pragma unroll 4
-      for (int i = tid; i < nk; i += kSelThreads) {
-        const uint32_t key = key_at(r0 + i);
-        if (key != 0u && (key & pmask) == prefix) atomicAdd(&wh[(key >> shift) & 255u], 1u);
-      }
-      __syncthreads();
-      for (int i = tid; i < 256; i += kSelThreads) {
-        uint32_t c = 0;
-#pragma unroll
-        for (int g = 0; g < 8; ++g) c += whist[g][i];
-        hist[pass & 1][i] = c;
-      }
-      cluster.sync();  // every CTA's histogram of this pass is complete
-      for (int i = tid; i < 256; i += kSelThreads) {
-        uint32_t c = 0;
-#pragma unroll
-        for (int r = 0; r < kSelCL; ++r) c += cluster.map_shared_rank(&hist[pass & 1][0], r)[i];
-        ghist[i] = c;
-      }
-      __syncthreads();
-      if (warp == 0) {  // the digit where the descending cumulative count reaches `need`
-        int cnt[8], tot8 = 0;
-#pragma unroll
-        for (int e = 0; e < 8; ++e) {
-          cnt[e] = static_cast<int>(ghist[255 - (lane * 8 + e)]);
-          tot8 += cnt[e];
-        }
-        int incl = tot8;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-          const int y = __shfl_up_sync(kFull, incl, o);
-          if (lane >= o) incl += y;
-        }
-        const int excl = incl - tot8;
-        if (excl < need && incl >= need) {
-          int cum = excl, e = 0;
-          for (; e < 7; ++e) {
-            if (cum + cnt[e] >= need) break;
-            cum += cnt[e];
-          }
-          s_need = need - cum;
-          s_prefix = prefix | (static_cast<uint32_t>(255 - (lane * 8 + e)) << shift);
-        }
-      }
-      __syncthreads();
-      need = s_need;
-      prefix = s_prefix;
-      pmask |= 255u << shift;
-    }
-  }
-  // per-thread counts: protected or above the threshold key (certain), and
-  // ties with it; scanned over the block, then over the cluster's ranks
-  int n_tie = 0, n_sure = 0;
-  for (int t = t0; t < t1; ++t) {
-    const uint32_t key = key_at(t);
-    if (key == 0u) {
-      ++n_sure;  // protected
-    } else if (k > 0) {
-      n_sure += key > prefix ? 1 : 0;
-      n_tie += key == prefix ? 1 : 0;
-    }
-  }
-  const int tie_excl = block_excl_sum(n_tie, wsum, &tot);
-  if (tid == 0) ex_cnt[0] = tot;
-  const int sure_excl = block_excl_sum(n_sure, wsum, &tot);
-  if (tid == 0) ex_cnt[1] = tot;
-  (void)sure_excl;
-  cluster.sync();
+  const int T = a.T, W = a.W, hs = a.hs, N = hs * T;
+  const int k = hs * (a.B - protected_count(T, W, a.sink, a.keep_window));  // >= 0 (validated), < candidates
+  const float* sc = a.scores + (size_t)grp * N;  // the group's units are consecutive
+  // warp w of CTA r takes the contiguous pairs [w0, w1)
+  const int per = (N + kSelCL * kSelWarps - 1) / (kSelCL * kSelWarps);
+  const int w0 = min(N, (rank * kSelWarps + warp) * per), w1 = min(N, w0 + per);
   if (tid == 0) {
-    int ties_before = 0, sel_before = 0;
-    for (int r = 0; r < rank; ++r) {
-      const int* rc = cluster.map_shared_rank(ex_cnt, r);
-      const int nt = rc[0], ns = rc[1];
-      const int take = min(max(need - ties_before, 0), nt);  // this rank's ties that are selected
-      sel_before += ns + take;
-      ties_before += nt;
-    }
-    s_before[0] = ties_before;
-    s_before[1] = sel_before;
+    s_n = 0;
+    s_bin = kBins;
+    s_need = 0;
+    s_last = ~0ull;
   }
+  if (tid < hs) s_hcnt[tid] = 0;
   __syncthreads();
-  const int cta_ties_before = s_before[0], cta_sel_before = s_before[1];
-  // this thread's selections: its certain ones and the ties that still fit
-  int tb = cta_ties_before + tie_excl;
-  const int my_sel = n_sure + min(max(need - tb, 0), n_tie);
-  const int sel_excl = block_excl_sum(my_sel, wsum, &tot);
-  int o = cta_sel_before + sel_excl;
+  cluster_arrive_relaxed();  // every CTA has started: awaited before the first remote store
+  grid_dependency_wait();
+  grid_launch_dependents();
+
+  // pairs are ordered by (key, ~f): a higher key first, at equal keys the lower f
+  auto pair_of = [&](int f) -> unsigned long long {  // 0: protected (or past the end)
+    const int t = hs == 1 ? f : f % T;
+    if (is_protected(t, T, W, a.sink, a.keep_window)) return 0ull;
+    return (static_cast<unsigned long long>(score_key(sc[f])) << 32) | (0xffffffffu - static_cast<unsigned>(f));
+  };
+  // exclusive sum over the block of one count per warp (`mine` from lane 0); the total in *total
+  auto block_counts = [&](int mine, int* total) -> int {
+    __syncthreads();
+    if (lane == 0) s_w[warp] = mine;
+    __syncthreads();
+    int before = 0, all = 0;
+#pragma unroll 4
+    for (int w = 0; w < kSelWarps; ++w) {
+      before += w < warp ? s_w[w] : 0;
+      all += s_w[w];
+    }
+    *total = all;
+    return before;
+  };
+
+  // ---- the bin of the k-th highest key: thread t takes four bins, descending
+  if (k > 0) {
+    uint4 c = make_uint4(0u, 0u, 0u, 0u);
+#pragma unroll 2
+    for (int h = 0; h < hs; ++h) {
+      const uint4 x = reinterpret_cast<const uint4*>(a.hist + ((size_t)grp * hs + h) * kBins)[kBins / 4 - 1 - tid];
+      c.x += x.x;
+      c.y += x.y;
+      c.z += x.z;
+      c.w += x.w;
+    }
+    const int b[4] = {(int)c.w, (int)c.z, (int)c.y, (int)c.x};
+    int incl = b[0] + b[1] + b[2] + b[3];
+    const int mine = incl;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const int y = __shfl_up_sync(kFull, incl, o);
+      if (lane >= o) incl += y;
+    }
+    int total;
+    int above = block_counts(__shfl_sync(kFull, incl, 31), &total) + incl - mine;
+#pragma unroll
+    for (int e = 0; e < 4; ++e) {
+      if (above < k && above + b[e] >= k) {  // one bin of the block
+        s_bin = kBins - 1 - (tid * 4 + e);
+        s_need = k - above;
+      }
+      above += b[e];
+    }
+    __syncthreads();
+    const int bin = s_bin;
+    // ---- the contested keys: this CTA's into every CTA's list
+#pragma unroll 4
+    for (int f0 = w0; f0 < w1; f0 += 32) {
+      const unsigned long long p = f0 + lane < w1 ? pair_of(f0 + lane) : 0ull;
+      if (p != 0ull && key_bin(static_cast<uint32_t>(p >> 32)) == bin) {
+        const int slot = atomicAdd(&s_n, 1);
+        if (slot < kMaxCont) s_cont[rank][slot] = p;
+      }
+    }
+    __syncthreads();
+    cluster_wait_acquire();
+    const int mn = s_n;
+    if (tid < kSelCL) *cluster.map_shared_rank(&s_cn[rank], tid) = mn;
+    for (int i = tid; i < min(mn, kMaxCont) * kSelCL; i += kSelThreads) {
+      const int r = i % kSelCL;
+      if (r != rank) *cluster.map_shared_rank(&s_cont[rank][i / kSelCL], r) = s_cont[rank][i / kSelCL];
+    }
+    cluster.sync();
+    bool over = false;
+    int m = 0;
+    for (int r = 0; r < kSelCL; ++r) {
+      over |= s_cn[r] > kMaxCont;
+      m += s_cn[r];
+    }
+    const int need = s_need;
+    if (!over) {
+      // the need-th of them: the one that need - 1 others precede
+      for (int i = tid; i < m; i += kSelThreads) {
+        int j = i, r = 0;
+        while (j >= s_cn[r]) j -= s_cn[r++];
+        const unsigned long long p = s_cont[r][j];
+        int before = 0;
+        for (int r2 = 0; r2 < kSelCL; ++r2) {
+          const int c2 = s_cn[r2];
+#pragma unroll 4
+          for (int j2 = 0; j2 < c2; ++j2) before += s_cont[r2][j2] > p ? 1 : 0;
+        }
+        if (before == need - 1) s_last = p;
+      }
+      __syncthreads();
+    } else {
+      // bisect: the largest p that at least k unprotected pairs reach
+      unsigned long long lo = 0ull;
+#pragma unroll 1
+      for (int bit = 63; bit >= 0; --bit) {
+        const unsigned long long mid = lo | (1ull << bit);
+        int c = 0;
+        for (int f = w0 + lane; f < w1; f += 32) c += pair_of(f) >= mid ? 1 : 0;
+        c = __reduce_add_sync(kFull, c);
+        int tot;
+        (void)block_counts(c, &tot);
+        if (tid < kSelCL) *cluster.map_shared_rank(&s_tot[bit & 1][rank], tid) = tot;
+        cluster.sync();
+        int all = 0;
+        for (int r = 0; r < kSelCL; ++r) all += s_tot[bit & 1][r];
+        if (all >= k) lo = mid;
+      }
+      if (tid == 0) s_last = lo;
+      cluster.sync();  // s_tot is written again below
+    }
+  } else {
+    cluster_wait_acquire();
+  }
+
+  // ---- this CTA's selections, then everybody's: protected pairs and those not below the last
+  const unsigned long long last = s_last;
+  auto selected = [&](int f) -> bool {
+    const unsigned long long p = pair_of(f);
+    return p == 0ull || p >= last;
+  };
+  int c = 0;
+#pragma unroll 4
+  for (int f0 = w0; f0 < w1; f0 += 32) c += __popc(__ballot_sync(kFull, f0 + lane < w1 && selected(f0 + lane)));
+  int tot;
+  int o = block_counts(c, &tot);
+  if (tid < kSelCL) *cluster.map_shared_rank(&s_tot[0][rank], tid) = tot;
+  cluster.sync();
+  for (int r = 0; r < rank; ++r) o += s_tot[0][r];
   const int n_sel = hs * a.B;  // the group's selections (protected included)
   int32_t* out = a.idx + (size_t)grp * n_sel;
-  int cur_h = 0, cur_n = 0;  // this thread's run of selections in one head (ranges rarely span two)
-  for (int t = t0; t < t1; ++t) {
-    const uint32_t key = key_at(t);
-    bool sel = true;  // protected
-    if (key != 0u) {
-      const bool tie = k > 0 && key == prefix;
-      sel = (k > 0 && key > prefix) || (tie && tb < need);
-      tb += tie ? 1 : 0;
+#pragma unroll 2
+  for (int f0 = w0; f0 < w1; f0 += 32) {
+    const int f = f0 + lane;
+    const bool sel = f < w1 && selected(f);
+    const unsigned mask = __ballot_sync(kFull, sel);
+    const int at = o + __popc(mask & ((1u << lane) - 1u));
+    if (sel && at < n_sel) {
+      out[at] = f;
+      if (a.diag_idx) a.diag_idx[(size_t)grp * n_sel + at] = f;
+      if (hs > 1) atomicAdd(&s_hcnt[f / T], 1);
     }
-    if (sel) {
-      if (o < n_sel) {  // stored as h * T + position
-        int h;
-        const int pt = pos_of(t, h);
-        out[o] = h * T + pt;
-        if (a.diag_idx) a.diag_idx[(size_t)grp * n_sel + o] = h * T + pt;
-        if (h != cur_h) {
-          if (cur_n) atomicAdd(&s_hcnt[cur_h], cur_n);
-          cur_h = h;
-          cur_n = 0;
-        }
-        ++cur_n;
-      }
-      ++o;
-    }
+    o += __popc(mask);
   }
-  if (hs > 1) {
-    // each head's slots are a contiguous run of the ascending list, as long
-    // as the head's selections in all CTAs of the cluster
-    if (cur_n) atomicAdd(&s_hcnt[cur_h], cur_n);
-    cluster.sync();
+  if (hs == 1) {
+    if (rank == 0 && tid == 0) {
+      a.cnt[grp] = a.B;
+      a.hbeg[grp] = grp * n_sel;
+    }
+    return;  // no remote access follows the last cluster barrier
+  }
+  // each head's slots are a contiguous run of the ascending list, as long as
+  // the head's selections in all CTAs of the cluster
+  cluster.sync();
+  if (rank == 0) {
     if (tid < hs) {
-      int c = 0;
-#pragma unroll
-      for (int r = 0; r < kSelCL; ++r) c += cluster.map_shared_rank(s_hcnt, r)[tid];
-      s_hstart[tid + 1] = c;
+      int x = 0;
+      for (int r = 0; r < kSelCL; ++r) x += cluster.map_shared_rank(s_hcnt, r)[tid];
+      s_hstart[tid + 1] = x;
     }
     __syncthreads();
     if (tid == 0) {
       s_hstart[0] = 0;
       for (int h = 0; h < hs; ++h) s_hstart[h + 1] += s_hstart[h];
     }
-  } else if (tid == 0) {
-    s_hstart[0] = 0;
-    s_hstart[1] = a.B;
-  }
-  __syncthreads();
-  if (rank == 0 && tid < hs) {
-    const int u = grp * hs + tid, c = s_hstart[tid + 1] - s_hstart[tid];
-    if (a.cnt) a.cnt[u] = c;
-    if (a.hbeg) a.hbeg[u] = grp * n_sel + s_hstart[tid];
+    __syncthreads();
+    if (tid < hs) {
+      a.cnt[grp * hs + tid] = s_hstart[tid + 1] - s_hstart[tid];
+      a.hbeg[grp * hs + tid] = grp * n_sel + s_hstart[tid];
+    }
   }
   cluster.sync();  // no CTA leaves while another may still read its shared memory
 }
@@ -1066,12 +1035,12 @@ __global__ void __cluster_dims__(kSelCL, 1, 1) __launch_bounds__(kSelThreads, 2)
 // The first stage writes C0' as the residual pass's operand image, the final
 // one the caller's moments and, from the same tiles, the retained cache.
 //
-// Grid (CL * D/64, units), clusters of CL CTAs: CTA (rank, kh) takes the row
-// tiles rank, rank + CL, ... and the key dims [64 kh, 64 kh + 64); the CL
-// partial sums meet through distributed shared memory, each rank finishing
-// 128 / CL value dims.  A set of 128..1024 rows is one tile per CTA: the kernel
-// is a chain of round trips (list, rows, MMA, exchange), 5-7 us, where the
-// dense gather, the per-tile records and their merge took 25-40.
+// Grid (CL * D/64, units), clusters of CL CTAs of 2048 / CL threads: CTA (rank,
+// kh) takes the row tiles rank, rank + CL, ... and the key dims [64 kh,
+// 64 kh + 64); the CL partial sums meet through distributed shared memory,
+// each rank finishing 128 / CL value dims, four elements of C per thread.  A
+// chain of round trips (list, rows, MMA, exchange) over code that runs once:
+// its time is latency and instruction fetch, so the loops stay rolled.
 //
 // The all-token co-moment is the multi-way Chan merge of the chunk records,
 // taken about the first chunk's means x0 so that no global mean is needed first:
@@ -1081,10 +1050,9 @@ __global__ void __cluster_dims__(kSelCL, 1, 1) __launch_bounds__(kSelThreads, 2)
 // records are stats_tc's, complete before the selection's predecessor (which
 // the selection has waited for when this kernel may start) began.
 // R's centred record is then removed with the reverse pairwise formula.
-constexpr int kRsThreads = 256;
-constexpr int kFinCH = 32;              // chunk records staged per pass
-constexpr int kRsRed = 64 + 4;          // row stride of a CTA's partial sums (floats)
-constexpr size_t kRsSmem = 1024 + kBoxBytes + kTileBytes;  // one K half, one V tile
+constexpr int kFinCH = 32;      // chunk records staged per pass
+constexpr int kRsRed = 64 + 4;  // row stride of a CTA's partial sums (floats)
+constexpr size_t kRsSmem = 1024 + kBoxBytes + kTileBytes + 2048;  // one K half, one V tile, ones
 
 struct RsetArgs {
   Layout L;
@@ -1106,96 +1074,81 @@ __device__ __forceinline__ void cp_async16(void* dst, const void* src, uint32_t 
 }
 
 template <int CL, bool FINAL>
-__global__ void __launch_bounds__(kRsThreads, 2) rset_kernel(const RsetArgs a) {
-  constexpr int NI = 8 / CL;       // value dims per thread in the merges (16 apart)
-  constexpr int RW = kDP / CL;     // value dims a rank finishes
+__global__ void __launch_bounds__(2048 / CL) rset_kernel(const RsetArgs a) {
+  constexpr int kThr = 2048 / CL;
+  constexpr int RW = kDP / CL;  // value dims a rank finishes
   extern __shared__ __align__(1024) uint8_t smraw[];
   uint8_t* sm = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smraw) + 1023) & ~uintptr_t(1023));
-  uint8_t* sK = sm;              // [128 rows][64 key dims]
-  uint8_t* sV = sm + kBoxBytes;  // [2 boxes][128 rows][64 value dims]
-  float* red = reinterpret_cast<float*>(sm);  // [128][kRsRed] this CTA's V^T K (after the tiles)
+  uint8_t* sK = sm;                               // [128 rows][64 key dims]
+  uint8_t* sV = sm + kBoxBytes;                   // [2 boxes][128 rows][64 value dims]
+  uint8_t* sOnes = sm + kBoxBytes + kTileBytes;   // [16 rows][128 B] of bf16 1.0
+  float* red = reinterpret_cast<float*>(sm);      // [128][kRsRed] this CTA's V^T K (after the tiles)
   __shared__ __align__(8) uint64_t done;
   __shared__ uint32_t tmem_base;
   __shared__ int s_ok;
-  __shared__ __align__(16) float s_pk[32][64], s_pv[16][kDP];  // column sums per row group
-  __shared__ __align__(16) float s_sk[64], s_sv[kDP];          // this CTA's column sums (read remotely)
+  __shared__ int s_t[kTok];                              // positions of a tile's rows, -1 past the unit's rows
+  __shared__ __align__(16) float s_sk[kDP], s_sv[kDP];  // this CTA's column sums (read remotely)
   const Layout& L = a.L;
   const int D = L.D, T = L.T;
   const int rank = blockIdx.x % CL, kh = blockIdx.x / CL, u = blockIdx.y;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const int cq = tid % 16, ar = tid / 16;  // merges: columns kh*64 + 4 cq.., value dims rank*RW + ar + 16 i
+  const int cq = tid % 16, row = rank * RW + tid / 16;  // this thread's four elements: (row, kh*64 + 4 cq ..)
 
   if (tid == 0) {
     mbar_init(&done, 1);
     mbar_fence_init();
     s_ok = 1;
   }
-  if (warp == 0) tmem_alloc(&tmem_base, 64);
+  if (warp == 0) tmem_alloc(&tmem_base, 128);
 
   // ---- the all-token set: this thread's elements of M and its means
   const size_t rf = L.rec;
   const float* recs = L.mpart + (size_t)u * L.n_chunks * rf;
-  float n = 0.f, sk[4] = {0.f, 0.f, 0.f, 0.f}, x0k[4] = {0.f, 0.f, 0.f, 0.f};
-  float sv[NI], x0v[NI], M[NI][4];
-#pragma unroll
-  for (int i = 0; i < NI; ++i) {
-    sv[i] = x0v[i] = 0.f;
-#pragma unroll
-    for (int j = 0; j < 4; ++j) M[i][j] = 0.f;
-  }
+  float n = 0.f, sv = 0.f, x0v = 0.f, sk[4] = {0.f, 0.f, 0.f, 0.f}, x0k[4] = {0.f, 0.f, 0.f, 0.f};
+  float M[4] = {0.f, 0.f, 0.f, 0.f};
   {
     float* s_n = reinterpret_cast<float*>(sm);  // [kFinCH]
     float* s_mk = s_n + kFinCH;                 // [kFinCH][64]
     float* s_mv = s_mk + kFinCH * 64;           // [kFinCH][RW]
+#pragma unroll 1
     for (int g0 = 0; g0 < L.n_chunks; g0 += kFinCH) {
       const int nb = min(kFinCH, L.n_chunks - g0);
       if (g0 > 0) __syncthreads();
       constexpr int per = 1 + 16 + RW / 4;  // float4s per record: n, 64 key means, RW value means
-#pragma unroll 4
-      for (int i = tid; i < nb * per; i += kRsThreads) {
+#pragma unroll 2
+      for (int i = tid; i < nb * per; i += kThr) {
         const int ch = i / per, j = i % per;
         const float* r = recs + (size_t)(g0 + ch) * rf;
-        if (j == 0) {
-          s_n[ch] = r[0];
-        } else if (j <= 16) {
-          *reinterpret_cast<float4*>(s_mk + ch * 64 + (j - 1) * 4) =
-              *reinterpret_cast<const float4*>(r + 4 + kh * 64 + (j - 1) * 4);
-        } else {
-          const int c = rank * RW + (j - 17) * 4;
-          *reinterpret_cast<float4*>(s_mv + ch * RW + (j - 17) * 4) =
-              c < D ? *reinterpret_cast<const float4*>(r + 4 + D + c) : make_float4(0.f, 0.f, 0.f, 0.f);
-        }
+        const int c = rank * RW + (j - 17) * 4;  // value dims past D are zero
+        const float* src = j == 0 ? r : j <= 16 ? r + 4 + kh * 64 + (j - 1) * 4 : r + 4 + D + c;
+        float* dst = j <= 16 ? s_mk + ch * 64 + (j - 1) * 4 : s_mv + ch * RW + (j - 17) * 4;
+        const float4 v =
+            j <= 16 || c < D ? *reinterpret_cast<const float4*>(src) : make_float4(0.f, 0.f, 0.f, 0.f);
+        if (j == 0) s_n[ch] = v.x;
+        else *reinterpret_cast<float4*>(dst) = v;
       }
       __syncthreads();
       if (g0 == 0) {
 #pragma unroll
         for (int j = 0; j < 4; ++j) x0k[j] = s_mk[cq * 4 + j];
-#pragma unroll
-        for (int i = 0; i < NI; ++i) x0v[i] = s_mv[ar + 16 * i];
+        x0v = s_mv[tid / 16];
       }
-#pragma unroll(CL >= 4 ? 8 : 2)
+      const float* m = recs + (size_t)g0 * rf + 4 + 2 * D + (size_t)min(row, D - 1) * D + kh * 64 + cq * 4;
+#pragma unroll 4
       for (int ch = 0; ch < nb; ++ch) {
-        const float* m = recs + (size_t)(g0 + ch) * rf + 4 + 2 * D + kh * 64 + cq * 4;
-        float4 m4[NI];
-#pragma unroll
-        for (int i = 0; i < NI; ++i) {
-          const int row = rank * RW + ar + 16 * i;
-          m4[i] = row < D ? *reinterpret_cast<const float4*>(m + (size_t)row * D) : make_float4(0.f, 0.f, 0.f, 0.f);
-        }
+        const float4 m4 = *reinterpret_cast<const float4*>(m + (size_t)ch * rf);
         const float nc = s_n[ch];
         if (nc > 0.f) {  // an empty record's co-moment is never written
           const float4 k4 = *reinterpret_cast<const float4*>(s_mk + ch * 64 + cq * 4);
           const float dk[4] = {k4.x - x0k[0], k4.y - x0k[1], k4.z - x0k[2], k4.w - x0k[3]};
+          const float mm[4] = {m4.x, m4.y, m4.z, m4.w};
+          const float dv = s_mv[ch * RW + tid / 16] - x0v;
           n += nc;
+          sv = fmaf(nc, dv, sv);
 #pragma unroll
-          for (int j = 0; j < 4; ++j) sk[j] = fmaf(nc, dk[j], sk[j]);
-#pragma unroll
-          for (int i = 0; i < NI; ++i) {
-            const float dv = s_mv[ch * RW + ar + 16 * i] - x0v[i];
-            sv[i] = fmaf(nc, dv, sv[i]);
-            const float mm[4] = {m4[i].x, m4[i].y, m4[i].z, m4[i].w};
-#pragma unroll
-            for (int j = 0; j < 4; ++j) M[i][j] += mm[j] + nc * dv * dk[j];
+          for (int j = 0; j < 4; ++j) {
+            sk[j] = fmaf(nc, dk[j], sk[j]);
+            M[j] += mm[j] + nc * dv * dk[j];
           }
         }
       }
@@ -1203,8 +1156,10 @@ __global__ void __launch_bounds__(kRsThreads, 2) rset_kernel(const RsetArgs a) {
   }
   __syncthreads();  // the staged records give way to the row tiles
   if (D < kDP)      // no second box of value dims
-    for (int i = tid; i < kBoxBytes / 16; i += kRsThreads)
+    for (int i = tid; i < kBoxBytes / 16; i += kThr)
       reinterpret_cast<uint4*>(sV + kBoxBytes)[i] = make_uint4(0u, 0u, 0u, 0u);
+  if (tid < 2048 / 16)  // the ones operand of the column sums
+    reinterpret_cast<uint4*>(sOnes)[tid] = make_uint4(0x3F803F80u, 0x3F803F80u, 0x3F803F80u, 0x3F803F80u);
   grid_dependency_wait();
   grid_launch_dependents();
 
@@ -1215,18 +1170,10 @@ __global__ void __launch_bounds__(kRsThreads, 2) rset_kernel(const RsetArgs a) {
   const int n_tiles = (cnt + kTok - 1) / kTok;
   const __nv_bfloat16* Ku = a.K + (size_t)u * T * D + kh * 64;
   const __nv_bfloat16* Vu = a.V + (size_t)u * T * D;
-  const uint32_t id = idesc_bf16(128, 64, 1, 1);  // V^T K: both MN-major (reduction over rows)
-  const uint32_t aK = smem_addr(sK), aV = smem_addr(sV);
   const int vch = D / 8;  // 16-byte chunks of a value row
-  float ks[8], vs[8];     // this thread's column sums: key chunk tid % 8, value chunk tid % 16
-#pragma unroll
-  for (int j = 0; j < 8; ++j) ks[j] = vs[j] = 0.f;
   int it = 0;
   bool ok = true;
-  tc_fence_before();
-  __syncthreads();
-  tc_fence_after();
-  const uint32_t tm = tmem_base;
+#pragma unroll 1
   for (int ti = rank; ti < n_tiles; ti += CL, ++it) {
     if (it > 0) {  // the operands are free once their MMAs have completed
       if (tid == 0 && !mbar_wait(&done, (it - 1) & 1, a.polls)) {
@@ -1238,57 +1185,56 @@ __global__ void __launch_bounds__(kRsThreads, 2) rset_kernel(const RsetArgs a) {
       if (!ok) break;  // uniform: s_ok changes only before a barrier
     }
     const int r0 = ti * kTok;
-#pragma unroll
-    for (int j = 0; j < 4; ++j) {  // 128 rows x 8 chunks of the key half
-      const int r = tid / 8 + 32 * j, c = tid % 8;
-      const int t = r0 + r < cnt ? min(max(lst[r0 + r] - hT, 0), T - 1) : 0;  // never outside the unit's slab
-      cp_async16(sK + r * 128 + ((c ^ (r & 7)) << 4), Ku + (size_t)t * D + c * 8, r0 + r < cnt ? 16u : 0u);
+    if (tid < kTok)  // never outside the unit's slab
+      s_t[tid] = r0 + tid < cnt ? min(max(lst[r0 + tid] - hT, 0), T - 1) : -1;
+    __syncthreads();
+#pragma unroll 1
+    for (int i = tid; i < kTok * 8; i += kThr) {  // the key half: 8 chunks a row
+      const int r = i / 8, c = i % 8, t = s_t[r];
+      cp_async16(sK + r * 128 + ((c ^ (r & 7)) << 4), Ku + (size_t)max(t, 0) * D + c * 8, t >= 0 ? 16u : 0u);
     }
-#pragma unroll
-    for (int j = 0; j < 8; ++j) {  // 128 rows x 16 chunks of the value rows
-      const int r = tid / 16 + 16 * j, c = tid % 16;
-      const int t = r0 + r < cnt ? min(max(lst[r0 + r] - hT, 0), T - 1) : 0;
-      if (c < vch)
-        cp_async16(sV + (c >> 3) * kBoxBytes + r * 128 + (((c & 7) ^ (r & 7)) << 4), Vu + (size_t)t * D + c * 8,
-                   r0 + r < cnt ? 16u : 0u);
+#pragma unroll 1
+    for (int i = tid; i < kTok * vch; i += kThr) {  // the value rows
+      const int r = i / vch, c = i % vch, t = s_t[r];
+      cp_async16(sV + (c >> 3) * kBoxBytes + r * 128 + (((c & 7) ^ (r & 7)) << 4), Vu + (size_t)max(t, 0) * D + c * 8,
+                 t >= 0 ? 16u : 0u);
     }
     asm volatile("cp.async.wait_all;" ::: "memory");
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");  // generic writes -> tensor-core reads
+    tc_fence_before();
     __syncthreads();
     if (tid == 0) {
-      for (int kk = 0; kk < 8; ++kk)
-        umma_bf16(tm, sdesc_sw128(aV + kk * 2048, kBoxBytes, 1024), sdesc_sw128(aK + kk * 2048, kBoxBytes, 1024), id,
-                  (it > 0 || kk > 0) ? 1u : 0u);
+      // V^T K, and the column sums of [K half | V's first box] and of V against
+      // ones (the boxes lie one after another), all MN-major over the rows
+      tc_fence_after();
+      const uint32_t tm = tmem_base, aK = smem_addr(sK), aV = smem_addr(sV), a1 = smem_addr(sOnes);
+      const uint32_t id = idesc_bf16(128, 64, 1, 1), id1 = idesc_bf16(128, 16, 1, 0);
+#pragma unroll 1
+      for (int kk = 0; kk < 8; ++kk) {
+        const uint64_t dk = sdesc_sw128(aK + kk * 2048, kBoxBytes, 1024), dv = sdesc_sw128(aV + kk * 2048, kBoxBytes, 1024);
+        const uint64_t d1 = sdesc_sw128(a1 + (kk & 3) * 32, 16, 1024);
+        const uint32_t acc = (it > 0 || kk > 0) ? 1u : 0u;
+        umma_bf16(tm, dv, dk, id, acc);
+        umma_bf16(tm + 64, dk, d1, id1, acc);
+        umma_bf16(tm + 80, dv, d1, id1, acc);
+      }
       umma_commit(&done);
     }
-    // column sums, and in the final stage the cache rows, from the same tile
-#pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      const int r = tid / 8 + 32 * j, c = tid % 8, row = r0 + r;
-      const uint4 w = *reinterpret_cast<const uint4*>(sK + r * 128 + ((c ^ (r & 7)) << 4));
-      float f[8];
-      unpack8(w, f);
-#pragma unroll
-      for (int e = 0; e < 8; ++e) ks[e] += f[e];
-      // (a joint selection's cache is zero up to the next tile past a unit's rows)
-      if (FINAL && (row < cnt || (L.hs > 1 && row < a.dst_cap)))
-        *reinterpret_cast<uint4*>(a.dst_K + ((size_t)u * a.dst_cap + row) * D + kh * 64 + c * 8) = w;
-    }
-#pragma unroll
-    for (int j = 0; j < 8; ++j) {
-      const int r = tid / 16 + 16 * j, c = tid % 16, row = r0 + r;
-      if (c < vch) {
-        const uint4 w = *reinterpret_cast<const uint4*>(sV + (c >> 3) * kBoxBytes + r * 128 + (((c & 7) ^ (r & 7)) << 4));
-        float f[8];
-        unpack8(w, f);
-#pragma unroll
-        for (int e = 0; e < 8; ++e) vs[e] += f[e];
-        if (FINAL && (c >> 3) == kh && (row < cnt || (L.hs > 1 && row < a.dst_cap)))
-          *reinterpret_cast<uint4*>(a.dst_V + ((size_t)u * a.dst_cap + row) * D + c * 8) = w;
+    if constexpr (FINAL) {
+      // the cache rows from the same tile, this CTA's halves (a joint
+      // selection's cache is zero up to the next tile past a unit's rows)
+#pragma unroll 1
+      for (int i = tid; i < kTok * 8; i += kThr) {
+        const int r = i / 8, c = i % 8, to = r0 + r;
+        if (to < cnt || (L.hs > 1 && to < a.dst_cap)) {
+          const size_t o = ((size_t)u * a.dst_cap + to) * D + kh * 64 + c * 8;
+          const uint32_t at = r * 128 + ((c ^ (r & 7)) << 4);
+          *reinterpret_cast<uint4*>(a.dst_K + o) = *reinterpret_cast<const uint4*>(sK + at);
+          *reinterpret_cast<uint4*>(a.dst_V + o) = *reinterpret_cast<const uint4*>(sV + kh * kBoxBytes + at);
+        }
       }
+      if (kh == 0 && tid < kTok && r0 + tid < cnt) a.dst_pos[(size_t)u * a.dst_cap + r0 + tid] = s_t[tid];
     }
-    if (FINAL && kh == 0 && tid < kTok && r0 + tid < cnt)
-      a.dst_pos[(size_t)u * a.dst_cap + r0 + tid] = lst[r0 + tid] - hT;
   }
   // ---- this CTA's sums and V^T K into shared memory
   if (it > 0 && ok) {
@@ -1301,133 +1247,103 @@ __global__ void __launch_bounds__(kRsThreads, 2) rset_kernel(const RsetArgs a) {
   }
   if (!ok && tid == 0) (void)mbar_wait(&done, (it - 1) & 1);  // drain: the MMAs still read shared memory
   __syncthreads();
-  tc_fence_after();
-#pragma unroll
-  for (int e = 0; e < 8; ++e) {
-    s_pk[tid / 8][(tid % 8) * 8 + e] = ks[e];
-    s_pv[tid / 16][(tid % 16) * 8 + e] = vs[e];
-  }
-  {
-    float x[32];
-    const int row = (warp & 3) * 32 + lane, c0 = (warp >> 2) * 32;
-    if (it > 0 && ok) {
-      tmem_ld32(tm + (static_cast<uint32_t>((warp & 3) * 32) << 16) + c0, x);
-    } else {
-#pragma unroll
-      for (int j = 0; j < 32; ++j) x[j] = 0.f;
-    }
-#pragma unroll
-    for (int j = 0; j < 32; j += 4)
-      *reinterpret_cast<float4*>(red + row * kRsRed + c0 + j) = make_float4(x[j], x[j + 1], x[j + 2], x[j + 3]);
-  }
-  tc_fence_before();
-  __syncthreads();
-  if (warp == 0) {
+  if (warp < 4) {
     tc_fence_after();
-    tmem_dealloc(tm, 64);
-  }
-  if (tid < 64) {
-    float x = 0.f;
-    for (int g = 0; g < 32; ++g) x += s_pk[g][tid];
-    s_sk[tid] = x;
-  } else if (tid < 64 + kDP) {
-    float x = 0.f;
-    for (int g = 0; g < 16; ++g) x += s_pv[g][tid - 64];
-    s_sv[tid - 64] = x;
+    const uint32_t tm = tmem_base + (static_cast<uint32_t>(warp * 32) << 16);
+    const int r = warp * 32 + lane;
+    const bool have = it > 0 && ok;
+    float x[32];
+#pragma unroll 1
+    for (int c0 = 0; c0 < 96; c0 += 32) {
+      if (have) {
+        tmem_ld32(tm + c0, x);
+      } else {
+#pragma unroll
+        for (int j = 0; j < 32; ++j) x[j] = 0.f;
+      }
+      if (c0 < 64) {
+#pragma unroll
+        for (int j = 0; j < 32; j += 4)
+          *reinterpret_cast<float4*>(red + r * kRsRed + c0 + j) = make_float4(x[j], x[j + 1], x[j + 2], x[j + 3]);
+      } else {
+        s_sk[r] = x[0];  // lanes 64.. hold sums of V's first box: not read
+        s_sv[r] = x[16];
+      }
+    }
+    tc_fence_before();
   }
   cg::cluster_group cluster = cg::this_cluster();
-  if constexpr (CL > 1) cluster.sync();
-  else __syncthreads();
+  cluster.sync();
+  if (warp == 0) {
+    tc_fence_after();
+    tmem_dealloc(tmem_base, 128);
+  }
 
   // ---- R's sums over the cluster, and E = all \ R
   const float nR = ok ? static_cast<float>(cnt) : 0.f;
-  float SR[NI][4], rv[NI], rk[4] = {0.f, 0.f, 0.f, 0.f};
-#pragma unroll
-  for (int i = 0; i < NI; ++i) {
-    rv[i] = 0.f;
-#pragma unroll
-    for (int j = 0; j < 4; ++j) SR[i][j] = 0.f;
-  }
-#pragma unroll
-  for (int r = 0; r < CL; ++r) {
-    const float* pr = CL > 1 ? cluster.map_shared_rank(red, r) : red;
-    const float* pk = CL > 1 ? cluster.map_shared_rank(s_sk, r) : s_sk;
-    const float* pv = CL > 1 ? cluster.map_shared_rank(s_sv, r) : s_sv;
-    const float4 k4 = *reinterpret_cast<const float4*>(pk + cq * 4);
+  float SR[4] = {0.f, 0.f, 0.f, 0.f}, rk[4] = {0.f, 0.f, 0.f, 0.f}, rv = 0.f;
+#pragma unroll 2
+  for (int r = 0; r < min(CL, max(1, n_tiles)); ++r) {  // ranks past the tiles hold zeros
+    const float4 k4 = *reinterpret_cast<const float4*>(cluster.map_shared_rank(s_sk, r) + cq * 4);
+    const float4 s4 = *reinterpret_cast<const float4*>(cluster.map_shared_rank(red, r) + row * kRsRed + cq * 4);
+    rv += cluster.map_shared_rank(s_sv, r)[row];
     rk[0] += k4.x;
     rk[1] += k4.y;
     rk[2] += k4.z;
     rk[3] += k4.w;
-#pragma unroll
-    for (int i = 0; i < NI; ++i) {
-      const int row = rank * RW + ar + 16 * i;
-      const float4 s4 = *reinterpret_cast<const float4*>(pr + row * kRsRed + cq * 4);
-      SR[i][0] += s4.x;
-      SR[i][1] += s4.y;
-      SR[i][2] += s4.z;
-      SR[i][3] += s4.w;
-      rv[i] += pv[row];
-    }
+    SR[0] += s4.x;
+    SR[1] += s4.y;
+    SR[2] += s4.z;
+    SR[3] += s4.w;
   }
   const float nE = n - nR;
-  float mk[4], mkR[4], mkE[4];
+  const float mv = x0v + sv / n, mvR = nR > 0.f ? rv / nR : 0.f, mvE = nE > 0.f ? (n * mv - nR * mvR) / nE : 0.f;
+  float CE[4], mkE[4];
 #pragma unroll
   for (int j = 0; j < 4; ++j) {
-    mk[j] = x0k[j] + sk[j] / n;
-    mkR[j] = nR > 0.f ? rk[j] / nR : 0.f;
-    mkE[j] = nE > 0.f ? (n * mk[j] - nR * mkR[j]) / nE : 0.f;
-  }
-#pragma unroll
-  for (int i = 0; i < NI; ++i) {
-    const int row = rank * RW + ar + 16 * i;
-    const float mv = x0v[i] + sv[i] / n;
-    const float mvR = nR > 0.f ? rv[i] / nR : 0.f;
-    const float mvE = nE > 0.f ? (n * mv - nR * mvR) / nE : 0.f;
-    float CE[4];
-#pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      CE[j] = 0.f;
-      if (nE > 0.f) {
-        const float Mall = M[i][j] - sv[i] * sk[j] / n;
-        const float MR = nR > 0.f ? SR[i][j] - rv[i] * rk[j] / nR : 0.f;
-        const float ME = Mall - MR - (nE * nR / n) * (mvR - mvE) * (mkR[j] - mkE[j]);
-        CE[j] = ME / nE;
-      }
-    }
-    if constexpr (FINAL) {
-      if (row < D) {
-        *reinterpret_cast<float4*>(a.mom.C + ((size_t)u * D + row) * D + kh * 64 + cq * 4) =
-            make_float4(CE[0], CE[1], CE[2], CE[3]);
-        if (kh == 0 && cq == 0) a.mom.mu_v[(size_t)u * D + row] = mvE;
-        if (row == 0)
-#pragma unroll
-          for (int j = 0; j < 4; ++j) a.mom.mu_k[(size_t)u * D + kh * 64 + cq * 4 + j] = mkE[j];
-      }
-    } else {
-      // C0' (clamped where |n0 C0| < tau) as three bf16 parts, K-major operand
-      // rows (value dims; zero past D) in the swizzled layout
-      float r4[4];
-#pragma unroll
-      for (int j = 0; j < 4; ++j) r4[j] = (row < D && !(fabsf(CE[j] * nE) < a.tau)) ? CE[j] : 0.f;
-      uint8_t* img = L.cimg + (size_t)u * 3 * kTileBytes + swz_off(row, kh * 64 + cq * 4, kTok);
-#pragma unroll
-      for (int part = 0; part < 3; ++part) {
-        uint2 w;
-        w.x = pack_bf16x2(r4[0], r4[1]);
-        w.y = pack_bf16x2(r4[2], r4[3]);
-        *reinterpret_cast<uint2*>(img + (size_t)part * kTileBytes) = w;
-#pragma unroll
-        for (int j = 0; j < 4; ++j) r4[j] = bf16_residual(r4[j]);
-      }
-      if (kh == 0 && cq == 0) L.mv0[(size_t)u * kDP + row] = row < D ? mvE : 0.f;
+    const float mk = x0k[j] + sk[j] / n, mkR = nR > 0.f ? rk[j] / nR : 0.f;
+    CE[j] = mkE[j] = 0.f;
+    if (nE > 0.f) {
+      mkE[j] = (n * mk - nR * mkR) / nE;
+      const float Mall = M[j] - sv * sk[j] / n;
+      const float MR = nR > 0.f ? SR[j] - rv * rk[j] / nR : 0.f;
+      const float ME = Mall - MR - (nE * nR / n) * (mvR - mvE) * (mkR - mkE[j]);
+      CE[j] = ME / nE;
     }
   }
-  if (FINAL && kh == 0 && rank == 0 && tid == 0) {
-    a.mom.n[u] = static_cast<int32_t>(nE);
-    a.dst_len[u] = cnt;
-    a.dst_seen[u] = T;
+  if constexpr (FINAL) {
+    if (row < D) {
+      *reinterpret_cast<float4*>(a.mom.C + ((size_t)u * D + row) * D + kh * 64 + cq * 4) =
+          make_float4(CE[0], CE[1], CE[2], CE[3]);
+      if (kh == 0 && cq == 0) a.mom.mu_v[(size_t)u * D + row] = mvE;
+      if (row == 0)
+#pragma unroll
+        for (int j = 0; j < 4; ++j) a.mom.mu_k[(size_t)u * D + kh * 64 + cq * 4 + j] = mkE[j];
+    }
+    if (kh == 0 && rank == 0 && tid == 0) {
+      a.mom.n[u] = static_cast<int32_t>(nE);
+      a.dst_len[u] = cnt;
+      a.dst_seen[u] = T;
+    }
+  } else {
+    // C0' (clamped where |n0 C0| < tau) as three bf16 parts, K-major operand
+    // rows (value dims; zero past D) in the swizzled layout
+    float r4[4];
+#pragma unroll
+    for (int j = 0; j < 4; ++j) r4[j] = (row < D && !(fabsf(CE[j] * nE) < a.tau)) ? CE[j] : 0.f;
+    uint8_t* img = L.cimg + (size_t)u * 3 * kTileBytes + swz_off(row, kh * 64 + cq * 4, kTok);
+#pragma unroll
+    for (int part = 0; part < 3; ++part) {
+      uint2 w;
+      w.x = pack_bf16x2(r4[0], r4[1]);
+      w.y = pack_bf16x2(r4[2], r4[3]);
+      *reinterpret_cast<uint2*>(img + (size_t)part * kTileBytes) = w;
+#pragma unroll
+      for (int j = 0; j < 4; ++j) r4[j] = bf16_residual(r4[j]);
+    }
+    if (kh == 0 && cq == 0) L.mv0[(size_t)u * kDP + row] = row < D ? mvE : 0.f;
   }
-  if constexpr (CL > 1) cluster.sync();  // no CTA leaves while another reads its shared memory
+  cluster.sync();  // no CTA leaves while another reads its shared memory
 }
 
 // ---------------------------------------------------------- keep-all path
@@ -1492,14 +1408,11 @@ cudaError_t smem_attr(const void* f, size_t bytes) {
   return cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(bytes));
 }
 
-// CTAs per unit and key half of rset_kernel: one row tile each, and no more
-// chunk records to merge than about 300 KB, as long as all CTAs run at once
-// (two per SM).
+// CTAs per unit and key half of rset_kernel: the more, the fewer records and
+// rows each takes; as many as run at once (shared memory: four per SM).
 int rset_cluster(const Layout& L, int num_sms) {
-  const long tiles = (L.B + kTok - 1) / kTok, nh = L.D / 64;
-  const long want = std::max(tiles, (long)L.n_chunks / 9);
-  int cl = 1;
-  while (cl < 8 && cl < want && 2L * cl * nh * L.units <= 2L * num_sms) cl *= 2;
+  int cl = 8;
+  while (cl > 2 && (long)cl * (L.D / 64) * L.units > 4L * num_sms) cl /= 2;
   return cl;
 }
 
@@ -1508,18 +1421,17 @@ cudaError_t launch_rset(const RsetArgs& a, int cl, cudaStream_t st) {
   const dim3 grid(cl * (a.L.D / 64), a.L.units);
   auto go = [&](void (*f)(RsetArgs)) -> cudaError_t {
     const cudaError_t e = smem_attr(reinterpret_cast<const void*>(f), kRsSmem);
-    return e != cudaSuccess ? e : launch_pdl(f, grid, kRsThreads, kRsSmem, st, cl, a);
+    return e != cudaSuccess ? e : launch_pdl(f, grid, 2048 / cl, kRsSmem, st, cl, a);
   };
   switch (cl) {
     case 8: return go(rset_kernel<8, FINAL>);
     case 4: return go(rset_kernel<4, FINAL>);
-    case 2: return go(rset_kernel<2, FINAL>);
-    default: return go(rset_kernel<1, FINAL>);
+    default: return go(rset_kernel<2, FINAL>);
   }
 }
 
 cudaError_t run(const CompressArgs& a, const mkv_geom& g, int num_sms, cudaStream_t st) {
-  Layout L = make_layout(g, a.T, a.budget, a.window, a.sink, a.keep_window, a.adaptive, num_sms);
+  Layout L = make_layout(g, a.T, a.budget, a.window, a.adaptive, num_sms);
   carve(L, a.ws);
   const int D = g.head_dim, T = a.T, B = a.budget, U = L.units;
   const bool keep_all = T <= B;
@@ -1551,6 +1463,8 @@ cudaError_t run(const CompressArgs& a, const mkv_geom& g, int num_sms, cudaStrea
   tp.qscale = rsqrtf(static_cast<float>(D)) * kLog2e;
   tp.rowpart = L.rowpart;
   tp.mrec = L.mpart;
+  tp.hist = L.hist;
+  tp.units = U;
   tp.ws = a.ws;
   tp.polls = pipeline_poll_limit();
   const dim3 cg(L.n_chunks, U);
@@ -1568,47 +1482,21 @@ cudaError_t run(const CompressArgs& a, const mkv_geom& g, int num_sms, cudaStrea
     return cudaGetLastError();
   }
 
-  SelectArgs sa{};
-  const int n_groups = U / L.hs;
-  const bool prefilter = L.cand != nullptr;
-  // keys a CTA caches when its range fits, for the joint (or per-unit) selection and the prefilter
-  auto cached_keys = [](long per) { return per <= kSelSmemKeys ? static_cast<int>(per) : 0; };
-  sa.smem_keys = cached_keys((L.hs * (long)L.Tc + kSelCL - 1) / kSelCL);
-  const int pf_keys = cached_keys((T + kSelCL - 1) / kSelCL);
-  const size_t sel_smem = (size_t)sa.smem_keys * sizeof(uint32_t), pf_smem = (size_t)pf_keys * sizeof(uint32_t);
-  if ((e = smem_attr((const void*)select_kernel, std::max(sel_smem, pf_smem))) != cudaSuccess) return e;
-  sa.T = T;
-  sa.Tc = L.Tc;
-  sa.cand = L.cand;
-  sa.W = a.window;
-  sa.B = B;
-  sa.sink = a.sink;
-  sa.keep_window = a.keep_window;
-  sa.idx = L.idx;
-  sa.hs = L.hs;
-  sa.cnt = L.cnt;
-  sa.hbeg = L.hbeg;
-  // one selection over `scores`; a joint one first keeps each unit's protected
-  // rows and its top Tc - |protected| as candidates (a per-unit selection)
-  auto select = [&](const float* scores, int32_t* diag_idx) -> cudaError_t {
-    if (prefilter) {
-      SelectArgs pf = sa;
-      pf.scores = scores;
-      pf.hs = 1;
-      pf.Tc = T;
-      pf.cand = nullptr;
-      pf.B = L.Tc;
-      pf.idx = L.cand;
-      pf.smem_keys = pf_keys;
-      pf.cnt = nullptr;
-      pf.hbeg = nullptr;
-      const cudaError_t pe = launch_pdl(select_kernel, dim3(U * kSelCL), kSelThreads, pf_smem, st, 0, pf);
-      if (pe != cudaSuccess) return pe;
-    }
-    SelectArgs s0 = sa;
-    s0.scores = scores;
-    s0.diag_idx = diag_idx;
-    return launch_pdl(select_kernel, dim3(n_groups * kSelCL), kSelThreads, sel_smem, st, 0, s0);
+  auto select = [&](const float* scores, const uint32_t* hist, int32_t* diag_idx) -> cudaError_t {
+    SelectArgs sa{};
+    sa.scores = scores;
+    sa.hist = hist;
+    sa.diag_idx = diag_idx;
+    sa.T = T;
+    sa.W = a.window;
+    sa.B = B;
+    sa.sink = a.sink;
+    sa.keep_window = a.keep_window;
+    sa.idx = L.idx;
+    sa.hs = L.hs;
+    sa.cnt = L.cnt;
+    sa.hbeg = L.hbeg;
+    return launch_pdl(select_kernel, dim3(U / L.hs * kSelCL), kSelThreads, 0, st, 0, sa);
   };
   RsetArgs ra{};
   ra.L = L;
@@ -1626,7 +1514,8 @@ cudaError_t run(const CompressArgs& a, const mkv_geom& g, int num_sms, cudaStrea
   ra.polls = tp.polls;
   const int cl = rset_cluster(L, num_sms);
 
-  if ((e = select(L.s, a.diag_idx1)) != cudaSuccess) return e;
+  uint32_t* hist2 = L.hist + (size_t)U * kBins;
+  if ((e = select(L.s, L.hist, a.diag_idx1)) != cudaSuccess) return e;
   if (a.mi) {
     if ((e = launch_rset<false>(ra, cl, st)) != cudaSuccess) return e;
     TcArgs r = tp;
@@ -1634,9 +1523,10 @@ cudaError_t run(const CompressArgs& a, const mkv_geom& g, int num_sms, cudaStrea
     r.mv0 = L.mv0;
     r.s_in = L.s;
     r.s_out = L.s2;
+    r.hist = hist2;
     r.diag = a.diag_score2;
     if ((e = launch_pdl(residual_tc, cg, kStatsThreads, kResidualSmem, st, 0, r, tmK, tmV)) != cudaSuccess) return e;
-    if ((e = select(L.s2, nullptr)) != cudaSuccess) return e;
+    if ((e = select(L.s2, hist2, nullptr)) != cudaSuccess) return e;
   }
   return launch_rset<true>(ra, cl, st);
 }
@@ -1644,7 +1534,7 @@ cudaError_t run(const CompressArgs& a, const mkv_geom& g, int num_sms, cudaStrea
 }  // namespace
 
 size_t compress_workspace_bytes(const mkv_geom& g, int32_t T, const mkv_compress_params& p, int num_sms) {
-  Layout L = make_layout(g, T, p.budget, p.window, p.sink, p.keep_window, p.adaptive, num_sms);
+  Layout L = make_layout(g, T, p.budget, p.window, p.adaptive, num_sms);
   return carve(L, nullptr);
 }
 
