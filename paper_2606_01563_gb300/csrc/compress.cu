@@ -51,11 +51,16 @@ constexpr int kTok = 128;                   // tokens per tile
 constexpr int kDP = 128;                    // padded head dim of every MMA
 constexpr int kTileBytes = kTok * kDP * 2;  // one [128 x 128] bf16 tile: 2 boxes of 16 KB
 constexpr int kBoxBytes = kTok * 128;
-// stats_tc: two epilogue groups of 4 warps (2..5 and 6..9), each taking half
-// of a tile's tokens, so that two warps per scheduler share the softmax work
+// stats_tc, residual_tc: two epilogue groups of 4 warps (2..5 and 6..9), so
+// that two warps per scheduler share the work
 constexpr int kStatsThreads = 320;
+constexpr int kMaxHs = 64;  // KV heads of a batch item with the adaptive budget
+// stats_tc's K/V stages: shared memory holds a third beside one block of window rows
+__host__ __device__ constexpr int stats_stages(int RWb) { return RWb == 1 ? 3 : 2; }
+__host__ __device__ constexpr size_t stats_smem(int RWb) {
+  return 1024 + (size_t)stats_stages(RWb) * 2 * kTileBytes + (size_t)RWb * 2 * kBoxBytes;
+}
 constexpr int kBins = 2048;  // bins of the scores' keys (select_kernel)
-constexpr int kPF = 0;  // tiles prefetched into L2 ahead of the one being loaded (0: none)
 constexpr unsigned kFull = 0xffffffffu;
 
 struct Layout {
@@ -74,6 +79,9 @@ struct Layout {
   int32_t* hbeg;      // [units] first slot of each unit in idx
   uint8_t* cimg;      // [units][3][128 x 128] C0' as three bf16 parts, in the residual's operand layout
   float* mv0;         // [units][kDP] mu_v of E0
+  float* fro;         // [units][kDP] parts of ||C0'||_F^2
+  float* norms;       // [units][T][2] ||k_t||^2, ||v_t||^2
+  int32_t* cand;      // [units][T] positions residual_tc has left to compute
 };
 
 __host__ __device__ inline size_t rec_floats(int D) { return align_up(4 + 2 * (size_t)D + (size_t)D * D, 4); }
@@ -126,6 +134,9 @@ size_t carve(Layout& L, void* ws) {
   L.hbeg = reinterpret_cast<int32_t*>(take(U * sizeof(int32_t)));
   L.cimg = take(U * (size_t)3 * kTileBytes);
   L.mv0 = reinterpret_cast<float*>(take(U * (size_t)kDP * sizeof(float)));
+  L.fro = reinterpret_cast<float*>(take(U * (size_t)kDP * sizeof(float)));
+  L.norms = reinterpret_cast<float*>(take(U * (size_t)L.T * 2 * sizeof(float)));
+  L.cand = reinterpret_cast<int32_t*>(take(U * (size_t)L.T * sizeof(int32_t)));
   return off;
 }
 
@@ -140,12 +151,50 @@ __device__ __forceinline__ int key_bin(uint32_t key) {
   return (key & 0x80000000u) ? static_cast<int>((key >> 20) & (kBins - 1)) : 0;
 }
 
-__device__ __forceinline__ void epi_sync() { asm volatile("bar.sync 1, 128;" ::: "memory"); }
-// whether v holds in all 128 threads of the first epilogue group (barrier 1)
+// 16 bytes global -> shared, asynchronously (src_bytes 0: zeros)
+__device__ __forceinline__ void cp_async16(void* dst, const void* src, uint32_t src_bytes) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(smem_addr(dst)), "l"(src), "r"(src_bytes)
+               : "memory");
+}
+
+// Eight bf16 of a 16-byte chunk added to `acc` (pairs of floats), and the sum
+// of their squares returned: two elements per instruction.
+__device__ __forceinline__ float sum_chunk(const uint4& w, uint64_t (&acc)[4]) {
+  const uint32_t x[4] = {w.x, w.y, w.z, w.w};
+  uint64_t sq = 0ull;
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    uint64_t v;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(v) : "r"(x[i] << 16), "r"(x[i] & 0xffff0000u));
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(acc[i]) : "l"(acc[i]), "l"(v));
+    asm("fma.rn.f32x2 %0, %1, %1, %2;" : "=l"(sq) : "l"(v), "l"(sq));
+  }
+  float a, b;
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(sq));
+  return a + b;
+}
+
+// Sums over each half warp of eight values per lane: lanes 2x and 2x + 1 of a
+// half get the sum of v[x] (x < 8).
+__device__ __forceinline__ float half_warp_sums(float (&v)[8], int lane) {
+#pragma unroll
+  for (int w = 4; w >= 1; w >>= 1) {
+    const bool hi = (lane & (2 * w)) != 0;
+#pragma unroll
+    for (int i = 0; i < w; ++i) {
+      const float send = hi ? v[i] : v[i + w], keep = hi ? v[i + w] : v[i];
+      v[i] = keep + __shfl_xor_sync(kFull, send, 2 * w);
+    }
+  }
+  return v[0] + __shfl_xor_sync(kFull, v[0], 1);
+}
+
+__device__ __forceinline__ void epi_sync() { asm volatile("bar.sync 1, 256;" ::: "memory"); }
+// whether v holds in all 256 threads of the epilogue warps (barrier 1)
 __device__ __forceinline__ bool epi_all(bool v) {
   uint32_t r;
   asm volatile(
-      "{\n\t.reg .pred p, q;\n\tsetp.ne.u32 p, %1, 0;\n\tbar.red.and.pred q, 1, 128, p;\n\t"
+      "{\n\t.reg .pred p, q;\n\tsetp.ne.u32 p, %1, 0;\n\tbar.red.and.pred q, 1, 256, p;\n\t"
       "selp.u32 %0, 1, 0, q;\n\t}"
       : "=r"(r)
       : "r"((uint32_t)v)
@@ -162,6 +211,12 @@ __device__ __forceinline__ bool pwait(uint64_t* bar, uint32_t parity, volatile i
   *abort_flag = 1;
   record_error(ws, MKV_ERR_TIMEOUT, u);
   return false;
+}
+
+// pwait by a whole warp: all its lanes go on or none.
+__device__ __forceinline__ bool pwait_warp(uint64_t* bar, uint32_t parity, volatile int* abort_flag, void* ws, int u,
+                                           uint32_t polls) {
+  return __all_sync(kFull, pwait(bar, parity, abort_flag, ws, u, polls)) != 0;
 }
 
 // After an abort, before a CTA frees its tensor memory and exits: wait (with
@@ -196,44 +251,65 @@ struct TcArgs {
   float* diag;
   const uint8_t* cimg;  // [units][3][128 x 128] operand image of C0'
   const float* mv0;     // [units][kDP]
+  float* norms;         // [units][T][2] ||k_t||^2, ||v_t||^2
+  // residual_tc's pruning
+  int prune, hs, B;     // hs: units per selection group
+  const int32_t* idx;   // [groups][hs * B] the first stage's selections
+  const float* fro;     // [units][kDP] parts (n_fro of them) of ||C0'||_F^2
+  int n_fro;
+  int32_t* cand;        // [units][T] positions left to compute, per CTA from its first position on
+  const void* K;
+  const void* V;
   void* ws;
   uint32_t polls;  // poll limit of the pipeline waits
 };
 
 // --------------------------------------------------------------- stats_tc
-// Window-row statistics and chunk moments of the prompt.
+// Window-row statistics, chunk moments and row norms of the prompt, in one
+// pass over K and V.  Bounded by that read (64 KB a tile and SM): the tensor
+// cores do the two products only, 1024 cycles a tile (column sums by products
+// with ones cost as many again), the epilogue warps take the column sums and
+// the norms from shared memory while a tile's logits are computed, and with up
+// to 128 window rows three stages are in flight and the logits double-buffered.
 __global__ void __launch_bounds__(kStatsThreads, 1)
     stats_tc(const TcArgs p, const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtensorMap tmV,
              const __grid_constant__ CUtensorMap tmQ) {
-  constexpr int kS = 2;
+  constexpr int kMaxS = 3;
   constexpr uint32_t kTmemCols = 512;
-  constexpr int cS = 256, cSum = 384;  // TMEM columns of V^T K and the sums
+  constexpr int cS = 256;  // TMEM columns: the logits [0, 256), V^T K
   extern __shared__ __align__(1024) uint8_t smraw[];
   uint8_t* sm = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smraw) + 1023) & ~uintptr_t(1023));
-  uint8_t* sK = sm;                        // [kS][128 x 128]
-  uint8_t* sV = sm + kS * kTileBytes;      // [kS][128 x 128]
-  uint8_t* sQ = sm + 2 * kS * kTileBytes;  // [2 boxes][RWb*128 rows][128 B]
-  uint8_t* sOnes = sQ + 2 * 2 * kBoxBytes;  // [2 boxes][16 rows][128 B] of bf16 1.0
-  __shared__ __align__(8) uint64_t full[kS], empty[kS], lfull, lempty, qfull, sdone;
+  const int RWb = p.RWb, kS = stats_stages(RWb), NB = RWb == 1 ? 2 : 1;  // stages, logits buffers
+  uint8_t* sKV = sm;                           // [kS][K tile, V tile]
+  uint8_t* sQ = sm + (size_t)kS * 2 * kTileBytes;  // [2 boxes][RWb*128 rows][128 B]
+  // after the last tile the first stage holds the epilogue's staging
+  float* stg = reinterpret_cast<float*>(sm);                  // [2 groups][128][36]
+  float* s_pk = stg + 2 * 128 * 36;                           // [16][128] column sums of K per row group
+  float* s_pv = s_pk + 16 * 128;                              // the same of V
+  float* s_m1 = s_pv + 16 * 128;                              // [2][128] the second group's row maxima
+  float* s_l1 = s_m1 + 2 * 128;                               // and sums
+  float* sum_k = s_l1 + 2 * 128;                              // [128]
+  float* sum_v = sum_k + kDP;                                 // [128]
+  __shared__ __align__(8) uint64_t full[kMaxS], empty[kMaxS], lfull[2], lempty[2], qfull, sdone;
   __shared__ uint32_t tmem_base;
   __shared__ int abort_flag, s_issued;
-  __shared__ float sum_k[kDP], sum_v[kDP];
-  __shared__ float s_m1[2][128], s_l1[2][128];  // the second epilogue group's row stats
 
   const int chunk = blockIdx.x, u = blockIdx.y;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int t_begin = chunk * p.chunk;
   const int t_end = min(p.n_rows, t_begin + p.chunk);
   const int n_tiles = (max(0, t_end - t_begin) + kTok - 1) / kTok;
-  const int RWb = p.RWb;
   volatile int* abrt = &abort_flag;
+
   if (tid == 0) {
     for (int i = 0; i < kS; ++i) {
       mbar_init(&full[i], 1);
-      mbar_init(&empty[i], 1);  // the stage is free once its MMAs have completed
+      mbar_init(&empty[i], 1 + 8);  // the stage's MMAs and the epilogue warps' reads
     }
-    mbar_init(&lfull, 1);
-    mbar_init(&lempty, 8);
+    for (int i = 0; i < 2; ++i) {
+      mbar_init(&lfull[i], 1);
+      mbar_init(&lempty[i], 8);
+    }
     mbar_init(&qfull, 1);
     mbar_init(&sdone, 1);
     abort_flag = 0;
@@ -241,45 +317,25 @@ __global__ void __launch_bounds__(kStatsThreads, 1)
     mbar_fence_init();
   }
   if (warp == 1) tmem_alloc(&tmem_base, kTmemCols);
-  if (warp >= 2 && warp < 6) {  // the ones operand of the column sums K^T 1 and V^T 1
-    for (int i = tid - 64; i < 2 * 16 * 128 / 16; i += 128)
-      reinterpret_cast<uint4*>(sOnes)[i] = make_uint4(0x3F803F80u, 0x3F803F80u, 0x3F803F80u, 0x3F803F80u);
-    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-  }
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
   const uint32_t tm = tmem_base;
   grid_dependency_wait();
   grid_launch_dependents();
-  if (chunk == 0)  // the unit's two tables of key counts
-    for (int i = tid; i < 2 * kBins / 4; i += kStatsThreads) {
-      const int tab = i / (kBins / 4), b4 = i % (kBins / 4);
-      reinterpret_cast<uint4*>(p.hist + ((size_t)tab * p.units + u) * kBins)[b4] = make_uint4(0u, 0u, 0u, 0u);
-    }
 
   if (warp == 0) {
     if (lane == 0) {  // ---- producer
       mbar_arrive_expect_tx(&qfull, 2u * RWb * kBoxBytes);
       for (int bx = 0; bx < 2; ++bx) tma_load_3d(sQ + bx * RWb * kBoxBytes, &tmQ, bx * 64, 0, u, &qfull);
-      for (int i = 0; i < min(kPF, n_tiles); ++i)
-        for (int bx = 0; bx < 2; ++bx) {
-          tma_prefetch_3d(&tmK, bx * 64, t_begin + i * kTok, u);
-          tma_prefetch_3d(&tmV, bx * 64, t_begin + i * kTok, u);
-        }
       for (int i = 0; i < n_tiles; ++i) {
         const int s = i % kS, j = i / kS;
-        if (kPF > 0 && i + kPF < n_tiles)
-          for (int bx = 0; bx < 2; ++bx) {
-            tma_prefetch_3d(&tmK, bx * 64, t_begin + (i + kPF) * kTok, u);
-            tma_prefetch_3d(&tmV, bx * 64, t_begin + (i + kPF) * kTok, u);
-          }
         if (j >= 1 && !pwait(&empty[s], (j - 1) & 1, abrt, p.ws, u, p.polls)) break;
+        uint8_t* dst = sKV + (size_t)s * 2 * kTileBytes;
         mbar_arrive_expect_tx(&full[s], 2u * kTileBytes);
-        for (int bx = 0; bx < 2; ++bx) {
-          tma_load_3d(sK + s * kTileBytes + bx * kBoxBytes, &tmK, bx * 64, t_begin + i * kTok, u, &full[s]);
-          tma_load_3d(sV + s * kTileBytes + bx * kBoxBytes, &tmV, bx * 64, t_begin + i * kTok, u, &full[s]);
-        }
+        for (int bx = 0; bx < 2; ++bx) tma_load_3d(dst + bx * kBoxBytes, &tmK, bx * 64, t_begin + i * kTok, u, &full[s]);
+        for (int bx = 0; bx < 2; ++bx)
+          tma_load_3d(dst + kTileBytes + bx * kBoxBytes, &tmV, bx * 64, t_begin + i * kTok, u, &full[s]);
         s_issued = i + 1;
       }
     }
@@ -287,42 +343,41 @@ __global__ void __launch_bounds__(kStatsThreads, 1)
     if (lane == 0) {  // ---- MMA issuer
       const uint32_t idL = idesc_bf16(128, 128, 0, 0);  // logits: rows x tokens, both K-major
       const uint32_t idS = idesc_bf16(128, 128, 1, 1);  // V^T K: both MN-major (reduction over tokens)
-      const uint32_t id1 = idesc_bf16(128, 16, 1, 0);   // X^T 1: X MN-major, ones K-major
-      const uint32_t aQ = smem_addr(sQ), a1 = smem_addr(sOnes);
+      const uint32_t aQ = smem_addr(sQ);
       const bool ok = pwait(&qfull, 0, abrt, p.ws, u, p.polls);
       for (int i = 0; ok && i < n_tiles; ++i) {
-        const int s = i % kS, j = i / kS;
+        const int s = i % kS, j = i / kS, b = i % NB;
         if (!pwait(&full[s], j & 1, abrt, p.ws, u, p.polls)) break;
+        if (i >= NB && !pwait(&lempty[b], (i / NB - 1) & 1, abrt, p.ws, u, p.polls)) break;
         tc_fence_after();
-        const uint32_t aK = smem_addr(sK + s * kTileBytes), aV = smem_addr(sV + s * kTileBytes);
-        if (i >= 1 && !pwait(&lempty, (i - 1) & 1, abrt, p.ws, u, p.polls)) break;
-        tc_fence_after();
+        const uint32_t aK = smem_addr(sKV + (size_t)s * 2 * kTileBytes), aV = aK + kTileBytes;
         for (int rb = 0; rb < RWb; ++rb)
           for (int kk = 0; kk < 8; ++kk) {
             const uint64_t dq =
                 sdesc_sw128(aQ + (kk >> 2) * RWb * kBoxBytes + rb * kBoxBytes + (kk & 3) * 32, 16, 1024);
             const uint64_t dk = sdesc_sw128(aK + (kk >> 2) * kBoxBytes + (kk & 3) * 32, 16, 1024);
-            umma_bf16(tm + rb * 128, dq, dk, idL, kk > 0 ? 1u : 0u);
+            umma_bf16(tm + (b + rb) * 128, dq, dk, idL, kk > 0 ? 1u : 0u);
           }
-        umma_commit(&lfull);
+        umma_commit(&lfull[b]);
         for (int kk = 0; kk < 8; ++kk) {
           const uint64_t dv = sdesc_sw128(aV + kk * 2048, kBoxBytes, 1024);
           const uint64_t dk = sdesc_sw128(aK + kk * 2048, kBoxBytes, 1024);
-          const uint64_t d1 = sdesc_sw128(a1 + (kk >> 2) * 2048 + (kk & 3) * 32, 16, 1024);
-          const uint32_t acc = (i > 0 || kk > 0) ? 1u : 0u;
-          umma_bf16(tm + cS, dv, dk, idS, acc);
-          umma_bf16(tm + cSum, dk, d1, id1, acc);       // column sums of K (lane = key dim)
-          umma_bf16(tm + cSum + 16, dv, d1, id1, acc);  // column sums of V (lane = value dim)
+          umma_bf16(tm + cS, dv, dk, idS, (i > 0 || kk > 0) ? 1u : 0u);
         }
         umma_commit(&empty[s]);
       }
       umma_commit(&sdone);
     }
   } else {
-    // ---- epilogue: group 0 = warps 2..5 (tokens 0..63 of a tile), group 1 =
-    // warps 6..9 (tokens 64..127); TMEM lane quarter qd = warp % 4
-    const int grp = (warp - 2) >> 2;
+    // ---- epilogue: group 0 = warps 2..5 (tokens 0..63 of a tile's logits),
+    // group 1 = warps 6..9 (tokens 64..127); TMEM lane quarter qd = warp % 4
+    const int ew = warp - 2, grp = ew >> 2;
     const int et = tid - 64 - grp * 128, qd = warp & 3;
+    if (chunk == 0)  // the unit's two tables of key counts
+      for (int i = tid - 64; i < 2 * kBins / 4; i += 256) {
+        const int tab = i / (kBins / 4), b4 = i % (kBins / 4);
+        reinterpret_cast<uint4*>(p.hist + ((size_t)tab * p.units + u) * kBins)[b4] = make_uint4(0u, 0u, 0u, 0u);
+      }
     const uint32_t lane_base = static_cast<uint32_t>(qd * 32) << 16;
     float m[2] = {-INFINITY, -INFINITY}, l[2] = {0.f, 0.f};
     int tmax_vis[2];
@@ -331,10 +386,31 @@ __global__ void __launch_bounds__(kStatsThreads, 1)
       tmax_vis[rb] = p.causal ? p.T - p.W + r % p.W : 0x7fffffff;
     }
     const int t_safe = p.causal ? p.T - p.W : 0x7fffffff;  // tokens every window row sees
+    // column sums: this lane's 8 dims (chunk lane % 16) over the rows 16 ew + lane / 16 + 2 j
+    const int ch = lane & 15, rh = lane >> 4;
+    uint64_t ksum[4] = {0ull, 0ull, 0ull, 0ull}, vsum[4] = {0ull, 0ull, 0ull, 0ull};
     for (int i = 0; i < n_tiles; ++i) {
-      if (!pwait(&lfull, i & 1, abrt, p.ws, u, p.polls)) break;
-      tc_fence_after();
+      const int s = i % kS, b = i % NB;
+      if (!pwait_warp(&full[s], (i / kS) & 1, abrt, p.ws, u, p.polls)) break;
       const int tt0 = t_begin + i * kTok;
+      {
+        const uint8_t* tk = sKV + (size_t)s * 2 * kTileBytes + (ch >> 3) * kBoxBytes + (ew * 16 + rh) * 128;
+        float kn[8], vn[8];
+#pragma unroll
+        for (int j = 0; j < 8; ++j) {
+          const uint32_t off = 2 * j * 128 + (((ch & 7) ^ ((rh + 2 * j) & 7)) << 4);
+          kn[j] = sum_chunk(*reinterpret_cast<const uint4*>(tk + off), ksum);
+          vn[j] = sum_chunk(*reinterpret_cast<const uint4*>(tk + kTileBytes + off), vsum);
+        }
+        __syncwarp();
+        if (lane == 0) mbar_arrive(&empty[s]);
+        // squared norms of 16 rows over the 16 lanes of each: lane 2 x holds row x / 8 + 2 (x % 8)
+        const float kq = half_warp_sums(kn, lane), vq = half_warp_sums(vn, lane);
+        const int t = tt0 + ew * 16 + rh + 2 * ((lane >> 1) & 7);
+        if (t < t_end) p.norms[((size_t)u * p.T + t) * 2 + (lane & 1)] = (lane & 1) ? vq : kq;
+      }
+      if (!pwait_warp(&lfull[b], (i / NB) & 1, abrt, p.ws, u, p.polls)) break;
+      tc_fence_after();
       const bool fast = tt0 + kTok <= t_end && tt0 + kTok - 1 <= t_safe;  // no masking in this tile
       // rb runs over a constant range (guarded by RWb), so that m, l and
       // tmax_vis stay in registers
@@ -343,7 +419,7 @@ __global__ void __launch_bounds__(kStatsThreads, 1)
         if (rb >= RWb) break;
         for (int c0 = grp * 64; c0 < grp * 64 + 64; c0 += 32) {
           float x[32];
-          tmem_ld32(tm + lane_base + rb * 128 + c0, x);
+          tmem_ld32(tm + lane_base + (b + rb) * 128 + c0, x);
           const int t0 = tt0 + c0;
           float mx = -INFINITY;
           if (fast) {
@@ -374,78 +450,80 @@ __global__ void __launch_bounds__(kStatsThreads, 1)
       }
       tc_fence_before();
       __syncwarp();
-      if (lane == 0) mbar_arrive(&lempty);
+      if (lane == 0) mbar_arrive(&lempty[b]);
     }
-    {  // merge the two groups' (max, sum) of each row
+    // uniform over the epilogue warps: after an abort the MMAs may still write
+    // TMEM and read the stages, so neither is touched and the chunk's record
+    // is left empty
+    const bool got = epi_all(pwait_warp(&sdone, 0, abrt, p.ws, u, p.polls));
+    float* rec = p.mrec + ((size_t)u * p.n_chunks + chunk) * rec_floats(p.D);
+    if (got) {
+      tc_fence_after();
+      // the per-warp column sums and the second group's row statistics
+#pragma unroll
+      for (int e = 0; e < 4; ++e) {
+        reinterpret_cast<uint64_t*>(s_pk + (ew * 2 + rh) * 128 + ch * 8)[e] = ksum[e];
+        reinterpret_cast<uint64_t*>(s_pv + (ew * 2 + rh) * 128 + ch * 8)[e] = vsum[e];
+      }
       if (grp == 1)
 #pragma unroll
         for (int rb = 0; rb < 2; ++rb) {
-          if (rb < RWb) {
-            s_m1[rb][qd * 32 + lane] = m[rb];
-            s_l1[rb][qd * 32 + lane] = l[rb];
-          }
+          s_m1[rb * 128 + qd * 32 + lane] = m[rb];
+          s_l1[rb * 128 + qd * 32 + lane] = l[rb];
         }
-      asm volatile("bar.sync 2, 256;" ::: "memory");
+      epi_sync();
+      {
+        const float* part = grp == 0 ? s_pk : s_pv;
+        float x = 0.f;
+#pragma unroll
+        for (int g = 0; g < 16; ++g) x += part[g * 128 + et];
+        (grp == 0 ? sum_k : sum_v)[et] = x;
+      }
       if (grp == 0)
 #pragma unroll
         for (int rb = 0; rb < 2; ++rb) {
           if (rb >= RWb) break;
           const int r = rb * 128 + qd * 32 + lane;
-          const float m1 = s_m1[rb][qd * 32 + lane], l1 = s_l1[rb][qd * 32 + lane];
-          const float M = fmaxf(m[rb], m1);
-          float L = 0.f;
-          if (M != -INFINITY) {
-            if (m[rb] != -INFINITY) L += l[rb] * fast_exp2(m[rb] - M);
-            if (m1 != -INFINITY) L += l1 * fast_exp2(m1 - M);
+          const float m1 = s_m1[r], l1 = s_l1[r];
+          const float Mx = fmaxf(m[rb], m1);
+          float Ls = 0.f;
+          if (Mx != -INFINITY) {
+            if (m[rb] != -INFINITY) Ls += l[rb] * fast_exp2(m[rb] - Mx);
+            if (m1 != -INFINITY) Ls += l1 * fast_exp2(m1 - Mx);
           }
-          if (r < p.RW) {
-            float* rp = p.rowpart + (((size_t)u * p.n_chunks + chunk) * p.RW + r) * 2;
-            rp[0] = M;
-            rp[1] = L;
-          }
+          if (r < p.RW)
+            *reinterpret_cast<float2*>(p.rowpart + (((size_t)u * p.n_chunks + chunk) * p.RW + r) * 2) =
+                make_float2(Mx, Ls);
         }
-    }
-    if (grp == 0) {
-    // uniform over the group: after an abort the MMAs may still write TMEM,
-    // so it is not read and the chunk's record is left empty
-    const bool got = epi_all(pwait(&sdone, 0, abrt, p.ws, u, p.polls));
-    float* rec = p.mrec + ((size_t)u * p.n_chunks + chunk) * rec_floats(p.D);
-    const float nc = got ? static_cast<float>(max(0, t_end - t_begin)) : 0.f;
-    if (got) {
-    tc_fence_after();
-    {
-      float x[32];
-      tmem_ld32(tm + lane_base + cSum, x);  // [0]: sum of K's column (this lane), [16]: of V's
-      sum_k[qd * 32 + lane] = x[0];
-      sum_v[qd * 32 + lane] = x[16];
-    }
-    epi_sync();
-    const float inv_nc = nc > 0.f ? 1.f / nc : 0.f;
-    const int a = qd * 32 + lane;  // value dim = TMEM lane
-    // centred co-moment rows staged 32 columns at a time through the (now
-    // free) K stage, so that the record is written in coalesced rows
-    float* stg = reinterpret_cast<float*>(sK);  // [128][33]
-    for (int c0 = 0; c0 < kDP; c0 += 32) {
-      float srow[32];
-      tmem_ld32(tm + lane_base + cS + c0, srow);
+      epi_sync();
+      const float nc = static_cast<float>(max(0, t_end - t_begin)), inv_nc = nc > 0.f ? 1.f / nc : 0.f;
+      const int a = qd * 32 + lane;  // value dim = TMEM lane
+      const float sva = sum_v[a] * inv_nc;
+      // centred co-moment rows, 32 columns at a time and group, through shared
+      // memory so that the record is written in whole 128-byte lines
+      float* sg = stg + grp * 128 * 36;
+#pragma unroll 1
+      for (int c0 = grp * 64; c0 < grp * 64 + 64; c0 += 32) {
+        float x[32];
+        tmem_ld32(tm + lane_base + cS + c0, x);
 #pragma unroll
-      for (int jj = 0; jj < 32; ++jj) stg[a * 33 + jj] = srow[jj] - sum_v[a] * sum_k[c0 + jj] * inv_nc;
-      epi_sync();
-      if (nc > 0.f)
-        for (int idx = et; idx < 128 * 32; idx += 128) {
-          const int r = idx >> 5, c = c0 + (idx & 31);
-          if (r < p.D && c < p.D) rec[4 + 2 * p.D + (size_t)r * p.D + c] = stg[r * 33 + (idx & 31)];
+        for (int jj = 0; jj < 32; jj += 4) {
+          const float4 k4 = *reinterpret_cast<const float4*>(sum_k + c0 + jj);
+          *reinterpret_cast<float4*>(sg + a * 36 + jj) =
+              make_float4(x[jj] - sva * k4.x, x[jj + 1] - sva * k4.y, x[jj + 2] - sva * k4.z, x[jj + 3] - sva * k4.w);
         }
-      epi_sync();
-    }
-    if (a < p.D) {
-      rec[4 + a] = nc > 0.f ? sum_k[a] / nc : 0.f;
-      rec[4 + p.D + a] = nc > 0.f ? sum_v[a] / nc : 0.f;
-    }
-    } else if (et < 4 + 2 * p.D) {
-      rec[et] = 0.f;  // an empty record: n = 0, zero means
-    }
-    if (et == 0) rec[0] = nc;
+        named_sync(2 + grp, 128);
+        if (c0 < p.D)
+#pragma unroll 4
+          for (int r = et / 8; r < p.D; r += 16)
+            *reinterpret_cast<float4*>(rec + 4 + 2 * p.D + (size_t)r * p.D + c0 + (et % 8) * 4) =
+                *reinterpret_cast<const float4*>(sg + r * 36 + (et % 8) * 4);
+        named_sync(2 + grp, 128);
+      }
+      if (et < p.D) rec[4 + grp * p.D + et] = (grp == 0 ? sum_k : sum_v)[et] * inv_nc;
+      if (tid == 64) rec[0] = nc;
+    } else if (tid - 64 < 4 + 2 * p.D) {  // an empty record: n = 0, zero means
+      for (int i = tid - 64; i < 4 + 2 * p.D; i += 256) rec[i] = 0.f;
     }
   }
   tc_fence_before();
@@ -461,36 +539,42 @@ __global__ void __launch_bounds__(kStatsThreads, 1)
 }
 
 // -------------------------------------------------------------- scores_tc
-__global__ void __launch_bounds__(kStatsThreads, 1)
+// Token scores: the logits again, token-major.  Four epilogue groups of four
+// warps, each on a TMEM buffer of 128 logits columns: with up to 128 window
+// rows they take every fourth tile, with more each tile is shared by two
+// groups (rows 0..127 and the others).  Two groups left the kernel bound by
+// the latency of their loads and exponentials (57 us at 32K, batch 4).
+constexpr int kScoreThreads = 64 + 4 * 128;
+__global__ void __launch_bounds__(kScoreThreads, 1)
     scores_tc(const TcArgs p, const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtensorMap tmQ) {
-  constexpr int kS = 3;
+  constexpr int kS = 4;
   extern __shared__ __align__(1024) uint8_t smraw[];
   uint8_t* sm = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smraw) + 1023) & ~uintptr_t(1023));
   uint8_t* sK = sm;                    // [kS][128 x 128]
   uint8_t* sQ = sm + kS * kTileBytes;  // [2 boxes][RWb*128][128 B]
-  __shared__ __align__(8) uint64_t full[kS], empty[kS], lfull[2], lempty[2], qfull, mma_done;
+  __shared__ __align__(8) uint64_t full[kS], empty[kS], lfull[4], lempty[4], pfull[2], qfull, mma_done;
   __shared__ uint32_t tmem_base;
   __shared__ int abort_flag, s_issued;
   __shared__ __align__(16) float s_b[256];  // log2(1 / l_r) - m_r (-inf for padding rows)
-  __shared__ int s_wi[256];                   // window index of row r (r mod W)
+  __shared__ int s_wi[256];                 // window index of row r (r mod W)
+  __shared__ float s_part[2][128];          // the upper rows' sums of a tile shared by two groups
 
   const int chunk = blockIdx.x, u = blockIdx.y;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int t_begin = chunk * p.chunk;
   const int t_end = min(p.n_rows, t_begin + p.chunk);
   const int n_tiles = (max(0, t_end - t_begin) + kTok - 1) / kTok;
-  const int RWb = p.RWb, RWp = RWb * 128;
+  const int RWb = p.RWb, RWp = RWb * 128, NB = 4 / RWb;  // TMEM buffers of RWp columns
   volatile int* abrt = &abort_flag;
 
   if (tid == 0) {
     for (int i = 0; i < kS; ++i) {
       mbar_init(&full[i], 1);
       mbar_init(&empty[i], 1);
-    }
-    for (int i = 0; i < 2; ++i) {
       mbar_init(&lfull[i], 1);
-      mbar_init(&lempty[i], 4);
+      mbar_init(&lempty[i], 4 * RWb);
     }
+    for (int i = 0; i < 2; ++i) mbar_init(&pfull[i], 4);
     mbar_init(&qfull, 1);
     mbar_init(&mma_done, 1);
     abort_flag = 0;
@@ -502,23 +586,16 @@ __global__ void __launch_bounds__(kStatsThreads, 1)
   __syncthreads();
   tc_fence_after();
   const uint32_t tm = tmem_base;
-  // The prompt and the queries were complete before stats_tc passed its own
-  // wait, so the copies need not wait for stats_tc; its row statistics do.
-  if (warp != 0) {
-    grid_dependency_wait();
-    grid_launch_dependents();
-  }
 
+  // The prompt and the queries were complete before stats_tc passed its own
+  // wait, so the copies and products need not wait for stats_tc; its row
+  // statistics do.
   if (warp == 0) {
     if (lane == 0) {
       mbar_arrive_expect_tx(&qfull, 2u * RWb * kBoxBytes);
       for (int bx = 0; bx < 2; ++bx) tma_load_3d(sQ + bx * RWb * kBoxBytes, &tmQ, bx * 64, 0, u, &qfull);
-      for (int i = kS; i < min(kS + kPF, n_tiles); ++i)
-        for (int bx = 0; bx < 2; ++bx) tma_prefetch_3d(&tmK, bx * 64, t_begin + i * kTok, u);
       for (int i = 0; i < n_tiles; ++i) {
         const int s = i % kS, j = i / kS;
-        if (kPF > 0 && i + kS + kPF < n_tiles)
-          for (int bx = 0; bx < 2; ++bx) tma_prefetch_3d(&tmK, bx * 64, t_begin + (i + kS + kPF) * kTok, u);
         if (j >= 1 && !pwait(&empty[s], (j - 1) & 1, abrt, p.ws, u, p.polls)) break;
         mbar_arrive_expect_tx(&full[s], kTileBytes);
         for (int bx = 0; bx < 2; ++bx)
@@ -532,15 +609,15 @@ __global__ void __launch_bounds__(kStatsThreads, 1)
       const uint32_t aQ = smem_addr(sQ);
       const bool ok = pwait(&qfull, 0, abrt, p.ws, u, p.polls);
       for (int i = 0; ok && i < n_tiles; ++i) {
-        const int s = i % kS, j = i / kS, b = i & 1;
+        const int s = i % kS, j = i / kS, b = i % NB;
         if (!pwait(&full[s], j & 1, abrt, p.ws, u, p.polls)) break;
-        if (i >= 2 && !pwait(&lempty[b], ((i >> 1) - 1) & 1, abrt, p.ws, u, p.polls)) break;
+        if (i >= NB && !pwait(&lempty[b], (i / NB - 1) & 1, abrt, p.ws, u, p.polls)) break;
         tc_fence_after();
         const uint32_t aK = smem_addr(sK + s * kTileBytes);
         for (int kk = 0; kk < 8; ++kk) {
           const uint64_t dk = sdesc_sw128(aK + (kk >> 2) * kBoxBytes + (kk & 3) * 32, 16, 1024);
           const uint64_t dq = sdesc_sw128(aQ + (kk >> 2) * RWb * kBoxBytes + (kk & 3) * 32, 16, 1024);
-          umma_bf16(tm + b * 256, dk, dq, id, kk > 0 ? 1u : 0u);
+          umma_bf16(tm + b * RWp, dk, dq, id, kk > 0 ? 1u : 0u);
         }
         umma_commit(&lfull[b]);
         umma_commit(&empty[s]);
@@ -548,51 +625,69 @@ __global__ void __launch_bounds__(kStatsThreads, 1)
       umma_commit(&mma_done);  // every MMA issued has completed
     }
   } else {
-    // two epilogue groups (warps 2..5 and 6..9) take alternate tiles; group g
-    // always reads TMEM buffer g
     const int grp = (warp - 2) >> 2, qd = warp & 3;
-    const uint32_t lane_base = static_cast<uint32_t>(qd * 32) << 16;
+    const int b = grp % NB, half = grp / NB;  // this group's buffer, and its 128 columns of it
+    const uint32_t cols = tm + (static_cast<uint32_t>(qd * 32) << 16) + b * RWp + half * 128;
+    grid_dependency_wait();
+    grid_launch_dependents();
     // merged row statistics of every window row
-    for (int r = tid - 64; r < RWp; r += 256) {
+    for (int r = tid - 64; r < RWp; r += 512) {
       float M = -INFINITY, Lsum = 0.f;
       if (r < p.RW) {
-        for (int c = 0; c < p.n_chunks; ++c)
-          M = fmaxf(M, p.rowpart[(((size_t)u * p.n_chunks + c) * p.RW + r) * 2]);
+        const float2* rp = reinterpret_cast<const float2*>(p.rowpart) + (size_t)u * p.n_chunks * p.RW + r;
+#pragma unroll 8
+        for (int c = 0; c < p.n_chunks; ++c) M = fmaxf(M, rp[(size_t)c * p.RW].x);
         if (M != -INFINITY)
+#pragma unroll 8
           for (int c = 0; c < p.n_chunks; ++c) {
-            const float* rp = p.rowpart + (((size_t)u * p.n_chunks + c) * p.RW + r) * 2;
-            if (rp[0] != -INFINITY) Lsum += rp[1] * fast_exp2(rp[0] - M);
+            const float2 v = rp[(size_t)c * p.RW];
+            if (v.x != -INFINITY) Lsum += v.y * fast_exp2(v.x - M);
           }
       }
       s_b[r] = (Lsum > 0.f) ? -log2f(Lsum) - M : -INFINITY;
       s_wi[r] = r % p.W;
     }
-    asm volatile("bar.sync 1, 256;" ::: "memory");
+    named_sync(1, 512);
     const int t_safe = p.causal ? p.T - p.W : 0x7fffffff;  // tokens every window row sees
-    for (int i = grp; i < n_tiles; i += 2) {
-      const int b = i & 1;
-      if (!pwait(&lfull[b], (i >> 1) & 1, abrt, p.ws, u, p.polls)) break;
+    const float* sb = s_b + half * 128;
+    for (int i = b; i < n_tiles; i += NB) {
+      if (!pwait_warp(&lfull[b], (i / NB) & 1, abrt, p.ws, u, p.polls)) break;
       tc_fence_after();
       const int t = t_begin + i * kTok + qd * 32 + lane;  // token of this thread (TMEM lane)
       const bool fast = t <= t_safe;  // every window row sees this token
       float acc = 0.f;
-      for (int c0 = 0; c0 < RWp; c0 += 32) {
+#pragma unroll 2
+      for (int c0 = 0; c0 < 128; c0 += 32) {
         float x[32];
-        tmem_ld32(tm + lane_base + b * 256 + c0, x);
+        tmem_ld32(cols + c0, x);
         if (fast) {  // p = 2^(x qscale + b_r); padding rows have b_r = -inf
 #pragma unroll
           for (int jj = 0; jj < 32; jj += 4) {
-            const float4 b4 = *reinterpret_cast<const float4*>(s_b + c0 + jj);
+            const float4 b4 = *reinterpret_cast<const float4*>(sb + c0 + jj);
             acc += fast_exp2(fmaf(x[jj], p.qscale, b4.x)) + fast_exp2(fmaf(x[jj + 1], p.qscale, b4.y)) +
                    fast_exp2(fmaf(x[jj + 2], p.qscale, b4.z)) + fast_exp2(fmaf(x[jj + 3], p.qscale, b4.w));
           }
         } else {
 #pragma unroll
           for (int jj = 0; jj < 32; ++jj) {
-            const int r = c0 + jj;
+            const int r = half * 128 + c0 + jj;
             if (t <= p.T - p.W + s_wi[r]) acc += fast_exp2(fmaf(x[jj], p.qscale, s_b[r]));
           }
         }
+      }
+      if (half == 1) {  // the upper rows' sums go to the group of the lower ones
+        s_part[b][qd * 32 + lane] = acc;
+        tc_fence_before();
+        __syncwarp();
+        if (lane == 0) {
+          mbar_arrive(&pfull[b]);
+          mbar_arrive(&lempty[b]);
+        }
+        continue;
+      }
+      if (RWb == 2) {
+        if (!pwait_warp(&pfull[b], (i / NB) & 1, abrt, p.ws, u, p.polls)) break;
+        acc += s_part[b][qd * 32 + lane];
       }
       tc_fence_before();
       __syncwarp();
@@ -618,6 +713,18 @@ __global__ void __launch_bounds__(kStatsThreads, 1)
 }
 
 // ------------------------------------------------------------ residual_tc
+// score2 = s_t ||v_t - mu_v0 - scale C0' k_t||.  Only the top k of it matter,
+// and ||r_t|| lies within c_t = ||mu_v0|| + scale ||C0'||_F ||k_t|| of ||v_t||:
+// with theta the smallest s_t (||v_t|| - c_t) over the first stage's k free
+// rows, at least k positions reach theta, so a position with
+// s_t (||v_t|| + c_t) < theta is not among the top k.  With `prune` a CTA
+// compares its positions' scores and norms against theta, gathers the rows
+// that remain (a few times the budget where C0' is small beside the values)
+// and computes score2 of those; the others get 0, which the k higher ones keep
+// out.  Reading K and V a second time is what the full pass costs: 128 us at
+// 32K, batch 4, against about 10 for the gathered rows.  When more than half
+// of a CTA's positions remain, or the caller wants score2 itself, the full
+// pass runs; a position's score2 is the same bits either way.
 __global__ void __launch_bounds__(kStatsThreads, 1)
     residual_tc(const TcArgs p, const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtensorMap tmV) {
   constexpr int kS = 2;
@@ -628,21 +735,33 @@ __global__ void __launch_bounds__(kStatsThreads, 1)
   uint8_t* sC = sm + 2 * kS * kTileBytes;  // [3 parts][128 x 128]: C0' = hi + mid + lo
   __shared__ __align__(8) uint64_t full[kS], empty[kS], yfull[2], yempty[2], cfull, mma_done;
   __shared__ uint32_t tmem_base;
-  __shared__ int abort_flag, s_issued;
+  __shared__ int abort_flag, s_issued, s_cnt;
+  __shared__ uint32_t s_theta;              // bits of a float >= 0
   __shared__ float s_mv[kDP];
+  __shared__ float s_mvn[kMaxHs], s_fro[kMaxHs];  // per head of the selection group: ||mu_v0||, scale ||C0'||_F
 
   const int chunk = blockIdx.x, u = blockIdx.y;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int t_begin = chunk * p.chunk;
   const int t_end = min(p.n_rows, t_begin + p.chunk);
-  const int n_tiles = (max(0, t_end - t_begin) + kTok - 1) / kTok;
   volatile int* abrt = &abort_flag;
   const int D = p.D;
+  const float scale = rsqrtf(static_cast<float>(D));
+  auto load_tile = [&](int i) {  // whole tile i of the chunk into stage i % kS
+    const int s = i % kS;
+    mbar_arrive_expect_tx(&full[s], 2u * kTileBytes);
+    for (int bx = 0; bx < 2; ++bx) {
+      tma_load_3d(sK + s * kTileBytes + bx * kBoxBytes, &tmK, bx * 64, t_begin + i * kTok, u, &full[s]);
+      tma_load_3d(sV + s * kTileBytes + bx * kBoxBytes, &tmV, bx * 64, t_begin + i * kTok, u, &full[s]);
+    }
+    s_issued = i + 1;
+  };
+  int n_tiles = (max(0, t_end - t_begin) + kTok - 1) / kTok;
 
   if (tid == 0) {
     for (int i = 0; i < kS; ++i) {
-      mbar_init(&full[i], 1);
-      mbar_init(&empty[i], 1 + 4);  // MMA commit + the 4 epilogue warps (value rows)
+      mbar_init(&full[i], p.prune ? 4 : 1);  // (set again when a pruning CTA turns to the full pass)
+      mbar_init(&empty[i], 1 + 4);           // MMA commit + the 4 epilogue warps (value rows)
     }
     for (int i = 0; i < 2; ++i) {
       mbar_init(&yfull[i], 1);
@@ -651,22 +770,14 @@ __global__ void __launch_bounds__(kStatsThreads, 1)
     mbar_init(&cfull, 1);
     mbar_init(&mma_done, 1);
     abort_flag = 0;
+    s_issued = 0;
+    s_cnt = 0;
+    s_theta = 0x7f800000u;
     mbar_fence_init();
     // the first stages' copies go out before the dependency wait: the prompt
     // was complete before the compression began
-    for (int i = kS; i < min(kS + kPF, n_tiles); ++i)
-      for (int bx = 0; bx < 2; ++bx) {
-        tma_prefetch_3d(&tmK, bx * 64, t_begin + i * kTok, u);
-        tma_prefetch_3d(&tmV, bx * 64, t_begin + i * kTok, u);
-      }
-    for (int i = 0; i < min(kS, n_tiles); ++i) {
-      mbar_arrive_expect_tx(&full[i], 2u * kTileBytes);
-      for (int bx = 0; bx < 2; ++bx) {
-        tma_load_3d(sK + i * kTileBytes + bx * kBoxBytes, &tmK, bx * 64, t_begin + i * kTok, u, &full[i]);
-        tma_load_3d(sV + i * kTileBytes + bx * kBoxBytes, &tmV, bx * 64, t_begin + i * kTok, u, &full[i]);
-      }
-    }
-    s_issued = min(kS, n_tiles);
+    if (!p.prune)
+      for (int i = 0; i < min(kS, n_tiles); ++i) load_tile(i);
   }
   if (warp == 1) tmem_alloc(&tmem_base, 256);
   if (D < kDP) {  // no second box of key dims: that part of the operand image is zero
@@ -688,24 +799,85 @@ __global__ void __launch_bounds__(kStatsThreads, 1)
   __syncthreads();
   tc_fence_after();
   const uint32_t tm = tmem_base;
-  const float scale = rsqrtf(static_cast<float>(D));
+
+  bool gather = false;
+  int32_t* list = p.cand + (size_t)u * p.T + t_begin;  // this CTA's remaining positions, in any order
+  if (p.prune) {
+    const int g0 = u / p.hs * p.hs;  // the selection group's first unit
+    for (int h = warp; h < p.hs; h += kStatsThreads / 32) {
+      float a2 = 0.f, f2 = 0.f;
+#pragma unroll
+      for (int j = 0; j < kDP; j += 32) {
+        const float x = p.mv0[(size_t)(g0 + h) * kDP + j + lane];
+        a2 = fmaf(x, x, a2);
+        if (j < p.n_fro) f2 += p.fro[(size_t)(g0 + h) * kDP + j + lane];
+      }
+      a2 = warp_sum(a2);
+      f2 = warp_sum(f2);
+      if (lane == 0) {
+        s_mvn[h] = sqrtf(a2);
+        s_fro[h] = scale * sqrtf(f2);
+      }
+    }
+    __syncthreads();
+    // theta: the smallest lower bound over the first stage's free rows (0 where a bound says nothing)
+    float lowest = INFINITY;
+#pragma unroll 4
+    for (int i = tid; i < p.hs * p.B; i += kStatsThreads) {
+      const int f = min(max(p.idx[(size_t)(g0 / p.hs) * p.hs * p.B + i], 0), p.hs * p.T - 1);
+      const int h = p.hs == 1 ? 0 : f / p.T, t = f - h * p.T;
+      if (!is_protected(t, p.T, p.W, p.sink, p.keep_window)) {
+        const float2 nn = reinterpret_cast<const float2*>(p.norms)[(size_t)g0 * p.T + f];
+        float lb = sqrtf(nn.y) - s_mvn[h] - s_fro[h] * sqrtf(nn.x);
+        lb = p.s_in[(size_t)g0 * p.T + f] * (lb > 0.f ? lb : 0.f);
+        lowest = fminf(lowest, lb > 0.f ? lb : 0.f);  // a NaN counts as 0
+      }
+    }
+    const uint32_t wmin = __reduce_min_sync(kFull, __float_as_uint(lowest));
+    if (lane == 0) atomicMin(&s_theta, wmin);
+    __syncthreads();
+    const float theta = __uint_as_float(s_theta) * 0.9999f;  // rounding of both sides: below 1e-6
+    const int h = u - g0;
+    const float mvn = s_mvn[h], fro = s_fro[h];
+#pragma unroll 4
+    for (int t0 = t_begin + warp * 32; t0 < t_end; t0 += kStatsThreads) {
+      const int t = t0 + lane;
+      bool cand = false;
+      if (t < t_end) {
+        const float2 nn = reinterpret_cast<const float2*>(p.norms)[(size_t)u * p.T + t];
+        const float ub = p.s_in[(size_t)u * p.T + t] * (sqrtf(nn.y) + mvn + fro * sqrtf(nn.x));
+        cand = !(ub < theta) && !is_protected(t, p.T, p.W, p.sink, p.keep_window);  // a NaN remains
+        if (!cand) p.s_out[(size_t)u * p.T + t] = 0.f;
+      }
+      const unsigned mask = __ballot_sync(kFull, cand);
+      if (mask != 0u) {
+        int at = 0;
+        if (lane == 0) at = atomicAdd(&s_cnt, __popc(mask));
+        at = __shfl_sync(kFull, at, 0) + __popc(mask & ((1u << lane) - 1u));
+        if (cand) list[at] = t;
+      }
+    }
+    __syncthreads();
+    gather = 2 * s_cnt <= t_end - t_begin;
+    if (gather) {
+      n_tiles = (s_cnt + kTok - 1) / kTok;
+    } else {
+      if (tid == 0) {
+        for (int i = 0; i < kS; ++i) {
+          asm volatile("mbarrier.inval.shared::cta.b64 [%0];" ::"r"(smem_addr(&full[i])) : "memory");
+          mbar_init(&full[i], 1);
+        }
+        mbar_fence_init();
+      }
+      __syncthreads();
+    }
+  }
 
   if (warp == 0) {
-    if (lane == 0) {
-      for (int i = kS; i < n_tiles; ++i) {
-        const int s = i % kS, j = i / kS;
-        if (kPF > 0 && i + kPF < n_tiles)
-          for (int bx = 0; bx < 2; ++bx) {
-            tma_prefetch_3d(&tmK, bx * 64, t_begin + (i + kPF) * kTok, u);
-            tma_prefetch_3d(&tmV, bx * 64, t_begin + (i + kPF) * kTok, u);
-          }
-        if (!pwait(&empty[s], (j - 1) & 1, abrt, p.ws, u, p.polls)) break;
-        mbar_arrive_expect_tx(&full[s], 2u * kTileBytes);
-        for (int bx = 0; bx < 2; ++bx) {
-          tma_load_3d(sK + s * kTileBytes + bx * kBoxBytes, &tmK, bx * 64, t_begin + i * kTok, u, &full[s]);
-          tma_load_3d(sV + s * kTileBytes + bx * kBoxBytes, &tmV, bx * 64, t_begin + i * kTok, u, &full[s]);
-        }
-        s_issued = i + 1;
+    if (lane == 0 && !gather) {
+      for (int i = s_issued; i < n_tiles; ++i) {
+        if (i >= kS && !pwait(&empty[i % kS], (i / kS - 1) & 1, abrt, p.ws, u, p.polls)) break;
+        load_tile(i);
       }
     }
   } else if (warp == 1) {
@@ -733,14 +905,36 @@ __global__ void __launch_bounds__(kStatsThreads, 1)
     }
   } else {
     // two epilogue groups (warps 2..5 and 6..9) take alternate tiles; group g
-    // always reads TMEM buffer g
+    // always reads stage g and TMEM buffer g
     const int grp = (warp - 2) >> 2, qd = warp & 3;
     const uint32_t lane_base = static_cast<uint32_t>(qd * 32) << 16;
-    const int row = qd * 32 + lane;  // token within the tile = TMEM lane
+    const int row = qd * 32 + lane;  // row within the tile = TMEM lane
     for (int i = grp; i < n_tiles; i += 2) {
       const int s = i % kS, j = i / kS, b = i & 1;
-      if (!pwait(&yfull[b], (i >> 1) & 1, abrt, p.ws, u, p.polls)) break;
-      if (!pwait(&full[s], j & 1, abrt, p.ws, u, p.polls)) break;
+      int t = t_begin + i * kTok + row;
+      bool live = t < t_end;
+      if (gather) {
+        // this warp's 32 rows of the list into the stage (free: the group is
+        // done with its tile i - 2, whose MMAs it waited for): 16 chunks of k
+        // and 16 of v a row, a row per step
+        live = i * kTok + row < s_cnt;
+        t = live ? list[i * kTok + row] : -1;
+#pragma unroll 4
+        for (int r = 0; r < 32; ++r) {
+          const int tr = __shfl_sync(kFull, t, r), c = lane & 15, rr = qd * 32 + r;
+          const uint8_t* src = reinterpret_cast<const uint8_t*>(lane < 16 ? p.K : p.V) +
+                               (((size_t)u * p.T + max(tr, 0)) * D + (c < D / 8 ? c * 8 : 0)) * 2;
+          uint8_t* dst = (lane < 16 ? sK : sV) + s * kTileBytes + (c >> 3) * kBoxBytes + rr * 128 +
+                         (((c & 7) ^ (rr & 7)) << 4);
+          cp_async16(dst, src, tr >= 0 && c < D / 8 ? 16u : 0u);
+        }
+        asm volatile("cp.async.wait_all;" ::: "memory");
+        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");  // generic writes -> tensor-core reads
+        __syncwarp();
+        if (lane == 0) mbar_arrive(&full[s]);
+      }
+      if (!pwait_warp(&yfull[b], (i >> 1) & 1, abrt, p.ws, u, p.polls)) break;
+      if (!pwait_warp(&full[s], j & 1, abrt, p.ws, u, p.polls)) break;
       tc_fence_after();
       const uint8_t* tv = sV + s * kTileBytes;
       float ss = 0.f;
@@ -769,8 +963,7 @@ __global__ void __launch_bounds__(kStatsThreads, 1)
         mbar_arrive(&yempty[b]);
         mbar_arrive(&empty[s]);
       }
-      const int t = t_begin + i * kTok + row;
-      if (t < t_end) {
+      if (live) {
         const bool prot = is_protected(t, p.T, p.W, p.sink, p.keep_window);
         const float v = prot ? 0.f : p.s_in[(size_t)u * p.T + t] * sqrtf(ss);
         p.s_out[(size_t)u * p.T + t] = v;
@@ -804,7 +997,8 @@ __global__ void __launch_bounds__(kStatsThreads, 1)
 // (key, f); one more pass counts and one writes.  Two cluster barriers, where
 // a radix select over the keys took four passes of three barriers each.  When
 // a CTA holds more than kMaxCont keys of that bin (many equal scores), the
-// cluster bisects the key and then f instead.
+// cluster bisects the key and then f instead.  512 threads for a unit (64
+// CTAs a wave at 8 units), 1024 for the longer joint lists.
 struct SelectArgs {
   const float* scores;   // [units][T]
   const uint32_t* hist;  // [units][kBins] counts of the unprotected scores' keys
@@ -816,13 +1010,14 @@ struct SelectArgs {
   int32_t* hbeg;      // [units] the unit's first slot in idx
 };
 
-constexpr int kSelThreads = 512;
-constexpr int kSelWarps = kSelThreads / 32;
 constexpr int kSelCL = 8;      // CTAs per selection group (one cluster), each over a contiguous range of pairs
 constexpr int kMaxCont = 256;  // keys of the contested bin a CTA may hold
-constexpr int kMaxHs = 64;     // KV heads of a batch item with the adaptive budget
 
-__global__ void __cluster_dims__(kSelCL, 1, 1) __launch_bounds__(kSelThreads, 2) select_kernel(const SelectArgs a) {
+template <int kSelThreads>
+__global__ void __cluster_dims__(kSelCL, 1, 1) __launch_bounds__(kSelThreads, 1024 / kSelThreads)
+    select_kernel(const SelectArgs a) {
+  constexpr int kSelWarps = kSelThreads / 32;
+  constexpr int kBatch = 8;  // pairs per lane loaded together
   __shared__ int s_w[kSelWarps];
   __shared__ int s_bin, s_need;
   __shared__ int s_n;                                          // this CTA's contested keys
@@ -852,11 +1047,30 @@ __global__ void __cluster_dims__(kSelCL, 1, 1) __launch_bounds__(kSelThreads, 2)
   grid_dependency_wait();
   grid_launch_dependents();
 
-  // pairs are ordered by (key, ~f): a higher key first, at equal keys the lower f
-  auto pair_of = [&](int f) -> unsigned long long {  // 0: protected (or past the end)
+  // pairs are ordered by (key, ~f): a higher key first, at equal keys the lower f;
+  // a protected pair stands above all
+  auto pair_of = [&](int f, float s) -> unsigned long long {
     const int t = hs == 1 ? f : f % T;
-    if (is_protected(t, T, W, a.sink, a.keep_window)) return 0ull;
-    return (static_cast<unsigned long long>(score_key(sc[f])) << 32) | (0xffffffffu - static_cast<unsigned>(f));
+    if (is_protected(t, T, W, a.sink, a.keep_window)) return ~0ull;
+    return (static_cast<unsigned long long>(score_key(s)) << 32) | (0xffffffffu - static_cast<unsigned>(f));
+  };
+  // fn(f, in range, pair) for every pair of this warp, kBatch x 32 loads in flight
+  auto each_pair = [&](auto&& fn) {
+#pragma unroll 1
+    for (int f0 = w0; f0 < w1; f0 += 32 * kBatch) {
+      float s[kBatch];
+#pragma unroll
+      for (int i = 0; i < kBatch; ++i) {
+        const int f = f0 + i * 32 + lane;
+        s[i] = f < w1 ? sc[f] : 0.f;
+      }
+#pragma unroll
+      for (int i = 0; i < kBatch; ++i) {
+        if (f0 + i * 32 >= w1) break;  // warp-uniform
+        const int f = f0 + i * 32 + lane;
+        fn(f, f < w1, pair_of(f, s[i]));
+      }
+    }
   };
   // exclusive sum over the block of one count per warp (`mine` from lane 0); the total in *total
   auto block_counts = [&](int mine, int* total) -> int {
@@ -876,14 +1090,15 @@ __global__ void __cluster_dims__(kSelCL, 1, 1) __launch_bounds__(kSelThreads, 2)
   // ---- the bin of the k-th highest key: thread t takes four bins, descending
   if (k > 0) {
     uint4 c = make_uint4(0u, 0u, 0u, 0u);
-#pragma unroll 2
-    for (int h = 0; h < hs; ++h) {
-      const uint4 x = reinterpret_cast<const uint4*>(a.hist + ((size_t)grp * hs + h) * kBins)[kBins / 4 - 1 - tid];
-      c.x += x.x;
-      c.y += x.y;
-      c.z += x.z;
-      c.w += x.w;
-    }
+    if (tid < kBins / 4)
+#pragma unroll 4
+      for (int h = 0; h < hs; ++h) {
+        const uint4 x = reinterpret_cast<const uint4*>(a.hist + ((size_t)grp * hs + h) * kBins)[kBins / 4 - 1 - tid];
+        c.x += x.x;
+        c.y += x.y;
+        c.z += x.z;
+        c.w += x.w;
+      }
     const int b[4] = {(int)c.w, (int)c.z, (int)c.y, (int)c.x};
     int incl = b[0] + b[1] + b[2] + b[3];
     const int mine = incl;
@@ -905,14 +1120,12 @@ __global__ void __cluster_dims__(kSelCL, 1, 1) __launch_bounds__(kSelThreads, 2)
     __syncthreads();
     const int bin = s_bin;
     // ---- the contested keys: this CTA's into every CTA's list
-#pragma unroll 4
-    for (int f0 = w0; f0 < w1; f0 += 32) {
-      const unsigned long long p = f0 + lane < w1 ? pair_of(f0 + lane) : 0ull;
-      if (p != 0ull && key_bin(static_cast<uint32_t>(p >> 32)) == bin) {
+    each_pair([&](int f, bool in, unsigned long long p) {
+      if (in && p != ~0ull && key_bin(static_cast<uint32_t>(p >> 32)) == bin) {
         const int slot = atomicAdd(&s_n, 1);
         if (slot < kMaxCont) s_cont[rank][slot] = p;
       }
-    }
+    });
     __syncthreads();
     cluster_wait_acquire();
     const int mn = s_n;
@@ -951,7 +1164,7 @@ __global__ void __cluster_dims__(kSelCL, 1, 1) __launch_bounds__(kSelThreads, 2)
       for (int bit = 63; bit >= 0; --bit) {
         const unsigned long long mid = lo | (1ull << bit);
         int c = 0;
-        for (int f = w0 + lane; f < w1; f += 32) c += pair_of(f) >= mid ? 1 : 0;
+        each_pair([&](int f, bool in, unsigned long long p) { c += in && p != ~0ull && p >= mid ? 1 : 0; });
         c = __reduce_add_sync(kFull, c);
         int tot;
         (void)block_counts(c, &tot);
@@ -970,13 +1183,8 @@ __global__ void __cluster_dims__(kSelCL, 1, 1) __launch_bounds__(kSelThreads, 2)
 
   // ---- this CTA's selections, then everybody's: protected pairs and those not below the last
   const unsigned long long last = s_last;
-  auto selected = [&](int f) -> bool {
-    const unsigned long long p = pair_of(f);
-    return p == 0ull || p >= last;
-  };
   int c = 0;
-#pragma unroll 4
-  for (int f0 = w0; f0 < w1; f0 += 32) c += __popc(__ballot_sync(kFull, f0 + lane < w1 && selected(f0 + lane)));
+  each_pair([&](int f, bool in, unsigned long long p) { c += __popc(__ballot_sync(kFull, in && p >= last)); });
   int tot;
   int o = block_counts(c, &tot);
   if (tid < kSelCL) *cluster.map_shared_rank(&s_tot[0][rank], tid) = tot;
@@ -984,10 +1192,8 @@ __global__ void __cluster_dims__(kSelCL, 1, 1) __launch_bounds__(kSelThreads, 2)
   for (int r = 0; r < rank; ++r) o += s_tot[0][r];
   const int n_sel = hs * a.B;  // the group's selections (protected included)
   int32_t* out = a.idx + (size_t)grp * n_sel;
-#pragma unroll 2
-  for (int f0 = w0; f0 < w1; f0 += 32) {
-    const int f = f0 + lane;
-    const bool sel = f < w1 && selected(f);
+  each_pair([&](int f, bool in, unsigned long long p) {
+    const bool sel = in && p >= last;
     const unsigned mask = __ballot_sync(kFull, sel);
     const int at = o + __popc(mask & ((1u << lane) - 1u));
     if (sel && at < n_sel) {
@@ -996,7 +1202,7 @@ __global__ void __cluster_dims__(kSelCL, 1, 1) __launch_bounds__(kSelThreads, 2)
       if (hs > 1) atomicAdd(&s_hcnt[f / T], 1);
     }
     o += __popc(mask);
-  }
+  });
   if (hs == 1) {
     if (rank == 0 && tid == 0) {
       a.cnt[grp] = a.B;
@@ -1067,11 +1273,6 @@ struct RsetArgs {
   void* ws;
   uint32_t polls;
 };
-
-__device__ __forceinline__ void cp_async16(void* dst, const void* src, uint32_t src_bytes) {
-  asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(smem_addr(dst)), "l"(src), "r"(src_bytes)
-               : "memory");
-}
 
 template <int CL, bool FINAL>
 __global__ void __launch_bounds__(2048 / CL) rset_kernel(const RsetArgs a) {
@@ -1282,8 +1483,8 @@ __global__ void __launch_bounds__(2048 / CL) rset_kernel(const RsetArgs a) {
   // ---- R's sums over the cluster, and E = all \ R
   const float nR = ok ? static_cast<float>(cnt) : 0.f;
   float SR[4] = {0.f, 0.f, 0.f, 0.f}, rk[4] = {0.f, 0.f, 0.f, 0.f}, rv = 0.f;
-#pragma unroll 2
-  for (int r = 0; r < min(CL, max(1, n_tiles)); ++r) {  // ranks past the tiles hold zeros
+#pragma unroll
+  for (int r = 0; r < CL; ++r) {  // ranks past the tiles hold zeros; all loads in flight
     const float4 k4 = *reinterpret_cast<const float4*>(cluster.map_shared_rank(s_sk, r) + cq * 4);
     const float4 s4 = *reinterpret_cast<const float4*>(cluster.map_shared_rank(red, r) + row * kRsRed + cq * 4);
     rv += cluster.map_shared_rank(s_sv, r)[row];
@@ -1331,6 +1532,8 @@ __global__ void __launch_bounds__(2048 / CL) rset_kernel(const RsetArgs a) {
     float r4[4];
 #pragma unroll
     for (int j = 0; j < 4; ++j) r4[j] = (row < D && !(fabsf(CE[j] * nE) < a.tau)) ? CE[j] : 0.f;
+    const float fro = warp_sum(r4[0] * r4[0] + r4[1] * r4[1] + r4[2] * r4[2] + r4[3] * r4[3]);
+    if (lane == 0) L.fro[(size_t)u * kDP + kh * 64 + rank * (RW / 2) + warp] = fro;  // two rows' part of ||C0'||_F^2
     uint8_t* img = L.cimg + (size_t)u * 3 * kTileBytes + swz_off(row, kh * 64 + cq * 4, kTok);
 #pragma unroll
     for (int part = 0; part < 3; ++part) {
@@ -1378,9 +1581,12 @@ __global__ void __launch_bounds__(256) keep_all_kernel(const CompressArgs a, int
 }
 
 // ------------------------------------------------------------------- host
-constexpr size_t kStatsSmem = 1024 + 2 * 2 * kTileBytes + 2 * 2 * kBoxBytes + 4096;  // K, V stages, Q, ones
-constexpr size_t kScoresSmem = 1024 + 3 * kTileBytes + 2 * 2 * kBoxBytes;
+constexpr size_t kScoresSmem = 1024 + 4 * kTileBytes + 2 * 2 * kBoxBytes;
 constexpr size_t kResidualSmem = 1024 + 2 * 2 * kTileBytes + 3 * kTileBytes;
+
+// residual_tc compares scores and norms before it reads rows when its CTAs
+// have at least this many tiles; below, the full pass takes no longer.
+constexpr int kPruneTiles = 8;
 
 // A launch that may begin while the kernel before it on the stream drains (it
 // waits for that kernel's end by itself); cl > 0: in clusters of cl CTAs
@@ -1436,7 +1642,7 @@ cudaError_t run(const CompressArgs& a, const mkv_geom& g, int num_sms, cudaStrea
   const int D = g.head_dim, T = a.T, B = a.budget, U = L.units;
   const bool keep_all = T <= B;
   cudaError_t e = cudaSuccess;
-  if ((e = smem_attr((const void*)stats_tc, kStatsSmem)) != cudaSuccess) return e;
+  if ((e = smem_attr((const void*)stats_tc, std::max(stats_smem(1), stats_smem(2)))) != cudaSuccess) return e;
   if ((e = smem_attr((const void*)scores_tc, kScoresSmem)) != cudaSuccess) return e;
   if ((e = smem_attr((const void*)residual_tc, kResidualSmem)) != cudaSuccess) return e;
 
@@ -1465,16 +1671,17 @@ cudaError_t run(const CompressArgs& a, const mkv_geom& g, int num_sms, cudaStrea
   tp.mrec = L.mpart;
   tp.hist = L.hist;
   tp.units = U;
+  tp.norms = L.norms;
   tp.ws = a.ws;
   tp.polls = pipeline_poll_limit();
   const dim3 cg(L.n_chunks, U);
 
   if (!keep_all || a.diag_scores != nullptr) {
-    if ((e = launch_pdl(stats_tc, cg, kStatsThreads, kStatsSmem, st, 0, tp, tmK, tmV, tmQ)) != cudaSuccess) return e;
+    if ((e = launch_pdl(stats_tc, cg, kStatsThreads, stats_smem(L.RWb), st, 0, tp, tmK, tmV, tmQ)) != cudaSuccess) return e;
     TcArgs p2 = tp;
     p2.s_out = L.s;
     p2.diag = a.diag_scores;
-    if ((e = launch_pdl(scores_tc, cg, kStatsThreads, kScoresSmem, st, 0, p2, tmK, tmQ)) != cudaSuccess) return e;
+    if ((e = launch_pdl(scores_tc, cg, kScoreThreads, kScoresSmem, st, 0, p2, tmK, tmQ)) != cudaSuccess) return e;
   }
   if (keep_all) {
     if (D == 128) keep_all_kernel<128><<<dim3((T + 7) / 8, U), 256, 0, st>>>(a, T);
@@ -1496,7 +1703,8 @@ cudaError_t run(const CompressArgs& a, const mkv_geom& g, int num_sms, cudaStrea
     sa.hs = L.hs;
     sa.cnt = L.cnt;
     sa.hbeg = L.hbeg;
-    return launch_pdl(select_kernel, dim3(U / L.hs * kSelCL), kSelThreads, 0, st, 0, sa);
+    if (L.hs == 1) return launch_pdl(select_kernel<512>, dim3(U * kSelCL), 512, 0, st, 0, sa);
+    return launch_pdl(select_kernel<1024>, dim3(U / L.hs * kSelCL), 1024, 0, st, 0, sa);
   };
   RsetArgs ra{};
   ra.L = L;
@@ -1525,6 +1733,16 @@ cudaError_t run(const CompressArgs& a, const mkv_geom& g, int num_sms, cudaStrea
     r.s_out = L.s2;
     r.hist = hist2;
     r.diag = a.diag_score2;
+    // a second pass over the prompt is worth avoiding from eight tiles a CTA on
+    r.prune = a.diag_score2 == nullptr && L.chunk >= kPruneTiles * kTok ? 1 : 0;
+    r.hs = L.hs;
+    r.B = B;
+    r.idx = L.idx;
+    r.fro = L.fro;
+    r.n_fro = D;
+    r.cand = L.cand;
+    r.K = a.K;
+    r.V = a.V;
     if ((e = launch_pdl(residual_tc, cg, kStatsThreads, kResidualSmem, st, 0, r, tmK, tmV)) != cudaSuccess) return e;
     if ((e = select(L.s2, hist2, nullptr)) != cudaSuccess) return e;
   }

@@ -1,0 +1,99 @@
+"""The selections of mkv_compress where its shortcuts could go wrong, on the GPU.
+
+Second stage: without the score2 output the residual pass computes only the
+positions whose score bound reaches the first stage's; with it, all of them.
+Both must leave the same bits in the cache and the moments (a computed
+position's score2 is the same either way), whatever the bound is worth.
+First stage: long runs of equal scores, where the threshold bin holds more
+keys than the selection exchanges, against a stable sort of the kernel's own
+scores."""
+import numpy as np
+import pytest
+import torch
+
+import oracle as O
+from paper_2606_01563_gb300 import mkv
+
+pytestmark = pytest.mark.gpu
+
+
+def compress(b, H, G, D, T, B, w, K, V, Q, adaptive, diag, pool=1, mi=1):
+    g = mkv.geom(b, H, G, D)
+    p = mkv.mkv_compress_params(B, w, 1, 1, pool, mi, 1, 1e-6, adaptive)
+    prot = 1 + w
+    cap = min(T, H * (B - prot) + prot) if adaptive else B
+    cache, mom = mkv.alloc_cache(g, cap), mkv.alloc_moments(g)
+    ws = mkv.alloc_workspace(mkv.mkv_compress_workspace_size(g, T, p))
+    ws.fill_(0xA5)  # the workspace needs no initialisation
+    s, s2 = torch.zeros(b, H, T, device="cuda"), torch.zeros(b, H, T, device="cuda")
+    mkv.mkv_compress(g, T, K, V, Q, p, cache, mom, ws, diag=(s, s2, None) if diag else None)
+    # the error word sits in the workspace, which held no valid status before the call
+    torch.cuda.synchronize()
+    return dict(K=cache.K, V=cache.V, pos=cache.pos, len=cache.len, n=mom.n, mu_k=mom.mu_k, mu_v=mom.mu_v, C=mom.C,
+                s=s, s2=s2)
+
+
+def draw(seed, b, H, G, D, T, w, kind):
+    gen = torch.Generator(device="cuda")
+    gen.manual_seed(seed)
+    r = lambda *s: torch.randn(*s, generator=gen, device="cuda")
+    K, V = r(b, H, T, D), r(b, H, T, D)
+    if kind == "outlier":  # a few long keys: loose bounds for their positions
+        K[:, :, ::97] *= 30.0
+    elif kind == "correlated":  # C0' as large as the values: the bound says little
+        V = 0.9 * K + 0.1 * V
+    elif kind == "offset":  # values far from zero
+        V = V + 8.0
+    elif kind == "zero_values":  # every score2 is the residual of nothing
+        V = torch.zeros_like(V)
+    elif kind == "infinite":  # bounds and scores that are not finite
+        V[:, :, T // 3, 0] = float("inf")
+    rows = torch.randint(0, T, (b, H, G * w, 3), generator=gen, device="cuda")
+    q = torch.stack([K[i, j][rows[i, j]].sum(1) for i in range(b) for j in range(H)]).view(b, H, G, w, D)
+    q = D ** 0.5 * q / torch.linalg.norm(q, dim=-1, keepdim=True) + 0.3 * r(b, H, G, w, D)
+    return K.to(torch.bfloat16), V.to(torch.bfloat16), q.to(torch.bfloat16)
+
+
+@pytest.mark.parametrize("kind", ["plain", "outlier", "correlated", "offset", "zero_values", "infinite"])
+@pytest.mark.parametrize("b,H,G,D,T,B,w,adaptive", [
+    (4, 8, 4, 128, 8192, 256, 32, 0),   # 16 tiles per CTA
+    (2, 16, 2, 64, 4100, 100, 16, 0),   # ragged last tile, half-width rows
+    (4, 8, 4, 128, 5001, 200, 32, 1),   # the bound shared by eight heads
+])
+def test_pruned_residual_selects_the_same(kind, b, H, G, D, T, B, w, adaptive):
+    K, V, Q = draw(b * 1000 + D, b, H, G, D, T, w, kind)
+    full = compress(b, H, G, D, T, B, w, K, V, Q, adaptive, True)
+    pruned = compress(b, H, G, D, T, B, w, K, V, Q, adaptive, False)
+    np.testing.assert_array_equal(pruned["len"].cpu(), full["len"].cpu())
+    for name in ("pos", "K", "V", "n", "mu_k", "mu_v", "C"):
+        x, y = pruned[name].cpu(), full[name].cpu()
+        if x.dtype == torch.bfloat16:
+            x, y = x.view(torch.int16), y.view(torch.int16)
+        elif x.dtype == torch.float32:
+            x, y = x.view(torch.int32), y.view(torch.int32)
+        assert torch.equal(x, y), f"{name} differs at {int((x != y).sum())} of {x.numel()} places"
+
+
+@pytest.mark.parametrize("T,B,adaptive,pool", [(700, 64, 0, 1), (9000, 500, 0, 32), (30000, 900, 0, 1), (6000, 300, 1, 1)])
+def test_equal_scores_take_the_lowest_positions(T, B, adaptive, pool):
+    """Keys that repeat every few rows: most scores are equal to many others,
+    and a tie that crosses the budget is broken by position (head first)."""
+    H, G, D, w = 2, 2, 64, 16
+    gen = torch.Generator(device="cuda")
+    gen.manual_seed(T)
+    base = torch.randn(1, H, 3, D, generator=gen, device="cuda").to(torch.bfloat16)
+    K = base[:, :, torch.arange(T, device="cuda") % 3].contiguous()
+    V = torch.randn(1, H, T, D, generator=gen, device="cuda").to(torch.bfloat16)
+    Q = torch.randn(1, H, G, w, D, generator=gen, device="cuda").to(torch.bfloat16)
+    out = compress(1, H, G, D, T, B, w, K, V, Q, adaptive, True, pool=pool, mi=0)
+    t = np.arange(T)
+    prot = (t < 1) | (t >= T - w)
+    s = out["s"][0].double().cpu().numpy()
+    k = B - int(prot.sum())
+    if adaptive:
+        want, _ = O.select_topk_joint(s, H * k, np.stack([prot] * H))
+    else:
+        want = [O.select_topk(s[h], k, prot)[0] for h in range(H)]
+    for h in range(H):
+        got = out["pos"][0, h, :int(out["len"][0, h])].cpu().numpy()
+        np.testing.assert_array_equal(got, want[h])
