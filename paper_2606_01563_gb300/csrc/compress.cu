@@ -51,10 +51,15 @@ constexpr int kTok = 128;                   // tokens per tile
 constexpr int kDP = 128;                    // padded head dim of every MMA
 constexpr int kTileBytes = kTok * kDP * 2;  // one [128 x 128] bf16 tile: 2 boxes of 16 KB
 constexpr int kBoxBytes = kTok * 128;
-// stats_tc, residual_tc: two epilogue groups of 4 warps (2..5 and 6..9), so
-// that two warps per scheduler share the work
-constexpr int kStatsThreads = 320;
+// residual_tc: two epilogue groups of 4 warps (2..5 and 6..9), so that two
+// warps per scheduler share the work
+constexpr int kResThreads = 320;
 constexpr int kMaxHs = 64;  // KV heads of a batch item with the adaptive budget
+// scores_tc's K stages, and its shared memory
+__host__ __device__ constexpr int score_stages(int RWb) { return RWb == 1 ? 6 : 4; }
+__host__ __device__ constexpr size_t score_smem(int RWb) {
+  return (size_t)score_stages(RWb) * kTileBytes + (size_t)RWb * 2 * kBoxBytes + 256 * 4 + 256 + (RWb - 1) * 2 * 128 * 4;
+}
 // stats_tc's K/V stages: shared memory holds a third beside one block of window rows
 __host__ __device__ constexpr int stats_stages(int RWb) { return RWb == 1 ? 3 : 2; }
 __host__ __device__ constexpr size_t stats_smem(int RWb) {
@@ -189,12 +194,12 @@ __device__ __forceinline__ float half_warp_sums(float (&v)[8], int lane) {
   return v[0] + __shfl_xor_sync(kFull, v[0], 1);
 }
 
-__device__ __forceinline__ void epi_sync() { asm volatile("bar.sync 1, 256;" ::: "memory"); }
-// whether v holds in all 256 threads of the epilogue warps (barrier 1)
+__device__ __forceinline__ void epi_sync() { asm volatile("bar.sync 1, 384;" ::: "memory"); }
+// whether v holds in all 384 threads of stats_tc's epilogue and summing warps (barrier 1)
 __device__ __forceinline__ bool epi_all(bool v) {
   uint32_t r;
   asm volatile(
-      "{\n\t.reg .pred p, q;\n\tsetp.ne.u32 p, %1, 0;\n\tbar.red.and.pred q, 1, 256, p;\n\t"
+      "{\n\t.reg .pred p, q;\n\tsetp.ne.u32 p, %1, 0;\n\tbar.red.and.pred q, 1, 384, p;\n\t"
       "selp.u32 %0, 1, 0, q;\n\t}"
       : "=r"(r)
       : "r"((uint32_t)v)
@@ -268,10 +273,14 @@ struct TcArgs {
 // Window-row statistics, chunk moments and row norms of the prompt, in one
 // pass over K and V.  Bounded by that read (64 KB a tile and SM): the tensor
 // cores do the two products only, 1024 cycles a tile (column sums by products
-// with ones cost as many again), the epilogue warps take the column sums and
-// the norms from shared memory while a tile's logits are computed, and with up
-// to 128 window rows three stages are in flight and the logits double-buffered.
-__global__ void __launch_bounds__(kStatsThreads, 1)
+// with ones cost as many again); eight warps turn the logits into row
+// statistics, four others take the column sums and row norms from shared
+// memory (in the same warps the two cost 32 us of 125 at 32K, batch 4); with
+// up to 128 window rows three stages are in flight and the logits
+// double-buffered.  V streams through L2, so that more of K is still there for
+// the scores, which start from the end of the chunk.
+constexpr int kStatThreads = 64 + 256 + 128;
+__global__ void __launch_bounds__(kStatThreads, 1)
     stats_tc(const TcArgs p, const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtensorMap tmV,
              const __grid_constant__ CUtensorMap tmQ) {
   constexpr int kMaxS = 3;
@@ -284,9 +293,9 @@ __global__ void __launch_bounds__(kStatsThreads, 1)
   uint8_t* sQ = sm + (size_t)kS * 2 * kTileBytes;  // [2 boxes][RWb*128 rows][128 B]
   // after the last tile the first stage holds the epilogue's staging
   float* stg = reinterpret_cast<float*>(sm);                  // [2 groups][128][36]
-  float* s_pk = stg + 2 * 128 * 36;                           // [16][128] column sums of K per row group
-  float* s_pv = s_pk + 16 * 128;                              // the same of V
-  float* s_m1 = s_pv + 16 * 128;                              // [2][128] the second group's row maxima
+  float* s_pk = stg + 2 * 128 * 36;                           // [8][128] column sums of K per row group
+  float* s_pv = s_pk + 8 * 128;                               // the same of V
+  float* s_m1 = s_pv + 8 * 128;                              // [2][128] the second group's row maxima
   float* s_l1 = s_m1 + 2 * 128;                               // and sums
   float* sum_k = s_l1 + 2 * 128;                              // [128]
   float* sum_v = sum_k + kDP;                                 // [128]
@@ -304,7 +313,7 @@ __global__ void __launch_bounds__(kStatsThreads, 1)
   if (tid == 0) {
     for (int i = 0; i < kS; ++i) {
       mbar_init(&full[i], 1);
-      mbar_init(&empty[i], 1 + 8);  // the stage's MMAs and the epilogue warps' reads
+      mbar_init(&empty[i], 1 + 4);  // the stage's MMAs and the summing warps' reads
     }
     for (int i = 0; i < 2; ++i) {
       mbar_init(&lfull[i], 1);
@@ -326,47 +335,91 @@ __global__ void __launch_bounds__(kStatsThreads, 1)
 
   if (warp == 0) {
     if (lane == 0) {  // ---- producer
+      const uint64_t pol_v = l2_evict_first();
       mbar_arrive_expect_tx(&qfull, 2u * RWb * kBoxBytes);
       for (int bx = 0; bx < 2; ++bx) tma_load_3d(sQ + bx * RWb * kBoxBytes, &tmQ, bx * 64, 0, u, &qfull);
+      int s = 0;
+      uint32_t ph = 1;
       for (int i = 0; i < n_tiles; ++i) {
-        const int s = i % kS, j = i / kS;
-        if (j >= 1 && !pwait(&empty[s], (j - 1) & 1, abrt, p.ws, u, p.polls)) break;
+        if (i >= kS && !pwait(&empty[s], ph, abrt, p.ws, u, p.polls)) break;
         uint8_t* dst = sKV + (size_t)s * 2 * kTileBytes;
         mbar_arrive_expect_tx(&full[s], 2u * kTileBytes);
         for (int bx = 0; bx < 2; ++bx) tma_load_3d(dst + bx * kBoxBytes, &tmK, bx * 64, t_begin + i * kTok, u, &full[s]);
         for (int bx = 0; bx < 2; ++bx)
-          tma_load_3d(dst + kTileBytes + bx * kBoxBytes, &tmV, bx * 64, t_begin + i * kTok, u, &full[s]);
+          tma_load_3d_hint(dst + kTileBytes + bx * kBoxBytes, &tmV, bx * 64, t_begin + i * kTok, u, &full[s], pol_v);
         s_issued = i + 1;
+        if (++s == kS) {
+          s = 0;
+          ph ^= 1u;
+        }
       }
     }
   } else if (warp == 1) {
     if (lane == 0) {  // ---- MMA issuer
       const uint32_t idL = idesc_bf16(128, 128, 0, 0);  // logits: rows x tokens, both K-major
       const uint32_t idS = idesc_bf16(128, 128, 1, 1);  // V^T K: both MN-major (reduction over tokens)
-      const uint32_t aQ = smem_addr(sQ);
+      const uint64_t dq = sdesc_sw128(smem_addr(sQ), 16, 1024), dk0 = sdesc_sw128(smem_addr(sKV), 16, 1024);
+      const uint64_t ds0 = sdesc_sw128(smem_addr(sKV), kBoxBytes, 1024);
       const bool ok = pwait(&qfull, 0, abrt, p.ws, u, p.polls);
+      int s = 0, b = 0;               // stage and logits buffer of tile i, and their phases
+      uint32_t ph = 0, bph = 1;
       for (int i = 0; ok && i < n_tiles; ++i) {
-        const int s = i % kS, j = i / kS, b = i % NB;
-        if (!pwait(&full[s], j & 1, abrt, p.ws, u, p.polls)) break;
-        if (i >= NB && !pwait(&lempty[b], (i / NB - 1) & 1, abrt, p.ws, u, p.polls)) break;
+        if (!pwait(&full[s], ph, abrt, p.ws, u, p.polls)) break;
+        if (i >= NB && !pwait(&lempty[b], bph, abrt, p.ws, u, p.polls)) break;
         tc_fence_after();
-        const uint32_t aK = smem_addr(sKV + (size_t)s * 2 * kTileBytes), aV = aK + kTileBytes;
+        const uint32_t st = s * (2 * kTileBytes >> 4);  // in descriptor units
         for (int rb = 0; rb < RWb; ++rb)
-          for (int kk = 0; kk < 8; ++kk) {
-            const uint64_t dq =
-                sdesc_sw128(aQ + (kk >> 2) * RWb * kBoxBytes + rb * kBoxBytes + (kk & 3) * 32, 16, 1024);
-            const uint64_t dk = sdesc_sw128(aK + (kk >> 2) * kBoxBytes + (kk & 3) * 32, 16, 1024);
-            umma_bf16(tm + (b + rb) * 128, dq, dk, idL, kk > 0 ? 1u : 0u);
-          }
+          umma_k128(tm + (b + rb) * 128, dq + rb * (kBoxBytes >> 4), dk0 + st, RWb * kBoxBytes, kBoxBytes, idL, 0u);
         umma_commit(&lfull[b]);
-        for (int kk = 0; kk < 8; ++kk) {
-          const uint64_t dv = sdesc_sw128(aV + kk * 2048, kBoxBytes, 1024);
-          const uint64_t dk = sdesc_sw128(aK + kk * 2048, kBoxBytes, 1024);
-          umma_bf16(tm + cS, dv, dk, idS, (i > 0 || kk > 0) ? 1u : 0u);
-        }
+        umma_mn128(tm + cS, ds0 + st + (kTileBytes >> 4), ds0 + st, idS, i > 0 ? 1u : 0u);
         umma_commit(&empty[s]);
+        if (++s == kS) {
+          s = 0;
+          ph ^= 1u;
+        }
+        if (++b == NB) {
+          b = 0;
+          bph ^= 1u;
+        }
       }
       umma_commit(&sdone);
+    }
+  } else if (warp >= 10) {
+    // ---- column sums and row norms: warp w takes rows 32 w .. 32 w + 31, this
+    // lane the 8 dims of chunk lane % 16 in the rows lane / 16 + 2 j of them
+    const int sw = warp - 10, ch = lane & 15, rh = lane >> 4;
+    uint64_t ksum[4] = {0ull, 0ull, 0ull, 0ull}, vsum[4] = {0ull, 0ull, 0ull, 0ull};
+    for (int i = 0; i < n_tiles; ++i) {
+      const int s = i % kS;
+      if (!pwait_warp(&full[s], (i / kS) & 1, abrt, p.ws, u, p.polls)) break;
+#pragma unroll 1
+      for (int r16 = 0; r16 < 32; r16 += 16) {
+        const uint8_t* tk = sKV + (size_t)s * 2 * kTileBytes + (ch >> 3) * kBoxBytes + (sw * 32 + r16 + rh) * 128;
+        float kn[8], vn[8];
+#pragma unroll
+        for (int j = 0; j < 8; ++j) {
+          const uint32_t off = 2 * j * 128 + (((ch & 7) ^ ((rh + 2 * j) & 7)) << 4);
+          kn[j] = sum_chunk(*reinterpret_cast<const uint4*>(tk + off), ksum);
+          vn[j] = sum_chunk(*reinterpret_cast<const uint4*>(tk + kTileBytes + off), vsum);
+        }
+        // squared norms over the 16 lanes of each row: lanes 2 x, 2 x + 1 of a half hold its row 2 x
+        const float kq = half_warp_sums(kn, lane), vq = half_warp_sums(vn, lane);
+        const int t = t_begin + i * kTok + sw * 32 + r16 + rh + 2 * ((lane >> 1) & 7);
+        if (t < t_end) p.norms[((size_t)u * p.T + t) * 2 + (lane & 1)] = (lane & 1) ? vq : kq;
+      }
+      __syncwarp();
+      if (lane == 0) mbar_arrive(&empty[s]);
+    }
+    // the first stage is free once every MMA is done and every summing warp is
+    // past its tiles: then the sums go there (after an abort they are not read)
+    const bool got = epi_all(pwait_warp(&sdone, 0, abrt, p.ws, u, p.polls));
+    if (got) {
+#pragma unroll
+      for (int e = 0; e < 4; ++e) {
+        reinterpret_cast<uint64_t*>(s_pk + (sw * 2 + rh) * 128 + ch * 8)[e] = ksum[e];
+        reinterpret_cast<uint64_t*>(s_pv + (sw * 2 + rh) * 128 + ch * 8)[e] = vsum[e];
+      }
+      epi_sync();
     }
   } else {
     // ---- epilogue: group 0 = warps 2..5 (tokens 0..63 of a tile's logits),
@@ -386,29 +439,8 @@ __global__ void __launch_bounds__(kStatsThreads, 1)
       tmax_vis[rb] = p.causal ? p.T - p.W + r % p.W : 0x7fffffff;
     }
     const int t_safe = p.causal ? p.T - p.W : 0x7fffffff;  // tokens every window row sees
-    // column sums: this lane's 8 dims (chunk lane % 16) over the rows 16 ew + lane / 16 + 2 j
-    const int ch = lane & 15, rh = lane >> 4;
-    uint64_t ksum[4] = {0ull, 0ull, 0ull, 0ull}, vsum[4] = {0ull, 0ull, 0ull, 0ull};
     for (int i = 0; i < n_tiles; ++i) {
-      const int s = i % kS, b = i % NB;
-      if (!pwait_warp(&full[s], (i / kS) & 1, abrt, p.ws, u, p.polls)) break;
-      const int tt0 = t_begin + i * kTok;
-      {
-        const uint8_t* tk = sKV + (size_t)s * 2 * kTileBytes + (ch >> 3) * kBoxBytes + (ew * 16 + rh) * 128;
-        float kn[8], vn[8];
-#pragma unroll
-        for (int j = 0; j < 8; ++j) {
-          const uint32_t off = 2 * j * 128 + (((ch & 7) ^ ((rh + 2 * j) & 7)) << 4);
-          kn[j] = sum_chunk(*reinterpret_cast<const uint4*>(tk + off), ksum);
-          vn[j] = sum_chunk(*reinterpret_cast<const uint4*>(tk + kTileBytes + off), vsum);
-        }
-        __syncwarp();
-        if (lane == 0) mbar_arrive(&empty[s]);
-        // squared norms of 16 rows over the 16 lanes of each: lane 2 x holds row x / 8 + 2 (x % 8)
-        const float kq = half_warp_sums(kn, lane), vq = half_warp_sums(vn, lane);
-        const int t = tt0 + ew * 16 + rh + 2 * ((lane >> 1) & 7);
-        if (t < t_end) p.norms[((size_t)u * p.T + t) * 2 + (lane & 1)] = (lane & 1) ? vq : kq;
-      }
+      const int b = i % NB, tt0 = t_begin + i * kTok;
       if (!pwait_warp(&lfull[b], (i / NB) & 1, abrt, p.ws, u, p.polls)) break;
       tc_fence_after();
       const bool fast = tt0 + kTok <= t_end && tt0 + kTok - 1 <= t_safe;  // no masking in this tile
@@ -452,19 +484,14 @@ __global__ void __launch_bounds__(kStatsThreads, 1)
       __syncwarp();
       if (lane == 0) mbar_arrive(&lempty[b]);
     }
-    // uniform over the epilogue warps: after an abort the MMAs may still write
+    // uniform over the epilogue and summing warps: after an abort the MMAs may still write
     // TMEM and read the stages, so neither is touched and the chunk's record
     // is left empty
     const bool got = epi_all(pwait_warp(&sdone, 0, abrt, p.ws, u, p.polls));
     float* rec = p.mrec + ((size_t)u * p.n_chunks + chunk) * rec_floats(p.D);
     if (got) {
       tc_fence_after();
-      // the per-warp column sums and the second group's row statistics
-#pragma unroll
-      for (int e = 0; e < 4; ++e) {
-        reinterpret_cast<uint64_t*>(s_pk + (ew * 2 + rh) * 128 + ch * 8)[e] = ksum[e];
-        reinterpret_cast<uint64_t*>(s_pv + (ew * 2 + rh) * 128 + ch * 8)[e] = vsum[e];
-      }
+      // the second group's row statistics
       if (grp == 1)
 #pragma unroll
         for (int rb = 0; rb < 2; ++rb) {
@@ -476,7 +503,7 @@ __global__ void __launch_bounds__(kStatsThreads, 1)
         const float* part = grp == 0 ? s_pk : s_pv;
         float x = 0.f;
 #pragma unroll
-        for (int g = 0; g < 16; ++g) x += part[g * 128 + et];
+        for (int g = 0; g < 8; ++g) x += part[g * 128 + et];
         (grp == 0 ? sum_k : sum_v)[et] = x;
       }
       if (grp == 0)
@@ -495,7 +522,7 @@ __global__ void __launch_bounds__(kStatsThreads, 1)
             *reinterpret_cast<float2*>(p.rowpart + (((size_t)u * p.n_chunks + chunk) * p.RW + r) * 2) =
                 make_float2(Mx, Ls);
         }
-      epi_sync();
+      named_sync(4, 256);
       const float nc = static_cast<float>(max(0, t_end - t_begin)), inv_nc = nc > 0.f ? 1.f / nc : 0.f;
       const int a = qd * 32 + lane;  // value dim = TMEM lane
       const float sva = sum_v[a] * inv_nc;
@@ -542,35 +569,39 @@ __global__ void __launch_bounds__(kStatsThreads, 1)
 // Token scores: the logits again, token-major.  Four epilogue groups of four
 // warps, each on a TMEM buffer of 128 logits columns: with up to 128 window
 // rows they take every fourth tile, with more each tile is shared by two
-// groups (rows 0..127 and the others).  Two groups left the kernel bound by
-// the latency of their loads and exponentials (57 us at 32K, batch 4).
+// groups (rows 0..127 and the others).  Bounded by the read of K, whose rate
+// follows the bytes in flight (four stages: 4.5 TB/s with no epilogue at all),
+// so shared memory goes to stages; from the chunk's end, where L2 still holds
+// what stats_tc read last.
 constexpr int kScoreThreads = 64 + 4 * 128;
 __global__ void __launch_bounds__(kScoreThreads, 1)
     scores_tc(const TcArgs p, const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtensorMap tmQ) {
-  constexpr int kS = 4;
-  extern __shared__ __align__(1024) uint8_t smraw[];
-  uint8_t* sm = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smraw) + 1023) & ~uintptr_t(1023));
-  uint8_t* sK = sm;                    // [kS][128 x 128]
-  uint8_t* sQ = sm + kS * kTileBytes;  // [2 boxes][RWb*128][128 B]
-  __shared__ __align__(8) uint64_t full[kS], empty[kS], lfull[4], lempty[4], pfull[2], qfull, mma_done;
+  constexpr int kMaxS = 6;
+  extern __shared__ __align__(1024) uint8_t sm[];  // a multiple of 1024 bytes from the block's base
+  const int RWb = p.RWb, RWp = RWb * 128, NB = 4 / RWb;  // TMEM buffers of RWp columns
+  const int kS = score_stages(RWb);
+  uint8_t* sK = sm;                            // [kS][128 x 128]
+  uint8_t* sQ = sm + (size_t)kS * kTileBytes;  // [2 boxes][RWb*128][128 B]
+  float* s_b = reinterpret_cast<float*>(sQ + (size_t)RWb * 2 * kBoxBytes);  // [256] log2(1 / l_r) - m_r (-inf: padding)
+  uint8_t* s_wi = reinterpret_cast<uint8_t*>(s_b + 256);                    // [256] window index of row r (r mod W)
+  float(*s_part)[128] = reinterpret_cast<float(*)[128]>(s_wi + 256);        // [2] the upper rows' sums (RWb = 2)
+  __shared__ __align__(8) uint64_t full[kMaxS], empty[kMaxS], lfull[4], lempty[4], pfull[2], qfull, mma_done;
   __shared__ uint32_t tmem_base;
   __shared__ int abort_flag, s_issued;
-  __shared__ __align__(16) float s_b[256];  // log2(1 / l_r) - m_r (-inf for padding rows)
-  __shared__ int s_wi[256];                 // window index of row r (r mod W)
-  __shared__ float s_part[2][128];          // the upper rows' sums of a tile shared by two groups
 
   const int chunk = blockIdx.x, u = blockIdx.y;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int t_begin = chunk * p.chunk;
   const int t_end = min(p.n_rows, t_begin + p.chunk);
   const int n_tiles = (max(0, t_end - t_begin) + kTok - 1) / kTok;
-  const int RWb = p.RWb, RWp = RWb * 128, NB = 4 / RWb;  // TMEM buffers of RWp columns
   volatile int* abrt = &abort_flag;
 
   if (tid == 0) {
     for (int i = 0; i < kS; ++i) {
       mbar_init(&full[i], 1);
       mbar_init(&empty[i], 1);
+    }
+    for (int i = 0; i < 4; ++i) {
       mbar_init(&lfull[i], 1);
       mbar_init(&lempty[i], 4 * RWb);
     }
@@ -594,33 +625,43 @@ __global__ void __launch_bounds__(kScoreThreads, 1)
     if (lane == 0) {
       mbar_arrive_expect_tx(&qfull, 2u * RWb * kBoxBytes);
       for (int bx = 0; bx < 2; ++bx) tma_load_3d(sQ + bx * RWb * kBoxBytes, &tmQ, bx * 64, 0, u, &qfull);
+      int s = 0;
+      uint32_t ph = 1;
       for (int i = 0; i < n_tiles; ++i) {
-        const int s = i % kS, j = i / kS;
-        if (j >= 1 && !pwait(&empty[s], (j - 1) & 1, abrt, p.ws, u, p.polls)) break;
+        if (i >= kS && !pwait(&empty[s], ph, abrt, p.ws, u, p.polls)) break;
         mbar_arrive_expect_tx(&full[s], kTileBytes);
         for (int bx = 0; bx < 2; ++bx)
-          tma_load_3d(sK + s * kTileBytes + bx * kBoxBytes, &tmK, bx * 64, t_begin + i * kTok, u, &full[s]);
+          tma_load_3d(sK + s * kTileBytes + bx * kBoxBytes, &tmK, bx * 64, t_begin + (n_tiles - 1 - i) * kTok, u,
+                      &full[s]);
         s_issued = i + 1;
+        if (++s == kS) {
+          s = 0;
+          ph ^= 1u;
+        }
       }
     }
   } else if (warp == 1) {
     if (lane == 0) {
       const uint32_t id = idesc_bf16(128, RWp, 0, 0);  // tokens x window rows, both K-major
-      const uint32_t aQ = smem_addr(sQ);
+      const uint64_t dq = sdesc_sw128(smem_addr(sQ), 16, 1024), dk0 = sdesc_sw128(smem_addr(sK), 16, 1024);
       const bool ok = pwait(&qfull, 0, abrt, p.ws, u, p.polls);
+      int s = 0, b = 0;  // stage and buffer of tile i, and their phases
+      uint32_t ph = 0, bph = 1;
       for (int i = 0; ok && i < n_tiles; ++i) {
-        const int s = i % kS, j = i / kS, b = i % NB;
-        if (!pwait(&full[s], j & 1, abrt, p.ws, u, p.polls)) break;
-        if (i >= NB && !pwait(&lempty[b], (i / NB - 1) & 1, abrt, p.ws, u, p.polls)) break;
+        if (!pwait(&full[s], ph, abrt, p.ws, u, p.polls)) break;
+        if (i >= NB && !pwait(&lempty[b], bph, abrt, p.ws, u, p.polls)) break;
         tc_fence_after();
-        const uint32_t aK = smem_addr(sK + s * kTileBytes);
-        for (int kk = 0; kk < 8; ++kk) {
-          const uint64_t dk = sdesc_sw128(aK + (kk >> 2) * kBoxBytes + (kk & 3) * 32, 16, 1024);
-          const uint64_t dq = sdesc_sw128(aQ + (kk >> 2) * RWb * kBoxBytes + (kk & 3) * 32, 16, 1024);
-          umma_bf16(tm + b * RWp, dk, dq, id, kk > 0 ? 1u : 0u);
-        }
+        umma_k128(tm + b * RWp, dk0 + s * (kTileBytes >> 4), dq, kBoxBytes, RWb * kBoxBytes, id, 0u);
         umma_commit(&lfull[b]);
         umma_commit(&empty[s]);
+        if (++s == kS) {
+          s = 0;
+          ph ^= 1u;
+        }
+        if (++b == NB) {
+          b = 0;
+          bph ^= 1u;
+        }
       }
       umma_commit(&mma_done);  // every MMA issued has completed
     }
@@ -645,7 +686,7 @@ __global__ void __launch_bounds__(kScoreThreads, 1)
           }
       }
       s_b[r] = (Lsum > 0.f) ? -log2f(Lsum) - M : -INFINITY;
-      s_wi[r] = r % p.W;
+      s_wi[r] = static_cast<uint8_t>(r % p.W);
     }
     named_sync(1, 512);
     const int t_safe = p.causal ? p.T - p.W : 0x7fffffff;  // tokens every window row sees
@@ -653,7 +694,7 @@ __global__ void __launch_bounds__(kScoreThreads, 1)
     for (int i = b; i < n_tiles; i += NB) {
       if (!pwait_warp(&lfull[b], (i / NB) & 1, abrt, p.ws, u, p.polls)) break;
       tc_fence_after();
-      const int t = t_begin + i * kTok + qd * 32 + lane;  // token of this thread (TMEM lane)
+      const int t = t_begin + (n_tiles - 1 - i) * kTok + qd * 32 + lane;  // token of this thread (TMEM lane)
       const bool fast = t <= t_safe;  // every window row sees this token
       float acc = 0.f;
 #pragma unroll 2
@@ -725,9 +766,9 @@ __global__ void __launch_bounds__(kScoreThreads, 1)
 // 32K, batch 4, against about 10 for the gathered rows.  When more than half
 // of a CTA's positions remain, or the caller wants score2 itself, the full
 // pass runs; a position's score2 is the same bits either way.
-__global__ void __launch_bounds__(kStatsThreads, 1)
+__global__ void __launch_bounds__(kResThreads, 1)
     residual_tc(const TcArgs p, const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtensorMap tmV) {
-  constexpr int kS = 2;
+  constexpr int kS = 2;  // tile i is in stage and TMEM buffer i % 2
   extern __shared__ __align__(1024) uint8_t smraw[];
   uint8_t* sm = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smraw) + 1023) & ~uintptr_t(1023));
   uint8_t* sK = sm;                        // [kS][128 x 128]
@@ -781,7 +822,7 @@ __global__ void __launch_bounds__(kStatsThreads, 1)
   }
   if (warp == 1) tmem_alloc(&tmem_base, 256);
   if (D < kDP) {  // no second box of key dims: that part of the operand image is zero
-    for (int i = tid; i < 3 * kBoxBytes / 16; i += kStatsThreads)
+    for (int i = tid; i < 3 * kBoxBytes / 16; i += kResThreads)
       reinterpret_cast<uint4*>(sC + (i / (kBoxBytes / 16)) * kTileBytes + kBoxBytes)[i % (kBoxBytes / 16)] =
           make_uint4(0u, 0u, 0u, 0u);
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");  // generic writes -> tensor-core reads
@@ -804,7 +845,7 @@ __global__ void __launch_bounds__(kStatsThreads, 1)
   int32_t* list = p.cand + (size_t)u * p.T + t_begin;  // this CTA's remaining positions, in any order
   if (p.prune) {
     const int g0 = u / p.hs * p.hs;  // the selection group's first unit
-    for (int h = warp; h < p.hs; h += kStatsThreads / 32) {
+    for (int h = warp; h < p.hs; h += kResThreads / 32) {
       float a2 = 0.f, f2 = 0.f;
 #pragma unroll
       for (int j = 0; j < kDP; j += 32) {
@@ -823,7 +864,7 @@ __global__ void __launch_bounds__(kStatsThreads, 1)
     // theta: the smallest lower bound over the first stage's free rows (0 where a bound says nothing)
     float lowest = INFINITY;
 #pragma unroll 4
-    for (int i = tid; i < p.hs * p.B; i += kStatsThreads) {
+    for (int i = tid; i < p.hs * p.B; i += kResThreads) {
       const int f = min(max(p.idx[(size_t)(g0 / p.hs) * p.hs * p.B + i], 0), p.hs * p.T - 1);
       const int h = p.hs == 1 ? 0 : f / p.T, t = f - h * p.T;
       if (!is_protected(t, p.T, p.W, p.sink, p.keep_window)) {
@@ -840,7 +881,7 @@ __global__ void __launch_bounds__(kStatsThreads, 1)
     const int h = u - g0;
     const float mvn = s_mvn[h], fro = s_fro[h];
 #pragma unroll 4
-    for (int t0 = t_begin + warp * 32; t0 < t_end; t0 += kStatsThreads) {
+    for (int t0 = t_begin + warp * 32; t0 < t_end; t0 += kResThreads) {
       const int t = t0 + lane;
       bool cand = false;
       if (t < t_end) {
@@ -883,22 +924,18 @@ __global__ void __launch_bounds__(kStatsThreads, 1)
   } else if (warp == 1) {
     if (lane == 0) {
       const uint32_t id = idesc_bf16(128, 128, 0, 0);
-      const uint32_t aC = smem_addr(sC);
+      const uint64_t dk0 = sdesc_sw128(smem_addr(sK), 16, 1024), dc0 = sdesc_sw128(smem_addr(sC), 16, 1024);
       const bool ok = pwait(&cfull, 0, abrt, p.ws, u, p.polls);
       for (int i = 0; ok && i < n_tiles; ++i) {
-        const int s = i % kS, j = i / kS, b = i & 1;
-        if (!pwait(&full[s], j & 1, abrt, p.ws, u, p.polls)) break;
-        if (i >= 2 && !pwait(&yempty[b], ((i >> 1) - 1) & 1, abrt, p.ws, u, p.polls)) break;
+        const int s = i & 1;
+        if (!pwait(&full[s], (i >> 1) & 1, abrt, p.ws, u, p.polls)) break;
+        if (i >= 2 && !pwait(&yempty[s], ((i >> 1) - 1) & 1, abrt, p.ws, u, p.polls)) break;
         tc_fence_after();
-        const uint32_t aK = smem_addr(sK + s * kTileBytes);
+#pragma unroll
         for (int part = 0; part < 3; ++part)
-          for (int kk = 0; kk < 8; ++kk) {
-            const uint64_t dk = sdesc_sw128(aK + (kk >> 2) * kBoxBytes + (kk & 3) * 32, 16, 1024);
-            const uint64_t dc =
-                sdesc_sw128(aC + part * kTileBytes + (kk >> 2) * kBoxBytes + (kk & 3) * 32, 16, 1024);
-            umma_bf16(tm + b * 128, dk, dc, id, (part > 0 || kk > 0) ? 1u : 0u);
-          }
-        umma_commit(&yfull[b]);
+          umma_k128(tm + s * 128, dk0 + s * (kTileBytes >> 4), dc0 + part * (kTileBytes >> 4), kBoxBytes, kBoxBytes, id,
+                    part > 0 ? 1u : 0u);
+        umma_commit(&yfull[s]);
         umma_commit(&empty[s]);
       }
       umma_commit(&mma_done);  // every MMA issued has completed
@@ -1581,7 +1618,6 @@ __global__ void __launch_bounds__(256) keep_all_kernel(const CompressArgs a, int
 }
 
 // ------------------------------------------------------------------- host
-constexpr size_t kScoresSmem = 1024 + 4 * kTileBytes + 2 * 2 * kBoxBytes;
 constexpr size_t kResidualSmem = 1024 + 2 * 2 * kTileBytes + 3 * kTileBytes;
 
 // residual_tc compares scores and norms before it reads rows when its CTAs
@@ -1643,7 +1679,7 @@ cudaError_t run(const CompressArgs& a, const mkv_geom& g, int num_sms, cudaStrea
   const bool keep_all = T <= B;
   cudaError_t e = cudaSuccess;
   if ((e = smem_attr((const void*)stats_tc, std::max(stats_smem(1), stats_smem(2)))) != cudaSuccess) return e;
-  if ((e = smem_attr((const void*)scores_tc, kScoresSmem)) != cudaSuccess) return e;
+  if ((e = smem_attr((const void*)scores_tc, std::max(score_smem(1), score_smem(2)))) != cudaSuccess) return e;
   if ((e = smem_attr((const void*)residual_tc, kResidualSmem)) != cudaSuccess) return e;
 
   CUtensorMap tmK, tmV, tmQ;
@@ -1677,11 +1713,11 @@ cudaError_t run(const CompressArgs& a, const mkv_geom& g, int num_sms, cudaStrea
   const dim3 cg(L.n_chunks, U);
 
   if (!keep_all || a.diag_scores != nullptr) {
-    if ((e = launch_pdl(stats_tc, cg, kStatsThreads, stats_smem(L.RWb), st, 0, tp, tmK, tmV, tmQ)) != cudaSuccess) return e;
+    if ((e = launch_pdl(stats_tc, cg, kStatThreads, stats_smem(L.RWb), st, 0, tp, tmK, tmV, tmQ)) != cudaSuccess) return e;
     TcArgs p2 = tp;
     p2.s_out = L.s;
     p2.diag = a.diag_scores;
-    if ((e = launch_pdl(scores_tc, cg, kScoreThreads, kScoresSmem, st, 0, p2, tmK, tmQ)) != cudaSuccess) return e;
+    if ((e = launch_pdl(scores_tc, cg, kScoreThreads, score_smem(L.RWb), st, 0, p2, tmK, tmQ)) != cudaSuccess) return e;
   }
   if (keep_all) {
     if (D == 128) keep_all_kernel<128><<<dim3((T + 7) / 8, U), 256, 0, st>>>(a, T);
@@ -1743,7 +1779,7 @@ cudaError_t run(const CompressArgs& a, const mkv_geom& g, int num_sms, cudaStrea
     r.cand = L.cand;
     r.K = a.K;
     r.V = a.V;
-    if ((e = launch_pdl(residual_tc, cg, kStatsThreads, kResidualSmem, st, 0, r, tmK, tmV)) != cudaSuccess) return e;
+    if ((e = launch_pdl(residual_tc, cg, kResThreads, kResidualSmem, st, 0, r, tmK, tmV)) != cudaSuccess) return e;
     if ((e = select(L.s2, hist2, nullptr)) != cudaSuccess) return e;
   }
   return launch_rset<true>(ra, cl, st);

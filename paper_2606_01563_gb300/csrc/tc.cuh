@@ -74,6 +74,25 @@ __device__ __forceinline__ void umma_bf16(uint32_t d_tmem, uint64_t da, uint64_t
       "l"(da), "l"(db), "r"(idesc), "r"(accumulate));
 }
 
+// The eight k-steps of a 128-deep product of K-major operands whose two
+// 64-column boxes lie a_box and b_box bytes apart: da, db the descriptors of
+// the first step.  One thread issues every MMA of a kernel, so a step is two
+// additions and the MMA itself.
+__device__ __forceinline__ void umma_k128(uint32_t d_tmem, uint64_t da, uint64_t db, uint32_t a_box, uint32_t b_box,
+                                          uint32_t idesc, uint32_t accumulate) {
+#pragma unroll
+  for (int kk = 0; kk < 8; ++kk)
+    umma_bf16(d_tmem, da + (kk >> 2) * (a_box >> 4) + (kk & 3) * 2, db + (kk >> 2) * (b_box >> 4) + (kk & 3) * 2, idesc,
+              kk > 0 ? 1u : accumulate);
+}
+// The same for MN-major operands (128 rows of the reduction, 16 per step).
+__device__ __forceinline__ void umma_mn128(uint32_t d_tmem, uint64_t da, uint64_t db, uint32_t idesc,
+                                           uint32_t accumulate) {
+#pragma unroll
+  for (int kk = 0; kk < 8; ++kk)
+    umma_bf16(d_tmem, da + kk * 128, db + kk * 128, idesc, kk > 0 ? 1u : accumulate);
+}
+
 // Arrive on `bar` once every MMA this thread issued so far has completed.
 __device__ __forceinline__ void umma_commit(uint64_t* bar) {
   asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(smem_addr(bar))
@@ -89,12 +108,14 @@ __device__ __forceinline__ void tma_load_3d(void* dst, const CUtensorMap* map, i
       : "memory");
 }
 
-// Prefetch a box of a 3-D tensor into L2 (no shared memory, no completion).
-__device__ __forceinline__ void tma_prefetch_3d(const CUtensorMap* map, int x, int y, int z) {
-  asm volatile("cp.async.bulk.prefetch.tensor.3d.L2.global [%0, {%1, %2, %3}];" ::"l"(
-                   reinterpret_cast<uint64_t>(map)),
-               "r"(x), "r"(y), "r"(z)
-               : "memory");
+// The same with an L2 cache policy on the bytes it reads.
+__device__ __forceinline__ void tma_load_3d_hint(void* dst, const CUtensorMap* map, int x, int y, int z, uint64_t* bar,
+                                                 uint64_t pol) {
+  asm volatile(
+      "cp.async.bulk.tensor.3d.shared::cluster.global.mbarrier::complete_tx::bytes.L2::cache_hint [%0], [%1, {%2, %3, "
+      "%4}], [%5], %6;" ::"r"(smem_addr(dst)),
+      "l"(reinterpret_cast<uint64_t>(map)), "r"(x), "r"(y), "r"(z), "r"(smem_addr(bar)), "l"(pol)
+      : "memory");
 }
 
 // Host: bf16 slabs [units][rows][inner] (unit stride in bytes) as a 3-D
