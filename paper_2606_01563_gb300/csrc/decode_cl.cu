@@ -91,14 +91,16 @@ __host__ __device__ constexpr size_t cl_smem_bytes(int D, int G, int S) {
   return cl_stages(D, G, S) * cl_stage_bytes(D) + cl_extra_bytes(D, G, S) + 1024;  // + alignment slack
 }
 
-template <int D, int G, bool C16, bool EARLY, bool CS>
+// ONE: one split per unit (many units): the CTA owns all dims and finishes them
+// from its own merged state, without the exchange.
+template <int D, int G, bool C16, bool EARLY, bool CS, bool ONE>
 __global__ void __launch_bounds__(kClThreads, 2)
     decode_cl_kernel(const DecodeArgs a, const __grid_constant__ CUtensorMap tmK,
                      const __grid_constant__ CUtensorMap tmV) {
   constexpr int MT = D / 16;  // 16-dim blocks of the output (and 16-row blocks of C')
   constexpr int KS = D / 16;  // k-steps of a dot product over the head dim
   constexpr int kTileBytes = kRows * D * 2;
-  const int S = a.S;
+  const int S = ONE ? 1 : a.S;
   const int NST = cl_stages(D, G, S);
   const int OD = cl_own_dims(D, S);
   extern __shared__ __align__(128) uint8_t dsm_raw[];
@@ -112,7 +114,7 @@ __global__ void __launch_bounds__(kClThreads, 2)
   __shared__ __align__(8) uint64_t full[kMaxStages], empty[kMaxStages], recv;
   __shared__ float sE[G], sSn[G];   // log2 of the moment weight n exp(scale q.mu_k); new token's logit
   __shared__ float sMuk[D], sKn[D];
-  __shared__ int sOwner[MT], sLo[MT], sFail;
+  __shared__ int sOwner[MT], sLo[MT], sFail, sBlk;
 
   const int s = blockIdx.x, kv = blockIdx.y, b = blockIdx.z;
   const int u = b * a.n_kv + kv;
@@ -131,9 +133,10 @@ __global__ void __launch_bounds__(kClThreads, 2)
     }
     // the receive barrier completes when every CTA's state for the owned dims has landed
     mbar_init(&recv, 1);
-    mbar_arrive_expect_tx(&recv, own_d > 0 ? static_cast<uint32_t>(S * G * (own_d + 2) * 4) : 0u);
+    if constexpr (!ONE) mbar_arrive_expect_tx(&recv, own_d > 0 ? static_cast<uint32_t>(S * G * (own_d + 2) * 4) : 0u);
     mbar_fence_init();
     sFail = 0;
+    sBlk = 2;  // the first two owned blocks of C' are the side warps'
     asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&tmK)) : "memory");
     asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&tmV)) : "memory");
   }
@@ -144,7 +147,7 @@ __global__ void __launch_bounds__(kClThreads, 2)
     sLo[tid] = own_lo(r, S, MT);
   }
   __syncthreads();
-  cluster_arrive_relaxed();  // paired with the wait before the first remote store
+  if constexpr (!ONE) cluster_arrive_relaxed();  // paired with the wait before the first remote store
 
   const bool corr = a.correction != 0 && a.n != nullptr;
   const bool do_c = corr && a.order == 1;
@@ -280,6 +283,68 @@ __global__ void __launch_bounds__(kClThreads, 2)
   }
   const bool use_m = n_e > 0;
   const float qscale = scale * kLog2e;
+  constexpr int kOwn = (G * D / 4 + kConsumerWarps * 32 - 1) / (kConsumerWarps * 32);
+  float4 own[kOwn];  // with one split: the attending threads' merged states, four dims of a head each
+  float own_m[kOwn], own_l[kOwn];
+  // C'q rows of the owned block j (operands in cf), on the tensor cores: A = C'
+  // rows split into bf16 hi + lo parts, clamp of Eq. fused applied here, or
+  // both read ready-made from the operand form; B = the q fragments; written
+  // as sF[row][head].  Four independent accumulator chains (k-step parity x
+  // part): these products share the tensor pipe with the attending warps' tiles.
+  auto cq_block = [&](int j) {
+    const float nf = static_cast<float>(n_e), tau = a.tau;
+    float dc[4][4] = {};
+    if constexpr (CS) {
+      if (do_c) {  // operand words as loaded
+#pragma unroll
+        for (int kk = 0; kk < KS; ++kk) {
+          mma_m16n8k16(dc[kk & 1], __float_as_uint(cf[kk][0].x), __float_as_uint(cf[kk][1].x),
+                       __float_as_uint(cf[kk][2].x), __float_as_uint(cf[kk][3].x), qa[kk][0], qa[kk][1]);
+          mma_m16n8k16(dc[2 + (kk & 1)], __float_as_uint(cf[kk][0].y), __float_as_uint(cf[kk][1].y),
+                       __float_as_uint(cf[kk][2].y), __float_as_uint(cf[kk][3].y), qa[kk][0], qa[kk][1]);
+        }
+      }
+    } else if (do_c) {
+#pragma unroll
+      for (int kk = 0; kk < KS; ++kk) {
+        uint32_t hi[4], lo[4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+          const float x = (fabsf(cf[kk][i].x * nf) < tau) ? 0.f : cf[kk][i].x;
+          const float y = (fabsf(cf[kk][i].y * nf) < tau) ? 0.f : cf[kk][i].y;
+          hi[i] = pack_bf16x2(x, y);
+          lo[i] = pack_bf16x2(bf16_residual(x), bf16_residual(y));
+        }
+        mma_m16n8k16(dc[kk & 1], hi[0], hi[1], hi[2], hi[3], qa[kk][0], qa[kk][1]);
+        if constexpr (!C16) mma_m16n8k16(dc[2 + (kk & 1)], lo[0], lo[1], lo[2], lo[3], qa[kk][0], qa[kk][1]);
+      }
+    }
+    float d[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) d[i] = (dc[0][i] + dc[1][i]) + (dc[2][i] + dc[3][i]);
+    const int ra = j * 16 + g, rb = ra + 8;  // local rows (owned dims)
+    if (2 * t < G) {
+      sF[ra * G + 2 * t] = d[0];
+      sF[rb * G + 2 * t] = d[2];
+    }
+    if (2 * t + 1 < G) {
+      sF[ra * G + 2 * t + 1] = d[1];
+      sF[rb * G + 2 * t + 1] = d[3];
+    }
+  };
+  // The blocks past the side warps' first two (few splits: up to eight blocks a
+  // CTA) go to whichever warp is free: the side warps alone finished 3-4 us
+  // after the tiles at one split, head dim 128.
+  auto cq_rest = [&]() {
+    for (;;) {
+      int j = 0;
+      if (lane == 0) j = atomicAdd(&sBlk, 1);
+      j = __shfl_sync(0xffffffffu, j, 0);
+      if (j >= nmt) break;
+      load_cf(j);
+      cq_block(j);
+    }
+  };
 
   if (side) {
     // the new token: 16 bytes of k (lanes < D/8) or v (lanes < D/4) per lane
@@ -301,59 +366,11 @@ __global__ void __launch_bounds__(kClThreads, 2)
       __syncwarp();
     }
     __syncwarp();
-    named_sync(3, 64);  // the moment warp's mu_v and mu_k rows are in place
     if (use_m) {
-      // f_hat_E rows of the owned blocks, blocks alternating between the two
-      // side warps: mu_v + scale C'q on the tensor cores (A = C' rows split
-      // into bf16 hi + lo parts, clamp of Eq. fused applied here, or both
-      // read ready-made from the operand form; B = the q fragments), written
-      // as sF[row][head].  Four independent accumulator
-      // chains (k-step parity x part): these products share the tensor pipe
-      // with an attending warp's tiles.
-      const float nf = static_cast<float>(n_e), tau = a.tau;
-      for (int j = warp - kLoaderWarp; j < nmt; j += 2) {
-        if (j > 1) load_cf(j);
-        float dc[4][4] = {};
-        if constexpr (CS) {
-          if (do_c) {  // operand words as loaded
-#pragma unroll
-            for (int kk = 0; kk < KS; ++kk) {
-              mma_m16n8k16(dc[kk & 1], __float_as_uint(cf[kk][0].x), __float_as_uint(cf[kk][1].x),
-                           __float_as_uint(cf[kk][2].x), __float_as_uint(cf[kk][3].x), qa[kk][0], qa[kk][1]);
-              mma_m16n8k16(dc[2 + (kk & 1)], __float_as_uint(cf[kk][0].y), __float_as_uint(cf[kk][1].y),
-                           __float_as_uint(cf[kk][2].y), __float_as_uint(cf[kk][3].y), qa[kk][0], qa[kk][1]);
-            }
-          }
-        } else if (do_c) {
-#pragma unroll
-          for (int kk = 0; kk < KS; ++kk) {
-            uint32_t hi[4], lo[4];
-#pragma unroll
-            for (int i = 0; i < 4; ++i) {
-              const float x = (fabsf(cf[kk][i].x * nf) < tau) ? 0.f : cf[kk][i].x;
-              const float y = (fabsf(cf[kk][i].y * nf) < tau) ? 0.f : cf[kk][i].y;
-              hi[i] = pack_bf16x2(x, y);
-              lo[i] = pack_bf16x2(bf16_residual(x), bf16_residual(y));
-            }
-            mma_m16n8k16(dc[kk & 1], hi[0], hi[1], hi[2], hi[3], qa[kk][0], qa[kk][1]);
-            if constexpr (!C16) mma_m16n8k16(dc[2 + (kk & 1)], lo[0], lo[1], lo[2], lo[3], qa[kk][0], qa[kk][1]);
-          }
-        }
-        float d[4];
-#pragma unroll
-        for (int i = 0; i < 4; ++i) d[i] = (dc[0][i] + dc[1][i]) + (dc[2][i] + dc[3][i]);
-        const int ra = j * 16 + g, rb = ra + 8;  // local rows (owned dims)
-        const float mva = sMuv[ra], mvb = sMuv[rb];
-        if (2 * t < G) {
-          sF[ra * G + 2 * t] = fmaf(scale, d[0], mva);
-          sF[rb * G + 2 * t] = fmaf(scale, d[2], mvb);
-        }
-        if (2 * t + 1 < G) {
-          sF[ra * G + 2 * t + 1] = fmaf(scale, d[1], mva);
-          sF[rb * G + 2 * t + 1] = fmaf(scale, d[3], mvb);
-        }
-      }
+      if (warp - kLoaderWarp < nmt) cq_block(warp - kLoaderWarp);
+      if (nmt > 2) cq_rest();
     }
+    named_sync(3, 64);  // the moment warp's mu_v and mu_k rows are in place
     if (producer) {
       if (has_new && lane < D / 4) {  // the token as floats: all of k, the owned dims of v
         const __nv_bfloat162* h2 = reinterpret_cast<const __nv_bfloat162*>(&kvc);
@@ -400,7 +417,7 @@ __global__ void __launch_bounds__(kClThreads, 2)
     }
     if (!producer && EARLY && s == 0 && lane == 0 && ldcg_hint(a.len + u, pol_keep) != len_read)
       record_error(a.ws, MKV_ERR_INVALID_ARG, u);  // the cache changed under an early load
-    cluster_wait_acquire();
+    if constexpr (!ONE) cluster_wait_acquire();
   } else {
     // ---- attending warps: rows [warp*16, warp*16 + 16) of every tile
     const int r0 = warp * 16;
@@ -496,6 +513,7 @@ __global__ void __launch_bounds__(kClThreads, 2)
       __syncwarp();
       if (lane == 0) mbar_arrive(&empty[st]);
     }
+    if (use_m && nmt > 2) cq_rest();
     if (!ok) {
       if (lane == 0) sFail = 1;
       m0 = m1 = kNegInf;
@@ -538,9 +556,13 @@ __global__ void __launch_bounds__(kClThreads, 2)
       }
     }
     named_sync(2, kConsumerWarps * 32);
-    cluster_wait_acquire();  // every CTA of the cluster has started and armed its receive barrier
-    // thread -> (head, 4 dims): the CTA's state for them goes to the owner of those dims
-    for (int it = tid; it < G * D / 4; it += kConsumerWarps * 32) {
+    if constexpr (!ONE) cluster_wait_acquire();  // every CTA has started and armed its receive barrier
+    // thread -> (head, 4 dims): the CTA's state for them goes to the owner of
+    // those dims (itself when there is one split: straight to the finish)
+#pragma unroll
+    for (int i = 0; i < kOwn; ++i) {
+      const int it = i * kConsumerWarps * 32 + tid;
+      if (it >= G * D / 4) break;
       const int h = it / (D / 4), d0 = (it % (D / 4)) * 4;
       float mw[kConsumerWarps], lw[kConsumerWarps], M = kNegInf;
 #pragma unroll
@@ -565,6 +587,12 @@ __global__ void __launch_bounds__(kClThreads, 2)
           }
         }
       }
+      if constexpr (ONE) {
+        own[i] = acc;
+        own_m[i] = M;
+        own_l[i] = L;
+        continue;
+      }
       const int rr = sOwner[d0 >> 4], lo = sLo[d0 >> 4] * 16;
       const uint32_t bar = cluster_map(&recv, rr);
       st_async_v4(cluster_map(rcv_o + ((size_t)s * G + h) * OD + (d0 - lo), rr), acc, bar);
@@ -576,58 +604,101 @@ __global__ void __launch_bounds__(kClThreads, 2)
   // ---- local parts (f_hat_E rows, per-head weights, v_new) in place; the
   // other CTAs' states for the owned dims landed
   __syncthreads();
-  const bool got_all = mbar_wait(&recv, 0);
-  if (!got_all && tid == 0) record_error(a.ws, MKV_ERR_TIMEOUT, u);
-
-  // ---- owner merge (log2 domain): one (head, owned dim) output per thread
-  for (int idx = tid; idx < G * own_d; idx += kClThreads) {
-    const int h = idx / own_d, j = idx % own_d;
-    float2 ml[kMaxSplits];
-    float M = has_new ? sSn[h] : kNegInf;
-#pragma unroll
-    for (int sl = 0; sl < kMaxSplits; ++sl) {
-      ml[sl] = sl < S ? *reinterpret_cast<const float2*>(rcv_ml + ((size_t)sl * G + h) * 2) : make_float2(kNegInf, 0.f);
-      if (ml[sl].y > 0.f) M = fmaxf(M, ml[sl].x);
+  // the merged normaliser of a head in the log2 domain, and the output of one
+  // dim: attention state (M, L, O) with the appended token, moment
+  // pseudo-state (e, fh)
+  auto finish = [&](int h, float M, float L, float O, float fh, float& lse2) -> float {
+    const bool have_r = L > 0.f;
+    if (use_m) {
+      const float e = sE[h];
+      if (!have_r) {
+        lse2 = e;
+        return fh;
+      }
+      const float a2 = M + fast_log2(L);
+      const float top = fmaxf(a2, e);
+      const float wr = fast_exp2(a2 - top), we = fast_exp2(e - top);
+      const float inv = fast_rcp(wr + we);
+      lse2 = top + fast_log2(wr + we);
+      return (wr * inv) * (O * fast_rcp(L)) + (we * inv) * fh;
     }
-    float L = 0.f, O = 0.f;
-    if (M != kNegInf) {
+    lse2 = have_r ? M + fast_log2(L) : kNegInf;
+    return have_r ? O * fast_rcp(L) : 0.f;
+  };
+  if constexpr (ONE) {
+    // ---- one split: each attending thread finishes the four dims it merged
+    if (!side) {
+#pragma unroll
+      for (int i = 0; i < kOwn; ++i) {
+        const int it = i * kConsumerWarps * 32 + tid;
+        if (it >= G * D / 4) break;
+        const int h = it / (D / 4), d0 = (it % (D / 4)) * 4;
+        const float Mr = own_l[i] > 0.f ? own_m[i] : kNegInf, sn = has_new ? sSn[h] : kNegInf;
+        const float M = fmaxf(Mr, sn);
+        float L = 0.f, O[4] = {0.f, 0.f, 0.f, 0.f};
+        if (own_l[i] > 0.f) {
+          const float w = fast_exp2(Mr - M);
+          L = own_l[i] * w;
+          O[0] = w * own[i].x;
+          O[1] = w * own[i].y;
+          O[2] = w * own[i].z;
+          O[3] = w * own[i].w;
+        }
+        if (has_new) {
+          const float w = fast_exp2(sn - M);
+          L += w;
+#pragma unroll
+          for (int e = 0; e < 4; ++e) O[e] = fmaf(w, sVn[d0 + e], O[e]);
+        }
+        if (!use_m && !(L > 0.f) && d0 == 0) record_error(a.ws, MKV_ERR_INVALID_ARG, u);
+        float res[4], lse2 = 0.f;
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+          const float fh = use_m ? fmaf(scale, sF[(d0 + e) * G + h], sMuv[d0 + e]) : 0.f;
+          res[e] = finish(h, M, L, O[e], fh, lse2);
+        }
+        *reinterpret_cast<float4*>(a.out + ((size_t)u * G + h) * D + d0) = make_float4(res[0], res[1], res[2], res[3]);
+        if (a.lse != nullptr && d0 == 0) a.lse[(size_t)u * G + h] = lse2 * kLn2;
+      }
+    }
+  } else {
+    const bool got_all = mbar_wait(&recv, 0);
+    if (!got_all && tid == 0) record_error(a.ws, MKV_ERR_TIMEOUT, u);
+    // ---- owner merge (log2 domain): one (head, owned dim) output per thread
+    for (int idx = tid; idx < G * own_d; idx += kClThreads) {
+      const int h = idx / own_d, j = idx % own_d;
+      float2 ml[kMaxSplits];
+      float M = has_new ? sSn[h] : kNegInf;
 #pragma unroll
       for (int sl = 0; sl < kMaxSplits; ++sl) {
-        if (ml[sl].y > 0.f) {
-          const float w = fast_exp2(ml[sl].x - M);
-          L = fmaf(ml[sl].y, w, L);
-          O = fmaf(w, rcv_o[((size_t)sl * G + h) * OD + j], O);
+        ml[sl] =
+            sl < S ? *reinterpret_cast<const float2*>(rcv_ml + ((size_t)sl * G + h) * 2) : make_float2(kNegInf, 0.f);
+        if (ml[sl].y > 0.f) M = fmaxf(M, ml[sl].x);
+      }
+      float L = 0.f, O = 0.f;
+      if (M != kNegInf) {
+#pragma unroll
+        for (int sl = 0; sl < kMaxSplits; ++sl) {
+          if (ml[sl].y > 0.f) {
+            const float w = fast_exp2(ml[sl].x - M);
+            L = fmaf(ml[sl].y, w, L);
+            O = fmaf(w, rcv_o[((size_t)sl * G + h) * OD + j], O);
+          }
+        }
+        if (has_new) {
+          const float w = fast_exp2(sSn[h] - M);
+          L += w;
+          O = fmaf(w, sVn[j], O);
         }
       }
-      if (has_new) {
-        const float w = fast_exp2(sSn[h] - M);
-        L += w;
-        O = fmaf(w, sVn[j], O);
-      }
+      const float fh = use_m ? fmaf(scale, sF[j * G + h], sMuv[j]) : 0.f;
+      if (!use_m && !(L > 0.f) && j == 0) record_error(a.ws, MKV_ERR_INVALID_ARG, u);
+      float lse2;
+      const float res = finish(h, M, L, O, fh, lse2);
+      const int dim = mlo * 16 + j;
+      a.out[((size_t)u * G + h) * D + dim] = res;
+      if (a.lse != nullptr && dim == 0) a.lse[(size_t)u * G + h] = lse2 * kLn2;
     }
-    const bool have_r = L > 0.f;
-    float res, lse2;  // output, log2 of the normaliser
-    if (use_m) {
-      const float e = sE[h], fh = sF[j * G + h];
-      if (have_r) {
-        const float a2 = M + fast_log2(L);
-        const float top = fmaxf(a2, e);
-        const float wr = fast_exp2(a2 - top), we = fast_exp2(e - top);
-        const float inv = fast_rcp(wr + we);
-        res = (wr * inv) * (O * fast_rcp(L)) + (we * inv) * fh;
-        lse2 = top + fast_log2(wr + we);
-      } else {
-        res = fh;
-        lse2 = e;
-      }
-    } else {
-      if (!have_r && j == 0) record_error(a.ws, MKV_ERR_INVALID_ARG, u);
-      res = have_r ? O * fast_rcp(L) : 0.f;
-      lse2 = have_r ? M + fast_log2(L) : kNegInf;
-    }
-    const int dim = mlo * 16 + j;
-    a.out[((size_t)u * G + h) * D + dim] = res;
-    if (a.lse != nullptr && dim == 0) a.lse[(size_t)u * G + h] = lse2 * kLn2;
   }
 
   if (producer && lane == 0) {
@@ -660,7 +731,7 @@ int cl_active_clusters(int S) {
   if (known[dev][S] == 0) {
     const size_t smem = cl_smem_bytes(D, G, S);
     int n = 0;
-    cudaError_t e = cudaFuncSetAttribute(decode_cl_kernel<D, G, C16, EARLY, false>,
+    cudaError_t e = cudaFuncSetAttribute(decode_cl_kernel<D, G, C16, EARLY, false, false>,
                                          cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
     if (e == cudaSuccess) {
       cudaLaunchConfig_t cfg{};
@@ -674,7 +745,7 @@ int cl_active_clusters(int S) {
       at[0].val.clusterDim.z = 1;
       cfg.attrs = at;
       cfg.numAttrs = 1;
-      e = cudaOccupancyMaxActiveClusters(&n, decode_cl_kernel<D, G, C16, EARLY, false>, &cfg);
+      e = cudaOccupancyMaxActiveClusters(&n, decode_cl_kernel<D, G, C16, EARLY, false, false>, &cfg);
     }
     if (e != cudaSuccess) {
       (void)cudaGetLastError();
@@ -685,13 +756,13 @@ int cl_active_clusters(int S) {
   return known[dev][S];
 }
 
-template <int D, int G, bool C16, bool EARLY, bool CS>
-cudaError_t launch_cl(const DecodeArgs& args, cudaStream_t stream) {
+template <int D, int G, bool C16, bool EARLY, bool CS, bool ONE>
+cudaError_t launch_cl_one(const DecodeArgs& args, cudaStream_t stream) {
   DecodeArgs a = args;
   a.S = a.S_cl;
   a.polls = pipeline_poll_limit();
   const size_t smem = cl_smem_bytes(D, G, a.S);
-  cudaError_t e = cudaFuncSetAttribute(decode_cl_kernel<D, G, C16, EARLY, CS>,
+  cudaError_t e = cudaFuncSetAttribute(decode_cl_kernel<D, G, C16, EARLY, CS, ONE>,
                                        cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
   if (e != cudaSuccess) return e;
   const uint64_t rows = (uint64_t)a.batch * a.n_kv * a.cap;  // the cache slabs of all units as one matrix
@@ -712,8 +783,14 @@ cudaError_t launch_cl(const DecodeArgs& args, cudaStream_t stream) {
   at[1].val.clusterDim.y = 1;
   at[1].val.clusterDim.z = 1;
   cfg.attrs = at;
-  cfg.numAttrs = 2;
-  return cudaLaunchKernelEx(&cfg, decode_cl_kernel<D, G, C16, EARLY, CS>, a, tmK, tmV);
+  cfg.numAttrs = ONE ? 1 : 2;
+  return cudaLaunchKernelEx(&cfg, decode_cl_kernel<D, G, C16, EARLY, CS, ONE>, a, tmK, tmV);
+}
+
+template <int D, int G, bool C16, bool EARLY, bool CS>
+cudaError_t launch_cl(const DecodeArgs& a, cudaStream_t stream) {
+  if (a.S_cl == 1) return launch_cl_one<D, G, C16, EARLY, CS, true>(a, stream);
+  return launch_cl_one<D, G, C16, EARLY, CS, false>(a, stream);
 }
 
 // C as fp32, as its bf16 copy, or in the operand form (validation rejects both copies at once)
