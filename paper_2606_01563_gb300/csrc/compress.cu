@@ -880,22 +880,31 @@ __global__ void __launch_bounds__(kResThreads, 1)
     const float theta = __uint_as_float(s_theta) * 0.9999f;  // rounding of both sides: below 1e-6
     const int h = u - g0;
     const float mvn = s_mvn[h], fro = s_fro[h];
-#pragma unroll 4
-    for (int t0 = t_begin + warp * 32; t0 < t_end; t0 += kResThreads) {
-      const int t = t0 + lane;
-      bool cand = false;
-      if (t < t_end) {
-        const float2 nn = reinterpret_cast<const float2*>(p.norms)[(size_t)u * p.T + t];
-        const float ub = p.s_in[(size_t)u * p.T + t] * (sqrtf(nn.y) + mvn + fro * sqrtf(nn.x));
-        cand = !(ub < theta) && !is_protected(t, p.T, p.W, p.sink, p.keep_window);  // a NaN remains
-        if (!cand) p.s_out[(size_t)u * p.T + t] = 0.f;
+    constexpr int kBatch = 8;  // positions per lane whose loads are in flight together
+#pragma unroll 1
+    for (int t0 = t_begin + warp * 32; t0 < t_end; t0 += kResThreads * kBatch) {
+      float2 nn[kBatch];
+      float sc[kBatch];
+#pragma unroll
+      for (int i = 0; i < kBatch; ++i) {
+        const int t = min(t0 + i * kResThreads + lane, t_end - 1);
+        nn[i] = reinterpret_cast<const float2*>(p.norms)[(size_t)u * p.T + t];
+        sc[i] = p.s_in[(size_t)u * p.T + t];
       }
-      const unsigned mask = __ballot_sync(kFull, cand);
-      if (mask != 0u) {
-        int at = 0;
-        if (lane == 0) at = atomicAdd(&s_cnt, __popc(mask));
-        at = __shfl_sync(kFull, at, 0) + __popc(mask & ((1u << lane) - 1u));
-        if (cand) list[at] = t;
+#pragma unroll
+      for (int i = 0; i < kBatch; ++i) {
+        const int t = t0 + i * kResThreads + lane;
+        const float ub = sc[i] * (sqrtf(nn[i].y) + mvn + fro * sqrtf(nn[i].x));
+        const bool cand = t < t_end && !(ub < theta) &&  // a NaN remains
+                          !is_protected(t, p.T, p.W, p.sink, p.keep_window);
+        if (t < t_end && !cand) p.s_out[(size_t)u * p.T + t] = 0.f;
+        const unsigned mask = __ballot_sync(kFull, cand);
+        if (mask != 0u) {
+          int at = 0;
+          if (lane == 0) at = atomicAdd(&s_cnt, __popc(mask));
+          at = __shfl_sync(kFull, at, 0) + __popc(mask & ((1u << lane) - 1u));
+          if (cand) list[at] = t;
+        }
       }
     }
     __syncthreads();
@@ -1402,8 +1411,8 @@ __global__ void __launch_bounds__(2048 / CL) rset_kernel(const RsetArgs a) {
   grid_launch_dependents();
 
   // ---- row tiles
-  const int cnt = L.cnt[u];
-  const int32_t* lst = L.idx + L.hbeg[u];
+  const int cnt = L.hs == 1 ? L.B : L.cnt[u];  // a unit's own selection has fixed size and place
+  const int32_t* lst = L.idx + (L.hs == 1 ? (size_t)u * L.B : (size_t)L.hbeg[u]);
   const int hT = (u % L.hs) * T;  // list entries are h * T + position
   const int n_tiles = (cnt + kTok - 1) / kTok;
   const __nv_bfloat16* Ku = a.K + (size_t)u * T * D + kh * 64;
