@@ -120,14 +120,17 @@ def lib():
     return _lib
 
 
+# Addresses go to ctypes as plain integers, and the current stream's handle
+# comes from torch without a Stream object around it: the marshalling of a
+# decode step took 8 of its 12 us on the host, most of it in those wrappers.
 def _ptr(t):
-    return None if t is None else ctypes.c_void_p(t.data_ptr())
+    return None if t is None else t.data_ptr()
 
 
 def _stream(stream):
     if stream is None:
-        stream = torch.cuda.current_stream()
-    return ctypes.c_void_p(stream.cuda_stream)
+        return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device())
+    return stream.cuda_stream
 
 
 def _check(code, where):
@@ -225,8 +228,7 @@ def mkv_compress(g, T, K, V, Q_obs, p: mkv_compress_params, cache: Cache, mom: M
                  stream=None):
     d = mkv_compress_diag(*(None if x is None else x.data_ptr() for x in (diag or (None, None, None))))
     c, m = cache.c(), mom.c()
-    code = lib().mkv_compress(g, T, _ptr(K), _ptr(V), _ptr(Q_obs), ctypes.byref(p), ctypes.byref(c),
-                              ctypes.byref(m), ctypes.byref(d), _ptr(ws), ws.numel(), _stream(stream))
+    code = lib().mkv_compress(g, T, _ptr(K), _ptr(V), _ptr(Q_obs), p, c, m, d, _ptr(ws), ws.numel(), _stream(stream))
     _check(code, "mkv_compress")
 
 
@@ -234,8 +236,7 @@ def mkv_decode_step(g, q, k_new, v_new, cache: Cache, mom: Moments | None, p: mk
                     ws, stream=None):
     c = cache.c()
     m = mom.c() if mom is not None else None
-    code = lib().mkv_decode_step(g, _ptr(q), _ptr(k_new), _ptr(v_new), ctypes.byref(c),
-                                 ctypes.byref(m) if m is not None else None, ctypes.byref(p), _ptr(out),
+    code = lib().mkv_decode_step(g, _ptr(q), _ptr(k_new), _ptr(v_new), c, m, p, _ptr(out),
                                  _ptr(lse), _ptr(ws), ws.numel(), _stream(stream))
     _check(code, "mkv_decode_step")
 
@@ -245,16 +246,15 @@ def mkv_decode_step_noalloc(g, q, k_new, v_new, cache: Cache, mom: Moments | Non
     """mkv_decode_step with the library's fixed device scratch instead of a workspace."""
     c = cache.c()
     m = mom.c() if mom is not None else None
-    code = lib().mkv_decode_step_noalloc(g, _ptr(q), _ptr(k_new), _ptr(v_new), ctypes.byref(c),
-                                         ctypes.byref(m) if m is not None else None, ctypes.byref(p), _ptr(out),
+    code = lib().mkv_decode_step_noalloc(g, _ptr(q), _ptr(k_new), _ptr(v_new), c, m, p, _ptr(out),
                                          _ptr(lse), _stream(stream))
     _check(code, "mkv_decode_step_noalloc")
 
 
 def mkv_evict_append(g, q, k_new, v_new, budget, cache: Cache, mom: Moments, tau, ws, stream=None):
     c, m = cache.c(), mom.c()
-    code = lib().mkv_evict_append(g, _ptr(q), _ptr(k_new), _ptr(v_new), budget, ctypes.byref(c),
-                                  ctypes.byref(m), tau, _ptr(ws), ws.numel(), _stream(stream))
+    code = lib().mkv_evict_append(g, _ptr(q), _ptr(k_new), _ptr(v_new), budget, c, m, tau, _ptr(ws), ws.numel(),
+                                  _stream(stream))
     _check(code, "mkv_evict_append")
 
 
@@ -266,23 +266,22 @@ def mkv_decode_evict_step(g, q, k_new, v_new, budget, cache: Cache, mom: Moments
                           ws, stream=None):
     """Algorithm 1 for one generated token: append, evict down to `budget`, corrected output."""
     c, m = cache.c(), mom.c()
-    code = lib().mkv_decode_evict_step(g, _ptr(q), _ptr(k_new), _ptr(v_new), budget, ctypes.byref(c),
-                                       ctypes.byref(m), ctypes.byref(p), _ptr(out), _ptr(lse), _ptr(ws), ws.numel(),
-                                       _stream(stream))
+    code = lib().mkv_decode_evict_step(g, _ptr(q), _ptr(k_new), _ptr(v_new), budget, c, m, p, _ptr(out), _ptr(lse),
+                                       _ptr(ws), ws.numel(), _stream(stream))
     _check(code, "mkv_decode_evict_step")
 
 
 def mkv_moments_pack_bf16(g, mom: Moments, C16, stream=None):
     """C16 (bf16 [b, h_kv, d, d]) = bf16(mom.C): the 16-bit copy mkv_decode_params.C16 points at."""
     m = mom.c()
-    _check(lib().mkv_moments_pack_bf16(g, ctypes.byref(m), _ptr(C16), _stream(stream)), "mkv_moments_pack_bf16")
+    _check(lib().mkv_moments_pack_bf16(g, m, _ptr(C16), _stream(stream)), "mkv_moments_pack_bf16")
 
 
 def mkv_moments_pack_split(g, mom: Moments, tau, C_split, stream=None):
     """C_split (int32 [b, h_kv, d, d], as many bytes as C) = the (hi, lo) bf16x2
     operand words of the clamped C': what mkv_decode_params.C_split points at."""
     m = mom.c()
-    _check(lib().mkv_moments_pack_split(g, ctypes.byref(m), float(tau), _ptr(C_split), _stream(stream)),
+    _check(lib().mkv_moments_pack_split(g, m, float(tau), _ptr(C_split), _stream(stream)),
            "mkv_moments_pack_split")
 
 
