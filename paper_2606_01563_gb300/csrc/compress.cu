@@ -66,6 +66,7 @@ __host__ __device__ constexpr size_t stats_smem(int RWb) {
   return 1024 + (size_t)stats_stages(RWb) * 2 * kTileBytes + (size_t)RWb * 2 * kBoxBytes;
 }
 constexpr int kBins = 2048;  // bins of the scores' keys (select_kernel)
+constexpr int kGroupCont = 2048;  // contested pairs a joint selection's list holds
 constexpr unsigned kFull = 0xffffffffu;
 
 struct Layout {
@@ -78,10 +79,12 @@ struct Layout {
   float* mpart;       // [units][n_chunks][rec]    all-token chunk moments
   float* s;           // [units][T]
   float* s2;          // [units][T]
-  int32_t* idx;       // [units / hs][hs * B] selection lists (h * T + t), ascending
+  int lsel;           // most rows a unit keeps: B, or its share of a group's at most
+  int32_t* idx;       // [units][lsel] selected positions, ascending
   int32_t* cnt;       // [units] rows each unit retains
   uint32_t* hist;     // [2][units][kBins] keys of the unprotected scores per bin (s, s2)
-  int32_t* hbeg;      // [units] first slot of each unit in idx
+  unsigned long long* glist;  // [units / hs][kGroupCont] contested pairs of a joint selection
+  int32_t* gcnt;              // [2][units] their counts by group (s, s2)
   uint8_t* cimg;      // [units][3][128 x 128] C0' as three bf16 parts, in the residual's operand layout
   float* mv0;         // [units][kDP] mu_v of E0
   float* fro;         // [units][kDP] parts of ||C0'||_F^2
@@ -98,10 +101,15 @@ __host__ __device__ __forceinline__ int protected_count(int T, int W, int sink, 
   return s + w - overlap;
 }
 
-Layout make_layout(const mkv_geom& g, int T, int B, int W, int adaptive, int num_sms) {
+Layout make_layout(const mkv_geom& g, int T, int B, int W, int sink, int keep_window, int adaptive, int num_sms) {
   Layout L{};
   L.hs = 1;
-  if (adaptive && T > B) L.hs = g.n_kv_heads;
+  L.lsel = B;
+  if (adaptive && T > B) {  // a unit keeps its protected rows plus up to every joint selection
+    const long prot = protected_count(T, W, sink, keep_window);
+    L.hs = g.n_kv_heads;
+    L.lsel = static_cast<int>(std::min<long>(T, (long)g.n_kv_heads * (B - prot) + prot));
+  }
   L.D = g.head_dim;
   L.G = g.group;
   L.W = W;
@@ -133,10 +141,12 @@ size_t carve(Layout& L, void* ws) {
   L.mpart = reinterpret_cast<float*>(take(U * L.n_chunks * L.rec * sizeof(float)));
   L.s = reinterpret_cast<float*>(take(U * (size_t)L.T * sizeof(float)));
   L.s2 = reinterpret_cast<float*>(take(U * (size_t)L.T * sizeof(float)));
-  L.idx = reinterpret_cast<int32_t*>(take(U * (size_t)L.B * sizeof(int32_t)));
+  L.idx = reinterpret_cast<int32_t*>(take(U * (size_t)L.lsel * sizeof(int32_t)));
   L.cnt = reinterpret_cast<int32_t*>(take(U * sizeof(int32_t)));
   L.hist = reinterpret_cast<uint32_t*>(take(2 * U * (size_t)kBins * sizeof(uint32_t)));
-  L.hbeg = reinterpret_cast<int32_t*>(take(U * sizeof(int32_t)));
+  L.glist = reinterpret_cast<unsigned long long*>(
+      take(L.hs > 1 ? U / L.hs * (size_t)kGroupCont * sizeof(unsigned long long) : 0));
+  L.gcnt = reinterpret_cast<int32_t*>(take(2 * U * sizeof(int32_t)));
   L.cimg = take(U * (size_t)3 * kTileBytes);
   L.mv0 = reinterpret_cast<float*>(take(U * (size_t)kDP * sizeof(float)));
   L.fro = reinterpret_cast<float*>(take(U * (size_t)kDP * sizeof(float)));
@@ -252,6 +262,7 @@ struct TcArgs {
   const float* s_in;
   float* s_out;
   uint32_t* hist;  // stats_tc: both tables, zeroed; scores_tc, residual_tc: the table their scores are counted in
+  int32_t* gcnt;   // [2][units] counts of joint selections, zeroed by stats_tc
   int units;
   float* diag;
   const uint8_t* cimg;  // [units][3][128 x 128] operand image of C0'
@@ -259,7 +270,9 @@ struct TcArgs {
   float* norms;         // [units][T][2] ||k_t||^2, ||v_t||^2
   // residual_tc's pruning
   int prune, hs, B;     // hs: units per selection group
-  const int32_t* idx;   // [groups][hs * B] the first stage's selections
+  const int32_t* idx;   // [units][lsel] the first stage's selections
+  const int32_t* cnt;   // [units] their numbers (joint; B otherwise)
+  int lsel;
   const float* fro;     // [units][kDP] parts (n_fro of them) of ||C0'||_F^2
   int n_fro;
   int32_t* cand;        // [units][T] positions left to compute, per CTA from its first position on
@@ -426,6 +439,7 @@ __global__ void __launch_bounds__(kStatThreads, 1)
     // group 1 = warps 6..9 (tokens 64..127); TMEM lane quarter qd = warp % 4
     const int ew = warp - 2, grp = ew >> 2;
     const int et = tid - 64 - grp * 128, qd = warp & 3;
+    if (chunk == 0 && tid - 64 < 2) p.gcnt[(size_t)(tid - 64) * p.units + u] = 0;
     if (chunk == 0)  // the unit's two tables of key counts
       for (int i = tid - 64; i < 2 * kBins / 4; i += 256) {
         const int tab = i / (kBins / 4), b4 = i % (kBins / 4);
@@ -863,15 +877,22 @@ __global__ void __launch_bounds__(kResThreads, 1)
     __syncthreads();
     // theta: the smallest lower bound over the first stage's free rows (0 where a bound says nothing)
     float lowest = INFINITY;
+    auto bound = [&](int h, int i) {
+      const int t = min(max(p.idx[(size_t)(g0 + h) * p.lsel + i], 0), p.T - 1);
+      if (is_protected(t, p.T, p.W, p.sink, p.keep_window)) return;
+      const float2 nn = reinterpret_cast<const float2*>(p.norms)[(size_t)(g0 + h) * p.T + t];
+      float lb = sqrtf(nn.y) - s_mvn[h] - s_fro[h] * sqrtf(nn.x);
+      lb = p.s_in[(size_t)(g0 + h) * p.T + t] * (lb > 0.f ? lb : 0.f);
+      lowest = fminf(lowest, lb > 0.f ? lb : 0.f);  // a NaN counts as 0
+    };
+    if (p.hs == 1) {
 #pragma unroll 4
-    for (int i = tid; i < p.hs * p.B; i += kResThreads) {
-      const int f = min(max(p.idx[(size_t)(g0 / p.hs) * p.hs * p.B + i], 0), p.hs * p.T - 1);
-      const int h = p.hs == 1 ? 0 : f / p.T, t = f - h * p.T;
-      if (!is_protected(t, p.T, p.W, p.sink, p.keep_window)) {
-        const float2 nn = reinterpret_cast<const float2*>(p.norms)[(size_t)g0 * p.T + f];
-        float lb = sqrtf(nn.y) - s_mvn[h] - s_fro[h] * sqrtf(nn.x);
-        lb = p.s_in[(size_t)g0 * p.T + f] * (lb > 0.f ? lb : 0.f);
-        lowest = fminf(lowest, lb > 0.f ? lb : 0.f);  // a NaN counts as 0
+      for (int i = tid; i < p.B; i += kResThreads) bound(0, i);
+    } else {
+      for (int h = warp; h < p.hs; h += kResThreads / 32) {  // a warp per head
+        const int c = min(p.cnt[g0 + h], p.lsel);
+#pragma unroll 4
+        for (int i = lane; i < c; i += 32) bound(h, i);
       }
     }
     const uint32_t wmin = __reduce_min_sync(kFull, __float_as_uint(lowest));
@@ -1030,253 +1051,330 @@ __global__ void __launch_bounds__(kResThreads, 1)
 }
 
 // ----------------------------------------------------------------- select
-// One cluster of kSelCL CTAs per selection group -- a unit, or with the
-// adaptive budget the hs KV heads of a batch item, whose (head, position)
-// pairs f = h * T + t are ranked together.  R = protected + the k highest
-// keys among the other pairs (ties to the lower f), written ascending, with
-// each unit's count and first slot.
+// One cluster of kSelCL CTAs per unit.  R = protected + the k highest keys
+// among the unit's other positions (ties to the lower position), or with the
+// adaptive budget the unit's share of the highest keys among the (head,
+// position) pairs f = h * T + t of its batch item's KV heads (ties to the lower
+// f); its positions are written ascending, with their count.
 //
 // The kernel that computed the scores has counted their keys into kBins bins
 // (exponent and three mantissa bits), so the bin of the k-th highest is known
-// from one scan.  The keys of that bin (about a sixth of k) are exchanged
-// over the cluster and ranked by counting, which gives the last selected
-// (key, f); one more pass counts and one writes.  Two cluster barriers, where
-// a radix select over the keys took four passes of three barriers each.  When
-// a CTA holds more than kMaxCont keys of that bin (many equal scores), the
-// cluster bisects the key and then f instead.  512 threads for a unit (64
-// CTAs a wave at 8 units), 1024 for the longer joint lists.
+// from one scan.  The keys of that bin (about a sixth of k) are exchanged and
+// ranked by counting, which gives the last selected pair; one more pass counts
+// and one writes.  Two cluster barriers, where a radix select over the keys
+// took four passes of three barriers each.  A unit's contested keys are
+// exchanged over its cluster; the pairs of a batch item through global memory
+// (contest_kernel), so that a joint selection too has kSelCL CTAs per unit.
+// When there are more contested keys than the lists hold (many equal scores),
+// a radix select over the pairs takes the place of the ranking.
 struct SelectArgs {
   const float* scores;   // [units][T]
   const uint32_t* hist;  // [units][kBins] counts of the unprotected scores' keys
   int T, W, B, sink, keep_window;
-  int32_t* idx;       // [groups][hs * B] selection lists, h * T + position, ascending (workspace)
-  int32_t* diag_idx;  // optional copy
-  int hs;             // units per selection group (1: one unit; > 1: the KV heads of a batch item)
-  int32_t* cnt;       // [units] rows retained per unit
-  int32_t* hbeg;      // [units] the unit's first slot in idx
+  int32_t* idx;       // [units][lsel] selected positions, ascending (workspace)
+  int32_t* diag_idx;  // optional copy (one unit per group)
+  int lsel;
+  int hs;             // units per selection group (1, or the KV heads of a batch item)
+  int32_t* cnt;       // [units] rows each unit retains (joint)
+  unsigned long long* glist;  // [groups][kGroupCont] contested pairs of a group (joint)
+  int32_t* gcnt;              // [groups] their count
 };
 
-constexpr int kSelCL = 8;      // CTAs per selection group (one cluster), each over a contiguous range of pairs
-constexpr int kMaxCont = 256;  // keys of the contested bin a CTA may hold
+constexpr int kSelThreads = 512;
+constexpr int kSelWarps = kSelThreads / 32;
+constexpr int kSelCL = 8;         // CTAs per unit (one cluster), each over a contiguous range of positions
+constexpr int kMaxCont = 256;     // keys of the contested bin a CTA may hold
+constexpr int kSelBatch = 8;      // positions per lane loaded together
 
-template <int kSelThreads>
-__global__ void __cluster_dims__(kSelCL, 1, 1) __launch_bounds__(kSelThreads, 1024 / kSelThreads)
-    select_kernel(const SelectArgs a) {
-  constexpr int kSelWarps = kSelThreads / 32;
-  constexpr int kBatch = 8;  // pairs per lane loaded together
+// pairs are ordered by (key, ~f): a higher key first, at equal keys the lower f
+__device__ __forceinline__ unsigned long long select_pair(float s, int f) {
+  return (static_cast<unsigned long long>(score_key(s)) << 32) | (0xffffffffu - static_cast<unsigned>(f));
+}
+
+// Exclusive sum over the block of one count per warp; the total in *total.
+__device__ __forceinline__ int block_counts(int mine, int* s_w, int* total) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  __syncthreads();
+  if (lane == 0) s_w[warp] = mine;
+  __syncthreads();
+  int before = 0, all = 0;
+#pragma unroll 4
+  for (int w = 0; w < kSelWarps; ++w) {
+    before += w < warp ? s_w[w] : 0;
+    all += s_w[w];
+  }
+  *total = all;
+  return before;
+}
+
+// The bin of the group's k-th highest key (k > 0) and how many of its keys are
+// selected, into *s_bin and *s_need: thread t takes four bins, descending.
+__device__ __forceinline__ void threshold_bin(const SelectArgs& a, int grp, int k, int* s_w, int* s_bin, int* s_need) {
+  const int tid = threadIdx.x, lane = tid & 31;
+  static_assert(kBins == 4 * kSelThreads, "four bins per thread");
+  uint4 c = make_uint4(0u, 0u, 0u, 0u);
+#pragma unroll 4
+  for (int h = 0; h < a.hs; ++h) {
+    const uint4 x = reinterpret_cast<const uint4*>(a.hist + ((size_t)grp * a.hs + h) * kBins)[kBins / 4 - 1 - tid];
+    c.x += x.x;
+    c.y += x.y;
+    c.z += x.z;
+    c.w += x.w;
+  }
+  const int b[4] = {(int)c.w, (int)c.z, (int)c.y, (int)c.x};
+  int incl = b[0] + b[1] + b[2] + b[3];
+  const int mine = incl;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const int y = __shfl_up_sync(kFull, incl, o);
+    if (lane >= o) incl += y;
+  }
+  int total;
+  int above = block_counts(__shfl_sync(kFull, incl, 31), s_w, &total) + incl - mine;
+#pragma unroll
+  for (int e = 0; e < 4; ++e) {
+    if (above < k && above + b[e] >= k) {  // one bin of the block
+      *s_bin = kBins - 1 - (tid * 4 + e);
+      *s_need = k - above;
+    }
+    above += b[e];
+  }
+  __syncthreads();
+}
+
+// fn(position, in range, pair) for the positions [w0, w1) of one unit, a warp's
+// share, kSelBatch x 32 loads in flight; f0 = the unit's first pair.  A
+// protected position's pair stands above all.
+template <typename F>
+__device__ __forceinline__ void each_pair(const SelectArgs& a, const float* sc, int w0, int w1, int f0, F&& fn) {
+  const int lane = threadIdx.x & 31;
+#pragma unroll 1
+  for (int t0 = w0; t0 < w1; t0 += 32 * kSelBatch) {
+    float s[kSelBatch];
+#pragma unroll
+    for (int i = 0; i < kSelBatch; ++i) {
+      const int t = t0 + i * 32 + lane;
+      s[i] = t < w1 ? sc[t] : 0.f;
+    }
+#pragma unroll
+    for (int i = 0; i < kSelBatch; ++i) {
+      if (t0 + i * 32 >= w1) break;  // warp-uniform
+      const int t = t0 + i * 32 + lane;
+      fn(t, t < w1, is_protected(t, a.T, a.W, a.sink, a.keep_window) ? ~0ull : select_pair(s[i], f0 + t));
+    }
+  }
+}
+
+// The contested pairs of joint selections: grid (kSelCL, units), every CTA's
+// part of its unit's positions, into the group's list.
+__global__ void __launch_bounds__(kSelThreads) contest_kernel(const SelectArgs a) {
+  __shared__ int s_w[kSelWarps];
+  __shared__ int s_bin, s_need, s_n, s_at;
+  __shared__ unsigned long long s_cont[kGroupCont];
+  const int u = blockIdx.y, grp = u / a.hs, h = u % a.hs, tid = threadIdx.x, warp = tid >> 5;
+  const int k = a.hs * (a.B - protected_count(a.T, a.W, a.sink, a.keep_window));
+  if (tid == 0) {
+    s_n = 0;
+    s_bin = kBins;
+  }
+  grid_dependency_wait();
+  grid_launch_dependents();
+  if (k <= 0) return;
+  __syncthreads();
+  threshold_bin(a, grp, k, s_w, &s_bin, &s_need);
+  const int bin = s_bin, per = (a.T + kSelCL * kSelWarps - 1) / (kSelCL * kSelWarps);
+  const int w0 = min(a.T, (static_cast<int>(blockIdx.x) * kSelWarps + warp) * per), w1 = min(a.T, w0 + per);
+  each_pair(a, a.scores + (size_t)u * a.T, w0, w1, h * a.T, [&](int, bool in, unsigned long long p) {
+    if (in && p != ~0ull && key_bin(static_cast<uint32_t>(p >> 32)) == bin) {
+      const int slot = atomicAdd(&s_n, 1);
+      if (slot < kGroupCont) s_cont[slot] = p;
+    }
+  });
+  __syncthreads();
+  if (tid == 0) s_at = atomicAdd(a.gcnt + grp, s_n);
+  __syncthreads();
+  for (int i = tid; i < min(s_n, kGroupCont); i += kSelThreads)
+    if (s_at + i < kGroupCont) a.glist[(size_t)grp * kGroupCont + s_at + i] = s_cont[i];
+}
+
+template <bool JOINT>
+__global__ void __cluster_dims__(kSelCL, 1, 1) __launch_bounds__(kSelThreads, 2) select_kernel(const SelectArgs a) {
   __shared__ int s_w[kSelWarps];
   __shared__ int s_bin, s_need;
-  __shared__ int s_n;                                          // this CTA's contested keys
-  __shared__ int s_cn[kSelCL];                                 // every CTA's (written remotely)
-  __shared__ unsigned long long s_cont[kSelCL][kMaxCont];      // every CTA's contested (key, ~f) (written remotely)
-  __shared__ unsigned long long s_last;                        // the last selected (key, ~f)
-  __shared__ int s_tot[2][kSelCL];                             // every CTA's counts (written remotely)
-  __shared__ int s_hcnt[kMaxHs], s_hstart[kMaxHs + 1];         // selections per head
+  __shared__ int s_n;            // this CTA's contested keys
+  __shared__ int s_cn[kSelCL];   // every CTA's (written remotely)
+  // the unit's contested pairs by CTA (written remotely), or the group's list
+  __shared__ unsigned long long s_cont[JOINT ? kGroupCont : kSelCL * kMaxCont];
+  __shared__ unsigned long long s_last;  // the last selected pair (written remotely when joint)
+  __shared__ int s_tot[2][kSelCL];       // every CTA's counts (written remotely)
   cg::cluster_group cluster = cg::this_cluster();
   const int rank = static_cast<int>(cluster.block_rank());
-  const int grp = blockIdx.x / kSelCL, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const int T = a.T, W = a.W, hs = a.hs, N = hs * T;
-  const int k = hs * (a.B - protected_count(T, W, a.sink, a.keep_window));  // >= 0 (validated), < candidates
-  const float* sc = a.scores + (size_t)grp * N;  // the group's units are consecutive
-  // warp w of CTA r takes the contiguous pairs [w0, w1)
-  const int per = (N + kSelCL * kSelWarps - 1) / (kSelCL * kSelWarps);
-  const int w0 = min(N, (rank * kSelWarps + warp) * per), w1 = min(N, w0 + per);
+  const int u = blockIdx.x / kSelCL, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int T = a.T, hs = JOINT ? a.hs : 1, grp = u / hs, h = u % hs;
+  const int prot = protected_count(T, a.W, a.sink, a.keep_window);
+  const int k = hs * (a.B - prot);  // >= 0 (validated), < candidates
+  const float* sc = a.scores + (size_t)u * T;
+  // warp w of CTA r takes the contiguous positions [w0, w1)
+  const int per = (T + kSelCL * kSelWarps - 1) / (kSelCL * kSelWarps);
+  const int w0 = min(T, (rank * kSelWarps + warp) * per), w1 = min(T, w0 + per);
   if (tid == 0) {
     s_n = 0;
     s_bin = kBins;
     s_need = 0;
     s_last = ~0ull;
   }
-  if (tid < hs) s_hcnt[tid] = 0;
   __syncthreads();
   cluster_arrive_relaxed();  // every CTA has started: awaited before the first remote store
   grid_dependency_wait();
   grid_launch_dependents();
 
-  // pairs are ordered by (key, ~f): a higher key first, at equal keys the lower f;
-  // a protected pair stands above all
-  auto pair_of = [&](int f, float s) -> unsigned long long {
-    const int t = hs == 1 ? f : f % T;
-    if (is_protected(t, T, W, a.sink, a.keep_window)) return ~0ull;
-    return (static_cast<unsigned long long>(score_key(s)) << 32) | (0xffffffffu - static_cast<unsigned>(f));
-  };
-  // fn(f, in range, pair) for every pair of this warp, kBatch x 32 loads in flight
-  auto each_pair = [&](auto&& fn) {
-#pragma unroll 1
-    for (int f0 = w0; f0 < w1; f0 += 32 * kBatch) {
-      float s[kBatch];
-#pragma unroll
-      for (int i = 0; i < kBatch; ++i) {
-        const int f = f0 + i * 32 + lane;
-        s[i] = f < w1 ? sc[f] : 0.f;
-      }
-#pragma unroll
-      for (int i = 0; i < kBatch; ++i) {
-        if (f0 + i * 32 >= w1) break;  // warp-uniform
-        const int f = f0 + i * 32 + lane;
-        fn(f, f < w1, pair_of(f, s[i]));
-      }
-    }
-  };
-  // exclusive sum over the block of one count per warp (`mine` from lane 0); the total in *total
-  auto block_counts = [&](int mine, int* total) -> int {
-    __syncthreads();
-    if (lane == 0) s_w[warp] = mine;
-    __syncthreads();
-    int before = 0, all = 0;
-#pragma unroll 4
-    for (int w = 0; w < kSelWarps; ++w) {
-      before += w < warp ? s_w[w] : 0;
-      all += s_w[w];
-    }
-    *total = all;
-    return before;
-  };
-
-  // ---- the bin of the k-th highest key: thread t takes four bins, descending
   if (k > 0) {
-    uint4 c = make_uint4(0u, 0u, 0u, 0u);
-    if (tid < kBins / 4)
-#pragma unroll 4
-      for (int h = 0; h < hs; ++h) {
-        const uint4 x = reinterpret_cast<const uint4*>(a.hist + ((size_t)grp * hs + h) * kBins)[kBins / 4 - 1 - tid];
-        c.x += x.x;
-        c.y += x.y;
-        c.z += x.z;
-        c.w += x.w;
-      }
-    const int b[4] = {(int)c.w, (int)c.z, (int)c.y, (int)c.x};
-    int incl = b[0] + b[1] + b[2] + b[3];
-    const int mine = incl;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-      const int y = __shfl_up_sync(kFull, incl, o);
-      if (lane >= o) incl += y;
-    }
-    int total;
-    int above = block_counts(__shfl_sync(kFull, incl, 31), &total) + incl - mine;
-#pragma unroll
-    for (int e = 0; e < 4; ++e) {
-      if (above < k && above + b[e] >= k) {  // one bin of the block
-        s_bin = kBins - 1 - (tid * 4 + e);
-        s_need = k - above;
-      }
-      above += b[e];
-    }
-    __syncthreads();
-    const int bin = s_bin;
-    // ---- the contested keys: this CTA's into every CTA's list
-    each_pair([&](int f, bool in, unsigned long long p) {
-      if (in && p != ~0ull && key_bin(static_cast<uint32_t>(p >> 32)) == bin) {
-        const int slot = atomicAdd(&s_n, 1);
-        if (slot < kMaxCont) s_cont[rank][slot] = p;
-      }
-    });
-    __syncthreads();
-    cluster_wait_acquire();
-    const int mn = s_n;
-    if (tid < kSelCL) *cluster.map_shared_rank(&s_cn[rank], tid) = mn;
-    for (int i = tid; i < min(mn, kMaxCont) * kSelCL; i += kSelThreads) {
-      const int r = i % kSelCL;
-      if (r != rank) *cluster.map_shared_rank(&s_cont[rank][i / kSelCL], r) = s_cont[rank][i / kSelCL];
-    }
-    cluster.sync();
+    threshold_bin(a, grp, k, s_w, &s_bin, &s_need);
+    const int bin = s_bin, need = s_need;
     bool over = false;
-    int m = 0;
-    for (int r = 0; r < kSelCL; ++r) {
-      over |= s_cn[r] > kMaxCont;
-      m += s_cn[r];
-    }
-    const int need = s_need;
-    if (!over) {
-      // the need-th of them: the one that need - 1 others precede
-      for (int i = tid; i < m; i += kSelThreads) {
-        int j = i, r = 0;
-        while (j >= s_cn[r]) j -= s_cn[r++];
-        const unsigned long long p = s_cont[r][j];
-        int before = 0;
-        for (int r2 = 0; r2 < kSelCL; ++r2) {
-          const int c2 = s_cn[r2];
-#pragma unroll 4
-          for (int j2 = 0; j2 < c2; ++j2) before += s_cont[r2][j2] > p ? 1 : 0;
+    if constexpr (JOINT) {
+      cluster_wait_acquire();
+      const int m = a.gcnt[grp];
+      over = m > kGroupCont;
+      if (!over) {
+        for (int i = tid; i < m; i += kSelThreads) s_cont[i] = a.glist[(size_t)grp * kGroupCont + i];
+        __syncthreads();
+        // the need-th of them, the one that need - 1 others precede: the
+        // cluster's warps share the candidates
+        for (int i = rank * kSelWarps + warp; i < m; i += kSelCL * kSelWarps) {
+          const unsigned long long p = s_cont[i];
+          int before = 0;
+          for (int j = lane; j < m; j += 32) before += s_cont[j] > p ? 1 : 0;
+          before = __reduce_add_sync(kFull, before);
+          if (before == need - 1 && lane < kSelCL) *cluster.map_shared_rank(&s_last, lane) = p;
         }
-        if (before == need - 1) s_last = p;
-      }
-      __syncthreads();
-    } else {
-      // bisect: the largest p that at least k unprotected pairs reach
-      unsigned long long lo = 0ull;
-#pragma unroll 1
-      for (int bit = 63; bit >= 0; --bit) {
-        const unsigned long long mid = lo | (1ull << bit);
-        int c = 0;
-        each_pair([&](int f, bool in, unsigned long long p) { c += in && p != ~0ull && p >= mid ? 1 : 0; });
-        c = __reduce_add_sync(kFull, c);
-        int tot;
-        (void)block_counts(c, &tot);
-        if (tid < kSelCL) *cluster.map_shared_rank(&s_tot[bit & 1][rank], tid) = tot;
         cluster.sync();
-        int all = 0;
-        for (int r = 0; r < kSelCL; ++r) all += s_tot[bit & 1][r];
-        if (all >= k) lo = mid;
       }
-      if (tid == 0) s_last = lo;
-      cluster.sync();  // s_tot is written again below
+    } else {
+      // ---- the contested keys: this CTA's into every CTA's list
+      each_pair(a, sc, w0, w1, 0, [&](int, bool in, unsigned long long p) {
+        if (in && p != ~0ull && key_bin(static_cast<uint32_t>(p >> 32)) == bin) {
+          const int slot = atomicAdd(&s_n, 1);
+          if (slot < kMaxCont) s_cont[rank * kMaxCont + slot] = p;
+        }
+      });
+      __syncthreads();
+      cluster_wait_acquire();
+      const int mn = s_n;
+      if (tid < kSelCL) *cluster.map_shared_rank(&s_cn[rank], tid) = mn;
+      for (int i = tid; i < min(mn, kMaxCont) * kSelCL; i += kSelThreads) {
+        const int r = i % kSelCL, e = rank * kMaxCont + i / kSelCL;
+        if (r != rank) *cluster.map_shared_rank(&s_cont[e], r) = s_cont[e];
+      }
+      cluster.sync();
+      int m = 0;
+      for (int r = 0; r < kSelCL; ++r) {
+        over |= s_cn[r] > kMaxCont;
+        m += s_cn[r];
+      }
+      if (!over) {
+        // the need-th of them: the one that need - 1 others precede
+        for (int i = tid; i < m; i += kSelThreads) {
+          int j = i, r = 0;
+          while (j >= s_cn[r]) j -= s_cn[r++];
+          const unsigned long long p = s_cont[r * kMaxCont + j];
+          int before = 0;
+          for (int r2 = 0; r2 < kSelCL; ++r2) {
+            const int c2 = s_cn[r2];
+#pragma unroll 4
+            for (int j2 = 0; j2 < c2; ++j2) before += s_cont[r2 * kMaxCont + j2] > p ? 1 : 0;
+          }
+          if (before == need - 1) s_last = p;
+        }
+        __syncthreads();
+      }
+    }
+    if (over) {
+      // radix select over the group's pairs, eight bits at a time below those
+      // the bin fixes, until the digit's pairs are exactly the missing ones
+      // (each cluster of a group over all its units)
+      uint32_t* hist = reinterpret_cast<uint32_t*>(s_cont);  // [256] this CTA's counts (read remotely), [256] the cluster's
+      const int top = bin > 0 ? 12 : 0;
+      unsigned long long prefix = bin > 0 ? static_cast<unsigned long long>(0x800u | bin) << 52 : 0ull;
+      unsigned long long mask = bin > 0 ? 0xfffull << 52 : 0ull;
+      int left = bin > 0 ? need : k;
+#pragma unroll 1
+      for (int shift = 64 - top - 8;; shift = max(shift - 8, 0)) {
+        cluster.sync();  // the lists, or the counts of the pass before, are read
+        if (tid < 256) hist[tid] = 0u;
+        __syncthreads();
+#pragma unroll 1
+        for (int g = 0; g < hs; ++g)
+          each_pair(a, a.scores + ((size_t)grp * hs + g) * T, w0, w1, g * T, [&](int, bool in, unsigned long long p) {
+            if (in && p != ~0ull && (p & mask) == prefix) atomicAdd(&hist[(p >> shift) & 255u], 1u);
+          });
+        cluster.sync();
+        if (tid < 256) {
+          uint32_t x = 0u;
+          for (int r = 0; r < kSelCL; ++r) x += cluster.map_shared_rank(hist, r)[tid];
+          hist[256 + tid] = x;
+        }
+        __syncthreads();
+        if (tid == 0) {  // the digit where the descending count reaches `left`
+          int d = 255, above = 0;
+          while (d > 0 && above + static_cast<int>(hist[256 + d]) < left) above += hist[256 + d--];
+          s_bin = d;
+          s_need = left - above;
+        }
+        __syncthreads();
+        prefix |= static_cast<unsigned long long>(s_bin) << shift;
+        mask |= 255ull << shift;
+        left = s_need;
+        if (shift == 0 || static_cast<int>(hist[256 + s_bin]) == left) break;  // uniform over the cluster
+        __syncthreads();
+      }
+      if (tid == 0) s_last = prefix;
+      cluster.sync();  // no counts are read remotely any more
     }
   } else {
     cluster_wait_acquire();
   }
 
-  // ---- this CTA's selections, then everybody's: protected pairs and those not below the last
+  // ---- this CTA's selections, then everybody's: protected positions and those not below the last
   const unsigned long long last = s_last;
   int c = 0;
-  each_pair([&](int f, bool in, unsigned long long p) { c += __popc(__ballot_sync(kFull, in && p >= last)); });
+  each_pair(a, sc, w0, w1, h * T,
+            [&](int, bool in, unsigned long long p) { c += __popc(__ballot_sync(kFull, in && p >= last)); });
   int tot;
-  int o = block_counts(c, &tot);
+  int o = block_counts(c, s_w, &tot);
   if (tid < kSelCL) *cluster.map_shared_rank(&s_tot[0][rank], tid) = tot;
   cluster.sync();
   for (int r = 0; r < rank; ++r) o += s_tot[0][r];
-  const int n_sel = hs * a.B;  // the group's selections (protected included)
-  int32_t* out = a.idx + (size_t)grp * n_sel;
-  each_pair([&](int f, bool in, unsigned long long p) {
+  int32_t* out = a.idx + (size_t)u * a.lsel;
+  each_pair(a, sc, w0, w1, h * T, [&](int t, bool in, unsigned long long p) {
     const bool sel = in && p >= last;
     const unsigned mask = __ballot_sync(kFull, sel);
     const int at = o + __popc(mask & ((1u << lane) - 1u));
-    if (sel && at < n_sel) {
-      out[at] = f;
-      if (a.diag_idx) a.diag_idx[(size_t)grp * n_sel + at] = f;
-      if (hs > 1) atomicAdd(&s_hcnt[f / T], 1);
+    if (sel && at < a.lsel) {
+      out[at] = t;
+      if (!JOINT && a.diag_idx) a.diag_idx[(size_t)u * a.lsel + at] = t;
     }
     o += __popc(mask);
   });
-  if (hs == 1) {
-    if (rank == 0 && tid == 0) {
-      a.cnt[grp] = a.B;
-      a.hbeg[grp] = grp * n_sel;
-    }
-    return;  // no remote access follows the last cluster barrier
+  if (JOINT && rank == 0 && tid == 0) {
+    int x = 0;
+    for (int r = 0; r < kSelCL; ++r) x += s_tot[0][r];
+    a.cnt[u] = min(x, a.lsel);
   }
-  // each head's slots are a contiguous run of the ascending list, as long as
-  // the head's selections in all CTAs of the cluster
-  cluster.sync();
-  if (rank == 0) {
-    if (tid < hs) {
-      int x = 0;
-      for (int r = 0; r < kSelCL; ++r) x += cluster.map_shared_rank(s_hcnt, r)[tid];
-      s_hstart[tid + 1] = x;
-    }
-    __syncthreads();
-    if (tid == 0) {
-      s_hstart[0] = 0;
-      for (int h = 0; h < hs; ++h) s_hstart[h + 1] += s_hstart[h];
-    }
-    __syncthreads();
-    if (tid < hs) {
-      a.cnt[grp * hs + tid] = s_hstart[tid + 1] - s_hstart[tid];
-      a.hbeg[grp * hs + tid] = grp * n_sel + s_hstart[tid];
-    }
+  // no remote access follows the last cluster barrier
+}
+
+// The first stage's joint list for inspection, [groups][hs * B] of h * T + t,
+// ascending: one CTA per group, from its units' lists.
+__global__ void __launch_bounds__(256) diag_joint_kernel(const SelectArgs a) {
+  int o = 0;
+  for (int h = 0; h < a.hs; ++h) {
+    const int u = blockIdx.x * a.hs + h, c = a.cnt[u];
+    for (int i = threadIdx.x; i < c; i += 256)
+      if (o + i < a.hs * a.B)
+        a.diag_idx[(size_t)blockIdx.x * a.hs * a.B + o + i] = h * a.T + a.idx[(size_t)u * a.lsel + i];
+    o += c;
   }
-  cluster.sync();  // no CTA leaves while another may still read its shared memory
 }
 
 // ------------------------------------------------------------------- rset
@@ -1411,9 +1509,8 @@ __global__ void __launch_bounds__(2048 / CL) rset_kernel(const RsetArgs a) {
   grid_launch_dependents();
 
   // ---- row tiles
-  const int cnt = L.hs == 1 ? L.B : L.cnt[u];  // a unit's own selection has fixed size and place
-  const int32_t* lst = L.idx + (L.hs == 1 ? (size_t)u * L.B : (size_t)L.hbeg[u]);
-  const int hT = (u % L.hs) * T;  // list entries are h * T + position
+  const int cnt = L.hs == 1 ? L.B : L.cnt[u];
+  const int32_t* lst = L.idx + (size_t)u * L.lsel;
   const int n_tiles = (cnt + kTok - 1) / kTok;
   const __nv_bfloat16* Ku = a.K + (size_t)u * T * D + kh * 64;
   const __nv_bfloat16* Vu = a.V + (size_t)u * T * D;
@@ -1433,7 +1530,7 @@ __global__ void __launch_bounds__(2048 / CL) rset_kernel(const RsetArgs a) {
     }
     const int r0 = ti * kTok;
     if (tid < kTok)  // never outside the unit's slab
-      s_t[tid] = r0 + tid < cnt ? min(max(lst[r0 + tid] - hT, 0), T - 1) : -1;
+      s_t[tid] = r0 + tid < cnt ? min(max(lst[r0 + tid], 0), T - 1) : -1;
     __syncthreads();
 #pragma unroll 1
     for (int i = tid; i < kTok * 8; i += kThr) {  // the key half: 8 chunks a row
@@ -1682,7 +1779,7 @@ cudaError_t launch_rset(const RsetArgs& a, int cl, cudaStream_t st) {
 }
 
 cudaError_t run(const CompressArgs& a, const mkv_geom& g, int num_sms, cudaStream_t st) {
-  Layout L = make_layout(g, a.T, a.budget, a.window, a.adaptive, num_sms);
+  Layout L = make_layout(g, a.T, a.budget, a.window, a.sink, a.keep_window, a.adaptive, num_sms);
   carve(L, a.ws);
   const int D = g.head_dim, T = a.T, B = a.budget, U = L.units;
   const bool keep_all = T <= B;
@@ -1715,6 +1812,7 @@ cudaError_t run(const CompressArgs& a, const mkv_geom& g, int num_sms, cudaStrea
   tp.rowpart = L.rowpart;
   tp.mrec = L.mpart;
   tp.hist = L.hist;
+  tp.gcnt = L.gcnt;
   tp.units = U;
   tp.norms = L.norms;
   tp.ws = a.ws;
@@ -1734,10 +1832,10 @@ cudaError_t run(const CompressArgs& a, const mkv_geom& g, int num_sms, cudaStrea
     return cudaGetLastError();
   }
 
-  auto select = [&](const float* scores, const uint32_t* hist, int32_t* diag_idx) -> cudaError_t {
+  auto select = [&](int stage, const float* scores, int32_t* diag_idx) -> cudaError_t {
     SelectArgs sa{};
     sa.scores = scores;
-    sa.hist = hist;
+    sa.hist = L.hist + (size_t)stage * U * kBins;
     sa.diag_idx = diag_idx;
     sa.T = T;
     sa.W = a.window;
@@ -1745,11 +1843,19 @@ cudaError_t run(const CompressArgs& a, const mkv_geom& g, int num_sms, cudaStrea
     sa.sink = a.sink;
     sa.keep_window = a.keep_window;
     sa.idx = L.idx;
+    sa.lsel = L.lsel;
     sa.hs = L.hs;
     sa.cnt = L.cnt;
-    sa.hbeg = L.hbeg;
-    if (L.hs == 1) return launch_pdl(select_kernel<512>, dim3(U * kSelCL), 512, 0, st, 0, sa);
-    return launch_pdl(select_kernel<1024>, dim3(U / L.hs * kSelCL), 1024, 0, st, 0, sa);
+    sa.glist = L.glist;
+    sa.gcnt = L.gcnt + (size_t)stage * U;
+    if (L.hs == 1) return launch_pdl(select_kernel<false>, dim3(U * kSelCL), kSelThreads, 0, st, 0, sa);
+    cudaError_t se = launch_pdl(contest_kernel, dim3(kSelCL, U), kSelThreads, 0, st, 0, sa);
+    if (se == cudaSuccess) se = launch_pdl(select_kernel<true>, dim3(U * kSelCL), kSelThreads, 0, st, 0, sa);
+    if (se == cudaSuccess && diag_idx != nullptr) {
+      diag_joint_kernel<<<U / L.hs, 256, 0, st>>>(sa);
+      se = cudaGetLastError();
+    }
+    return se;
   };
   RsetArgs ra{};
   ra.L = L;
@@ -1767,8 +1873,7 @@ cudaError_t run(const CompressArgs& a, const mkv_geom& g, int num_sms, cudaStrea
   ra.polls = tp.polls;
   const int cl = rset_cluster(L, num_sms);
 
-  uint32_t* hist2 = L.hist + (size_t)U * kBins;
-  if ((e = select(L.s, L.hist, a.diag_idx1)) != cudaSuccess) return e;
+  if ((e = select(0, L.s, a.diag_idx1)) != cudaSuccess) return e;
   if (a.mi) {
     if ((e = launch_rset<false>(ra, cl, st)) != cudaSuccess) return e;
     TcArgs r = tp;
@@ -1776,20 +1881,22 @@ cudaError_t run(const CompressArgs& a, const mkv_geom& g, int num_sms, cudaStrea
     r.mv0 = L.mv0;
     r.s_in = L.s;
     r.s_out = L.s2;
-    r.hist = hist2;
+    r.hist = L.hist + (size_t)U * kBins;
     r.diag = a.diag_score2;
     // a second pass over the prompt is worth avoiding from eight tiles a CTA on
     r.prune = a.diag_score2 == nullptr && L.chunk >= kPruneTiles * kTok ? 1 : 0;
     r.hs = L.hs;
     r.B = B;
     r.idx = L.idx;
+    r.cnt = L.cnt;
+    r.lsel = L.lsel;
     r.fro = L.fro;
     r.n_fro = D;
     r.cand = L.cand;
     r.K = a.K;
     r.V = a.V;
     if ((e = launch_pdl(residual_tc, cg, kResThreads, kResidualSmem, st, 0, r, tmK, tmV)) != cudaSuccess) return e;
-    if ((e = select(L.s2, hist2, nullptr)) != cudaSuccess) return e;
+    if ((e = select(1, L.s2, nullptr)) != cudaSuccess) return e;
   }
   return launch_rset<true>(ra, cl, st);
 }
@@ -1797,7 +1904,7 @@ cudaError_t run(const CompressArgs& a, const mkv_geom& g, int num_sms, cudaStrea
 }  // namespace
 
 size_t compress_workspace_bytes(const mkv_geom& g, int32_t T, const mkv_compress_params& p, int num_sms) {
-  Layout L = make_layout(g, T, p.budget, p.window, p.adaptive, num_sms);
+  Layout L = make_layout(g, T, p.budget, p.window, p.sink, p.keep_window, p.adaptive, num_sms);
   return carve(L, nullptr);
 }
 

@@ -136,7 +136,7 @@ __global__ void __launch_bounds__(kClThreads, 2)
     if constexpr (!ONE) mbar_arrive_expect_tx(&recv, own_d > 0 ? static_cast<uint32_t>(S * G * (own_d + 2) * 4) : 0u);
     mbar_fence_init();
     sFail = 0;
-    sBlk = 2;  // the first two owned blocks of C' are the side warps'
+    if constexpr (ONE) sBlk = 2;  // the first two owned blocks of C' are the side warps'
     asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&tmK)) : "memory");
     asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&tmV)) : "memory");
   }
@@ -323,18 +323,23 @@ __global__ void __launch_bounds__(kClThreads, 2)
 #pragma unroll
     for (int i = 0; i < 4; ++i) d[i] = (dc[0][i] + dc[1][i]) + (dc[2][i] + dc[3][i]);
     const int ra = j * 16 + g, rb = ra + 8;  // local rows (owned dims)
+    // f_hat_E = mu_v + scale C'q: with one split, where an attending warp may
+    // get here before mu_v is staged, added at the finish
+    const float ka = ONE ? 1.f : scale, mva = ONE ? 0.f : sMuv[ra], mvb = ONE ? 0.f : sMuv[rb];
+    auto put = [&](int at, float x, float mv) { sF[at] = ONE ? x : fmaf(ka, x, mv); };
     if (2 * t < G) {
-      sF[ra * G + 2 * t] = d[0];
-      sF[rb * G + 2 * t] = d[2];
+      put(ra * G + 2 * t, d[0], mva);
+      put(rb * G + 2 * t, d[2], mvb);
     }
     if (2 * t + 1 < G) {
-      sF[ra * G + 2 * t + 1] = d[1];
-      sF[rb * G + 2 * t + 1] = d[3];
+      put(ra * G + 2 * t + 1, d[1], mva);
+      put(rb * G + 2 * t + 1, d[3], mvb);
     }
   };
-  // The blocks past the side warps' first two (few splits: up to eight blocks a
-  // CTA) go to whichever warp is free: the side warps alone finished 3-4 us
-  // after the tiles at one split, head dim 128.
+  // One split: the blocks past the side warps' first two go to whichever warp
+  // is free (the side warps alone finished 3-4 us after the tiles at head dim
+  // 128).  With more splits the side warps alternate: a claim costs the
+  // attending warps more than the block or two that are left.
   auto cq_rest = [&]() {
     for (;;) {
       int j = 0;
@@ -366,11 +371,20 @@ __global__ void __launch_bounds__(kClThreads, 2)
       __syncwarp();
     }
     __syncwarp();
-    if (use_m) {
-      if (warp - kLoaderWarp < nmt) cq_block(warp - kLoaderWarp);
-      if (nmt > 2) cq_rest();
+    if constexpr (ONE) {
+      if (use_m) {
+        cq_block(warp - kLoaderWarp);
+        cq_rest();
+      }
+      named_sync(3, 64);  // the moment warp's mu_v and mu_k rows are in place
+    } else {
+      named_sync(3, 64);
+      if (use_m)
+        for (int j = warp - kLoaderWarp; j < nmt; j += 2) {
+          if (j > 1) load_cf(j);
+          cq_block(j);
+        }
     }
-    named_sync(3, 64);  // the moment warp's mu_v and mu_k rows are in place
     if (producer) {
       if (has_new && lane < D / 4) {  // the token as floats: all of k, the owned dims of v
         const __nv_bfloat162* h2 = reinterpret_cast<const __nv_bfloat162*>(&kvc);
@@ -513,7 +527,9 @@ __global__ void __launch_bounds__(kClThreads, 2)
       __syncwarp();
       if (lane == 0) mbar_arrive(&empty[st]);
     }
-    if (use_m && nmt > 2) cq_rest();
+    if constexpr (ONE) {
+      if (use_m) cq_rest();
+    }
     if (!ok) {
       if (lane == 0) sFail = 1;
       m0 = m1 = kNegInf;
@@ -691,7 +707,7 @@ __global__ void __launch_bounds__(kClThreads, 2)
           O = fmaf(w, sVn[j], O);
         }
       }
-      const float fh = use_m ? fmaf(scale, sF[j * G + h], sMuv[j]) : 0.f;
+      const float fh = use_m ? sF[j * G + h] : 0.f;
       if (!use_m && !(L > 0.f) && j == 0) record_error(a.ws, MKV_ERR_INVALID_ARG, u);
       float lse2;
       const float res = finish(h, M, L, O, fh, lse2);
