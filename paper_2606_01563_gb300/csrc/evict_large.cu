@@ -23,6 +23,7 @@
 
 #include <algorithm>
 #include <mutex>
+#include <type_traits>
 
 #include "evict_common.cuh"
 #include "warp_mma.cuh"
@@ -69,6 +70,32 @@ struct LargeLayout {
   }
 };
 
+// A lane's DPL dims as pairs of floats, two per instruction (fma.f32x2).
+__device__ __forceinline__ uint64_t pair(float a, float b) {
+  uint64_t r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
+  return r;
+}
+__device__ __forceinline__ float pair_sum(uint64_t p) {
+  float a, b;
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(p));
+  return a + b;
+}
+__device__ __forceinline__ uint64_t fma2(uint64_t a, uint64_t b, uint64_t c) {
+  uint64_t r;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+  return r;
+}
+__device__ __forceinline__ uint64_t add2(uint64_t a, uint64_t b) {
+  uint64_t r;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+__device__ __forceinline__ uint64_t unpack2(uint32_t w) {  // two bf16
+  uint64_t r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "r"(w << 16), "r"(w & 0xffff0000u));
+  return r;
+}
 template <int DPL>
 __device__ __forceinline__ void unpack_bf16(const uint2& w, float (&o)[DPL]) {
   const float2 lo = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&w.x));
@@ -79,6 +106,21 @@ __device__ __forceinline__ void unpack_bf16(const uint2& w, float (&o)[DPL]) {
     o[2] = hi.x;
     o[3] = hi.y;
   }
+}
+template <int HP>
+__device__ __forceinline__ void ld_pairs(const float* p, uint64_t (&v)[HP]) {
+  if constexpr (HP == 2) {
+    const ulonglong2 t = *reinterpret_cast<const ulonglong2*>(p);
+    v[0] = t.x;
+    v[1] = t.y;
+  } else {
+    v[0] = *reinterpret_cast<const unsigned long long*>(p);
+  }
+}
+template <int HP>
+__device__ __forceinline__ void st_pairs(float* p, const uint64_t (&v)[HP]) {
+  if constexpr (HP == 2) *reinterpret_cast<ulonglong2*>(p) = make_ulonglong2(v[0], v[1]);
+  else *reinterpret_cast<unsigned long long*>(p) = v[0];
 }
 // a lane's DPL dims of a row, as raw bf16 words
 template <int DPL>
@@ -447,58 +489,70 @@ __global__ void __launch_bounds__(kLT, 1) evict_large_kernel(const EvictArgs a) 
         }
       }
     };
-    // ---- y_j' = y_j + (dk . k_j) dv, then ||v_j - mu_v - (scale / n) y_j||, 8 rows at a time
-    for (int i0 = 0; i0 < nri; i0 += kRB) {
-      const unsigned m = (s_alive[warp][i0 >> 5] >> (i0 & 31)) & 0xffu;
-      if (m == 0u) continue;  // warp-uniform
+    // ---- y_j' = y_j + (dk . k_j) dv, then ||v_j - mu_v - (scale / n) y_j||, 8
+    // rows at a time with all their loads in flight.  Rows evicted before are
+    // carried along; their scores are not posted.
+    constexpr int HP = DPL / 2;
+    uint64_t dk2[HP], dv2[HP], nmv2[HP];
+#pragma unroll
+    for (int d = 0; d < HP; ++d) {
+      dk2[d] = pair(sdk[2 * d], sdk[2 * d + 1]);
+      dv2[d] = pair(sdv[2 * d], sdv[2 * d + 1]);
+      nmv2[d] = pair(-mv[2 * d], -mv[2 * d + 1]);
+    }
+    const uint64_t nrs2 = pair(-rs, -rs);
+    auto batch = [&](int i0, auto full) {  // full: all 8 rows exist
+      constexpr bool F = decltype(full)::value;
       const size_t off = (size_t)(warp + kLW * i0) * D + lane * DPL;
+      const __nv_bfloat16 *kp = Kr + off, *vp = Vr + off;
+      float* yp = Y + off;
       uint2 kw[P], vw[P];
-      float y[P][DPL];
+      uint64_t y[P][HP];
 #pragma unroll
       for (int i = 0; i < P; ++i) {
         kw[i] = vw[i] = make_uint2(0u, 0u);
 #pragma unroll
-        for (int d = 0; d < DPL; ++d) y[i][d] = 0.f;
-        if ((m >> i) & 1u) {
-          const size_t o = off + (size_t)i * kLW * D;
-          if (e > 0) kw[i] = load_raw<DPL>(Kr + o);
-          vw[i] = load_raw<DPL>(Vr + o);
-          ld_vec<DPL>(Y + o, y[i]);
+        for (int d = 0; d < HP; ++d) y[i][d] = 0ull;
+        if (F || i0 + i < nri) {
+          if (e > 0) kw[i] = load_raw<DPL>(kp + i * kLW * D);
+          vw[i] = load_raw<DPL>(vp + i * kLW * D);
+          ld_pairs<HP>(yp + i * kLW * D, y[i]);
         }
       }
       if (e > 0) {
         float pv[P];
 #pragma unroll
         for (int i = 0; i < P; ++i) {
-          float kf[DPL];
-          unpack_bf16<DPL>(kw[i], kf);
-          pv[i] = 0.f;
-#pragma unroll
-          for (int d = 0; d < DPL; ++d) pv[i] = fmaf(sdk[d], kf[d], pv[i]);
+          uint64_t a2 = fma2(dk2[0], unpack2(kw[i].x), 0ull);
+          if constexpr (HP == 2) a2 = fma2(dk2[HP - 1], unpack2(kw[i].y), a2);
+          pv[i] = pair_sum(a2);
         }
         const float dsum = transpose_sum<P>(pv, lane);
 #pragma unroll
         for (int i = 0; i < P; ++i) {
           const float dot = __shfl_sync(kFull, dsum, i << SH);
 #pragma unroll
-          for (int d = 0; d < DPL; ++d) y[i][d] = fmaf(dot, sdv[d], y[i][d]);
-          if ((m >> i) & 1u) st_vec<DPL>(Y + off + (size_t)i * kLW * D, y[i]);
+          for (int d = 0; d < HP; ++d) y[i][d] = fma2(pair(dot, dot), dv2[d], y[i][d]);
+          if (F || i0 + i < nri) st_pairs<HP>(yp + i * kLW * D, y[i]);
         }
       }
       float ss[P];
 #pragma unroll
       for (int i = 0; i < P; ++i) {
-        float vf[DPL];
-        unpack_bf16<DPL>(vw[i], vf);
-        ss[i] = 0.f;
+        uint64_t s2 = 0ull;
 #pragma unroll
-        for (int d = 0; d < DPL; ++d) {
-          const float rr = vf[d] - mv[d] - rs * y[i][d];
-          ss[i] = fmaf(rr, rr, ss[i]);
+        for (int d = 0; d < HP; ++d) {
+          const uint64_t rr = fma2(nrs2, y[i][d], add2(unpack2(d == 0 ? vw[i].x : vw[i].y), nmv2[d]));
+          s2 = fma2(rr, rr, s2);
         }
+        ss[i] = pair_sum(s2);
       }
-      score_batch(i0, m, ss);
-    }
+      score_batch(i0, (s_alive[warp][i0 >> 5] >> (i0 & 31)) & 0xffu, ss);
+    };
+    int i0 = 0;
+#pragma unroll 1
+    for (; i0 + kRB <= nri; i0 += kRB) batch(i0, std::true_type{});
+    if (i0 < nri) batch(i0, std::false_type{});
     post_key();
     __syncthreads();
     post_mail(s_nz);
