@@ -250,16 +250,17 @@ __global__ void __launch_bounds__(kRT, 1) evict_reg_kernel(const EvictArgs a) {
   // that last changed the moments; the others (appended since) are computed
   // here: n (C k_j) on the tensor cores, C as three bf16 parts (exact to 24
   // bits), warp w taking 8 value dims, in blocks of 32 rows
-  float y[RPW][DPL];
+  constexpr int HP = DPL / 2;
+  uint64_t y[RPW][HP];  // pairs of floats
   unsigned alive = 0u;
 #pragma unroll
   for (int i = 0; i < RPW; ++i) {
     const int r = warp + kRW * i;
 #pragma unroll
-    for (int d = 0; d < DPL; ++d) y[i][d] = 0.f;
+    for (int d = 0; d < HP; ++d) y[i][d] = 0ull;
     if (r < nr) {
       alive |= 1u << i;
-      if (n > 0 && j0 + r < y_cur) ld_vec<DPL>(a.Y + (row0 + j0 + r) * D + lane * DPL, y[i]);
+      if (n > 0 && j0 + r < y_cur) ld_pairs<HP>(a.Y + (row0 + j0 + r) * D + lane * DPL, y[i]);
     }
   }
   if (n > 0 && nr > 0 && j1 > y_cur) {  // uniform over the CTA
@@ -307,7 +308,7 @@ __global__ void __launch_bounds__(kRT, 1) evict_reg_kernel(const EvictArgs a) {
 #pragma unroll
         for (int i = 2 * blk; i < 2 * blk + 2 && i < RPW; ++i) {
           const int r = warp + kRW * i;
-          if (r < nr && j0 + r >= y_cur) ld_vec<DPL>(yb + (r - rlo) * L::LDY + lane * DPL, y[i]);
+          if (r < nr && j0 + r >= y_cur) ld_pairs<HP>(yb + (r - rlo) * L::LDY + lane * DPL, y[i]);
         }
         __syncthreads();
       }
@@ -363,17 +364,25 @@ __global__ void __launch_bounds__(kRT, 1) evict_reg_kernel(const EvictArgs a) {
     for (int h = 0; h < G; ++h) ereg[h] = (i < RPW && r < nr) ? lg[h * L::R + r] : 0.f;
   }
 
-  // y_j' = y_j + (dk . k_j) dv of the warp's surviving rows
+  // y_j' = y_j + (dk . k_j) dv of the warp's rows, two elements per instruction.
+  // Rows evicted before, and those past the slice, are carried along without
+  // a test (their shared memory is this kernel's); only live rows are scored.
   auto fold_y = [&]() {
+    uint64_t dk2[HP], dv2[HP];
+#pragma unroll
+    for (int d = 0; d < HP; ++d) {
+      dk2[d] = pair(sdk[2 * d], sdk[2 * d + 1]);
+      dv2[d] = pair(sdv[2 * d], sdv[2 * d + 1]);
+    }
     float pv[P];
 #pragma unroll
     for (int i = 0; i < P; ++i) {
       pv[i] = 0.f;
-      if (i < RPW && ((alive >> i) & 1u)) {
-        float kf[DPL];
-        load_bf16<DPL>(Ks + (warp + kRW * i) * L::LDK + lane * DPL, kf);
-#pragma unroll
-        for (int d = 0; d < DPL; ++d) pv[i] = fmaf(sdk[d], kf[d], pv[i]);
+      if (i < RPW) {
+        const uint2 kw = load_raw<DPL>(Ks + (warp + kRW * i) * L::LDK + lane * DPL);
+        uint64_t a2 = fma2(dk2[0], unpack2(kw.x), 0ull);
+        if constexpr (HP == 2) a2 = fma2(dk2[HP - 1], unpack2(kw.y), a2);
+        pv[i] = pair_sum(a2);
       }
     }
     const float dsum = transpose_sum<P>(pv, lane);
@@ -381,7 +390,7 @@ __global__ void __launch_bounds__(kRT, 1) evict_reg_kernel(const EvictArgs a) {
     for (int i = 0; i < RPW; ++i) {
       const float dot = __shfl_sync(kFull, dsum, i << SH);
 #pragma unroll
-      for (int d = 0; d < DPL; ++d) y[i][d] = fmaf(dot, sdv[d], y[i][d]);
+      for (int d = 0; d < HP; ++d) y[i][d] = fma2(pair(dot, dot), dv2[d], y[i][d]);
     }
   };
   const int n_evict = len - a.budget;
@@ -458,16 +467,23 @@ __global__ void __launch_bounds__(kRT, 1) evict_reg_kernel(const EvictArgs a) {
       }
     };
     float part[P];
+    {
+      uint64_t nmv2[HP];
 #pragma unroll
-    for (int i = 0; i < P; ++i) {
-      part[i] = 0.f;
-      if (i < RPW && ((alive >> i) & 1u)) {
-        float vf[DPL];
-        load_bf16<DPL>(Vs + (warp + kRW * i) * D + lane * DPL, vf);
+      for (int d = 0; d < HP; ++d) nmv2[d] = pair(-mv[2 * d], -mv[2 * d + 1]);
+      const uint64_t nrs2 = pair(-rs, -rs);
 #pragma unroll
-        for (int d = 0; d < DPL; ++d) {
-          const float rr = vf[d] - mv[d] - rs * y[i < RPW ? i : 0][d];
-          part[i] = fmaf(rr, rr, part[i]);
+      for (int i = 0; i < P; ++i) {
+        part[i] = 0.f;
+        if (i < RPW) {
+          const uint2 vw = load_raw<DPL>(Vs + (warp + kRW * i) * D + lane * DPL);
+          uint64_t s2 = 0ull;
+#pragma unroll
+          for (int d = 0; d < HP; ++d) {
+            const uint64_t rr = fma2(nrs2, y[i < RPW ? i : 0][d], add2(unpack2(d == 0 ? vw.x : vw.y), nmv2[d]));
+            s2 = fma2(rr, rr, s2);
+          }
+          part[i] = pair_sum(s2);
         }
       }
     }
@@ -501,7 +517,7 @@ __global__ void __launch_bounds__(kRT, 1) evict_reg_kernel(const EvictArgs a) {
           float yc[DPL];
           if (!direct) {
 #pragma unroll
-            for (int d = 0; d < DPL; ++d) yc[d] = y[i < RPW ? i : 0][d];
+            for (int d = 0; d < HP; ++d) unpair(y[i < RPW ? i : 0][d], yc[2 * d], yc[2 * d + 1]);
             for (int z = 0; z < nz; ++z) {  // y'_a -= S_tilde_ab k_b for clamped (a, b)
               const int va = static_cast<int>(s_gidx[z] / D), kb = static_cast<int>(s_gidx[z] % D);
               if (va / DPL == lane) {
@@ -604,7 +620,7 @@ __global__ void __launch_bounds__(kRT, 1) evict_reg_kernel(const EvictArgs a) {
         }
         if (lane == 0) Pg[dst] = s_pos[r];
       }
-      if (has_y) st_vec<DPL>(a.Y + (row0 + dst) * D + lane * DPL, y[i]);
+      if (has_y) st_pairs<HP>(a.Y + (row0 + dst) * D + lane * DPL, y[i]);
     }
   }
   // ---- the moments back: this CTA's rows of C = S_tilde / n (each warp folded its own)

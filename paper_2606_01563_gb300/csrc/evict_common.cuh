@@ -58,6 +58,57 @@ __device__ __forceinline__ void st_vec(float* p, const float* v) {
   else *reinterpret_cast<float2*>(p) = make_float2(v[0], v[1]);
 }
 
+// A lane's DPL dims as pairs of floats, two per instruction (fma.f32x2).
+__device__ __forceinline__ uint64_t pair(float a, float b) {
+  uint64_t r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
+  return r;
+}
+__device__ __forceinline__ void unpair(uint64_t p, float& a, float& b) {
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(p));
+}
+__device__ __forceinline__ float pair_sum(uint64_t p) {
+  float a, b;
+  unpair(p, a, b);
+  return a + b;
+}
+__device__ __forceinline__ uint64_t fma2(uint64_t a, uint64_t b, uint64_t c) {
+  uint64_t r;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+  return r;
+}
+__device__ __forceinline__ uint64_t add2(uint64_t a, uint64_t b) {
+  uint64_t r;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+__device__ __forceinline__ uint64_t unpack2(uint32_t w) {  // two bf16
+  uint64_t r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "r"(w << 16), "r"(w & 0xffff0000u));
+  return r;
+}
+template <int HP>
+__device__ __forceinline__ void ld_pairs(const float* p, uint64_t (&v)[HP]) {
+  if constexpr (HP == 2) {
+    const ulonglong2 t = *reinterpret_cast<const ulonglong2*>(p);
+    v[0] = t.x;
+    v[1] = t.y;
+  } else {
+    v[0] = *reinterpret_cast<const unsigned long long*>(p);
+  }
+}
+template <int HP>
+__device__ __forceinline__ void st_pairs(float* p, const uint64_t (&v)[HP]) {
+  if constexpr (HP == 2) *reinterpret_cast<ulonglong2*>(p) = make_ulonglong2(v[0], v[1]);
+  else *reinterpret_cast<unsigned long long*>(p) = v[0];
+}
+// a lane's DPL dims of a row, as raw bf16 words
+template <int DPL>
+__device__ __forceinline__ uint2 load_raw(const __nv_bfloat16* p) {
+  if constexpr (DPL == 4) return *reinterpret_cast<const uint2*>(p);
+  else return make_uint2(*reinterpret_cast<const uint32_t*>(p), 0u);
+}
+
 // One round of a transposing butterfly: lanes with bit o set keep the upper
 // W values, the others the lower W, and each adds its partner's copy.
 template <int W>

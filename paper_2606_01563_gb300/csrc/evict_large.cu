@@ -70,32 +70,6 @@ struct LargeLayout {
   }
 };
 
-// A lane's DPL dims as pairs of floats, two per instruction (fma.f32x2).
-__device__ __forceinline__ uint64_t pair(float a, float b) {
-  uint64_t r;
-  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
-  return r;
-}
-__device__ __forceinline__ float pair_sum(uint64_t p) {
-  float a, b;
-  asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(p));
-  return a + b;
-}
-__device__ __forceinline__ uint64_t fma2(uint64_t a, uint64_t b, uint64_t c) {
-  uint64_t r;
-  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
-  return r;
-}
-__device__ __forceinline__ uint64_t add2(uint64_t a, uint64_t b) {
-  uint64_t r;
-  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
-  return r;
-}
-__device__ __forceinline__ uint64_t unpack2(uint32_t w) {  // two bf16
-  uint64_t r;
-  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "r"(w << 16), "r"(w & 0xffff0000u));
-  return r;
-}
 template <int DPL>
 __device__ __forceinline__ void unpack_bf16(const uint2& w, float (&o)[DPL]) {
   const float2 lo = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&w.x));
@@ -107,28 +81,6 @@ __device__ __forceinline__ void unpack_bf16(const uint2& w, float (&o)[DPL]) {
     o[3] = hi.y;
   }
 }
-template <int HP>
-__device__ __forceinline__ void ld_pairs(const float* p, uint64_t (&v)[HP]) {
-  if constexpr (HP == 2) {
-    const ulonglong2 t = *reinterpret_cast<const ulonglong2*>(p);
-    v[0] = t.x;
-    v[1] = t.y;
-  } else {
-    v[0] = *reinterpret_cast<const unsigned long long*>(p);
-  }
-}
-template <int HP>
-__device__ __forceinline__ void st_pairs(float* p, const uint64_t (&v)[HP]) {
-  if constexpr (HP == 2) *reinterpret_cast<ulonglong2*>(p) = make_ulonglong2(v[0], v[1]);
-  else *reinterpret_cast<unsigned long long*>(p) = v[0];
-}
-// a lane's DPL dims of a row, as raw bf16 words
-template <int DPL>
-__device__ __forceinline__ uint2 load_raw(const __nv_bfloat16* p) {
-  if constexpr (DPL == 4) return *reinterpret_cast<const uint2*>(p);
-  else return make_uint2(*reinterpret_cast<const uint32_t*>(p), 0u);
-}
-
 template <int D, int G>
 __global__ void __launch_bounds__(kLT, 1) evict_large_kernel(const EvictArgs a) {
   constexpr int NC = D / 32;   // float4 chunks per row for 8-lane row groups (logits)
