@@ -44,8 +44,8 @@ namespace {
 // mailbox beforehand).  Scores assume that no entry is clamped; when a mailbox
 // says otherwise, the lists are exchanged and the rows scored again.
 //
-// What bounds it: a chain of dependent steps, not memory: about 2 us per
-// eviction and a fixed part of a few round trips (length, rows and moments,
+// What bounds it: a chain of dependent steps, not memory: about 2.2 us per
+// further eviction (64 of 192 or 576 rows: 157, 160 us) and a fixed part of a few round trips (length, rows and moments,
 // one cluster exchange of the softmax maxima and sums, rows out).  Logits and
 // S_tilde k of rows without a kept y run on the tensor cores from the rows in
 // shared memory; survivors are written straight from there to their compacted
@@ -146,6 +146,17 @@ __global__ void __launch_bounds__(kRT, 1) evict_reg_kernel(const EvictArgs a) {
   // rows 0..y_cur-1 of the cache's y rows are current (none without them)
   const int y_cur = max(0, min(y_len_in, len_in));
 
+  // Continuous eviction: only the appended row has no y, and every CTA computes
+  // the elements of its own rows of S_tilde for it.  Computed where the row is,
+  // like a longer run of appended rows, n C k took 2.7 us of the call's 11 (all
+  // of C in one CTA): a step at 512 rows with its decode 18.4 -> 16.4 us.
+  // (the length is compared as read: nvcc 13.0.88 folded y_cur == len_in to true)
+  const bool one_fresh = n > 0 && has_new && y_len_in >= len_in;
+  const int y_have = one_fresh ? len : y_cur;  // rows from here on are computed row by row below
+  float kf_new[DPL];
+#pragma unroll
+  for (int d = 0; d < DPL; ++d) kf_new[d] = one_fresh ? __bfloat162float(kn[lane * DPL + d]) : 0.f;
+
   // ---- this slice's rows, the query, this CTA's rows of S_tilde, the means
   for (int idx = tid; idx < nr * CH; idx += kRT) {
     const int r = idx / CH, c = idx % CH;
@@ -244,6 +255,15 @@ __global__ void __launch_bounds__(kRT, 1) evict_reg_kernel(const EvictArgs a) {
     *cluster.map_shared_rank(&mail_m[rank][h], r) = m;
     *cluster.map_shared_rank(&mail_z[rank][h], r) = z;
   }
+  if (one_fresh)
+    for (int j = warp; j < SR; j += kRW) {
+      float s[DPL], dot = 0.f;
+      ld_vec<DPL>(S + (size_t)j * D + lane * DPL, s);
+#pragma unroll
+      for (int d = 0; d < DPL; ++d) dot = fmaf(s[d], kf_new[d], dot);
+      dot = warp_sum(dot);
+      if (lane == 0) *cluster.map_shared_rank(yb + a0 + j, len_in / rows_per) = dot;
+    }
   cluster_arrive_release();
 
   // ---- y_j = S_tilde k_j.  Rows below the cache's y_len carry it from the call
@@ -263,7 +283,7 @@ __global__ void __launch_bounds__(kRT, 1) evict_reg_kernel(const EvictArgs a) {
       if (n > 0 && j0 + r < y_cur) ld_pairs<HP>(a.Y + (row0 + j0 + r) * D + lane * DPL, y[i]);
     }
   }
-  if (n > 0 && nr > 0 && j1 > y_cur) {  // uniform over the CTA
+  if (n > 0 && nr > 0 && j1 > y_have) {  // uniform over the CTA
     constexpr int kHalves = kRW / NT;   // warps sharing 8 value dims: 1 at D = 128 (both 16-row halves), 2 at D = 64
     const int g = lane >> 2, t = lane & 3, nt = warp % NT, half = warp / NT;
     uint32_t b3[3][KS][2];
@@ -339,6 +359,9 @@ __global__ void __launch_bounds__(kRT, 1) evict_reg_kernel(const EvictArgs a) {
   // (Kahan) float, decremented per eviction: value zf - zc.  Every CTA
   // combines the same partials in the same order, so all hold the same values.
   cluster_wait_acquire();
+#pragma unroll
+  for (int i = 0; i < RPW; ++i)
+    if (one_fresh && warp + kRW * i == jn && jn < nr) ld_pairs<HP>(yb + lane * DPL, y[i]);
   float zf = 1.f, zc = 0.f, zinv = 1.f, Mh = 0.f;
   if (lane < G) {
     float m = -INFINITY, z = 0.f;

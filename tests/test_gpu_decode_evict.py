@@ -146,3 +146,19 @@ def test_eviction_state_several_evictions_per_step_d64():
     rng = np.random.default_rng(42)
     st = setup(rng, 2, 2, 2, 64, [40, 33, 45, 20], 48, [0, 25, 3, 7])
     run_steps(st, 2, 2, 2, 64, 24, steps=3, seed=9, evict_state=True)
+
+
+@pytest.mark.parametrize("b,H,G,D,budget,cap", [
+    (1, 2, 2, 64, 1, 4),         # one row per CTA, most of the cluster idle
+    (1, 2, 8, 64, 8, 12),        # the appended row alone in its slice
+    (1, 2, 4, 128, 1151, 1152),  # the largest capacity, 16 rows per warp
+    (3, 20, 2, 64, 90, 96),      # smaller clusters: more rows of S_tilde per CTA
+    (5, 16, 1, 128, 60, 64),
+])
+def test_appended_row_alone_without_y(b, H, G, D, budget, cap):
+    """From the second step on only the appended row has no kept y: its
+    elements come from all CTAs of the cluster to the one that holds it."""
+    rng = np.random.default_rng(70 + budget)
+    units = b * H
+    st = setup(rng, b, H, G, D, [budget] * units, cap, [0 if i == 1 else 300 for i in range(units)])
+    run_steps(st, b, H, G, D, budget, steps=3, seed=11, evict_state=True)
