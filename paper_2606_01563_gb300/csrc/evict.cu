@@ -44,12 +44,15 @@ namespace {
 // mailbox beforehand).  Scores assume that no entry is clamped; when a mailbox
 // says otherwise, the lists are exchanged and the rows scored again.
 //
-// What bounds it: a chain of dependent steps, not memory: about 2.2 us per
-// further eviction (64 of 192 or 576 rows: 157, 160 us) and a fixed part of a few round trips (length, rows and moments,
-// one cluster exchange of the softmax maxima and sums, rows out).  Logits and
-// S_tilde k of rows without a kept y run on the tensor cores from the rows in
-// shared memory; survivors are written straight from there to their compacted
-// places (every CTA has seen every evicted row, so no count is exchanged).
+// What bounds it: a chain of dependent steps, not memory: about 2 us per
+// further eviction (64 of 192 or 576 rows: 144, 147 us) and a fixed part of a
+// few round trips (length, rows and moments, one cluster exchange of the
+// softmax maxima and sums, rows out).  The block's minimum key goes through one
+// word pair per warp and warp-wide reductions: 64-bit minimum atomics on one
+// shared word made the same evictions 157 and 160 us.  Logits and S_tilde k of
+// rows without a kept y run on the tensor cores from the rows in shared memory;
+// survivors are written straight from there to their compacted places (every
+// CTA has seen every evicted row, so no count is exchanged).
 constexpr int kRegCap = 1152;  // largest capacity of this kernel
 constexpr int kRT = 512;       // threads per CTA
 constexpr int kRW = kRT / 32;  // warps per CTA
@@ -84,7 +87,7 @@ __global__ void __launch_bounds__(kRT, 1) evict_reg_kernel(const EvictArgs a) {
   __shared__ float s_mw[kRW][8], s_zw[kRW][8];          // (max, sum) of each warp's rows
   __shared__ float mail_m[kMaxCL][G], mail_z[kMaxCL][G];  // every CTA's (max, sum)
   __shared__ float mail_e[2][kMaxCL][G];                  // e_h of each CTA's candidate row
-  __shared__ unsigned long long s_best[2];
+  __shared__ uint2 s_key[kRW];  // each warp's minimum key: (row, score bits)
   __shared__ unsigned long long mail_key[2][kMaxCL];
   __shared__ int mail_nz[2][kMaxCL];
   __shared__ __align__(16) __nv_bfloat16 mail_row[2][kMaxCL][2 * D];
@@ -186,10 +189,7 @@ __global__ void __launch_bounds__(kRT, 1) evict_reg_kernel(const EvictArgs a) {
     mv[d] = n > 0 ? a.mu_v[(size_t)u * D + lane * DPL + d] : 0.f;
     sdk[d] = sdv[d] = 0.f;
   }
-  if (tid == 0) {
-    s_nz = 0;
-    s_best[0] = s_best[1] = ~0ull;
-  }
+  if (tid == 0) s_nz = 0;
   __syncthreads();
 
   // ---- logits of this CTA's rows: warp w takes rows 16 w .. 16 w + 15 against
@@ -438,7 +438,6 @@ __global__ void __launch_bounds__(kRT, 1) evict_reg_kernel(const EvictArgs a) {
         if (any) scan_row(j, s);
       }
     if (e == n_evict) break;  // uniform over the cluster
-    if (tid == 0) s_best[par ^ 1] = ~0ull;  // its readers finished one iteration ago
 
     // ---- y_j', then the residual norms of the warp's rows:
     // r_j = v_j - mu_v - (scale / n) y_j
@@ -455,29 +454,27 @@ __global__ void __launch_bounds__(kRT, 1) evict_reg_kernel(const EvictArgs a) {
       for (int i = 0; i < P; ++i) pv[i] = ss[i];
       const float sum = transpose_sum<P>(pv, lane);
       const int i = lane >> SH;
-      unsigned long long key = ~0ull;
+      unsigned hi = ~0u, lo = ~0u;  // score bits, row
       if ((lane & ((1 << SH) - 1)) == 0 && i < RPW && ((alive >> i) & 1u)) {
         float alpha = 0.f;
 #pragma unroll
         for (int h = 0; h < G; ++h) alpha = fmaf(ereg[h], invz[h], alpha);
         const float score = alpha * sqrtf(sum);
-        key = (static_cast<unsigned long long>(__float_as_uint(score)) << 32) |
-              static_cast<unsigned>(j0 + warp + kRW * i);
+        hi = __float_as_uint(score);
+        lo = static_cast<unsigned>(j0 + warp + kRW * i);
       }
-#pragma unroll
-      for (int o = 16; o >= (1 << SH); o >>= 1) {
-        const unsigned long long k2 = __shfl_xor_sync(kFull, key, o);
-        key = k2 < key ? k2 : key;
-      }
-      if (lane == 0 && key != ~0ull) atomicMin(&s_best[par], key);
+      min_key(hi, lo);
+      if (lane == 0) s_key[warp] = make_uint2(lo, hi);
     };
     // warp w < CL posts this CTA's key, candidate row and clamp count into rank w's mailbox
     auto post_mail = [&](int nz) {
       if (warp < CL) {
-        const unsigned long long b = s_best[par];
-        const int jb = (b == ~0ull) ? -1 : static_cast<int>(b & 0xffffffffu) - j0;
+        const uint2 wk = s_key[lane % kRW];
+        unsigned hi = wk.y, lo = wk.x;
+        min_key(hi, lo);
+        const int jb = (hi & lo) == ~0u ? -1 : static_cast<int>(lo) - j0;
         if (lane == 0) {
-          *cluster.map_shared_rank(&mail_key[par][rank], warp) = b;
+          *cluster.map_shared_rank(&mail_key[par][rank], warp) = (static_cast<unsigned long long>(hi) << 32) | lo;
           *cluster.map_shared_rank(&mail_nz[par][rank], warp) = nz;
         }
         if (jb >= 0 && lane < G) *cluster.map_shared_rank(&mail_e[par][rank][lane], warp) = lg[lane * L::R + jb];
@@ -530,7 +527,6 @@ __global__ void __launch_bounds__(kRT, 1) evict_reg_kernel(const EvictArgs a) {
         s_gidx[tid] = cluster.map_shared_rank(s_zidx, r)[z];
         s_gval[tid] = cluster.map_shared_rank(s_zval, r)[z];
       }
-      if (tid == 0) s_best[par] = ~0ull;
       cluster.sync();  // lists and mailboxes read, S_tilde written
 #pragma unroll
       for (int i = 0; i < P; ++i) {
@@ -582,8 +578,8 @@ __global__ void __launch_bounds__(kRT, 1) evict_reg_kernel(const EvictArgs a) {
     // differ), by two warp-wide minimum reductions (score bits, then row)
     const unsigned long long bk = (lane < CL) ? mail_key[par][lane] : ~0ull;
     const unsigned khi = static_cast<unsigned>(bk >> 32), klo = static_cast<unsigned>(bk);
-    const unsigned mhi = __reduce_min_sync(kFull, khi);
-    const unsigned mlo = __reduce_min_sync(kFull, khi == mhi ? klo : 0xffffffffu);
+    unsigned mhi = khi, mlo = klo;
+    min_key(mhi, mlo);
     const int src = __ffs(__ballot_sync(kFull, khi == mhi && klo == mlo)) - 1;
     const int js = (mhi == 0xffffffffu && mlo == 0xffffffffu) ? -1 : static_cast<int>(mlo);
     if (js < 0) {  // uniform: every rank read the same keys

@@ -8,15 +8,6 @@ namespace mkv {
 
 constexpr unsigned kFull = 0xffffffffu;
 
-__device__ __forceinline__ unsigned long long shfl_min_u64(unsigned long long v) {
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    const unsigned long long w = __shfl_xor_sync(kFull, v, o);
-    v = w < v ? w : v;
-  }
-  return v;
-}
-
 constexpr int kMaxClamp = 64;    // clamped entries corrected incrementally
 
 // Bytes of staging per unit (K and V rows, positions), padded so that every
@@ -86,6 +77,12 @@ __device__ __forceinline__ uint64_t unpack2(uint32_t w) {  // two bf16
   uint64_t r;
   asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "r"(w << 16), "r"(w & 0xffff0000u));
   return r;
+}
+// the warp's smallest (hi, lo), in every lane
+__device__ __forceinline__ void min_key(unsigned& hi, unsigned& lo) {
+  const unsigned m = __reduce_min_sync(kFull, hi);
+  lo = __reduce_min_sync(kFull, hi == m ? lo : ~0u);
+  hi = m;
 }
 template <int HP>
 __device__ __forceinline__ void ld_pairs(const float* p, uint64_t (&v)[HP]) {

@@ -95,7 +95,7 @@ __global__ void __launch_bounds__(kLT, 1) evict_large_kernel(const EvictArgs a) 
   __shared__ float s_M[G], s_Mg[G];  // this CTA's largest logit per head (read remotely), the unit's
   __shared__ double s_Z[G], s_Zg[G];
   __shared__ float mail_e[2][kMaxCL][G];  // e_h of each CTA's candidate row
-  __shared__ unsigned long long s_best[2];
+  __shared__ uint2 s_key[kLW];  // each warp's minimum key: (row, score bits)
   __shared__ unsigned long long mail_key[2][kMaxCL];
   // the mailboxes of candidate rows, and before the loop two K blocks of the set-up products
   constexpr int kMailBytes = 2 * kMaxCL * 2 * D * 2, kBlkBytes = 2 * kBlk * (D + 8) * 2;
@@ -176,10 +176,7 @@ __global__ void __launch_bounds__(kLT, 1) evict_large_kernel(const EvictArgs a) 
     Kr = Ks;
     Vr = Vs;
   }
-  if (tid == 0) {
-    s_nz = 0;
-    s_best[0] = s_best[1] = ~0ull;
-  }
+  if (tid == 0) s_nz = 0;
   for (int i = tid; i < kLW * kWords; i += kLT) {
     const int w = i / kWords, b0 = (i % kWords) * 32;  // rows w + 16 (b0 ..)
     const int have = w < nr ? (nr - w + kLW - 1) / kLW : 0;
@@ -394,7 +391,6 @@ __global__ void __launch_bounds__(kLT, 1) evict_large_kernel(const EvictArgs a) 
       scan_row();
     }
     if (e == n_evict) break;  // uniform over the cluster
-    if (tid == 0) s_best[par ^ 1] = ~0ull;  // its readers finished one iteration ago
 
     const float rs = (n > 0) ? scale / static_cast<float>(n) : 0.f;
     float invz[G];
@@ -420,16 +416,19 @@ __global__ void __launch_bounds__(kLT, 1) evict_large_kernel(const EvictArgs a) 
       }
     };
     auto post_key = [&]() {
-      const unsigned long long b = shfl_min_u64(key);
-      if (lane == 0 && b != ~0ull) atomicMin(&s_best[par], b);
+      unsigned hi = static_cast<unsigned>(key >> 32), lo = static_cast<unsigned>(key);
+      min_key(hi, lo);
+      if (lane == 0) s_key[warp] = make_uint2(lo, hi);
     };
     // warp w < CL posts this CTA's key, candidate row and clamp count into rank w's mailbox
     auto post_mail = [&](int nz) {
       if (warp < CL) {
-        const unsigned long long b = s_best[par];
-        const int jb = (b == ~0ull) ? -1 : static_cast<int>(b & 0xffffffffu) - j0;
+        const uint2 wk = s_key[lane % kLW];
+        unsigned hi = wk.y, lo = wk.x;
+        min_key(hi, lo);
+        const int jb = (hi & lo) == ~0u ? -1 : static_cast<int>(lo) - j0;
         if (lane == 0) {
-          *cluster.map_shared_rank(&mail_key[par][rank], warp) = b;
+          *cluster.map_shared_rank(&mail_key[par][rank], warp) = (static_cast<unsigned long long>(hi) << 32) | lo;
           *cluster.map_shared_rank(&mail_nz[par][rank], warp) = nz;
         }
         if (jb >= 0 && lane < G) *cluster.map_shared_rank(&mail_e[par][rank][lane], warp) = eb[(size_t)lane * es + jb];
@@ -525,7 +524,6 @@ __global__ void __launch_bounds__(kLT, 1) evict_large_kernel(const EvictArgs a) 
         s_gidx[tid] = cluster.map_shared_rank(s_zidx, r)[z];
         s_gval[tid] = cluster.map_shared_rank(s_zval, r)[z];
       }
-      if (tid == 0) s_best[par] = ~0ull;
       key = ~0ull;
       cluster.sync();  // lists and mailboxes read, S_tilde written
       for (int i0 = 0; i0 < nri; i0 += kRB) {
@@ -583,8 +581,8 @@ __global__ void __launch_bounds__(kLT, 1) evict_large_kernel(const EvictArgs a) 
     // two warp-wide minimum reductions (score bits, then row)
     const unsigned long long bk = (lane < CL) ? mail_key[par][lane] : ~0ull;
     const unsigned khi = static_cast<unsigned>(bk >> 32), klo = static_cast<unsigned>(bk);
-    const unsigned mhi = __reduce_min_sync(kFull, khi);
-    const unsigned mlo = __reduce_min_sync(kFull, khi == mhi ? klo : 0xffffffffu);
+    unsigned mhi = khi, mlo = klo;
+    min_key(mhi, mlo);
     const int src = __ffs(__ballot_sync(kFull, khi == mhi && klo == mlo)) - 1;
     const int js = (mhi == 0xffffffffu && mlo == 0xffffffffu) ? -1 : static_cast<int>(mlo);
     if (js < 0) {  // uniform: every rank read the same keys
