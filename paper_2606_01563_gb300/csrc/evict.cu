@@ -32,11 +32,13 @@ namespace {
 
 // ---------------------------------------------------------------------------
 // Register kernel: a cluster of 8, 4 or 2 CTAs of 512 threads per unit, each
-// with a contiguous slice of at most 16 RPW rows.  Warp w owns the slice rows
-// w, w + 16, ... and lane l the dims [l*DPL, (l+1)*DPL) of each, with
-// y_j = S_tilde k_j (raw co-moment form, S_tilde = n C) in registers.  The CTAs
-// share out S_tilde itself by rows, in shared memory: a fold costs a warp one
-// row or a few, and every CTA lists the clamped entries of its own rows.
+// with a contiguous slice of at most 16 RPW rows (RPW the smallest of 2, 5, 9
+// and 16 that holds a slice of the capacity: a warp computes all of its RPW
+// rows, there or not).  Warp w owns the slice rows w, w + 16, ... and lane l
+// the dims [l*DPL, (l+1)*DPL) of each, with y_j = S_tilde k_j (raw co-moment
+// form, S_tilde = n C) in registers.  The CTAs share out S_tilde itself by
+// rows, in shared memory: a fold costs a warp one row or a few, and every CTA
+// lists the clamped entries of its own rows.
 // Every thread computes the Welford fold of its own dims from the evicted row,
 // so the only barriers of an iteration are one block barrier (the block's
 // minimum key) and one cluster barrier (every CTA's key, candidate row, its
@@ -45,7 +47,8 @@ namespace {
 // says otherwise, the lists are exchanged and the rows scored again.
 //
 // What bounds it: a chain of dependent steps, not memory: about 2 us per
-// further eviction (64 of 192 or 576 rows: 144, 147 us) and a fixed part of a
+// further eviction (64 of 192, 576, 1152 rows: 117, 147, 177 us; 144 us
+// for the first with five rows per warp instead of two) and a fixed part of a
 // few round trips (length, rows and moments, one cluster exchange of the
 // softmax maxima and sums, rows out).  The block's minimum key goes through one
 // word pair per warp and warp-wide reductions: 64-bit minimum atomics on one
@@ -74,8 +77,8 @@ __global__ void __launch_bounds__(kRT, 1) evict_reg_kernel(const EvictArgs a) {
   using L = RegLayout<D, G, RPW>;
   constexpr int DPL = D / 32;  // dims per lane
   constexpr int KS = D / 16, NT = D / 8, CH = D / 8;
-  constexpr int P = RPW <= 8 ? 8 : 16;  // padded row count of the transposing sums
-  constexpr int SH = P == 8 ? 2 : 1;    // lane l scores row l >> SH
+  constexpr int P = RPW <= 2 ? 2 : RPW <= 8 ? 8 : 16;  // padded row count of the transposing sums
+  constexpr int SH = P == 2 ? 4 : P == 8 ? 2 : 1;      // lane l scores row l >> SH
   extern __shared__ __align__(16) uint8_t dsmem[];
   __nv_bfloat16* Ks = reinterpret_cast<__nv_bfloat16*>(dsmem + L::K);  // [R][LDK]
   __nv_bfloat16* Vs = reinterpret_cast<__nv_bfloat16*>(dsmem + L::V);  // [R][D]
@@ -723,12 +726,14 @@ cudaError_t launch_reg(const EvictArgs& a, int cl, cudaStream_t stream) {
 template <int D, int G>
 cudaError_t launch_rows(const EvictArgs& a, int cl, cudaStream_t stream) {
   const int slice = (a.cap + cl - 1) / cl;  // rows of one CTA's slice at most
+  if (slice <= kRW * 2) return launch_reg<D, G, 2>(a, cl, stream);
   if (slice <= kRW * 5) return launch_reg<D, G, 5>(a, cl, stream);
   if (slice <= kRW * 9) return launch_reg<D, G, 9>(a, cl, stream);
   return launch_reg<D, G, 16>(a, cl, stream);
 }
 template <int D, int G>
 int active_rows(int slice, int cl) {
+  if (slice <= kRW * 2) return active_clusters<D, G, 2>(cl);
   if (slice <= kRW * 5) return active_clusters<D, G, 5>(cl);
   if (slice <= kRW * 9) return active_clusters<D, G, 9>(cl);
   return active_clusters<D, G, 16>(cl);

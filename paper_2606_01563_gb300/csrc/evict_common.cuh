@@ -119,18 +119,21 @@ __device__ __forceinline__ void tsum_round(float* v, int lane, int o) {
   }
 }
 
-// Warp sums of P (8 or 16) values per lane in P - 1 + 5 - log2(P) shuffles:
+// Warp sums of P (2, 8 or 16) values per lane in P - 1 + 5 - log2(P) shuffles:
 // returns, in every lane, the sum over the warp of v[lane >> (5 - log2 P)].
 template <int P>
 __device__ __forceinline__ float transpose_sum(float (&v)[P], int lane) {
-  static_assert(P == 8 || P == 16, "8 or 16 values");
+  static_assert(P == 2 || P == 8 || P == 16, "2, 8 or 16 values");
   if constexpr (P == 16) tsum_round<8>(v, lane, 16);
-  tsum_round<4>(v, lane, P == 16 ? 8 : 16);
-  tsum_round<2>(v, lane, P == 16 ? 4 : 8);
-  tsum_round<1>(v, lane, P == 16 ? 2 : 4);
+  if constexpr (P >= 8) {
+    tsum_round<4>(v, lane, P == 16 ? 8 : 16);
+    tsum_round<2>(v, lane, P == 16 ? 4 : 8);
+  }
+  constexpr int kLast = 32 / P;
+  tsum_round<1>(v, lane, kLast);
   float r = v[0];
 #pragma unroll
-  for (int o = (P == 16 ? 1 : 2); o >= 1; o >>= 1) r += __shfl_xor_sync(kFull, r, o);
+  for (int o = kLast / 2; o >= 1; o >>= 1) r += __shfl_xor_sync(kFull, r, o);
   return r;
 }
 

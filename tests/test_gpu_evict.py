@@ -174,6 +174,20 @@ def test_evict_large_slices(units, G, D, cap, evict, tau):
     check(gpu, st)
 
 
+@pytest.mark.parametrize("G,D,cap,tau", [
+    (4, 128, 256, 1e-6),  # the largest slice of two rows per warp
+    (4, 128, 257, 1e-6),  # one row more: five rows per warp
+    (1, 64, 250, 0.05),   # clamped entries with two rows per warp
+    (8, 128, 129, 0.5),   # the direct clamped product
+])
+def test_evict_small_slices(G, D, cap, tau):
+    """Capacities around 8 slices of 32 rows, full caches, several evictions."""
+    rng = np.random.default_rng(83 + cap)
+    st = setup(rng, 1, 2, G, D, [cap - 1, cap - 6], cap, [200, 90])
+    gpu = run_case(st, 1, 2, G, D, cap - 12, True, tau=tau)
+    check(gpu, st)
+
+
 def test_evict_many_units():
     """24 units at capacity 200: three waves of 8-CTA clusters of the register
     kernel (5 rows per warp)."""
