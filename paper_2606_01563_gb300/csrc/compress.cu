@@ -291,7 +291,8 @@ struct TcArgs {
 // memory (in the same warps the two cost 32 us of 125 at 32K, batch 4); with
 // up to 128 window rows three stages are in flight and the logits
 // double-buffered.  V streams through L2, so that more of K is still there for
-// the scores, which start from the end of the chunk.
+// the scores, which start from the end of the chunk.  Alone at 32K, 32 units:
+// 115 us, 4.7 TB/s on 128 CTAs, one per SM; at 8K 17 us (21 before).
 constexpr int kStatThreads = 64 + 256 + 128;
 __global__ void __launch_bounds__(kStatThreads, 1)
     stats_tc(const TcArgs p, const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtensorMap tmV,
@@ -586,7 +587,8 @@ __global__ void __launch_bounds__(kStatThreads, 1)
 // groups (rows 0..127 and the others).  Bounded by the read of K, whose rate
 // follows the bytes in flight (four stages: 4.5 TB/s with no epilogue at all),
 // so shared memory goes to stages; from the chunk's end, where L2 still holds
-// what stats_tc read last.
+// what stats_tc read last.  Alone from a cold L2: 60 us at 32K, 32 units (4.5
+// TB/s); 85 us at 128K with 256 window rows, where the exponentials bound it.
 constexpr int kScoreThreads = 64 + 4 * 128;
 __global__ void __launch_bounds__(kScoreThreads, 1)
     scores_tc(const TcArgs p, const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtensorMap tmQ) {
@@ -776,8 +778,8 @@ __global__ void __launch_bounds__(kScoreThreads, 1)
 // compares its positions' scores and norms against theta, gathers the rows
 // that remain (a few times the budget where C0' is small beside the values)
 // and computes score2 of those; the others get 0, which the k higher ones keep
-// out.  Reading K and V a second time is what the full pass costs: 128 us at
-// 32K, batch 4, against about 10 for the gathered rows.  When more than half
+// out.  Reading K and V a second time is what the full pass costs: alone at
+// 32K, batch 4 (32 units) it takes 143 us, the bounded one 22.  When more than half
 // of a CTA's positions remain, or the caller wants score2 itself, the full
 // pass runs; a position's score2 is the same bits either way.
 __global__ void __launch_bounds__(kResThreads, 1)
@@ -1062,7 +1064,8 @@ __global__ void __launch_bounds__(kResThreads, 1)
 // from one scan.  The keys of that bin (about a sixth of k) are exchanged and
 // ranked by counting, which gives the last selected pair; one more pass counts
 // and one writes.  Two cluster barriers, where a radix select over the keys
-// took four passes of three barriers each.  A unit's contested keys are
+// took four passes of three barriers each: alone at 32K, 32 units, 13.5 us
+// against 24.5 (with the rows' gather, now rset's), at 128K 20 against 35.  A unit's contested keys are
 // exchanged over its cluster; the pairs of a batch item through global memory
 // (contest_kernel), so that a joint selection too has kSelCL CTAs per unit.
 // When there are more contested keys than the lists hold (many equal scores),
@@ -1390,7 +1393,10 @@ __global__ void __launch_bounds__(256) diag_joint_kernel(const SelectArgs a) {
 // 64 kh + 64); the CL partial sums meet through distributed shared memory,
 // each rank finishing 128 / CL value dims, four elements of C per thread.  A
 // chain of round trips (list, rows, MMA, exchange) over code that runs once:
-// its time is latency and instruction fetch, so the loops stay rolled.
+// its time is latency and instruction fetch, so the loops stay rolled.  Alone
+// at 32K, 32 units, it takes 25 us, what a second pass of stats_tc over gathered
+// rows (13.5) and a merge kernel (11.5) took before; but its merge runs while
+// the selection does, and the gathered copies are gone.
 //
 // The all-token co-moment is the multi-way Chan merge of the chunk records,
 // taken about the first chunk's means x0 so that no global mean is needed first:
