@@ -47,7 +47,7 @@ namespace {
 // says otherwise, the lists are exchanged and the rows scored again.
 //
 // What bounds it: a chain of dependent steps, not memory: about 2 us per
-// further eviction (64 of 192, 576, 1152 rows: 117, 147, 177 us; 144 us
+// further eviction (64 of 192, 576, 1152 rows: 119, 147, 177 us; 144 us
 // for the first with five rows per warp instead of two) and a fixed part of a
 // few round trips (length, rows and moments, one cluster exchange of the
 // softmax maxima and sums, rows out).  The block's minimum key goes through one
