@@ -1238,7 +1238,9 @@ __global__ void __cluster_dims__(kSelCL, 1, 1) __launch_bounds__(kSelThreads, 2)
     s_last = ~0ull;
   }
   __syncthreads();
-  cluster_arrive_relaxed();  // every CTA has started: awaited before the first remote store
+  // every CTA has started, its s_last initialised (release: another CTA may
+  // overwrite it): awaited before the first remote store
+  cluster_arrive_release();
   grid_dependency_wait();
   grid_launch_dependents();
 

@@ -97,3 +97,20 @@ def test_equal_scores_take_the_lowest_positions(T, B, adaptive, pool):
     for h in range(H):
         got = out["pos"][0, h, :int(out["len"][0, h])].cpu().numpy()
         np.testing.assert_array_equal(got, want[h])
+
+
+def test_joint_selection_of_many_groups():
+    """The last selected pair of a joint selection is found by one CTA of each
+    cluster and stored into the others, over the value they start with: 40
+    groups of 8 clusters, more than run at once, five times over."""
+    b, H, G, D, T, B, w = 40, 8, 1, 64, 640, 48, 16
+    K, V, Q = draw(17, b, H, G, D, T, w, "plain")
+    t = np.arange(T)
+    prot = np.stack([(t < 1) | (t >= T - w)] * H)
+    for _ in range(5):
+        out = compress(b, H, G, D, T, B, w, K, V, Q, 1, True, mi=0)
+        s, ln, pos = out["s"].double().cpu().numpy(), out["len"].cpu().numpy(), out["pos"].cpu().numpy()
+        for i in range(b):
+            want, _ = O.select_topk_joint(s[i], H * (B - 1 - w), prot)
+            for h in range(H):
+                np.testing.assert_array_equal(pos[i, h, :ln[i, h]], want[h])
