@@ -197,6 +197,7 @@ mkv_status mkv_decode_evict_step(mkv_geom geom, const void* q, const void* k_new
   e.y_len = cache->y_len;
   e.budget = budget;
   e.tau = p->tau;
+  e.release = 1;
   e.batch = geom.batch;
   e.n_kv = geom.n_kv_heads;
   evict_carve(e, geom, cache->capacity, workspace);

@@ -21,7 +21,7 @@
 //                            into the caller's mkv_moments
 // Every launch is a programmatic dependent of the one before it: a kernel's
 // set-up, and what it reads of the prompt or of launches further back, run
-// while its predecessor drains.
+// while its predecessor drains.  The last releases no launch after the call.
 //
 // With the budget shared by the KV heads of a batch item (adaptive), each
 // select ranks the (head, position) pairs of the batch item together.
@@ -1525,7 +1525,9 @@ __global__ void __launch_bounds__(2048 / CL) rset_kernel(const RsetArgs a) {
   if (tid < 2048 / 16)  // the ones operand of the column sums
     reinterpret_cast<uint4*>(sOnes)[tid] = make_uint4(0x3F803F80u, 0x3F803F80u, 0x3F803F80u, 0x3F803F80u);
   grid_dependency_wait();
-  grid_launch_dependents();
+  // The call's last kernel releases nothing early: a decode step with
+  // early_load reads the cache and the moments before its own wait.
+  if constexpr (!FINAL) grid_launch_dependents();
 
   // ---- row tiles
   const int cnt = L.hs == 1 ? L.B : L.cnt[u];

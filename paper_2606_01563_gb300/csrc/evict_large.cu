@@ -114,10 +114,11 @@ __global__ void __launch_bounds__(kLT, 1) evict_large_kernel(const EvictArgs a) 
     return reinterpret_cast<__nv_bfloat16*>(s_rows) + ((size_t)par * kMaxCL + r) * 2 * D;
   };
 
-  // The next kernel in the stream may be placed on free SMs while this one
-  // runs (it waits for this one's end); not before this one's own wait.
+  // In mkv_decode_evict_step the decode kernel may be placed on free SMs while
+  // this one runs: it waits before it reads.  After mkv_evict_append the next
+  // launch may be a decode step with early_load, which does not.
   grid_dependency_wait();
-  grid_launch_dependents();
+  if (a.release) grid_launch_dependents();
   cg::cluster_group cluster = cg::this_cluster();
   const int rank = static_cast<int>(cluster.block_rank()), CL = static_cast<int>(cluster.num_blocks());
   const int u = blockIdx.x / CL;

@@ -82,6 +82,7 @@ struct EvictArgs {
   float* Y;          // optional fp32 [units][cap][D]: y_j = S_tilde k_j of each row (mkv_cache.y)
   int32_t* y_len;    // optional [units]: rows 0..y_len-1 of Y are current (mkv_cache.y_len)
   int32_t rows_max;  // large kernel: rows per CTA slice = ceil(cap / CTAs per unit)
+  int32_t release;   // the next launch waits before it reads the cache: it may be placed early
   int32_t batch;
   int32_t n_kv;
 };
