@@ -749,6 +749,9 @@ __global__ void __launch_bounds__(kScoreThreads, 1)
       tc_fence_before();
       __syncwarp();
       if (lane == 0) mbar_arrive(&lempty[b]);
+      // rows past the unit's end hold zeros: without the causal mask their
+      // logits of 0 would add to the last chunk
+      if (t >= t_end) acc = 0.f;
       for (int o = 1; o < p.pool; o <<= 1) acc += __shfl_xor_sync(kFull, acc, o);  // aligned chunks
       if (t < t_end) {
         p.s_out[(size_t)u * p.T + t] = acc;

@@ -14,7 +14,7 @@ import torch
 
 import oracle as O
 from paper_2606_01563_gb300 import mkv
-from paper_2606_01563_gb300.inputs import WORKLOADS, Generator, Geometry, Workload
+from paper_2606_01563_gb300.inputs import WORKLOADS, Generator, Geometry, Workload, bf16_round
 from gpu_util import assert_moment_close, bf16, host
 from parity import check_compress_item_adaptive, check_compress_unit, evicted_moments
 
@@ -80,6 +80,28 @@ def test_batch_and_d128_ragged():
 
 def test_llama_layer_full_size():
     run(WORKLOADS["llama8b_layer_t8k"])
+
+
+@pytest.mark.parametrize("pool,G,w,T", [(4, 2, 16, 1001), (32, 2, 16, 1030), (32, 4, 64, 1003), (8, 1, 8, 129)])
+def test_partial_last_chunk_without_causal_mask(pool, G, w, T):
+    """A last chunk of fewer than `pool` positions: the tile's rows past T add
+    nothing to it (with the causal mask no window row sees them anyway)."""
+    H, D, B = 2, 64, 60
+    rng = np.random.default_rng(T)
+    K, V = bf16_round(rng.standard_normal((1, H, T, D))), bf16_round(rng.standard_normal((1, H, T, D)))
+    Q = bf16_round(rng.standard_normal((1, H, G, w, D)))
+    g = mkv.geom(1, H, G, D)
+    p = mkv.mkv_compress_params(B, w, 0, 0, pool, 0, 0, 1e-6)
+    cache, mom = mkv.alloc_cache(g, B), mkv.alloc_moments(g)
+    ws = mkv.alloc_workspace(mkv.mkv_compress_workspace_size(g, T, p))
+    s = torch.zeros(1, H, T, device="cuda")
+    mkv.mkv_compress(g, T, bf16(K), bf16(V), bf16(Q), p, cache, mom, ws, diag=(s, None, None))
+    assert mkv.mkv_get_device_error(ws)[0] == 0
+    for h in range(H):
+        ref = O.pool_scores(O.window_scores(Q[0, h], K[0, h], causal=False), pool)
+        np.testing.assert_allclose(host(s)[0, h], ref, rtol=2e-5, atol=2e-6 * ref.max())
+        want = O.select_topk(host(s)[0, h].astype(np.float64), B, np.zeros(T, bool))[0]
+        np.testing.assert_array_equal(host(cache.pos)[0, h], want)
 
 
 # ------------------------------------------------------- adaptive budget
@@ -209,7 +231,6 @@ def test_adaptive_head_with_no_retained_rows():
     point at two of its keys, head 1's keys are near zero (flat attention), so
     the joint top 2 are both head 0's and head 1 keeps nothing (len 0; its
     moments cover all T rows)."""
-    from paper_2606_01563_gb300.inputs import bf16_round
     rng = np.random.default_rng(41)
     T, d, g_, w = 256, 64, 2, 8
     K = np.empty((1, 2, T, d))
