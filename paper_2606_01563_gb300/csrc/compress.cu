@@ -1399,8 +1399,10 @@ __global__ void __launch_bounds__(256) diag_joint_kernel(const SelectArgs a) {
 // ------------------------------------------------------------------- rset
 // Moments of E = all \ R for the rows R a selection kept, in one kernel per
 // stage: the rows are gathered by their list straight into the tensor-core
-// operand layout (no dense copy of them), V^T K of them accumulates in TMEM,
-// and the epilogue takes their centred co-moment out of the all-token set's.
+// operand layout (no dense copy of them), V^T K of a 128-row tile forms in
+// TMEM, the tile's co-moment is centred as it is read from there and added to
+// the CTA's earlier ones, and the epilogue takes the sum out of the all-token
+// set's co-moment.
 // The first stage writes C0' as the residual pass's operand image, the final
 // one the caller's moments and, from the same tiles, the retained cache.
 //
@@ -1421,10 +1423,17 @@ __global__ void __launch_bounds__(256) diag_joint_kernel(const SelectArgs a) {
 // It is merged before the dependency wait, while the selection runs: the
 // records are stats_tc's, complete before the selection's predecessor (which
 // the selection has waited for when this kernel may start) began.
-// R's centred record is then removed with the reverse pairwise formula.
+// R's tiles and ranks are merged about the same x0, and R's centred record is
+// then removed with the reverse pairwise formula.  The centring tile by tile
+// matters where channels have means of several standard deviations: taken out
+// once over all of R (4096 of 8192 rows, means of 10 and 4), it left C 25 times
+// as far from 64 bits as fp32 sums need.
 constexpr int kFinCH = 32;      // chunk records staged per pass
 constexpr int kRsRed = 64 + 4;  // row stride of a CTA's partial sums (floats)
-constexpr size_t kRsSmem = 1024 + kBoxBytes + kTileBytes + 2048;  // one K half, one V tile, ones
+constexpr int kRsOperands = kBoxBytes + kTileBytes + 2048;  // one K half, one V tile, ones
+constexpr size_t rset_smem(bool several) {
+  return 1024 + kRsOperands + (several ? (size_t)kDP * kRsRed * 4 : 0);
+}
 
 struct RsetArgs {
   Layout L;
@@ -1438,10 +1447,11 @@ struct RsetArgs {
   mkv_moments mom;
   void* ws;
   uint32_t polls;
+  int several;  // a CTA may have more than one row tile
 };
 
 template <int CL, bool FINAL>
-__global__ void __launch_bounds__(2048 / CL) rset_kernel(const RsetArgs a) {
+__global__ void __launch_bounds__(2048 / CL, CL == 2 ? 1 : 2) rset_kernel(const RsetArgs a) {
   constexpr int kThr = 2048 / CL;
   constexpr int RW = kDP / CL;  // value dims a rank finishes
   extern __shared__ __align__(1024) uint8_t smraw[];
@@ -1449,12 +1459,14 @@ __global__ void __launch_bounds__(2048 / CL) rset_kernel(const RsetArgs a) {
   uint8_t* sK = sm;                               // [128 rows][64 key dims]
   uint8_t* sV = sm + kBoxBytes;                   // [2 boxes][128 rows][64 value dims]
   uint8_t* sOnes = sm + kBoxBytes + kTileBytes;   // [16 rows][128 B] of bf16 1.0
-  float* red = reinterpret_cast<float*>(sm);      // [128][kRsRed] this CTA's V^T K (after the tiles)
+  // [128][kRsRed] this CTA's V^T K about x0: over the operands of its only tile, or past them
+  float* red = reinterpret_cast<float*>(sm + (a.several ? kRsOperands : 0));
   __shared__ __align__(8) uint64_t done;
   __shared__ uint32_t tmem_base;
   __shared__ int s_ok;
   __shared__ int s_t[kTok];                              // positions of a tile's rows, -1 past the unit's rows
-  __shared__ __align__(16) float s_sk[kDP], s_sv[kDP];  // this CTA's column sums (read remotely)
+  __shared__ __align__(16) float s_sk[64], s_sv[kDP];  // this CTA's column sums about x0 (read remotely)
+  __shared__ __align__(16) float s_x0k[64], s_tk[64];   // x0 of the key half, and a tile's sums of K
   const Layout& L = a.L;
   const int D = L.D, T = L.T;
   const int rank = blockIdx.x % CL, kh = blockIdx.x / CL, u = blockIdx.y;
@@ -1499,6 +1511,7 @@ __global__ void __launch_bounds__(2048 / CL) rset_kernel(const RsetArgs a) {
 #pragma unroll
         for (int j = 0; j < 4; ++j) x0k[j] = s_mk[cq * 4 + j];
         x0v = s_mv[tid / 16];
+        if (tid < 64) s_x0k[tid] = s_mk[tid];
       }
       const float* m = recs + (size_t)g0 * rf + 4 + 2 * D + (size_t)min(row, D - 1) * D + kh * 64 + cq * 4;
 #pragma unroll 4
@@ -1539,19 +1552,17 @@ __global__ void __launch_bounds__(2048 / CL) rset_kernel(const RsetArgs a) {
   const __nv_bfloat16* Ku = a.K + (size_t)u * T * D + kh * 64;
   const __nv_bfloat16* Vu = a.V + (size_t)u * T * D;
   const int vch = D / 8;  // 16-byte chunks of a value row
+  // this thread's TMEM lane (a value dim) and its part of the 64 key columns
+  constexpr int kCols = 64 * 128 / kThr;
+  const int vrow = (warp & 3) * 32 + lane, c_lo = (warp >> 2) * kCols;
+  const uint32_t tm_lane = static_cast<uint32_t>((warp & 3) * 32) << 16;
+  const float x0row = vrow < D ? recs[4 + D + vrow] : 0.f;  // x0 of that dim
+  float rv_lane = 0.f, rk_lane = 0.f;  // R's sums about x0: of value dim vrow, of key dim tid (tid < 64)
+  float* my_red = red + vrow * kRsRed;
   int it = 0;
   bool ok = true;
 #pragma unroll 1
   for (int ti = rank; ti < n_tiles; ti += CL, ++it) {
-    if (it > 0) {  // the operands are free once their MMAs have completed
-      if (tid == 0 && !mbar_wait(&done, (it - 1) & 1, a.polls)) {
-        s_ok = 0;
-        record_error(a.ws, MKV_ERR_TIMEOUT, u);
-      }
-      __syncthreads();
-      ok = s_ok != 0;
-      if (!ok) break;  // uniform: s_ok changes only before a barrier
-    }
     const int r0 = ti * kTok;
     if (tid < kTok)  // never outside the unit's slab
       s_t[tid] = r0 + tid < cnt ? min(max(lst[r0 + tid], 0), T - 1) : -1;
@@ -1581,7 +1592,7 @@ __global__ void __launch_bounds__(2048 / CL) rset_kernel(const RsetArgs a) {
       for (int kk = 0; kk < 8; ++kk) {
         const uint64_t dk = sdesc_sw128(aK + kk * 2048, kBoxBytes, 1024), dv = sdesc_sw128(aV + kk * 2048, kBoxBytes, 1024);
         const uint64_t d1 = sdesc_sw128(a1 + (kk & 3) * 32, 16, 1024);
-        const uint32_t acc = (it > 0 || kk > 0) ? 1u : 0u;
+        const uint32_t acc = kk > 0 ? 1u : 0u;
         umma_bf16(tm, dv, dk, id, acc);
         umma_bf16(tm + 64, dk, d1, id1, acc);
         umma_bf16(tm + 80, dv, d1, id1, acc);
@@ -1603,43 +1614,50 @@ __global__ void __launch_bounds__(2048 / CL) rset_kernel(const RsetArgs a) {
       }
       if (kh == 0 && tid < kTok && r0 + tid < cnt) a.dst_pos[(size_t)u * a.dst_cap + r0 + tid] = s_t[tid];
     }
-  }
-  // ---- this CTA's sums and V^T K into shared memory
-  if (it > 0 && ok) {
-    if (tid == 0 && !mbar_wait(&done, (it - 1) & 1, a.polls)) {
+    if (tid == 0 && !mbar_wait(&done, it & 1, a.polls)) {
       s_ok = 0;
       record_error(a.ws, MKV_ERR_TIMEOUT, u);
     }
     __syncthreads();
     ok = s_ok != 0;
-  }
-  if (!ok && tid == 0) (void)mbar_wait(&done, (it - 1) & 1);  // drain: the MMAs still read shared memory
-  __syncthreads();
-  if (warp < 4) {
+    if (!ok) {  // uniform: s_ok changes only before a barrier
+      if (tid == 0) (void)mbar_wait(&done, it & 1);  // drain: the MMAs still read shared memory
+      break;
+    }
+    // ---- the tile's means, then its co-moment about x0 onto the tiles before
     tc_fence_after();
-    const uint32_t tm = tmem_base + (static_cast<uint32_t>(warp * 32) << 16);
-    const int r = warp * 32 + lane;
-    const bool have = it > 0 && ok;
-    float x[32];
-#pragma unroll 1
-    for (int c0 = 0; c0 < 96; c0 += 32) {
-      if (have) {
-        tmem_ld32(tm + c0, x);
-      } else {
+    const float nt = static_cast<float>(min(kTok, cnt - r0));
+    if (warp < 2) {  // lanes 64.. hold sums of V's first box: not read
+      const float tk = tmem_ld1(tmem_base + tm_lane + 64);
+      s_tk[tid] = tk;
+      rk_lane += fmaf(-nt, s_x0k[tid], tk);
+    }
+    const float tv = tmem_ld1(tmem_base + tm_lane + 80);
+    rv_lane += fmaf(-nt, x0row, tv);
+    float x[kCols];
+    tmem_ld<kCols>(tmem_base + tm_lane + c_lo, x);
+    __syncthreads();
+    const float inv = 1.f / nt, mv = tv / nt, w = nt * (mv - x0row);
 #pragma unroll
-        for (int j = 0; j < 32; ++j) x[j] = 0.f;
-      }
-      if (c0 < 64) {
-#pragma unroll
-        for (int j = 0; j < 32; j += 4)
-          *reinterpret_cast<float4*>(red + r * kRsRed + c0 + j) = make_float4(x[j], x[j + 1], x[j + 2], x[j + 3]);
-      } else {
-        s_sk[r] = x[0];  // lanes 64.. hold sums of V's first box: not read
-        s_sv[r] = x[16];
-      }
+    for (int j = 0; j < kCols; j += 4) {
+      const float4 tk = *reinterpret_cast<const float4*>(s_tk + c_lo + j);
+      const float4 xk = *reinterpret_cast<const float4*>(s_x0k + c_lo + j);
+      float4* to = reinterpret_cast<float4*>(my_red + c_lo + j);
+      float4 y = it > 0 ? *to : make_float4(0.f, 0.f, 0.f, 0.f);
+      y.x += fmaf(w, fmaf(tk.x, inv, -xk.x), fmaf(-mv, tk.x, x[j]));
+      y.y += fmaf(w, fmaf(tk.y, inv, -xk.y), fmaf(-mv, tk.y, x[j + 1]));
+      y.z += fmaf(w, fmaf(tk.z, inv, -xk.z), fmaf(-mv, tk.z, x[j + 2]));
+      y.w += fmaf(w, fmaf(tk.w, inv, -xk.w), fmaf(-mv, tk.w, x[j + 3]));
+      *to = y;
     }
     tc_fence_before();
   }
+  if (it == 0 || !ok) {
+    __syncthreads();  // what the operands' set-up wrote there
+    for (int c = c_lo; c < c_lo + kCols; c += 4) *reinterpret_cast<float4*>(my_red + c) = make_float4(0.f, 0.f, 0.f, 0.f);
+  }
+  if (tid < 64) s_sk[tid] = ok ? rk_lane : 0.f;
+  if (tid < kDP) s_sv[tid] = ok ? rv_lane : 0.f;
   cg::cluster_group cluster = cg::this_cluster();
   cluster.sync();
   if (warp == 0) {
@@ -1665,17 +1683,20 @@ __global__ void __launch_bounds__(2048 / CL) rset_kernel(const RsetArgs a) {
     SR[3] += s4.w;
   }
   const float nE = n - nR;
-  const float mv = x0v + sv / n, mvR = nR > 0.f ? rv / nR : 0.f, mvE = nE > 0.f ? (n * mv - nR * mvR) / nE : 0.f;
+  // means of R and E about x0
+  const float dvR = nR > 0.f ? rv / nR : 0.f, dvE = nE > 0.f ? (sv - rv) / nE : 0.f;
+  const float mvE = nE > 0.f ? x0v + dvE : 0.f;
   float CE[4], mkE[4];
 #pragma unroll
   for (int j = 0; j < 4; ++j) {
-    const float mk = x0k[j] + sk[j] / n, mkR = nR > 0.f ? rk[j] / nR : 0.f;
+    const float dkR = nR > 0.f ? rk[j] / nR : 0.f;
     CE[j] = mkE[j] = 0.f;
     if (nE > 0.f) {
-      mkE[j] = (n * mk - nR * mkR) / nE;
+      const float dkE = (sk[j] - rk[j]) / nE;
+      mkE[j] = x0k[j] + dkE;
       const float Mall = M[j] - sv * sk[j] / n;
       const float MR = nR > 0.f ? SR[j] - rv * rk[j] / nR : 0.f;
-      const float ME = Mall - MR - (nE * nR / n) * (mvR - mvE) * (mkR - mkE[j]);
+      const float ME = Mall - MR - (nE * nR / n) * (dvR - dvE) * (dkR - dkE);
       CE[j] = ME / nE;
     }
   }
@@ -1789,11 +1810,12 @@ int rset_cluster(const Layout& L, int num_sms) {
 }
 
 template <bool FINAL>
-cudaError_t launch_rset(const RsetArgs& a, int cl, cudaStream_t st) {
+cudaError_t launch_rset(RsetArgs a, int cl, cudaStream_t st) {
   const dim3 grid(cl * (a.L.D / 64), a.L.units);
+  a.several = a.L.lsel > cl * kTok ? 1 : 0;
   auto go = [&](void (*f)(RsetArgs)) -> cudaError_t {
-    const cudaError_t e = smem_attr(reinterpret_cast<const void*>(f), kRsSmem);
-    return e != cudaSuccess ? e : launch_pdl(f, grid, 2048 / cl, kRsSmem, st, cl, a);
+    const cudaError_t e = smem_attr(reinterpret_cast<const void*>(f), rset_smem(true));
+    return e != cudaSuccess ? e : launch_pdl(f, grid, 2048 / cl, rset_smem(a.several != 0), st, cl, a);
   };
   switch (cl) {
     case 8: return go(rset_kernel<8, FINAL>);

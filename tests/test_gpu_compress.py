@@ -104,6 +104,66 @@ def test_partial_last_chunk_without_causal_mask(pool, G, w, T):
         np.testing.assert_array_equal(host(cache.pos)[0, h], want)
 
 
+def tile_centred_moments(K, V, x0k, x0v):
+    """(n, sums, co-moment about (x0k, x0v)) of rows in fp32: every 128-row tile
+    centred about its own means, tiles merged about the common reference."""
+    f = np.float32
+    n, sk, sv = 0, np.zeros(K.shape[1], f), np.zeros(V.shape[1], f)
+    M = np.zeros((V.shape[1], K.shape[1]), f)
+    for i in range(0, len(K), 128):
+        k, v = K[i:i + 128].astype(f), V[i:i + 128].astype(f)
+        m = f(len(k))
+        ck, cv = k.sum(0, dtype=f), v.sum(0, dtype=f)
+        dk, dv = ck / m - x0k, cv / m - x0v
+        M += (v.T @ k - np.outer(cv / m, ck)) + m * np.outer(dv, dk)
+        n, sk, sv = n + len(k), sk + m * dk, sv + m * dv
+    return f(n), sk, sv, M
+
+
+@pytest.mark.parametrize("H,D,T,B,ok,ov", [
+    (1, 128, 8192, 4096, 10.0, 4.0),  # half of the prompt retained: four tiles per CTA
+    (8, 128, 2400, 2000, 4.0, 1.0),   # nearly all of it, a ragged last tile
+    (2, 64, 3000, 1500, 6.0, 6.0),
+    (1, 128, 2048, 300, 10.0, 4.0),   # fewer tiles than CTAs
+])
+def test_moments_of_keys_and_values_far_from_zero(H, D, T, B, ok, ov):
+    """Channels with means of several standard deviations: the error of C
+    against 64 bits stays within four times what the same rows give in fp32
+    with every 128-row tile centred before the merge.  Four: the tensor core's
+    sums drop bits where the reference rounds (twice the error, and of one
+    sign), and the order of the sums is another (sums centred once over all
+    rows gave 4.5 times at 1500 rows and 25 times at 4096)."""
+    rng = np.random.default_rng(D + B)
+    w, f = 32, np.float32
+    K = bf16_round(rng.standard_normal((1, H, T, D)) + ok * rng.standard_normal((1, H, 1, D)))
+    V = bf16_round(rng.standard_normal((1, H, T, D)) + ov * rng.standard_normal((1, H, 1, D)))
+    Q = bf16_round(0.3 * rng.standard_normal((1, H, 1, w, D)))
+    g = mkv.geom(1, H, 1, D)
+    p = mkv.mkv_compress_params(B, w, 1, 1, 1, 1, 1, 1e-6)
+    cache, mom = mkv.alloc_cache(g, B), mkv.alloc_moments(g)
+    ws = mkv.alloc_workspace(mkv.mkv_compress_workspace_size(g, T, p))
+    mkv.mkv_compress(g, T, bf16(K), bf16(V), bf16(Q), p, cache, mom, ws)
+    assert mkv.mkv_get_device_error(ws)[0] == 0
+    e2, m2 = 0.0, 0.0
+    for h in range(H):
+        keep = np.zeros(T, bool)
+        keep[host(cache.pos)[0, h, :B]] = True
+        ref = O.moments_of(K[0, h][~keep], V[0, h][~keep])
+        x0k, x0v = K[0, h, :128].mean(0).astype(f), V[0, h, :128].mean(0).astype(f)
+        n, sk, sv, M = tile_centred_moments(K[0, h], V[0, h], x0k, x0v)
+        nR, rk, rv, R = tile_centred_moments(K[0, h][keep], V[0, h][keep], x0k, x0v)
+        nE = n - nR
+        dk, dv = rk / nR - (sk - rk) / nE, rv / nR - (sv - rv) / nE
+        C = ((M - np.outer(sv, sk) / n) - (R - np.outer(rv, rk) / nR) - nE * nR / n * np.outer(dv, dk)) / nE
+        e2 += np.sum((host(mom.C)[0, h] - ref.C) ** 2)
+        m2 += np.sum((C - ref.C) ** 2)
+        # the means: a few roundings of the largest
+        np.testing.assert_allclose(host(mom.mu_k)[0, h], ref.mu_k, rtol=0, atol=1e-6 * np.abs(ref.mu_k).max())
+        np.testing.assert_allclose(host(mom.mu_v)[0, h], ref.mu_v, rtol=0, atol=1e-6 * np.abs(ref.mu_v).max())
+    print(f"C: {np.sqrt(e2):.3e} from 64 bits, the fp32 reference {np.sqrt(m2):.3e}")
+    assert np.sqrt(e2) <= 4 * np.sqrt(m2), (np.sqrt(e2), np.sqrt(m2))
+
+
 # ------------------------------------------------------- adaptive budget
 def run_adaptive(wl, T=None, pool=1, mi=1, tau=1e-6, seed=0, cap_extra=0):
     """mkv_compress with adaptive=1 against oracle.compress_adaptive, per batch
