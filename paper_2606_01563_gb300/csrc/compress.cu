@@ -1801,12 +1801,18 @@ cudaError_t smem_attr(const void* f, size_t bytes) {
   return cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(bytes));
 }
 
-// CTAs per unit and key half of rset_kernel: the more, the fewer records and
-// rows each takes; as many as run at once (shared memory: four per SM).
+// CTAs per unit and key half of rset_kernel (2048 threads of them in any case:
+// the count decides into how many parts a unit's row tiles fall and how often
+// its records' means are read).  Four, unless more would still find room and
+// have tiles, or fewer do with as many parts.  us of a call with 8 / 4 / 2:
+//   8 units, 8K, budgets 512, 1024, 4096: 69.5/63.8/70.3, 76.0/75.0/87.9, 142/156/208
+//   16 units, 16K, budget 2048: 177/190/207; 24 units: 230/210/227
+//   32 units, 32K, budgets 256, 1500, 4096: 274/246/239, 346/317/330, 530/510/549
+//   512 units, 1K, budget 128: 1167/772/726
 int rset_cluster(const Layout& L, int num_sms) {
-  int cl = 8;
-  while (cl > 2 && (long)cl * (L.D / 64) * L.units > 4L * num_sms) cl /= 2;
-  return cl;
+  const long pairs = (long)L.units * (L.D / 64);
+  if (L.B > 8 * kTok && 8 * pairs <= 2L * num_sms) return 8;
+  return L.B <= 2 * kTok && 4 * pairs > num_sms ? 2 : 4;
 }
 
 template <bool FINAL>

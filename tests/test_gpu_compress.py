@@ -164,6 +164,19 @@ def test_moments_of_keys_and_values_far_from_zero(H, D, T, B, ok, ov):
     assert np.sqrt(e2) <= 4 * np.sqrt(m2), (np.sqrt(e2), np.sqrt(m2))
 
 
+@pytest.mark.parametrize("b,H,D,T,B", [
+    (5, 8, 128, 600, 200),     # two row tiles, more units than SMs for four CTAs each
+    (10, 8, 64, 420, 100),     # one tile
+    (5, 8, 128, 1300, 1100),   # nine tiles over four CTAs
+    (1, 2, 128, 1500, 1153),   # ten over eight
+    (2, 2, 64, 3000, 2200),
+])
+def test_retained_set_clusters(b, H, D, T, B):
+    """The numbers of CTAs that share a unit's retained rows (2, 4 and 8), with
+    one and with several row tiles per CTA."""
+    run(Workload("rset", Geometry(b, H, 1, D), T, B, 16, "logscale"), seed=B)
+
+
 # ------------------------------------------------------- adaptive budget
 def run_adaptive(wl, T=None, pool=1, mi=1, tau=1e-6, seed=0, cap_extra=0):
     """mkv_compress with adaptive=1 against oracle.compress_adaptive, per batch
