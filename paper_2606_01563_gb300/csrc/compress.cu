@@ -785,6 +785,13 @@ __global__ void __launch_bounds__(kScoreThreads, 1)
 // 32K, batch 4 (32 units) it takes 143 us, the bounded one 22.  When more than half
 // of a CTA's positions remain, or the caller wants score2 itself, the full
 // pass runs; a position's score2 is the same bits either way.
+//
+// Roundings: each norm is a chain of at most 18 fp32 additions (1e-6 of it),
+// Y's elements come from 24 sums on the tensor core, which may drop a unit in
+// the last place each (3e-6 of ||C0'||_F ||k||), so a bound and the score2 it
+// stands for differ by less than 1e-5 (||v|| + c).  Relative to ||v|| + c that
+// is within theta's factor; ||v|| - c may be much smaller and gives it up.
+constexpr float kBoundSlack = 1e-5f;
 __global__ void __launch_bounds__(kResThreads, 1)
     residual_tc(const TcArgs p, const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtensorMap tmV) {
   constexpr int kS = 2;  // tile i is in stage and TMEM buffer i % 2
@@ -905,7 +912,8 @@ __global__ void __launch_bounds__(kResThreads, 1)
         t[i] = min(max(t[i], 0), p.T - 1);
         const size_t at = (size_t)(g0 + hs[i]) * p.T + t[i];
         const float2 nn = reinterpret_cast<const float2*>(p.norms)[at];
-        const float lb = sqrtf(nn.y) - s_mvn[hs[i]] - s_fro[hs[i]] * sqrtf(nn.x);
+        const float vn = sqrtf(nn.y), off = s_mvn[hs[i]] + s_fro[hs[i]] * sqrtf(nn.x);
+        const float lb = (vn - off) - kBoundSlack * (vn + off);
         const float b = p.s_in[at] * (lb > 0.f ? lb : 0.f);
         if (!is_protected(t[i], p.T, p.W, p.sink, p.keep_window))
           lowest = fminf(lowest, b > 0.f ? b : 0.f);  // a NaN counts as 0
@@ -914,7 +922,7 @@ __global__ void __launch_bounds__(kResThreads, 1)
     const uint32_t wmin = __reduce_min_sync(kFull, __float_as_uint(lowest));
     if (lane == 0) atomicMin(&s_theta, wmin);
     __syncthreads();
-    const float theta = __uint_as_float(s_theta) * 0.9999f;  // rounding of both sides: below 1e-6
+    const float theta = __uint_as_float(s_theta) * 0.9999f;  // relative roundings: theta's, ub's and score2's
     const int h = u - g0;
     const float mvn = s_mvn[h], fro = s_fro[h];
     constexpr int kBatch = 8;  // positions per lane whose loads are in flight together

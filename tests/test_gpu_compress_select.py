@@ -17,9 +17,9 @@ from paper_2606_01563_gb300 import mkv
 pytestmark = pytest.mark.gpu
 
 
-def compress(b, H, G, D, T, B, w, K, V, Q, adaptive, diag, pool=1, mi=1):
+def compress(b, H, G, D, T, B, w, K, V, Q, adaptive, diag, pool=1, mi=1, tau=1e-6):
     g = mkv.geom(b, H, G, D)
-    p = mkv.mkv_compress_params(B, w, 1, 1, pool, mi, 1, 1e-6, adaptive)
+    p = mkv.mkv_compress_params(B, w, 1, 1, pool, mi, 1, tau, adaptive)
     prot = 1 + w
     cap = min(T, H * (B - prot) + prot) if adaptive else B
     cache, mom = mkv.alloc_cache(g, cap), mkv.alloc_moments(g)
@@ -114,3 +114,43 @@ def test_joint_selection_of_many_groups():
             want, _ = O.select_topk_joint(s[i], H * (B - 1 - w), prot)
             for h in range(H):
                 np.testing.assert_array_equal(pos[i, h, :ln[i, h]], want[h])
+
+
+def test_pruning_bound_of_rounding_size():
+    """Values near one large constant, so that the first stage's lower bounds
+    ||v|| - ||mu_v0|| are differences of nearly equal norms, no larger than a
+    few of their roundings; in each unit one row of the opposite sign whose
+    score2 lies just above the weakest first-stage row's and meets its own
+    upper bound.  (tau clamps all of C0'.)"""
+    b, H, G, D, T, B, w = 4, 8, 2, 128, 32768, 64, 16
+    U, k, scale, q0, q1 = b * H, B - 1 - w, D ** -0.5, 16.0, 2.0 ** -4
+    gen = torch.Generator()
+    gen.manual_seed(9)
+    logit = torch.full((U, T), -17.0, dtype=torch.float64)
+    a = torch.full((U, T), 256.0)
+    opposite = torch.empty(U, dtype=torch.int64)
+    for u in range(U):
+        at = 1 + torch.randperm(T - w - 1, generator=gen)
+        n1 = 4 + u  # values of 255: mu_v0 = 256 - n1 / n0 per dim (one value of -256 against two of 512)
+        r = D ** 0.5 * n1 / (T - B)
+        first, opposite[u] = at[:k], at[k]
+        logit[u, first] = 0.2 * torch.arange(k, dtype=torch.float64)
+        # a quarter of a rounding of ||mu_v0|| = 2896 above the weakest row's score2
+        logit[u, at[k]] = np.log(r / (512 * D ** 0.5)) + 0.25 * 1.2e-4 / r
+        a[u, at[k]] = -256.0
+        a[u, at[k + 1:k + 3]] = 512.0
+        a[u, at[k + 3:k + 3 + n1]] = 255.0
+    K = torch.zeros(U, T, D)
+    x = torch.round(logit / (scale * q0) * 16) / 16
+    K[:, :, 0] = x
+    K[:, :, 1] = (logit - scale * q0 * x) / (scale * q1)
+    Q = torch.zeros(b, H, G, w, D)
+    Q[..., 0], Q[..., 1] = q0, q1
+    K = K.view(b, H, T, D).to(torch.bfloat16).cuda()
+    V = a[:, :, None].expand(U, T, D).reshape(b, H, T, D).to(torch.bfloat16).cuda()
+    Q = Q.to(torch.bfloat16).cuda()
+    full = compress(b, H, G, D, T, B, w, K, V, Q, 0, True, tau=1e30)
+    pruned = compress(b, H, G, D, T, B, w, K, V, Q, 0, False, tau=1e30)
+    pos = full["pos"].view(U, -1).cpu()
+    assert all(int(opposite[u]) in pos[u].tolist() for u in range(U))
+    assert torch.equal(pruned["pos"].view(U, -1).cpu(), pos)
