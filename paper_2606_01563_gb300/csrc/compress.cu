@@ -85,6 +85,7 @@ struct Layout {
   uint32_t* hist;     // [2][units][kBins] keys of the unprotected scores per bin (s, s2)
   unsigned long long* glist;  // [units / hs][kGroupCont] contested pairs of a joint selection
   int32_t* gcnt;              // [2][units] their counts by group (s, s2)
+  uint32_t* sub;              // [2][units / hs][kBins] and their keys per second-level bin (sub_bin)
   uint8_t* cimg;      // [units][3][128 x 128] C0' as three bf16 parts, in the residual's operand layout
   float* mv0;         // [units][kDP] mu_v of E0
   float* fro;         // [units][kDP] parts of ||C0'||_F^2
@@ -147,6 +148,7 @@ size_t carve(Layout& L, void* ws) {
   L.glist = reinterpret_cast<unsigned long long*>(
       take(L.hs > 1 ? U / L.hs * (size_t)kGroupCont * sizeof(unsigned long long) : 0));
   L.gcnt = reinterpret_cast<int32_t*>(take(2 * U * sizeof(int32_t)));
+  L.sub = reinterpret_cast<uint32_t*>(take(L.hs > 1 ? 2 * (U / L.hs) * (size_t)kBins * sizeof(uint32_t) : 0));
   L.cimg = take(U * (size_t)3 * kTileBytes);
   L.mv0 = reinterpret_cast<float*>(take(U * (size_t)kDP * sizeof(float)));
   L.fro = reinterpret_cast<float*>(take(U * (size_t)kDP * sizeof(float)));
@@ -164,6 +166,13 @@ __device__ __forceinline__ bool is_protected(int t, int T, int W, int sink, int 
 __device__ __forceinline__ uint32_t score_key(float s) { return max(1u, float_key(s)); }
 __device__ __forceinline__ int key_bin(uint32_t key) {
   return (key & 0x80000000u) ? static_cast<int>((key >> 20) & (kBins - 1)) : 0;
+}
+
+// The keys of one bin in second-level bins, in order: eleven of the 20 bits
+// below those that the bin fixes; bin 0's by the sign and ten bits below.
+__device__ __forceinline__ int sub_bin(int bin, uint32_t key) {
+  if (bin > 0) return static_cast<int>((key >> 9) & (kBins - 1));
+  return static_cast<int>((key & 0x80000000u) ? 1024u | ((key >> 10) & 1023u) : key >> 21);
 }
 
 // 16 bytes global -> shared, asynchronously (src_bytes 0: zeros)
@@ -263,13 +272,15 @@ struct TcArgs {
   float* s_out;
   uint32_t* hist;  // stats_tc: both tables, zeroed; scores_tc, residual_tc: the table their scores are counted in
   int32_t* gcnt;   // [2][units] counts of joint selections, zeroed by stats_tc
+  uint32_t* sub;   // [2][units / hs][kBins] second-level counts of joint selections (or null), zeroed by stats_tc
   int units;
   float* diag;
   const uint8_t* cimg;  // [units][3][128 x 128] operand image of C0'
   const float* mv0;     // [units][kDP]
   float* norms;         // [units][T][2] ||k_t||^2, ||v_t||^2
+  int hs;  // units per selection group
   // residual_tc's pruning
-  int prune, hs, B;     // hs: units per selection group
+  int prune, B;
   const int32_t* idx;   // [units][lsel] the first stage's selections
   const int32_t* cnt;   // [units] their numbers (joint; B otherwise)
   int lsel;
@@ -445,6 +456,8 @@ __global__ void __launch_bounds__(kStatThreads, 1)
       for (int i = tid - 64; i < 2 * kBins / 4; i += 256) {
         const int tab = i / (kBins / 4), b4 = i % (kBins / 4);
         reinterpret_cast<uint4*>(p.hist + ((size_t)tab * p.units + u) * kBins)[b4] = make_uint4(0u, 0u, 0u, 0u);
+        if (p.sub != nullptr && u % p.hs == 0)
+          reinterpret_cast<uint4*>(p.sub + ((size_t)tab * p.units + u) / p.hs * kBins)[b4] = make_uint4(0u, 0u, 0u, 0u);
       }
     const uint32_t lane_base = static_cast<uint32_t>(qd * 32) << 16;
     float m[2] = {-INFINITY, -INFINITY}, l[2] = {0.f, 0.f};
@@ -1090,8 +1103,10 @@ __global__ void __launch_bounds__(kResThreads, 1)
 // against 24.5 (with the rows' gather, now rset's), at 128K 20 against 35.  A unit's contested keys are
 // exchanged over its cluster; the pairs of a batch item through global memory
 // (contest_kernel), so that a joint selection too has kSelCL CTAs per unit.
-// When there are more contested keys than the lists hold (many equal scores),
-// a radix select over the pairs takes the place of the ranking.
+// When there are more contested keys than the lists hold (k above about
+// 12000, or many equal scores), counts of their next eleven bits, taken as they
+// were listed, narrow them down and the scan is repeated; equal keys that
+// still do not fit are counted by position.
 struct SelectArgs {
   const float* scores;   // [units][T]
   const uint32_t* hist;  // [units][kBins] counts of the unprotected scores' keys
@@ -1103,12 +1118,14 @@ struct SelectArgs {
   int32_t* cnt;       // [units] rows each unit retains (joint)
   unsigned long long* glist;  // [groups][kGroupCont] contested pairs of a group (joint)
   int32_t* gcnt;              // [groups] their count
+  uint32_t* sub;              // [groups][kBins] their second-level counts
 };
 
 constexpr int kSelThreads = 512;
 constexpr int kSelWarps = kSelThreads / 32;
 constexpr int kSelCL = 8;         // CTAs per unit (one cluster), each over a contiguous range of positions
 constexpr int kMaxCont = 256;     // keys of the contested bin a CTA may hold
+static_assert(kGroupCont == kSelCL * kMaxCont, "one list serves both");
 constexpr int kSelBatch = 8;      // positions per lane loaded together
 
 // pairs are ordered by (key, ~f): a higher key first, at equal keys the lower f
@@ -1132,20 +1149,13 @@ __device__ __forceinline__ int block_counts(int mine, int* s_w, int* total) {
   return before;
 }
 
-// The bin of the group's k-th highest key (k > 0) and how many of its keys are
-// selected, into *s_bin and *s_need: thread t takes four bins, descending.
-__device__ __forceinline__ void threshold_bin(const SelectArgs& a, int grp, int k, int* s_w, int* s_bin, int* s_need) {
+// Of kBins counts, thread t holding the four bins 4 (kSelThreads - 1 - t) ..,
+// the bin where their descending sum reaches k > 0, how many of its keys are
+// selected, and (if s_left) how many it has, into *s_bin, *s_need and *s_left.
+__device__ __forceinline__ void threshold_of(const uint4& c, int k, int* s_w, int* s_bin, int* s_need,
+                                             int* s_left = nullptr) {
   const int tid = threadIdx.x, lane = tid & 31;
   static_assert(kBins == 4 * kSelThreads, "four bins per thread");
-  uint4 c = make_uint4(0u, 0u, 0u, 0u);
-#pragma unroll 4
-  for (int h = 0; h < a.hs; ++h) {
-    const uint4 x = reinterpret_cast<const uint4*>(a.hist + ((size_t)grp * a.hs + h) * kBins)[kBins / 4 - 1 - tid];
-    c.x += x.x;
-    c.y += x.y;
-    c.z += x.z;
-    c.w += x.w;
-  }
   const int b[4] = {(int)c.w, (int)c.z, (int)c.y, (int)c.x};
   int incl = b[0] + b[1] + b[2] + b[3];
   const int mine = incl;
@@ -1161,10 +1171,26 @@ __device__ __forceinline__ void threshold_bin(const SelectArgs& a, int grp, int 
     if (above < k && above + b[e] >= k) {  // one bin of the block
       *s_bin = kBins - 1 - (tid * 4 + e);
       *s_need = k - above;
+      if (s_left != nullptr) *s_left = b[e];
     }
     above += b[e];
   }
   __syncthreads();
+}
+
+// The bin of the group's k-th highest key.
+__device__ __forceinline__ void threshold_bin(const SelectArgs& a, int grp, int k, int* s_w, int* s_bin, int* s_need) {
+  uint4 c = make_uint4(0u, 0u, 0u, 0u);
+#pragma unroll 4
+  for (int h = 0; h < a.hs; ++h) {
+    const uint4 x =
+        reinterpret_cast<const uint4*>(a.hist + ((size_t)grp * a.hs + h) * kBins)[kBins / 4 - 1 - threadIdx.x];
+    c.x += x.x;
+    c.y += x.y;
+    c.z += x.z;
+    c.w += x.w;
+  }
+  threshold_of(c, k, s_w, s_bin, s_need);
 }
 
 // fn(position, in range, pair) for the positions [w0, w1) of one unit, a warp's
@@ -1190,6 +1216,79 @@ __device__ __forceinline__ void each_pair(const SelectArgs& a, const float* sc, 
   }
 }
 
+// One addition to a slot counter and to a table of counts for the lanes of a
+// warp with `is`: the counter once per warp, the table once where all agree on
+// the bin (as equal scores do).  Returns the lane's slot.
+__device__ __forceinline__ int warp_append(bool is, int d, int* n, uint32_t* counts) {
+  const int lane = threadIdx.x & 31;
+  const unsigned mask = __ballot_sync(kFull, is);
+  if (mask == 0u) return 0;
+  const int first = __ffs(mask) - 1, d0 = __shfl_sync(kFull, d, first);
+  int slot = 0;
+  if (lane == first) slot = atomicAdd(n, __popc(mask));
+  slot = __shfl_sync(kFull, slot, first) + __popc(mask & ((1u << lane) - 1u));
+  if (__all_sync(kFull, !is || d == d0)) {
+    if (lane == first) atomicAdd(&counts[d0], static_cast<uint32_t>(__popc(mask)));
+  } else if (is) {
+    atomicAdd(&counts[d], 1u);
+  }
+  return slot;
+}
+
+// The need-th highest of the list's pairs (lists by CTA, s_cn[r] pairs at r *
+// kMaxCont, all with p >> bits == pre), into *s_last; need is at most their
+// number.  A pair's rank among
+// kRankMax or fewer is counted by comparing; more are narrowed down before by
+// counts of eleven of their bits at a time (32K, 8 units, budget 8192, about
+// 1400 pairs: a selection 108 us with all compared, 15 narrowed).
+constexpr int kRankMax = 64;
+__device__ __forceinline__ void list_select(const unsigned long long* s_cont, const int* s_cn, int m, int need,
+                                            unsigned long long pre, int bits, uint32_t* s_hist, unsigned long long* s_few, int* s_n, int* s_w, int* s_bin,
+                                            int* s_need, unsigned long long* s_last) {
+  const int tid = threadIdx.x;
+  auto each = [&](auto&& fn) {
+    for (int i = tid; i < m; i += kSelThreads) {
+      int j = i, r = 0;
+      while (j >= s_cn[r]) j -= s_cn[r++];
+      fn(s_cont[r * kMaxCont + j]);
+    }
+  };
+  int left = m;  // candidates: the pairs with p >> bits == pre
+  while (left > kRankMax && bits > 0) {
+    const int w = min(bits, 11), sh = bits - w;
+    for (int i = tid; i < kBins; i += kSelThreads) s_hist[i] = 0u;
+    __syncthreads();
+    each([&](unsigned long long p) {
+      if (bits > 63 || p >> bits == pre) atomicAdd(&s_hist[(p >> sh) & ((1u << w) - 1u)], 1u);
+    });
+    __syncthreads();
+    threshold_of(reinterpret_cast<const uint4*>(s_hist)[kBins / 4 - 1 - tid], need, s_w, s_bin, s_need);
+    pre = pre << w | static_cast<unsigned>(*s_bin);
+    bits = sh;
+    need = *s_need;
+    left = static_cast<int>(s_hist[*s_bin]);
+    __syncthreads();
+  }
+  if (tid == 0) *s_n = 0;
+  __syncthreads();
+  each([&](unsigned long long p) {
+    if (bits > 63 || p >> bits == pre) {
+      const int slot = atomicAdd(s_n, 1);
+      if (slot < kRankMax) s_few[slot] = p;
+    }
+  });
+  __syncthreads();
+  const int few = min(*s_n, kRankMax);
+  if (tid < few) {
+    const unsigned long long p = s_few[tid];
+    int before = 0;
+#pragma unroll 4
+    for (int j = 0; j < few; ++j) before += s_few[j] > p ? 1 : 0;
+    if (before == need - 1) *s_last = p;
+  }
+  __syncthreads();
+}
+
 // The contested pairs of joint selections: grid (kSelCL, units), every CTA's
 // part of its unit's positions, into the group's list.
 __global__ void __launch_bounds__(kSelThreads) contest_kernel(const SelectArgs a) {
@@ -1210,10 +1309,10 @@ __global__ void __launch_bounds__(kSelThreads) contest_kernel(const SelectArgs a
   const int bin = s_bin, per = (a.T + kSelCL * kSelWarps - 1) / (kSelCL * kSelWarps);
   const int w0 = min(a.T, (static_cast<int>(blockIdx.x) * kSelWarps + warp) * per), w1 = min(a.T, w0 + per);
   each_pair(a, a.scores + (size_t)u * a.T, w0, w1, h * a.T, [&](int, bool in, unsigned long long p) {
-    if (in && p != ~0ull && key_bin(static_cast<uint32_t>(p >> 32)) == bin) {
-      const int slot = atomicAdd(&s_n, 1);
-      if (slot < kGroupCont) s_cont[slot] = p;
-    }
+    const uint32_t key = static_cast<uint32_t>(p >> 32);
+    const bool is = in && p != ~0ull && key_bin(key) == bin;
+    const int slot = warp_append(is, sub_bin(bin, key), &s_n, a.sub + (size_t)grp * kBins);
+    if (is && slot < kGroupCont) s_cont[slot] = p;
   });
   __syncthreads();
   if (tid == 0) s_at = atomicAdd(a.gcnt + grp, s_n);
@@ -1225,11 +1324,14 @@ __global__ void __launch_bounds__(kSelThreads) contest_kernel(const SelectArgs a
 template <bool JOINT>
 __global__ void __cluster_dims__(kSelCL, 1, 1) __launch_bounds__(kSelThreads, 2) select_kernel(const SelectArgs a) {
   __shared__ int s_w[kSelWarps];
-  __shared__ int s_bin, s_need;
+  __shared__ int s_bin, s_need, s_left;
   __shared__ int s_n;            // this CTA's contested keys
   __shared__ int s_cn[kSelCL];   // every CTA's (written remotely)
   // the unit's contested pairs by CTA (written remotely), or the group's list
-  __shared__ unsigned long long s_cont[JOINT ? kGroupCont : kSelCL * kMaxCont];
+  __shared__ unsigned long long s_cont[kSelCL * kMaxCont];
+  __shared__ __align__(16) uint32_t s_hist[kBins];  // this CTA's counts of the contested keys' next bits (read remotely)
+  __shared__ int s_tie[kMaxHs];                     // and of its equal keys per unit (read remotely)
+  __shared__ unsigned long long s_few[kRankMax];
   __shared__ unsigned long long s_last;  // the last selected pair (written remotely when joint)
   __shared__ int s_tot[2][kSelCL];       // every CTA's counts (written remotely)
   cg::cluster_group cluster = cg::this_cluster();
@@ -1239,6 +1341,7 @@ __global__ void __cluster_dims__(kSelCL, 1, 1) __launch_bounds__(kSelThreads, 2)
   const int prot = protected_count(T, a.W, a.sink, a.keep_window);
   const int k = hs * (a.B - prot);  // >= 0 (validated), < candidates
   const float* sc = a.scores + (size_t)u * T;
+  const float* sc0 = a.scores + (size_t)grp * hs * T;  // the group's first unit
   // warp w of CTA r takes the contiguous positions [w0, w1)
   const int per = (T + kSelCL * kSelWarps - 1) / (kSelCL * kSelWarps);
   const int w0 = min(T, (rank * kSelWarps + warp) * per), w1 = min(T, w0 + per);
@@ -1249,33 +1352,106 @@ __global__ void __cluster_dims__(kSelCL, 1, 1) __launch_bounds__(kSelThreads, 2)
     s_last = ~0ull;
   }
   __syncthreads();
-  // every CTA has started, its s_last initialised (release: another CTA may
-  // overwrite it): awaited before the first remote store
+  // every CTA has started, with its initial values in place (release): awaited
+  // before the first remote store
   cluster_arrive_release();
   grid_dependency_wait();
   grid_launch_dependents();
 
   if (k > 0) {
     threshold_bin(a, grp, k, s_w, &s_bin, &s_need);
-    const int bin = s_bin, need = s_need;
-    bool over = false;
+    const int bin = s_bin;
+    int need = s_need;  // of the contested keys, how many are selected
+    // contested: the keys of the bin, or (bits >= 0) those with key >> bits == pre
+    uint32_t pre = 0u;
+    int bits = -1;
+    auto contested = [&](uint32_t key) { return bits < 0 ? key_bin(key) == bin : key >> bits == pre; };
+    int left = 0;  // keys contested, where known
+    auto narrow = [&](int d) {  // to the digit d that the counts gave, of the next 11 bits
+      need = s_need;
+      left = s_left;
+      if (bits >= 0) {
+        const int w = min(bits, 11);
+        pre = pre << w | static_cast<uint32_t>(d);
+        bits -= w;
+      } else if (bin > 0) {
+        pre = (0x800u | static_cast<uint32_t>(bin)) << 11 | static_cast<uint32_t>(d);
+        bits = 9;
+      } else {
+        pre = d >= 1024 ? 0x200000u | (d & 1023u) : static_cast<uint32_t>(d);
+        bits = d >= 1024 ? 10 : 21;
+      }
+    };
+    // the pair to find is in the lists, whose lengths are s_cn
+    auto from_lists = [&](int m) {
+      const unsigned long long p0 = bits >= 0 ? pre : bin > 0 ? 0x800u | static_cast<uint32_t>(bin) : 0u;
+      list_select(s_cont, s_cn, m, need, p0, bits >= 0 ? bits + 32 : bin > 0 ? 52 : 64, s_hist, s_few, &s_n, s_w, &s_bin,
+                  &s_need, &s_last);
+    };
+    // this CTA's list to every CTA, unless it overflowed; whether all fit, and their sum
+    auto exchange = [&](int& m) -> bool {
+      const int mn = s_n;
+      if (tid < kSelCL) *cluster.map_shared_rank(&s_cn[rank], tid) = mn;
+      if (mn <= kMaxCont)
+        for (int i = tid; i < mn * kSelCL; i += kSelThreads) {
+          const int r = i % kSelCL, e = rank * kMaxCont + i / kSelCL;
+          if (r != rank) *cluster.map_shared_rank(&s_cont[e], r) = s_cont[e];
+        }
+      cluster.sync();
+      bool fit = true;
+      m = 0;
+      for (int r = 0; r < kSelCL; ++r) {
+        fit &= s_cn[r] <= kMaxCont;
+        m += s_cn[r];
+      }
+      return fit;
+    };
+    // the cluster's counts of the contested keys' next digit
+    auto narrow_by_counts = [&]() {
+      uint4 c = make_uint4(0u, 0u, 0u, 0u);
+      for (int r = 0; r < kSelCL; ++r) {
+        const uint4 x = reinterpret_cast<const uint4*>(cluster.map_shared_rank(s_hist, r))[kBins / 4 - 1 - tid];
+        c.x += x.x;
+        c.y += x.y;
+        c.z += x.z;
+        c.w += x.w;
+      }
+      threshold_of(c, need, s_w, &s_bin, &s_need, &s_left);
+      narrow(s_bin);
+    };
+    // ---- scan of the group's units: the contested keys into this CTA's list,
+    // and their next digit counted
+    auto scan = [&]() {
+      for (int i = tid; i < kBins; i += kSelThreads) s_hist[i] = 0u;
+      if (tid == 0) s_n = 0;
+      __syncthreads();
+      const int w = min(max(bits, 0), 11), sh = max(bits, 0) - w;
+#pragma unroll 1
+      for (int g = 0; g < hs; ++g)
+        each_pair(a, sc0 + (size_t)g * T, w0, w1, g * T, [&](int, bool in, unsigned long long p) {
+          const uint32_t key = static_cast<uint32_t>(p >> 32);
+          const bool is = in && p != ~0ull && contested(key);
+          const int d = bits < 0 ? sub_bin(bin, key) : static_cast<int>((key >> sh) & ((1u << w) - 1u));
+          const int slot = warp_append(is, d, &s_n, s_hist);
+          if (is && slot < kMaxCont) s_cont[rank * kMaxCont + slot] = p;
+        });
+      __syncthreads();
+    };
+    int m;
+    bool found;
     if constexpr (JOINT) {
       cluster_wait_acquire();
-      const int m = a.gcnt[grp];
-      over = m > kGroupCont;
-      if (!over) {
+      m = a.gcnt[grp];
+      found = m <= kGroupCont;
+      if (found) {  // contest_kernel's list, in parts as the clusters' lists are
         for (int i = tid; i < m; i += kSelThreads) s_cont[i] = a.glist[(size_t)grp * kGroupCont + i];
+        if (tid < kSelCL) s_cn[tid] = min(max(m - tid * kMaxCont, 0), kMaxCont);
         __syncthreads();
-        // the need-th of them, the one that need - 1 others precede: the
-        // cluster's warps share the candidates
-        for (int i = rank * kSelWarps + warp; i < m; i += kSelCL * kSelWarps) {
-          const unsigned long long p = s_cont[i];
-          int before = 0;
-          for (int j = lane; j < m; j += 32) before += s_cont[j] > p ? 1 : 0;
-          before = __reduce_add_sync(kFull, before);
-          if (before == need - 1 && lane < kSelCL) *cluster.map_shared_rank(&s_last, lane) = p;
-        }
-        cluster.sync();
+        from_lists(m);
+      } else {
+        const uint4 c = reinterpret_cast<const uint4*>(a.sub + (size_t)grp * kBins)[kBins / 4 - 1 - tid];
+        threshold_of(c, need, s_w, &s_bin, &s_need, &s_left);
+        narrow(s_bin);
       }
     } else {
       // ---- the contested keys: this CTA's into every CTA's list
@@ -1287,76 +1463,73 @@ __global__ void __cluster_dims__(kSelCL, 1, 1) __launch_bounds__(kSelThreads, 2)
       });
       __syncthreads();
       cluster_wait_acquire();
-      const int mn = s_n;
-      if (tid < kSelCL) *cluster.map_shared_rank(&s_cn[rank], tid) = mn;
-      for (int i = tid; i < min(mn, kMaxCont) * kSelCL; i += kSelThreads) {
-        const int r = i % kSelCL, e = rank * kMaxCont + i / kSelCL;
-        if (r != rank) *cluster.map_shared_rank(&s_cont[e], r) = s_cont[e];
-      }
-      cluster.sync();
-      int m = 0;
-      for (int r = 0; r < kSelCL; ++r) {
-        over |= s_cn[r] > kMaxCont;
-        m += s_cn[r];
-      }
-      if (!over) {
-        // the need-th of them: the one that need - 1 others precede
-        for (int i = tid; i < m; i += kSelThreads) {
-          int j = i, r = 0;
-          while (j >= s_cn[r]) j -= s_cn[r++];
-          const unsigned long long p = s_cont[r * kMaxCont + j];
-          int before = 0;
-          for (int r2 = 0; r2 < kSelCL; ++r2) {
-            const int c2 = s_cn[r2];
-#pragma unroll 4
-            for (int j2 = 0; j2 < c2; ++j2) before += s_cont[r2 * kMaxCont + j2] > p ? 1 : 0;
-          }
-          if (before == need - 1) s_last = p;
-        }
-        __syncthreads();
+      found = exchange(m);
+      if (found) {
+        from_lists(m);
+      } else {
+        cluster.sync();  // every CTA is done with s_cn
+        scan();
+        cluster.sync();
+        narrow_by_counts();
       }
     }
-    if (over) {
-      // radix select over the group's pairs, eight bits at a time below those
-      // the bin fixes, until the digit's pairs are exactly the missing ones
-      // (each cluster of a group over all its units)
-      uint32_t* hist = reinterpret_cast<uint32_t*>(s_cont);  // [256] this CTA's counts (read remotely), [256] the cluster's
-      const int top = bin > 0 ? 12 : 0;
-      unsigned long long prefix = bin > 0 ? static_cast<unsigned long long>(0x800u | bin) << 52 : 0ull;
-      unsigned long long mask = bin > 0 ? 0xfffull << 52 : 0ull;
-      int left = bin > 0 ? need : k;
 #pragma unroll 1
-      for (int shift = 64 - top - 8;; shift = max(shift - 8, 0)) {
-        cluster.sync();  // the lists, or the counts of the pass before, are read
-        if (tid < 256) hist[tid] = 0u;
+    while (!found) {
+      cluster.sync();  // the lists and counts of the scan before are read
+      const bool equal = bits == 0 && left > kGroupCont;  // uniform over the cluster
+      if (!equal) scan();
+      if (!equal && exchange(m)) {
+        from_lists(m);
+        found = true;
+      } else if (bits != 0) {
+        narrow_by_counts();
+      } else {
+        // ---- equal keys: the need-th by unit and position, from the counts of every (unit, CTA)
+        for (int g = tid; g < hs; g += kSelThreads) s_tie[g] = 0;
         __syncthreads();
-#pragma unroll 1
-        for (int g = 0; g < hs; ++g)
-          each_pair(a, a.scores + ((size_t)grp * hs + g) * T, w0, w1, g * T, [&](int, bool in, unsigned long long p) {
-            if (in && p != ~0ull && (p & mask) == prefix) atomicAdd(&hist[(p >> shift) & 255u], 1u);
+        auto tied = [&](int g, auto&& fn) {
+          each_pair(a, sc0 + (size_t)g * T, w0, w1, g * T, [&](int, bool in, unsigned long long p) {
+            const bool is = in && p != ~0ull && static_cast<uint32_t>(p >> 32) == pre;
+            fn(__ballot_sync(kFull, is), p);
           });
+        };
+#pragma unroll 1
+        for (int g = 0; g < hs; ++g) {
+          int c = 0;
+          tied(g, [&](unsigned mask, unsigned long long) { c += __popc(mask); });
+          if (lane == 0) atomicAdd(&s_tie[g], c);
+        }
         cluster.sync();
-        if (tid < 256) {
-          uint32_t x = 0u;
-          for (int r = 0; r < kSelCL; ++r) x += cluster.map_shared_rank(hist, r)[tid];
-          hist[256 + tid] = x;
+        if (tid == 0) s_bin = -1;
+        static_assert(kMaxHs * kSelCL <= kSelThreads, "one count per thread");
+        const int mine = tid < hs * kSelCL ? cluster.map_shared_rank(s_tie, tid % kSelCL)[tid / kSelCL] : 0;
+        int incl = mine, total;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+          const int y = __shfl_up_sync(kFull, incl, o);
+          if (lane >= o) incl += y;
+        }
+        incl += block_counts(__shfl_sync(kFull, incl, 31), s_w, &total);
+        if (incl >= need && incl - mine < need) {  // one thread
+          s_bin = tid;
+          s_need = need - (incl - mine);
         }
         __syncthreads();
-        if (tid == 0) {  // the digit where the descending count reaches `left`
-          int d = 255, above = 0;
-          while (d > 0 && above + static_cast<int>(hist[256 + d]) < left) above += hist[256 + d--];
-          s_bin = d;
-          s_need = left - above;
+        if (s_bin % kSelCL == rank) {  // uniform over the CTA: it holds the pair
+          const int g = s_bin / kSelCL, left = s_need;
+          int c = 0;
+          tied(g, [&](unsigned mask, unsigned long long) { c += __popc(mask); });
+          int run = block_counts(c, s_w, &total);
+          if (run < left && run + c >= left)  // one warp
+            tied(g, [&](unsigned mask, unsigned long long p) {
+              if (((mask >> lane) & 1u) && run + __popc(mask & ((1u << lane) - 1u)) == left - 1)
+                for (int r = 0; r < kSelCL; ++r) *cluster.map_shared_rank(&s_last, r) = p;
+              run += __popc(mask);
+            });
         }
-        __syncthreads();
-        prefix |= static_cast<unsigned long long>(s_bin) << shift;
-        mask |= 255ull << shift;
-        left = s_need;
-        if (shift == 0 || static_cast<int>(hist[256 + s_bin]) == left) break;  // uniform over the cluster
-        __syncthreads();
+        found = true;
+        cluster.sync();
       }
-      if (tid == 0) s_last = prefix;
-      cluster.sync();  // no counts are read remotely any more
     }
   } else {
     cluster_wait_acquire();
@@ -1873,6 +2046,8 @@ cudaError_t run(const CompressArgs& a, const mkv_geom& g, int num_sms, cudaStrea
   tp.mrec = L.mpart;
   tp.hist = L.hist;
   tp.gcnt = L.gcnt;
+  tp.sub = L.hs > 1 ? L.sub : nullptr;
+  tp.hs = L.hs;
   tp.units = U;
   tp.norms = L.norms;
   tp.ws = a.ws;
@@ -1908,6 +2083,7 @@ cudaError_t run(const CompressArgs& a, const mkv_geom& g, int num_sms, cudaStrea
     sa.cnt = L.cnt;
     sa.glist = L.glist;
     sa.gcnt = L.gcnt + (size_t)stage * U;
+    sa.sub = L.sub + (size_t)stage * (U / L.hs) * kBins;
     if (L.hs == 1) return launch_pdl(select_kernel<false>, dim3(U * kSelCL), kSelThreads, 0, st, 0, sa);
     cudaError_t se = launch_pdl(contest_kernel, dim3(kSelCL, U), kSelThreads, 0, st, 0, sa);
     if (se == cudaSuccess) se = launch_pdl(select_kernel<true>, dim3(U * kSelCL), kSelThreads, 0, st, 0, sa);
@@ -1945,7 +2121,6 @@ cudaError_t run(const CompressArgs& a, const mkv_geom& g, int num_sms, cudaStrea
     r.diag = a.diag_score2;
     // a second pass over the prompt is worth avoiding from eight tiles a CTA on
     r.prune = a.diag_score2 == nullptr && L.chunk >= kPruneTiles * kTok ? 1 : 0;
-    r.hs = L.hs;
     r.B = B;
     r.idx = L.idx;
     r.cnt = L.cnt;

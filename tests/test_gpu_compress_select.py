@@ -154,3 +154,46 @@ def test_pruning_bound_of_rounding_size():
     pos = full["pos"].view(U, -1).cpu()
     assert all(int(opposite[u]) in pos[u].tolist() for u in range(U))
     assert torch.equal(pruned["pos"].view(U, -1).cpu(), pos)
+
+
+@pytest.mark.parametrize("kind,H,T,B,adaptive,pool", [
+    ("distinct", 2, 40000, 16000, 0, 1),   # more contested keys than a list holds, all different
+    ("distinct", 8, 24000, 2600, 1, 1),    # the same of a joint selection
+    ("chunks", 2, 30001, 9000, 0, 32),     # equal in runs of 32
+    ("chunks", 4, 30001, 4000, 1, 32),
+    ("close", 2, 40000, 6000, 0, 1),       # one bin, most keys apart in their last bits only
+    ("close", 4, 16000, 2000, 1, 1),
+    ("equal", 2, 20000, 900, 0, 1),        # all equal: by position alone
+    ("equal", 64, 700, 40, 1, 1),          # the last selected pair in one of the later heads
+    ("zero", 2, 30000, 700, 0, 1),         # fewer scores above zero than selections
+    ("zero", 8, 9000, 300, 1, 1),
+])
+def test_more_contested_keys_than_the_lists_hold(kind, H, T, B, adaptive, pool):
+    """Selections whose threshold bin holds more keys than the exchanged lists,
+    against a stable sort of the kernel's own scores."""
+    G, D, w = 1, 64, 8
+    gen = torch.Generator(device="cuda")
+    gen.manual_seed(T + B)
+    r = lambda *s: torch.randn(*s, generator=gen, device="cuda")
+    K, V, Q = r(1, H, T, D), r(1, H, T, D), r(1, H, G, w, D)
+    if kind == "close":
+        K *= 1e-3
+    elif kind == "equal":
+        K[:] = K[:, :1, :1]
+    elif kind == "zero":  # 400 keys hold all the weight
+        K[:, :, 400:] = -40.0 * Q[:, :, 0, :1]
+        Q[:] = Q[:, :, :, :1]
+    K, V, Q = (x.to(torch.bfloat16) for x in (K, V, Q))
+    out = compress(1, H, G, D, T, B, w, K, V, Q, adaptive, True, pool=pool, mi=0)
+    t = np.arange(T)
+    prot = (t < 1) | (t >= T - w)
+    s = out["s"][0].double().cpu().numpy()
+    if kind == "zero":
+        assert (s[:, 500:T - w] == 0).all()
+    k = B - int(prot.sum())
+    if adaptive:
+        want, _ = O.select_topk_joint(s, H * k, np.stack([prot] * H))
+    else:
+        want = [O.select_topk(s[h], k, prot)[0] for h in range(H)]
+    for h in range(H):
+        np.testing.assert_array_equal(out["pos"][0, h, :int(out["len"][0, h])].cpu().numpy(), want[h])
