@@ -55,10 +55,12 @@ constexpr int kBoxBytes = kTok * 128;
 // warps per scheduler share the work
 constexpr int kResThreads = 320;
 constexpr int kMaxHs = 64;  // KV heads of a batch item with the adaptive budget
+constexpr int kHot = 249, kHotLo = (127 - 20) * 8;  // bins a CTA counts in shared memory (count_bin)
 // scores_tc's K stages, and its shared memory
 __host__ __device__ constexpr int score_stages(int RWb) { return RWb == 1 ? 6 : 4; }
 __host__ __device__ constexpr size_t score_smem(int RWb) {
-  return (size_t)score_stages(RWb) * kTileBytes + (size_t)RWb * 2 * kBoxBytes + 256 * 4 + 256 + (RWb - 1) * 2 * 128 * 4;
+  return (size_t)score_stages(RWb) * kTileBytes + (size_t)RWb * 2 * kBoxBytes + 256 * 4 + kHot * 4 +
+         (RWb - 1) * 2 * 128 * 4;
 }
 // stats_tc's K/V stages: shared memory holds a third beside one block of window rows
 __host__ __device__ constexpr int stats_stages(int RWb) { return RWb == 1 ? 3 : 2; }
@@ -166,6 +168,20 @@ __device__ __forceinline__ bool is_protected(int t, int T, int W, int sink, int 
 __device__ __forceinline__ uint32_t score_key(float s) { return max(1u, float_key(s)); }
 __device__ __forceinline__ int key_bin(uint32_t key) {
   return (key & 0x80000000u) ? static_cast<int>((key >> 20) & (kBins - 1)) : 0;
+}
+
+// A CTA's counts of its scores' bins, one addition to the table in global memory
+// per bin and CTA: 31 octaves from 2^-20 up and bin 0 (zeros).  Others, rare or
+// far apart, are counted there at once.  (All of a unit's scores lie in a few
+// tens of bins: counting each in global memory, 1M positions of 2 units took
+// scores_tc 185 us where the pass alone takes 90.)
+__device__ __forceinline__ void count_bin(int bin, uint32_t* s_hot, uint32_t* table) {
+  const unsigned i = bin == 0 ? kHot - 1u : static_cast<unsigned>(bin - kHotLo);
+  atomicAdd(i < kHot - (bin != 0) ? s_hot + i : table + bin, 1u);
+}
+__device__ __forceinline__ void flush_bins(const uint32_t* s_hot, uint32_t* table) {
+  for (int i = threadIdx.x; i < kHot; i += blockDim.x)
+    if (s_hot[i] != 0u) atomicAdd(table + (i == kHot - 1 ? 0 : kHotLo + i), s_hot[i]);
 }
 
 // The keys of one bin in second-level bins, in order: eleven of the 20 bits
@@ -612,8 +628,9 @@ __global__ void __launch_bounds__(kScoreThreads, 1)
   uint8_t* sK = sm;                            // [kS][128 x 128]
   uint8_t* sQ = sm + (size_t)kS * kTileBytes;  // [2 boxes][RWb*128][128 B]
   float* s_b = reinterpret_cast<float*>(sQ + (size_t)RWb * 2 * kBoxBytes);  // [256] log2(1 / l_r) - m_r (-inf: padding)
-  uint8_t* s_wi = reinterpret_cast<uint8_t*>(s_b + 256);                    // [256] window index of row r (r mod W)
-  float(*s_part)[128] = reinterpret_cast<float(*)[128]>(s_wi + 256);        // [2] the upper rows' sums (RWb = 2)
+  uint32_t* s_hot = reinterpret_cast<uint32_t*>(s_b + 256);                 // [kHot] counts of the scores' bins
+  float(*s_part)[128] = reinterpret_cast<float(*)[128]>(s_hot + kHot);      // [2] the upper rows' sums (RWb = 2)
+  __shared__ uint8_t s_wi[256];                                             // window index of row r (r mod W)
   __shared__ __align__(8) uint64_t full[kMaxS], empty[kMaxS], lfull[4], lempty[4], pfull[2], qfull, mma_done;
   __shared__ uint32_t tmem_base;
   __shared__ int abort_flag, s_issued;
@@ -717,6 +734,7 @@ __global__ void __launch_bounds__(kScoreThreads, 1)
       s_b[r] = (Lsum > 0.f) ? -log2f(Lsum) - M : -INFINITY;
       s_wi[r] = static_cast<uint8_t>(r % p.W);
     }
+    for (int i = tid - 64; i < kHot; i += 512) s_hot[i] = 0u;
     named_sync(1, 512);
     const int t_safe = p.causal ? p.T - p.W : 0x7fffffff;  // tokens every window row sees
     const float* sb = s_b + half * 128;
@@ -769,7 +787,7 @@ __global__ void __launch_bounds__(kScoreThreads, 1)
       if (t < t_end) {
         p.s_out[(size_t)u * p.T + t] = acc;
         if (!is_protected(t, p.T, p.W, p.sink, p.keep_window))
-          atomicAdd(p.hist + (size_t)u * kBins + key_bin(score_key(acc)), 1u);
+          count_bin(key_bin(score_key(acc)), s_hot, p.hist + (size_t)u * kBins);
         if (p.diag) p.diag[(size_t)u * p.T + t] = acc;
       }
     }
@@ -778,6 +796,7 @@ __global__ void __launch_bounds__(kScoreThreads, 1)
   __syncthreads();
   // the MMA thread's final commit, and after an abort the copies in flight
   if (tid == 0) drain_after_abort(full, kS, abort_flag ? s_issued : 0, abort_flag ? &qfull : nullptr, &mma_done);
+  flush_bins(s_hot, p.hist + (size_t)u * kBins);
   __syncthreads();
   if (warp == 1) {
     tc_fence_after();
@@ -808,8 +827,7 @@ constexpr float kBoundSlack = 1e-5f;
 __global__ void __launch_bounds__(kResThreads, 1)
     residual_tc(const TcArgs p, const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtensorMap tmV) {
   constexpr int kS = 2;  // tile i is in stage and TMEM buffer i % 2
-  extern __shared__ __align__(1024) uint8_t smraw[];
-  uint8_t* sm = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smraw) + 1023) & ~uintptr_t(1023));
+  extern __shared__ __align__(1024) uint8_t sm[];  // a multiple of 1024 bytes from the block's base
   uint8_t* sK = sm;                        // [kS][128 x 128]
   uint8_t* sV = sm + kS * kTileBytes;      // [kS][128 x 128]
   uint8_t* sC = sm + 2 * kS * kTileBytes;  // [3 parts][128 x 128]: C0' = hi + mid + lo
@@ -820,6 +838,7 @@ __global__ void __launch_bounds__(kResThreads, 1)
   __shared__ float s_mv[kDP];
   __shared__ float s_mvn[kMaxHs], s_fro[kMaxHs];  // per head of the selection group: ||mu_v0||, scale ||C0'||_F
   __shared__ int s_sel[kMaxHs];                   // and the positions its first selection holds
+  __shared__ uint32_t s_hot[kHot];                // counts of the scores' bins
 
   const int chunk = blockIdx.x, u = blockIdx.y;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -876,6 +895,7 @@ __global__ void __launch_bounds__(kResThreads, 1)
       bulk_g2s(sC + part * kTileBytes, p.cimg + ((size_t)u * 3 + part) * kTileBytes, part_bytes, &cfull);
   }
   if (tid < kDP) s_mv[tid] = p.mv0[(size_t)u * kDP + tid];
+  for (int i = tid; i < kHot; i += kResThreads) s_hot[i] = 0u;
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
@@ -1071,7 +1091,7 @@ __global__ void __launch_bounds__(kResThreads, 1)
         const bool prot = is_protected(t, p.T, p.W, p.sink, p.keep_window);
         const float v = prot ? 0.f : p.s_in[(size_t)u * p.T + t] * sqrtf(ss);
         p.s_out[(size_t)u * p.T + t] = v;
-        if (!prot) atomicAdd(p.hist + (size_t)u * kBins + key_bin(score_key(v)), 1u);
+        if (!prot) count_bin(key_bin(score_key(v)), s_hot, p.hist + (size_t)u * kBins);
         if (p.diag) p.diag[(size_t)u * p.T + t] = v;
       }
     }
@@ -1080,6 +1100,7 @@ __global__ void __launch_bounds__(kResThreads, 1)
   __syncthreads();
   // the MMA thread's final commit, and after an abort the copies in flight
   if (tid == 0) drain_after_abort(full, kS, abort_flag ? s_issued : 0, &cfull, &mma_done);
+  flush_bins(s_hot, p.hist + (size_t)u * kBins);
   __syncthreads();
   if (warp == 1) {
     tc_fence_after();
@@ -1950,7 +1971,7 @@ __global__ void __launch_bounds__(256) keep_all_kernel(const CompressArgs a, int
 }
 
 // ------------------------------------------------------------------- host
-constexpr size_t kResidualSmem = 1024 + 2 * 2 * kTileBytes + 3 * kTileBytes;
+constexpr size_t kResidualSmem = 2 * 2 * kTileBytes + 3 * kTileBytes;
 
 // residual_tc compares scores and norms before it reads rows when its CTAs
 // have at least this many tiles; below, the full pass takes no longer.

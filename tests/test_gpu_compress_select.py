@@ -167,6 +167,8 @@ def test_pruning_bound_of_rounding_size():
     ("equal", 64, 700, 40, 1, 1),          # the last selected pair in one of the later heads
     ("zero", 2, 30000, 700, 0, 1),         # fewer scores above zero than selections
     ("zero", 8, 9000, 300, 1, 1),
+    ("tail", 2, 30000, 700, 0, 1),         # the threshold far below the bins a CTA counts on its own
+    ("tail", 8, 9000, 300, 1, 1),
 ])
 def test_more_contested_keys_than_the_lists_hold(kind, H, T, B, adaptive, pool):
     """Selections whose threshold bin holds more keys than the exchanged lists,
@@ -183,6 +185,12 @@ def test_more_contested_keys_than_the_lists_hold(kind, H, T, B, adaptive, pool):
     elif kind == "zero":  # 400 keys hold all the weight
         K[:, :, 400:] = -40.0 * Q[:, :, 0, :1]
         Q[:] = Q[:, :, :, :1]
+    elif kind == "tail":  # 100 keys hold all the weight, the others from e^-18 of theirs down to e^-28
+        Q[:] = Q[:, :, :, :1]
+        logit = -18.0 - 10.0 * torch.rand(1, H, T, 1, generator=gen, device="cuda")
+        logit[:, :, :100] = 0.0
+        q0 = Q[:, :, 0, :1]
+        K = logit * D ** 0.5 * q0 / (q0 * q0).sum(-1, keepdim=True)
     K, V, Q = (x.to(torch.bfloat16) for x in (K, V, Q))
     out = compress(1, H, G, D, T, B, w, K, V, Q, adaptive, True, pool=pool, mi=0)
     t = np.arange(T)
@@ -190,6 +198,8 @@ def test_more_contested_keys_than_the_lists_hold(kind, H, T, B, adaptive, pool):
     s = out["s"][0].double().cpu().numpy()
     if kind == "zero":
         assert (s[:, 500:T - w] == 0).all()
+    elif kind == "tail":
+        assert (s[:, 200:T - w] < 2.0 ** -21).all() and (s > 0).all()
     k = B - int(prot.sum())
     if adaptive:
         want, _ = O.select_topk_joint(s, H * k, np.stack([prot] * H))
