@@ -123,13 +123,19 @@ def lib():
 # Addresses go to ctypes as plain integers, and the current stream's handle
 # comes from torch without a Stream object around it: the marshalling of a
 # decode step took 8 of its 12 us on the host, most of it in those wrappers.
+# (A private function of torch: without it, the public one and its object.)
+_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+
+
 def _ptr(t):
     return None if t is None else t.data_ptr()
 
 
 def _stream(stream):
     if stream is None:
-        return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device())
+        if _raw_stream is None:
+            return torch.cuda.current_stream().cuda_stream
+        return _raw_stream(torch.cuda.current_device())
     return stream.cuda_stream
 
 

@@ -238,3 +238,15 @@ def test_evict_validation(L):
     assert run(tau=float("nan")) == 1
     assert run(wsb=8) == 7
     assert run(g=mkv.geom(1, 2, 5, 64)) == 2
+
+
+def test_current_stream_without_torchs_private_function(monkeypatch):
+    """A torch that lacks the raw-handle function still gives the current stream."""
+    import torch
+
+    class Stream:
+        cuda_stream = 1234
+
+    monkeypatch.setattr(mkv, "_raw_stream", None)
+    monkeypatch.setattr(torch.cuda, "current_stream", lambda *a: Stream())
+    assert mkv._stream(None) == 1234 and mkv._stream(Stream()) == 1234
