@@ -6,7 +6,7 @@ gap exceeds GAP_EXACT (relative).  Below that gap either side of the
 boundary is a correct answer, so these helpers check what is unique and
 that the rest is valid:
   - compress: each selection is replayed on the kernel's own fp32 scores
-    (the radix select must return exactly the top k of the values it
+    (the selection must return exactly the top k of the values it
     ranked, lower position first on ties); where the oracle's gap exceeds
     GAP_EXACT it must also equal the oracle's set; otherwise the oracle
     continues from the kernel's choice (score2 under the kernel's stage-1

@@ -6,8 +6,8 @@ gathered cache, and the evicted-set moments (1e-4 relative).  Includes the tiny 
 mi off, T <= budget, 256 window rows, and the full Llama-3.1-8B one-layer
 workload (T=8192, B=512, w=32); then the same with the budget shared by the
 KV heads of a batch item (adaptive=1, Ada-KV allocation of Sec. 5.1) against
-oracle.compress_adaptive, including a head count and prompt length whose
-joint selection lists exceed the select kernel's shared-memory key cache."""
+oracle.compress_adaptive, including a budget at which the threshold bin of the
+joint selection holds more pairs than a group's list of them."""
 import numpy as np
 import pytest
 import torch
@@ -235,8 +235,8 @@ def test_adaptive_budget_covers_prompt():
 
 
 def test_adaptive_uncached_select_keys():
-    # 8 heads x 60000 positions and a budget that leaves no per-head prefilter:
-    # each select CTA's range of the joint list exceeds its shared-memory key cache
+    # 8 heads x 60000 positions, 32000 of them kept: more contested pairs than a
+    # group's list holds
     wl = Workload("a-long", Geometry(1, 8, 1, 64), 60000, 4000, 16, "logscale")
     run_adaptive(wl, seed=14)
 

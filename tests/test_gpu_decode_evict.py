@@ -119,7 +119,7 @@ def test_evict_to_empty_cache_gives_moment_term():
 
 
 def test_large_cache_eviction_kernel():
-    """Capacity 1300 (> 8 x 144 rows): the shared-memory cluster eviction kernel."""
+    """Capacity 1300 (above the register kernel's 1152 rows)."""
     rng = np.random.default_rng(35)
     st = setup(rng, 1, 2, 2, 128, [1200, 1100], 1300, [500, 0])
     run_steps(st, 1, 2, 2, 128, 1150, steps=2, seed=6)
@@ -151,9 +151,11 @@ def test_eviction_state_several_evictions_per_step_d64():
 @pytest.mark.parametrize("b,H,G,D,budget,cap", [
     (1, 2, 2, 64, 1, 4),         # one row per CTA, most of the cluster idle
     (1, 2, 8, 64, 8, 12),        # the appended row alone in its slice
-    (1, 2, 4, 128, 1151, 1152),  # the largest capacity, 16 rows per warp
+    (1, 2, 4, 128, 1151, 1152),  # the largest capacity, 9 rows per warp
     (3, 20, 2, 64, 90, 96),      # smaller clusters: more rows of S_tilde per CTA
     (5, 16, 1, 128, 60, 64),
+    (3, 8, 4, 128, 699, 700),    # four CTAs, 16 rows per warp
+    (8, 8, 1, 64, 399, 400),     # the same with two
 ])
 def test_appended_row_alone_without_y(b, H, G, D, budget, cap):
     """From the second step on only the appended row has no kept y: its

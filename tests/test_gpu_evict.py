@@ -130,8 +130,7 @@ def test_evict_clamp_paths(tau):
 
 
 def test_evict_large_capacity_fallback():
-    """A capacity whose row slices do not fit in shared memory runs the
-    single-CTA kernel; results are the same."""
+    """A capacity past the register kernel's, one unit: 16 CTAs share its rows."""
     rng = np.random.default_rng(32)
     st = setup(rng, 1, 1, 4, 128, [2300], 2400, [500])
     gpu = run_case(st, 1, 1, 4, 128, 2260, False)
@@ -147,8 +146,8 @@ def test_evict_budget_zero_and_batch():
 
 @pytest.mark.parametrize("cap", [1000, 1200])
 def test_evict_slice_sizes(cap):
-    """Row slices of 125 rows (register-resident kernel, 9 rows per warp) and
-    150 rows (shared-memory cluster kernel): 30 evictions each."""
+    """1000 rows (register kernel, slices of 125 rows, 9 per warp) and 1200 (the
+    kernel for larger caches): 30 evictions each."""
     rng = np.random.default_rng(34 + cap)
     st = setup(rng, 1, 2, 4, 128, [cap - 11, cap - 20], cap, [300, 0])
     gpu = run_case(st, 1, 2, 4, 128, cap - 41, True)
@@ -189,11 +188,26 @@ def test_evict_small_slices(G, D, cap, tau):
 
 
 def test_evict_many_units():
-    """24 units at capacity 200: three waves of 8-CTA clusters of the register
-    kernel (5 rows per warp)."""
+    """24 units at capacity 200: more than one wave of 8-CTA clusters, so four
+    CTAs of 50 rows."""
     rng = np.random.default_rng(27)
     st = setup(rng, 3, 8, 2, 128, [190] * 24, 200, [400, 0] * 12)
     gpu = run_case(st, 3, 8, 2, 128, 140, True)
+    check(gpu, st)
+
+
+@pytest.mark.parametrize("units,G,D,cap,tau", [
+    (24, 4, 128, 700, 1e-6),   # clusters of four CTAs, slices of 175 rows: 16 per warp
+    (24, 1, 64, 1024, 0.05),   # the largest slice (256 rows), clamped entries
+    (64, 2, 128, 500, 1e-6),   # clusters of two CTAs, slices of 250 rows
+    (64, 8, 64, 290, 1e-6),
+])
+def test_evict_16_rows_per_warp(units, G, D, cap, tau):
+    """Enough units that clusters of eight CTAs would take several waves."""
+    rng = np.random.default_rng(91 + cap)
+    lens = [cap - 1 - 3 * (i % 4) for i in range(units)]
+    st = setup(rng, units // 8, 8, G, D, lens, cap, [0 if i == 1 else 300 for i in range(units)])
+    gpu = run_case(st, units // 8, 8, G, D, cap - 12, True, tau=tau)
     check(gpu, st)
 
 
@@ -257,7 +271,7 @@ def test_eviction_state_reset_by_compress_and_large_capacity():
     mkv.mkv_compress(g, wl.T, bf16(K), bf16(V), bf16(Q), p, cache, mkv.alloc_moments(g), ws)
     assert mkv.mkv_get_device_error(ws)[0] == 0
     assert (host(cache.y_len) == 0).all()
-    # capacity 2400 runs the single-CTA kernel: y_len goes to 0 after its evictions
+    # capacity 2400 runs the kernel for larger caches: y_len goes to 0 after its evictions
     rng = np.random.default_rng(32)
     st = setup(rng, 1, 1, 4, 128, [2300], 2400, [500])
     g = mkv.geom(1, 1, 4, 128)

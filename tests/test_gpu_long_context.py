@@ -9,7 +9,7 @@ recomputes a sampled unit (or batch item) from its own prompt slice.
 
 What is compared:
   - window scores and score2 within tolerance;
-  - each selection replayed on the kernel's own fp32 scores: the radix select
+  - each selection replayed on the kernel's own fp32 scores: the selection
     must return exactly the top k of the values it ranked, lower position
     first on ties;
   - the selection equal to the oracle's wherever the oracle's boundary gap
