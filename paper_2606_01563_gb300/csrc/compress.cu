@@ -1652,6 +1652,14 @@ struct RsetArgs {
   int several;  // a CTA may have more than one row tile
 };
 
+// x0 + (s - r) / n, the roundings of the difference and the quotient put back:
+// where the means are near zero they weigh as x0 (a chunk's mean) does.
+__device__ __forceinline__ float mean_about(float x0, float s, float r, float n, float inv) {  // inv = 1 / n
+  const float t = s - r, b = t - s, err = (s - (t - b)) - (r + b);
+  const float q = t * inv;
+  return (x0 + q) + (fmaf(-q, n, t) + err) * inv;
+}
+
 template <int CL, bool FINAL>
 __global__ void __launch_bounds__(2048 / CL, CL == 2 ? 1 : 2) rset_kernel(const RsetArgs a) {
   constexpr int kThr = 2048 / CL;
@@ -1886,16 +1894,17 @@ __global__ void __launch_bounds__(2048 / CL, CL == 2 ? 1 : 2) rset_kernel(const 
   }
   const float nE = n - nR;
   // means of R and E about x0
-  const float dvR = nR > 0.f ? rv / nR : 0.f, dvE = nE > 0.f ? (sv - rv) / nE : 0.f;
-  const float mvE = nE > 0.f ? x0v + dvE : 0.f;
+  const float invE = nE > 0.f ? 1.f / nE : 0.f;
+  const float dvR = nR > 0.f ? rv / nR : 0.f, dvE = (sv - rv) * invE;
+  const float mvE = nE > 0.f ? mean_about(x0v, sv, rv, nE, invE) : 0.f;
   float CE[4], mkE[4];
 #pragma unroll
   for (int j = 0; j < 4; ++j) {
     const float dkR = nR > 0.f ? rk[j] / nR : 0.f;
     CE[j] = mkE[j] = 0.f;
     if (nE > 0.f) {
-      const float dkE = (sk[j] - rk[j]) / nE;
-      mkE[j] = x0k[j] + dkE;
+      const float dkE = (sk[j] - rk[j]) * invE;
+      mkE[j] = mean_about(x0k[j], sk[j], rk[j], nE, invE);
       const float Mall = M[j] - sv * sk[j] / n;
       const float MR = nR > 0.f ? SR[j] - rv * rk[j] / nR : 0.f;
       const float ME = Mall - MR - (nE * nR / n) * (dvR - dvE) * (dkR - dkE);

@@ -177,6 +177,31 @@ def test_retained_set_clusters(b, H, D, T, B):
     run(Workload("rset", Geometry(b, H, 1, D), T, B, 16, "logscale"), seed=B)
 
 
+def test_means_near_zero():
+    """Means far below the spread of the rows, so that a chunk's mean, about
+    which sums are taken, is larger than the result: over twelve prompts they
+    are as near 64 bits as with R's uncentred sums taken out of the all-token
+    ones (9.1e-8 and 9.5e-8 of their norm), and a tenth more at most."""
+    wl = WORKLOADS["tiny_d64_t1k"]
+    G_, T, B = wl.geom, wl.T, wl.budget
+    g = mkv.geom(G_.batch, G_.n_kv_heads, G_.group, G_.head_dim)
+    p = mkv.mkv_compress_params(B, wl.window, 1, 1, 1, 1, 1, 1e-6)
+    cache, mom = mkv.alloc_cache(g, B), mkv.alloc_moments(g)
+    ws = mkv.alloc_workspace(mkv.mkv_compress_workspace_size(g, T, p))
+    err, ref = np.zeros(2), np.zeros(2)
+    for seed in range(12):
+        K, V, Q = Generator(wl, seed=seed).prefill()
+        mkv.mkv_compress(g, T, bf16(K), bf16(V), bf16(Q), p, cache, mom, ws)
+        for h in range(G_.n_kv_heads):
+            m = evicted_moments(K[0, h], V[0, h], host(cache.pos)[0, h, :B])
+            for i, (x, y) in enumerate(((host(mom.mu_k)[0, h], m.mu_k), (host(mom.mu_v)[0, h], m.mu_v))):
+                err[i] += np.sum((x - y) ** 2)
+                ref[i] += np.sum(y ** 2)
+    rel = np.sqrt(err / ref)
+    print(f"mu_k {rel[0]:.3e} mu_v {rel[1]:.3e}")
+    assert rel[0] <= 1.0e-7 and rel[1] <= 1.05e-7, rel
+
+
 # ------------------------------------------------------- adaptive budget
 def run_adaptive(wl, T=None, pool=1, mi=1, tau=1e-6, seed=0, cap_extra=0):
     """mkv_compress with adaptive=1 against oracle.compress_adaptive, per batch
