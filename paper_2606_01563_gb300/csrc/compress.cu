@@ -9,8 +9,9 @@
 //   scores_tc (chunk, unit)  logits again (token-major) -> s_t = sum over rows
 //                            of exp(l - m_row) / l_row, pooled
 //   select    (8-CTA cluster per unit) R0 = protected + top-k(s): the bin of the
-//                            k-th key from counts the score kernels keep, the
-//                            bin's keys ranked, ties to the lower position
+//                            k-th key from counts the score kernels keep, then
+//                            the k-th among the bin's keys, ties to the lower
+//                            position
 //   rset      (cluster, unit) M0 = moments(all) - moments(R0): the chunk records
 //                            merged, R0's rows gathered and their co-moment
 //                            removed; C0' written as three bf16 operand parts
@@ -29,7 +30,7 @@
 // The tensor-core kernels are warp-specialised: warp 0 issues the TMA copies
 // (3-D tensor maps over per-unit slabs: rows past a unit's end read as zeros),
 // warp 1 owns TMEM and issues tcgen05.mma, and the other warps run the
-// epilogue (two groups of four in stats_tc, scores_tc and residual_tc);
+// epilogue (two groups of four in stats_tc and residual_tc, four in scores_tc);
 // stages hand over through mbarriers whose waits are all bounded.  Head dims
 // below 128 use the same 128-wide MMAs: the missing 64-column box is
 // zero-filled.
@@ -616,8 +617,8 @@ __global__ void __launch_bounds__(kStatThreads, 1)
 // groups (rows 0..127 and the others).  Bounded by the read of K, whose rate
 // follows the bytes in flight (four stages: 4.5 TB/s with no epilogue at all),
 // so shared memory goes to stages; from the chunk's end, where L2 still holds
-// what stats_tc read last.  Alone from a cold L2: 60 us at 32K, 32 units (4.5
-// TB/s); 85 us at 128K with 256 window rows, where the exponentials bound it.
+// what stats_tc read last.  Alone from a cold L2: 62 us at 32K, 32 units (4.4
+// TB/s); 74 us at 128K with 256 window rows, where the exponentials bound it.
 constexpr int kScoreThreads = 64 + 4 * 128;
 __global__ void __launch_bounds__(kScoreThreads, 1)
     scores_tc(const TcArgs p, const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtensorMap tmQ) {
@@ -814,7 +815,7 @@ __global__ void __launch_bounds__(kScoreThreads, 1)
 // that remain (a few times the budget where C0' is small beside the values)
 // and computes score2 of those; the others get 0, which the k higher ones keep
 // out.  Reading K and V a second time is what the full pass costs: alone at
-// 32K, batch 4 (32 units) it takes 143 us, the bounded one 22.  When more than half
+// 32K, batch 4 (32 units) it takes 143 us, the bounded one 23.  When more than half
 // of a CTA's positions remain, or the caller wants score2 itself, the full
 // pass runs; a position's score2 is the same bits either way.
 //
@@ -924,8 +925,8 @@ __global__ void __launch_bounds__(kResThreads, 1)
     __syncthreads();
     // theta: the smallest lower bound over the first stage's free rows (0 where
     // a bound says nothing).  All threads walk the group's lists end to end: a
-    // warp per head waited for the longest list (adaptive, 16 units of 20K: a
-    // call 144.7 us, now 138.6).
+    // warp per head waited for the longest list (adaptive, 16 units of 20K: 6 us
+    // of the call).
     float lowest = INFINITY;
     int total = 0;
     for (int h = 0; h < p.hs; ++h) total += s_sel[h];
@@ -1118,12 +1119,13 @@ __global__ void __launch_bounds__(kResThreads, 1)
 // The kernel that computed the scores has counted their keys into kBins bins
 // (exponent and three mantissa bits), so the bin of the k-th highest is known
 // from one scan.  The keys of that bin (about a sixth of k) are exchanged and
-// ranked by counting, which gives the last selected pair; one more pass counts
+// the last selected pair found among them (list_select); one more pass counts
 // and one writes.  Two cluster barriers, where a radix select over the keys
-// took four passes of three barriers each: alone at 32K, 32 units, 13.5 us
-// against 24.5 (with the rows' gather, now rset's), at 128K 20 against 35.  A unit's contested keys are
-// exchanged over its cluster; the pairs of a batch item through global memory
-// (contest_kernel), so that a joint selection too has kSelCL CTAs per unit.
+// took four passes of three barriers each: alone at 32K, 32 units, 14 us
+// against 24.5 (with the rows' gather, now rset's), at 128K 22.6 against 35.
+// A unit's contested keys are exchanged over its cluster; the pairs of a batch
+// item through global memory (contest_kernel lists them), so that a joint
+// selection too has kSelCL CTAs per unit.
 // When there are more contested keys than the lists hold (k above about
 // 12000, or many equal scores), counts of their next eleven bits, taken as they
 // were listed, narrow them down and the scan is repeated; equal keys that
@@ -1614,8 +1616,8 @@ __global__ void __launch_bounds__(256) diag_joint_kernel(const SelectArgs a) {
 // each rank finishing 128 / CL value dims, four elements of C per thread.  A
 // chain of round trips (list, rows, MMA, exchange) over code that runs once:
 // its time is latency and instruction fetch, so the loops stay rolled.  Alone
-// at 32K, 32 units, it takes 25 us, what a second pass of stats_tc over gathered
-// rows (13.5) and a merge kernel (11.5) took before; but its merge runs while
+// at 32K, 32 units, it takes 16 us, where a second pass of stats_tc over
+// gathered rows (13.5) and a merge kernel (11.5) took 25; its merge runs while
 // the selection does, and the gathered copies are gone.
 //
 // The all-token co-moment is the multi-way Chan merge of the chunk records,

@@ -741,8 +741,13 @@ int active_rows(int slice, int cl) {
 }
 
 // Of 8, 4 and 2 CTAs per unit (slices of at most 256 rows) the one that takes
-// the fewest waves, at a tie the larger: an eviction is a chain of barriers
-// whose length hardly depends on the rows of a CTA, a second wave doubles it.
+// the fewest waves, at a tie the larger: a second wave doubles the time, while
+// an eviction's chain of barriers grows by half from 2 to 9 rows per warp and
+// by a third again to 16, whose instances spill at d = 128 (412 to 468 bytes).
+// us of a call with 8 / 4 / 2 CTAs, 64 evictions: 24 units of 192 rows
+// 233/143/185, of 364 rows 284/173/251; 32 units of 764 rows 510/231/-; 40 of
+// 264 rows 425/282/195; 64 of 192 rows 576/284/186, of 464 rows 706/341/250;
+// one eviction with y, 16 and 128 units of 513 rows: 19/12/- and 96/56/-.
 template <int D, int G>
 cudaError_t launch_dg(const EvictArgs& a, cudaStream_t stream) {
   if (a.cap > kRegCap) return launch_evict_large(a, D, G, stream);

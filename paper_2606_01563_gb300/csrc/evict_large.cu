@@ -14,10 +14,10 @@
 // the workspace and the cache, where L2 holds them.
 //
 // What bounds it: per eviction a CTA streams its slice once, 1.5 KB a row, so
-// at 4160 rows (8 units, 260 rows per CTA) the row pass is about 4 us beside
-// the 2 of the serial chain (fold, block barrier, mailboxes, cluster barrier):
-// 64 evictions 434 us, where one CTA per unit that recomputed C' k of every row
-// took 73.5 ms.  The pass
+// at 4160 rows (8 units of 12 CTAs, 347 rows per CTA) the row pass is about 4 us
+// beside the 2 of the serial chain (fold, block barrier, mailboxes, cluster
+// barrier): 64 evictions 430 us, the first of them 55 with the set-up, where one
+// CTA per unit that recomputed C' k of every row took 73.5 ms.  The pass
 // runs over 8 rows a warp at a time with all their loads in flight; the
 // update of y and the residual norm share it.  The set-up products C k_j run
 // on the tensor cores (keys exact in bf16, C split into three bf16 parts).
